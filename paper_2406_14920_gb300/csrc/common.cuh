@@ -211,6 +211,7 @@ struct WorkList {
   int64_t first;           // items [first, total) are processed (0 except in tuning trials)
   int tile;                // consecutive items per worker tile (warp kernels: per warp; thread kernel: per lane)
   int shard, nshard;       // this launch takes the tiles t with t % nshard == shard (work split over GPUs)
+  int mpb, mpk;            // most primitive pairs of a shell pair in the bra and in the ket class
 };
 
 // Boys F_0..F_M at T.  Below BOYS_TMAX: Taylor expansion of F_M around the

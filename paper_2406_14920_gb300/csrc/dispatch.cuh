@@ -3,6 +3,7 @@
 // in parallel.
 #pragma once
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 #include "kernels_g.cuh"
 #include "units.h"
@@ -21,51 +22,76 @@ template <> struct ClassL<7> { static constexpr int l1 = 3, l2 = 1; };
 template <> struct ClassL<8> { static constexpr int l1 = 3, l2 = 2; };
 template <> struct ClassL<9> { static constexpr int l1 = 3, l2 = 3; };
 
-struct LaunchInfo {
-  int grid, block;
-  size_t smem;
-};
-
-template <typename Kern>
-inline cudaError_t launch_persistent(Kern kern, size_t smem, int64_t items, int warps_per_block, int nsm,
-                                     LaunchInfo* info) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// Resident blocks per SM of a kernel with `smem` bytes of dynamic shared memory
+// (raising the kernel's limit first).  Both are constants of the kernel and the
+// device, so they are asked for once per device and kept: the two runtime calls
+// cost about 2 us, and a build of a small molecule is some fifty launches.
+constexpr int kMaxDev = 64;
+template <auto Kern>
+cudaError_t blocks_per_sm(int threads, size_t smem, int* occ) {
+  static std::atomic<int> known[kMaxDev] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * warps_per_block, smem);
-  if (e != cudaSuccess) return e;
-  if (occ < 1) return cudaErrorInvalidConfiguration;
-  int64_t need = (items + warps_per_block - 1) / warps_per_block;
-  int64_t grid = std::min<int64_t>(need, (int64_t)nsm * occ);
-  if (grid < 1) grid = 1;
-  info->grid = (int)grid;
-  info->block = 32 * warps_per_block;
-  info->smem = smem;
+  int n = dev < kMaxDev ? known[dev].load(std::memory_order_acquire) : 0;
+  if (n == 0) {
+    if (smem > 48 * 1024) {
+      e = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, Kern, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (n < 1) return cudaErrorInvalidConfiguration;
+    if (dev < kMaxDev) known[dev].store(n, std::memory_order_release);
+  }
+  *occ = n;
   return cudaSuccess;
+}
+
+// Persistent launch of Kern over `workers` independent work items of `per_block`
+// items per block: as many blocks as the items need, at most those the device holds.
+template <auto Kern, typename Args>
+cudaError_t launch_over(const Args& a, int64_t workers, int per_block, int threads, size_t smem, cudaStream_t s,
+                        int nsm) {
+  int occ = 0;
+  const cudaError_t e = blocks_per_sm<Kern>(threads, smem, &occ);
+  if (e != cudaSuccess) return e;
+  const int64_t grid = std::min<int64_t>((workers + per_block - 1) / per_block, (int64_t)nsm * occ);
+  Kern<<<(int)std::max<int64_t>(1, grid), threads, smem, s>>>(a);
+  cudaError_t r = cudaGetLastError();
+  if (r == cudaErrorInvalidValue && smem > 48 * 1024) {  // the limit was set in a context that cudaDeviceReset ended
+    r = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (r != cudaSuccess) return r;
+    Kern<<<(int)std::max<int64_t>(1, grid), threads, smem, s>>>(a);
+    r = cudaGetLastError();
+  }
+  return r;
+}
+
+// work items of a thread kernel over a list of n items (with the parts of a
+// short list, see prim_split; longer lists fill the grid by themselves)
+template <typename T>
+inline int64_t split_items(const WorkList& wl, int64_t n) {
+  return sizeof(T) == 4 || wl.nshard > 1 ? n : n * wl.mpb * wl.mpk;
 }
 
 template <int LA, int LB, int LC, int LD, typename T>
 cudaError_t launch_jk_t(const JKArgs& a, cudaStream_t s, int nsm) {
-  if (a.k.wl.total <= 0) return cudaSuccess;
-  LaunchInfo li;
+  const int64_t n = a.k.wl.total - a.k.wl.first;
+  if (n <= 0) return cudaSuccess;
   if constexpr (use_thread_kernel(LA, LB, LC, LD, sizeof(T) == 4)) {
-    auto kern = jk_thread_kernel<LA, LB, LC, LD, T>;
-    int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 128, 0);
-    if (e != cudaSuccess) return e;
-    int64_t need = (a.k.wl.total + 127) / 128;
-    int64_t grid = std::min<int64_t>(need, (int64_t)nsm * std::max(occ, 1));
-    kern<<<(int)grid, 128, 0, s>>>(a);
+    return launch_over<jk_thread_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.k.wl, n), 128, 128, 0, s, nsm);
+  } else if constexpr (use_block_kernel<LA, LB, LC, LD, T>()) {
+    using S = CShape<LA, LB, LC, LD, T>;
+    static_assert(S::smem() <= 227 * 1024, "block kernel exceeds 227 KB");
+    return launch_over<jk_block_kernel<LA, LB, LC, LD, T>>(a, n, 1, S::NT, S::smem(), s, nsm);
   } else {
     using S = BShape<LA, LB, LC, LD, T>;
     constexpr int WPB = 4;
-    static_assert(S::table_bytes() + WPB * S::smem_per_warp() <= 227 * 1024, "warp kernel block exceeds 227 KB");
-    auto kern = jk_warp_kernel<LA, LB, LC, LD, T>;
-    cudaError_t e = launch_persistent(kern, S::table_bytes() + WPB * S::smem_per_warp(), a.k.wl.total, WPB, nsm, &li);
-    if (e != cudaSuccess) return e;
-    kern<<<li.grid, li.block, li.smem, s>>>(a);
+    constexpr size_t smem = S::table_bytes() + WPB * S::smem_per_warp();
+    static_assert(smem <= 227 * 1024, "warp kernel block exceeds 227 KB");
+    return launch_over<jk_warp_kernel<LA, LB, LC, LD, T>>(a, n, WPB, 32 * WPB, smem, s, nsm);
   }
-  return cudaGetLastError();
 }
 
 // Launch of class pair (X, y) in precision P for y in YLO..YHI (compile-time
@@ -95,15 +121,14 @@ cudaError_t launch_grad_unit(int y, const GradArgs& a, cudaStream_t s, int nsm) 
       if (a.wl.total <= 0) return cudaSuccess;
       constexpr int LA = ClassL<X>::l1, LB = ClassL<X>::l2, LC = ClassL<Y>::l1, LD = ClassL<Y>::l2;
       using T = std::conditional_t<P == 1, float, double>;
-      using S = GShape<LA, LB, LC, LD, T>;
-      constexpr int WPB = 4;
-      static_assert(S::table_bytes() + WPB * S::smem_per_warp() <= 227 * 1024, "gradient block exceeds 227 KB");
-      LaunchInfo li;
-      auto kern = grad_warp_kernel<LA, LB, LC, LD, T>;
-      cudaError_t e = launch_persistent(kern, S::table_bytes() + WPB * S::smem_per_warp(), a.wl.total, WPB, nsm, &li);
-      if (e != cudaSuccess) return e;
-      kern<<<li.grid, li.block, li.smem, s>>>(a);
-      return cudaGetLastError();
+      const int64_t n = a.wl.total - a.wl.first;
+      if constexpr (use_grad_thread(LA, LB, LC, LD, P == 1)) {
+        return launch_over<grad_thread_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.wl, n), 128, 128, 0, s, nsm);
+      } else {
+        using S = GShape<LA, LB, LC, LD, T>;
+        static_assert(S::smem() <= 227 * 1024, "gradient block exceeds 227 KB");
+        return launch_over<grad_block_kernel<LA, LB, LC, LD, T>>(a, n, 1, S::NT, S::smem(), s, nsm);
+      }
     }
     return launch_grad_unit<X, P, Y + 1>(y, a, s, nsm);
   }
@@ -111,26 +136,15 @@ cudaError_t launch_grad_unit(int y, const GradArgs& a, cudaStream_t s, int nsm) 
 
 template <int LAB, int LCD, typename T>
 cudaError_t launch_j_t(const JArgs& a, cudaStream_t s, int nsm) {
-  if (a.wl.total <= 0) return cudaSuccess;
+  const int64_t n = a.wl.total - a.wl.first;
+  if (n <= 0) return cudaSuccess;
   if constexpr (use_j_thread(LAB, LCD)) {
-    auto kern = j_thread_kernel<LAB, LCD, T>;
-    int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 128, 0);
-    if (e != cudaSuccess) return e;
-    const int64_t need = (a.wl.total + 127) / 128;
-    const int64_t grid = std::min<int64_t>(need, (int64_t)nsm * std::max(occ, 1));
-    kern<<<(int)std::max<int64_t>(1, grid), 128, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_over<j_thread_kernel<LAB, LCD, T>>(a, split_items<T>(a.wl, n), 128, 128, 0, s, nsm);
   } else {
-    using S = JShape<LAB, LCD, T>;
     constexpr int WPB = 4;
-    static_assert(WPB * S::smem_per_warp() <= 227 * 1024, "J-engine block exceeds 227 KB");
-    LaunchInfo li;
-    auto kern = j_warp_kernel<LAB, LCD, T>;
-    cudaError_t e = launch_persistent(kern, WPB * S::smem_per_warp(), a.wl.total, WPB, nsm, &li);
-    if (e != cudaSuccess) return e;
-    kern<<<li.grid, li.block, li.smem, s>>>(a);
-    return cudaGetLastError();
+    constexpr size_t smem = WPB * JShape<LAB, LCD, T>::smem_per_warp();
+    static_assert(smem <= 227 * 1024, "J-engine block exceeds 227 KB");
+    return launch_over<j_warp_kernel<LAB, LCD, T>>(a, n, WPB, 32 * WPB, smem, s, nsm);
   }
 }
 

@@ -154,6 +154,44 @@ struct BraCursor {
   }
 };
 
+// Thread kernels on short lists: an item's primitive quartets are split into n =
+// sb * sk parts (sb ranges of bra primitives times sk of ket primitives), each a
+// work item of its own whose sums are added like any other, so that a contracted
+// (81 primitive quartets) item of a small molecule is not one thread's serial
+// chain.  n is the largest split that still gives every lane of the launch at
+// most one part; lists longer than the launch's lanes are not split (a part
+// repeats the contraction with D).  FP64 only: an FP32 item's sum is taken whole,
+// so that its rounding does not depend on the list it is in.  A split over GPUs
+// keeps whole items.
+struct PrimSplit {
+  int n, sb, sk;
+  __device__ __forceinline__ void range(int part, int npb, int npk, int& b0, int& b1, int& k0, int& k1) const {
+    const int pb = part / sk, pk = part - pb * sk;
+    b0 = npb * pb / sb;
+    b1 = npb * (pb + 1) / sb;
+    k0 = npk * pk / sk;
+    k1 = npk * (pk + 1) / sk;
+  }
+};
+template <typename T>
+__device__ __forceinline__ PrimSplit prim_split(const WorkList& wl, int64_t items, int64_t lanes) {
+  PrimSplit s{1, 1, 1};
+  if (sizeof(T) == 4 || wl.nshard > 1 || items <= 0 || 2 * items > lanes) return s;
+  const int64_t room = lanes / items;
+  s.sb = (int)(room < wl.mpb ? room : wl.mpb);
+  const int64_t rk = room / s.sb;
+  s.sk = (int)(rk < wl.mpk ? rk : wl.mpk);
+  s.n = s.sb * s.sk;
+  return s;
+}
+
+// Items per tile of a block kernel: wl.tile, fewer when that would leave blocks idle
+__device__ __forceinline__ int64_t block_tile(const WorkList& wl, int64_t items) {
+  if (wl.nshard > 1) return wl.tile;
+  const int64_t t = items / (2 * (int64_t)gridDim.x);
+  return t < 1 ? 1 : (t < wl.tile ? t : wl.tile);
+}
+
 template <typename T> __device__ __forceinline__ T ldT(const double* p) { return (T)__ldg(p); }
 
 // precision-explicit reciprocal square root (a plain overload inside this
@@ -370,9 +408,11 @@ __global__ void __launch_bounds__(128) j_thread_kernel(JArgs a) {
   const int64_t span = 32 * (int64_t)a.wl.tile, ntiles = (total - first + span - 1) / span;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   unsigned long long done = 0, doneq = 0, doneb = 0;
+  const PrimSplit sp = prim_split<T>(a.wl, total - first, 32 * nwarps);
   for (int64_t tl = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * nshard + shard;
-       tl < ntiles; tl += nwarps * nshard) {
-    const int64_t t0 = first + tl * span, i1 = t0 + span < total ? t0 + span : total;
+       tl < ntiles * sp.n; tl += nwarps * nshard) {
+    const int part = (int)(tl / ntiles);
+    const int64_t t0 = first + (tl - part * ntiles) * span, i1 = t0 + span < total ? t0 + span : total;
     BraCursor cur;
     if (!compact) cur.seek(a.wl, t0 + lane < i1 ? t0 + lane : t0);
     for (int64_t base = t0; base < i1; base += 32) {  // uniform over the warp
@@ -398,22 +438,26 @@ __global__ void __launch_bounds__(128) j_thread_kernel(JArgs a) {
         npk = __ldg(a.sp.np + pk_id);
         offk = __ldg(a.sp.poff + pk_id);
         hk = __ldg(a.sp.hoff + pk_id);
-        ++done;
-        doneq += (unsigned long long)npb * npk;
-        doneb += npb;
+        if (part == 0) {
+          ++done;
+          doneq += (unsigned long long)npb * npk;
+          doneb += npb;
+        }
       }
       // lane 0's item is always valid here
-      const int pb0 = __shfl_sync(0xffffffffu, pb_id, 0);
-      const bool uni = __all_sync(0xffffffffu, !ok || pb_id == pb0);
-      const int npb_loop = uni ? __shfl_sync(0xffffffffu, npb, 0) : npb;
-      for (int pb = 0; pb < npb_loop; ++pb) {
+      const int pair0 = __shfl_sync(0xffffffffu, pb_id, 0);
+      const bool uni = __all_sync(0xffffffffu, !ok || pb_id == pair0);
+      if (uni) npb = __shfl_sync(0xffffffffu, npb, 0);
+      int pb0, pb1, pk0, pk1;
+      sp.range(part, npb, npk, pb0, pb1, pk0, pk1);
+      for (int pb = pb0; pb < pb1; ++pb) {
         T acc[HAB];
 #pragma unroll
         for (int x = 0; x < HAB; ++x) acc[x] = T(0);
         if (ok) {
           Prim<T> bp;
           bp.load(a.pd, offb + pb);
-          for (int pk = 0; pk < npk; ++pk) {
+          for (int pk = pk0; pk < pk1; ++pk) {
             Prim<T> kp;
             kp.load(a.pd, offk + pk);
             const T ps = bp.p + kp.p;

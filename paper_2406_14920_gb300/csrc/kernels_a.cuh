@@ -6,11 +6,6 @@
 #pragma once
 #include "kernels.cuh"
 
-// 1: the register kernel sums the J_ab contributions of a warp's items over the
-// warp (shuffles) when they share the bra pair, one atomic per element
-#ifndef ERI_JAB_REDUCE
-#define ERI_JAB_REDUCE 0
-#endif
 // FP64 register kernel beyond the tiny classes: largest L and footprint
 // (doubles).  GB300 issues about 3.4 FP64 FMAs per clock per SM, so every warp
 // instruction with idle lanes is expensive; one quartet per lane keeps all 32
@@ -21,7 +16,7 @@
 #define ERI_THREAD64_LMAX 6
 #endif
 #ifndef ERI_THREAD64_FOOT
-#define ERI_THREAD64_FOOT 300
+#define ERI_THREAD64_FOOT 200
 #endif
 
 namespace eri {
@@ -95,18 +90,18 @@ __device__ __forceinline__ T ket_term(const T* ex, const T* ey, const T* ez, con
 // Variant for classes whose W (all ket pairs) does not fit in registers: the
 // bra transform runs per primitive quartet, one ket pair cd at a time.
 template <int LA, int LB, int LC, int LD, typename T>
-__device__ __forceinline__ void eri_block_reg_pq(const KArgs& a, int offb, int npb, int eb0, int offk, int npk, int ek0,
-                                                 T* X) {
+__device__ __forceinline__ void eri_block_reg_pq(const KArgs& a, int offb, int pb0, int pb1, int eb0, int offk, int pk0,
+                                                 int pk1, int ek0, T* X) {
   using S = AShape<LA, LB, LC, LD>;
   constexpr int LAB = S::LAB, LCD = S::LCD, L = S::L;
 #pragma unroll
   for (int x = 0; x < S::NAB * S::NCD; ++x) X[x] = T(0);
-  for (int pb = 0; pb < npb; ++pb) {
+  for (int pb = pb0; pb < pb1; ++pb) {
     Prim<T> bp;
     bp.load(a.pd, offb + pb);
     T eb[3 * S::NEB];
     load_or_build_e<LA, LB, T>(a.pd, eb0 + pb * 3 * S::NEB, bp, eb);
-    for (int pk = 0; pk < npk; ++pk) {
+    for (int pk = pk0; pk < pk1; ++pk) {
       Prim<T> kp;
       kp.load(a.pd, offk + pk);
       T ek[3 * S::NEK];
@@ -152,19 +147,19 @@ __device__ __forceinline__ void eri_block_reg_pq(const KArgs& a, int offb, int n
 }
 
 template <int LA, int LB, int LC, int LD, typename T>
-__device__ __forceinline__ void eri_block_reg(const KArgs& a, int offb, int npb, int eb0, int offk, int npk, int ek0,
-                                              T* X) {
+__device__ __forceinline__ void eri_block_reg(const KArgs& a, int offb, int pb0, int pb1, int eb0, int offk, int pk0,
+                                              int pk1, int ek0, T* X) {
   using S = AShape<LA, LB, LC, LD>;
   constexpr int LAB = S::LAB, LCD = S::LCD, L = S::L;
 #pragma unroll
   for (int x = 0; x < S::NAB * S::NCD; ++x) X[x] = T(0);
-  for (int pb = 0; pb < npb; ++pb) {
+  for (int pb = pb0; pb < pb1; ++pb) {
     Prim<T> bp;
     bp.load(a.pd, offb + pb);
     T W[S::NCD * S::HAB];
 #pragma unroll
     for (int x = 0; x < S::NCD * S::HAB; ++x) W[x] = T(0);
-    for (int pk = 0; pk < npk; ++pk) {
+    for (int pk = pk0; pk < pk1; ++pk) {
       Prim<T> kp;
       kp.load(a.pd, offk + pk);
       T ek[3 * S::NEK];
@@ -219,7 +214,7 @@ __device__ __forceinline__ void eri_block_reg(const KArgs& a, int offb, int npb,
 // transposes are added by the post kernels).
 template <int LA, int LB, int LC, int LD, typename T>
 __device__ __forceinline__ void contract_block(const JKArgs& A, const T* X, T w, int ao1, int ao2, int ao3, int ao4,
-                                               int64_t base, int n, T* jab_out = nullptr) {
+                                               int64_t base, int n) {
   using S = AShape<LA, LB, LC, LD>;
   const T* Dp = dens<T>(A.k) + base;
   double* Kh = A.k.Kh ? A.k.Kh + base : nullptr;
@@ -280,8 +275,7 @@ __device__ __forceinline__ void contract_block(const JKArgs& A, const T* X, T w,
 #pragma unroll
       for (int icd = 0; icd < S::NCD; ++icd)
         s = fma(X[iab * S::NCD + icd], __ldg(Dp + (size_t)(ao3 + icd / S::ND) * n + ao4 + icd % S::ND), s);
-      if (jab_out) jab_out[iab] = w2 * s;  // reduced over the warp by the caller
-      else acc_add(Jh + (size_t)(ao1 + iab / S::NB) * n + ao2 + iab % S::NB, (double)(w2 * s), A.k.det);
+      acc_add(Jh + (size_t)(ao1 + iab / S::NB) * n + ao2 + iab % S::NB, (double)(w2 * s), A.k.det);
     }
 #pragma unroll
     for (int icd = 0; icd < S::NCD; ++icd) {  // Jh_cd += 2w (ab|cd) D_ab
@@ -295,16 +289,10 @@ __device__ __forceinline__ void contract_block(const JKArgs& A, const T* X, T w,
 }
 
 // One quartet (bra position ib, ket position ik of the work list) of a thread-kernel class.
-// Where an item's J_ab contributions go when the caller reduces them over the warp.
-struct JabTarget {
-  int pb_id, ao1, ao2, n;
-  int64_t base;
-};
-
 template <int LA, int LB, int LC, int LD, typename T>
-__device__ __forceinline__ void thread_item(const JKArgs& A, int ib, int ik, unsigned long long& done,
-                                            unsigned long long& doneq, unsigned long long& doneb,
-                                            T* jab_out = nullptr, JabTarget* tgt = nullptr) {
+__device__ __forceinline__ void thread_item(const JKArgs& A, int ib, int ik, const PrimSplit& sp, int part,
+                                            unsigned long long& done, unsigned long long& doneq,
+                                            unsigned long long& doneb) {
   using S = AShape<LA, LB, LC, LD>;
   const KArgs& a = A.k;
   const int pb_id = __ldg(a.wl.bra + ib);
@@ -313,26 +301,29 @@ __device__ __forceinline__ void thread_item(const JKArgs& A, int ib, int ik, uns
   const int s1 = __ldg(a.sp.s1 + pb_id), s2 = __ldg(a.sp.s2 + pb_id);
   const int s3 = __ldg(a.sp.s1 + pk_id), s4 = __ldg(a.sp.s2 + pk_id);
   const int npb_ = __ldg(a.sp.np + pb_id), npk_ = __ldg(a.sp.np + pk_id);
-  ++done;
-  doneq += (unsigned long long)npb_ * npk_;
-  doneb += npb_;
+  if (part == 0) {
+    ++done;
+    doneq += (unsigned long long)npb_ * npk_;
+    doneb += npb_;
+  }
+  int pb0, pb1, pk0, pk1;
+  sp.range(part, npb_, npk_, pb0, pb1, pk0, pk1);
+  if (pb0 >= pb1 || pk0 >= pk1) return;
   T w = T(1);
   if (s1 == s2) w *= T(0.5);
   if (s3 == s4) w *= T(0.5);
   if (pb_id == pk_id) w *= T(0.5);
   T X[S::NAB * S::NCD];
   if constexpr (S::WACC)
-    eri_block_reg<LA, LB, LC, LD, T>(a, __ldg(a.sp.poff + pb_id), npb_, __ldg(a.sp.eoff + pb_id),
-                                     __ldg(a.sp.poff + pk_id), npk_, __ldg(a.sp.eoff + pk_id), X);
+    eri_block_reg<LA, LB, LC, LD, T>(a, __ldg(a.sp.poff + pb_id), pb0, pb1, __ldg(a.sp.eoff + pb_id),
+                                     __ldg(a.sp.poff + pk_id), pk0, pk1, __ldg(a.sp.eoff + pk_id), X);
   else
-    eri_block_reg_pq<LA, LB, LC, LD, T>(a, __ldg(a.sp.poff + pb_id), npb_, __ldg(a.sp.eoff + pb_id),
-                                        __ldg(a.sp.poff + pk_id), npk_, __ldg(a.sp.eoff + pk_id), X);
+    eri_block_reg_pq<LA, LB, LC, LD, T>(a, __ldg(a.sp.poff + pb_id), pb0, pb1, __ldg(a.sp.eoff + pb_id),
+                                        __ldg(a.sp.poff + pk_id), pk0, pk1, __ldg(a.sp.eoff + pk_id), X);
   const int ao1 = __ldg(a.sp.ao1 + pb_id), ao2 = __ldg(a.sp.ao2 + pb_id);
   const int64_t base = __ldg(a.sp.mat_off + mol);
   const int n = __ldg(a.sp.mat_n + mol);
-  if (tgt) *tgt = JabTarget{pb_id, ao1, ao2, n, base};
-  contract_block<LA, LB, LC, LD, T>(A, X, w, ao1, ao2, __ldg(a.sp.ao1 + pk_id), __ldg(a.sp.ao2 + pk_id), base, n,
-                                    jab_out);
+  contract_block<LA, LB, LC, LD, T>(A, X, w, ao1, ao2, __ldg(a.sp.ao1 + pk_id), __ldg(a.sp.ao2 + pk_id), base, n);
 }
 
 template <int LA, int LB, int LC, int LD, typename T>
@@ -348,68 +339,24 @@ __global__ void __launch_bounds__(128) jk_thread_kernel(JKArgs A) {
   // a warp shares a tile of 32 * tile consecutive items, lane l takes items l, l + 32, ...
   const int64_t span = 32 * (int64_t)a.wl.tile, ntiles = (total - first + span - 1) / span;
   const int lane = threadIdx.x & 31;
-  for (int64_t tl = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * nshard + shard; tl < ntiles;
+  const PrimSplit sp = prim_split<T>(a.wl, total - first, stride);
+  for (int64_t tl = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * nshard + shard; tl < ntiles * sp.n;
        tl += (stride >> 5) * nshard) {
-    const int64_t t0 = first + tl * span;
+    const int part = (int)(tl / ntiles);
+    const int64_t t0 = first + (tl - part * ntiles) * span;
     const int64_t i1 = t0 + span < total ? t0 + span : total;
-#if ERI_JAB_REDUCE
-    if (A.Jh && !a.det) {
-      // the list is bra-major: a warp's 32 items usually share the bra pair, so
-      // their J_ab contributions are summed with shuffles (in FP64) and added
-      // once; deterministic builds keep one fixed-point add per item, whose sum
-      // does not depend on how items fall into warps
-      using S = AShape<LA, LB, LC, LD>;
-      BraCursor cur;
-      if (!compact) cur.seek(a.wl, t0 + lane < i1 ? t0 + lane : t0);
-      for (int64_t b0 = t0; b0 < i1; b0 += 32) {  // uniform over the warp; lane 0 always has an item
-        const int64_t item = b0 + lane;
-        const bool ok = item < i1;
-        T jab[S::NAB];
-        JabTarget tg{-1, 0, 0, 0, 0};
-#pragma unroll
-        for (int x = 0; x < S::NAB; ++x) jab[x] = T(0);
-        if (ok) {
-          int ib, ik;
-          if (compact) {
-            const int2 v = __ldg(a.items + item);
-            ib = v.x;
-            ik = v.y;
-          } else {
-            ik = cur.at(a.wl, item);
-            ib = cur.ib;
-          }
-          thread_item<LA, LB, LC, LD, T>(A, ib, ik, done, doneq, doneb, jab, &tg);
-        }
-        const int pb0 = __shfl_sync(0xffffffffu, tg.pb_id, 0);
-        if (__all_sync(0xffffffffu, !ok || tg.pb_id == pb0)) {
-#pragma unroll
-          for (int x = 0; x < S::NAB; ++x) {
-            double v = (double)jab[x];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) atomicAdd(A.Jh + tg.base + (size_t)(tg.ao1 + x / S::NB) * tg.n + tg.ao2 + x % S::NB, v);
-          }
-        } else if (ok) {
-#pragma unroll
-          for (int x = 0; x < S::NAB; ++x)
-            acc_add(A.Jh + tg.base + (size_t)(tg.ao1 + x / S::NB) * tg.n + tg.ao2 + x % S::NB, (double)jab[x], a.det);
-        }
-      }
-      continue;
-    }
-#endif
     const int64_t i0 = t0 + lane;
     if (i0 >= i1) continue;
     if (compact) {
       for (int64_t item = i0; item < i1; item += 32) {
         const int2 v = __ldg(a.items + item);
-        thread_item<LA, LB, LC, LD, T>(A, v.x, v.y, done, doneq, doneb);
+        thread_item<LA, LB, LC, LD, T>(A, v.x, v.y, sp, part, done, doneq, doneb);
       }
     } else {
       BraCursor cur(a.wl, i0);
       for (int64_t item = i0; item < i1; item += 32) {
         const int ik = cur.at(a.wl, item);
-        thread_item<LA, LB, LC, LD, T>(A, cur.ib, ik, done, doneq, doneb);
+        thread_item<LA, LB, LC, LD, T>(A, cur.ib, ik, sp, part, done, doneq, doneb);
       }
     }
   }

@@ -847,6 +847,8 @@ WorkList eri_plan_impl::klist(int X, int Y) const {
   w.prefix = d_kpre + h_koff[X * NPAIRCLASS + Y];
   w.nbra = h_ccount[X];
   w.total = h_ktot[X * NPAIRCLASS + Y];
+  w.mpb = h_maxnp[X];
+  w.mpk = h_maxnp[Y];
   return w;
 }
 
@@ -862,6 +864,8 @@ WorkList eri_plan_impl::jlist(int X, int Y) const {
   w.prefix = d_jpre + h_joff[X * NPAIRCLASS + Y];
   w.nbra = h_ccount[X];
   w.total = h_jtot[X * NPAIRCLASS + Y];
+  w.mpb = h_maxnp[X];
+  w.mpk = h_maxnp[Y];
   return w;
 }
 
@@ -878,13 +882,13 @@ void eri_plan_impl::release() {
   prof_events.clear();
   if (gexec) cudaGraphExecDestroy(gexec);
   gexec = nullptr;
-  for (int b = 0; b < kBranches; ++b) {
+  for (int b = 0; b < kStreams; ++b) {
     if (branch[b]) cudaStreamDestroy(branch[b]);
     if (join_ev[b]) cudaEventDestroy(join_ev[b]);
     branch[b] = nullptr;
     join_ev[b] = nullptr;
   }
-  for (int b = 0; b < kBranches; ++b) {
+  for (int b = 0; b < kStreams; ++b) {
     if (tbuf[b]) cudaFree(tbuf[b]);
     tbuf[b] = nullptr;
   }
@@ -908,11 +912,34 @@ int eri_plan_impl::ensure_streams() {
   if (cap_stream) return ERI_OK;
   CK(cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking));
   CK(cudaEventCreateWithFlags(&fork_ev, cudaEventDisableTiming));
-  for (int b = 0; b < kBranches; ++b) {
+  for (int b = 0; b < kStreams; ++b) {
     CK(cudaStreamCreateWithFlags(&branch[b], cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&join_ev[b], cudaEventDisableTiming));
   }
   return ERI_OK;
+}
+
+int eri_plan_impl::fork(cudaStream_t s, int n) {
+  CK(cudaEventRecord(fork_ev, s));
+  for (int b = 0; b < n; ++b) CK(cudaStreamWaitEvent(branch[b], fork_ev, 0));
+  return ERI_OK;
+}
+
+int eri_plan_impl::join(cudaStream_t s, int n) {
+  for (int b = 0; b < n; ++b) {
+    CK(cudaEventRecord(join_ev[b], branch[b]));
+    CK(cudaStreamWaitEvent(s, join_ev[b], 0));
+  }
+  return ERI_OK;
+}
+
+// Eager calls overlap their class launches (independent sums into the same
+// accumulators) on the plan's side streams: a small molecule's fifty launches
+// hold a few blocks each, and one after another they leave most SMs idle.
+// Profiled calls run in order on the caller's stream, so that an event pair
+// times one launch.
+int eri_plan_impl::eager_branches() const {
+  return opts.profile ? 0 : kStreams;
 }
 
 // Compacted tier lists of mixed-precision builds: per branch, two lists of
@@ -927,14 +954,14 @@ int eri_plan_impl::ensure_tier_bufs(int nb) {
   const int64_t cap = std::min(mx, kTierCap);
   if (cap > tier_cap) {
     CK(cudaDeviceSynchronize());
-    for (int b = 0; b < kBranches; ++b) {
+    for (int b = 0; b < kStreams; ++b) {
       if (tbuf[b]) cudaFree(tbuf[b]);
       tbuf[b] = nullptr;
     }
     tier_nb = 0;
     tier_cap = cap;
   }
-  if (!tcnt) CK(dalloc(&tcnt, 2 * kBranches));
+  if (!tcnt) CK(dalloc(&tcnt, 2 * kStreams));
   for (int b = tier_nb; b < nb; ++b) CK(dalloc(&tbuf[b], 2 * (size_t)tier_cap));
   tier_nb = std::max(tier_nb, nb);
   return ERI_OK;
@@ -1254,6 +1281,7 @@ static int plan_create(int nmol, const eri_basis_t* const* bases, const double* 
         pcls[ip] = pair_class(l[x], l[y]);
         peoff[ip] = (int)std::min<int64_t>(ne_tot, INT32_MAX);
         pmol[ip] = m;
+        P->h_maxnp[pcls[ip]] = std::max(P->h_maxnp[pcls[ip]], pnp[ip]);
         nprimpair += pnp[ip];
         nherm_tot += (int64_t)pnp[ip] * nherm(l[x] + l[y]);
         ne_tot += (int64_t)pnp[ip] * 3 * (l[x] + 1) * (l[y] + 1) * (l[x] + l[y] + 1);
@@ -1307,6 +1335,7 @@ static int plan_create(int nmol, const eri_basis_t* const* bases, const double* 
     CKP(dalloc(&P->d_Dherm, nherm_tot)); CKP(dalloc(&P->d_Jherm, nherm_tot)); CKP(dalloc(&P->d_Dhermf, nherm_tot));
     CKP(dalloc(&P->d_status, 1));
     if (P->alloc_pairs() != ERI_OK) { rc = ERI_ENOMEM; goto fail; }
+    if ((rc = P->ensure_streams()) != ERI_OK) goto fail;  // here: builds allocate and create nothing
     CKP(upload(P->d_sh_l, l)); CKP(upload(P->d_sh_atom, atom)); CKP(upload(P->d_sh_np, np));
     CKP(upload(P->d_sh_po, po)); CKP(upload(P->d_sh_ao, ao)); CKP(upload(P->d_shloc, shloc));
     CKP(upload(P->d_exps, ex)); CKP(upload(P->d_coefs, co)); CKP(upload(P->d_coords, xyz));
@@ -1368,13 +1397,29 @@ extern "C" int eri_plan_set_coords(eri_plan_t* plan, const double* coords_dev, i
   return P->geometry(s, freeze_lists == 0);
 }
 
-// One J/K build on stream s, lists as they stand.  With `concurrent` the class
-// launches are spread over the plan's side streams (fork / join by events) in
-// decreasing order of estimated work; otherwise they run in order on s.
+// Class pairs of a build in launch order, and the side stream each goes to: by
+// decreasing estimated work, to the least-loaded of nbranch streams (nbranch = 0:
+// in class order, on the caller's stream).
+struct ClassLaunch {
+  int X, Y;
+  double cost;
+  int branch;
+};
+static void assign_branches(std::vector<ClassLaunch>& v, int nbranch) {
+  if (nbranch <= 0) return;
+  std::stable_sort(v.begin(), v.end(), [](const ClassLaunch& a, const ClassLaunch& b) { return a.cost > b.cost; });
+  double load[eri_plan_impl::kStreams] = {};
+  for (ClassLaunch& l : v) {
+    l.branch = (int)(std::min_element(load, load + nbranch) - load);
+    load[l.branch] += l.cost;
+  }
+}
+
+// One J/K build on stream s, lists as they stand.  nbranch > 0: the class
+// launches are spread over that many of the plan's side streams (fork / join by
+// events); 0: they run in order on s (profiled builds).
 static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, int precision, cudaStream_t s,
                       int nbranch) {
-  // nbranch = 0: eager build on s (profiling allowed); >= 1: graph capture,
-  // class launches forked onto nbranch branch streams (least-loaded first)
   const bool concurrent = nbranch > 0;
   const int64_t nn = P->nmat;
   const MolMats mm = molmats(P);
@@ -1397,11 +1442,8 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       k_dmax<<<grid1(P->npair, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_sh_l, P->d_pao1, P->d_pao2,
                                                   P->d_pmol, P->d_mat_off, P->d_mat_n, P->d_Dp, P->d_dmax);
       CK(cudaGetLastError());
-      if (!concurrent) {
-        const int rc = P->ensure_tier_bufs(1);
-        if (rc != ERI_OK) return rc;
-      }
-      if (P->tier_nb < (concurrent ? nbranch : 1)) return ERI_EINVAL;
+      const int rc = P->ensure_tier_bufs(std::max(1, nbranch));  // (a graph capture has them already)
+      if (rc != ERI_OK) return rc;
     }
     JArgs ja{};
     ja.pd = P->pairdata(); ja.sp = P->spinfo(); ja.bt = P->boystabs();
@@ -1415,17 +1457,12 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
     ka.Q = P->d_Q; ka.dmax = P->d_dmax; ka.pmaxp = P->d_pmaxp; ka.prefmaxp = P->d_prefmaxp;
     ka.shloc = P->d_shloc; ka.pbase = P->d_pbase;
     ka.tau = (float)P->opts.mixed_tau; ka.pmax32 = (float)kPmax32; ka.mixed = 1;
-    if (concurrent) {
-      CK(cudaEventRecord(P->fork_ev, s));
-      for (int b = 0; b < nbranch; ++b) CK(cudaStreamWaitEvent(P->branch[b], P->fork_ev, 0));
-    }
     // counters2 kinds 0 (J-engine FP64) and 3 (J-engine FP32)
     CK(cudaMemsetAsync(P->d_counters2, 0, sizeof(unsigned long long) * NPAIRCLASS * NPAIRCLASS * 3, s));
     CK(cudaMemsetAsync(P->d_counters2 + 3 * NPAIRCLASS * NPAIRCLASS * 3, 0,
                        sizeof(unsigned long long) * NPAIRCLASS * NPAIRCLASS * 3, s));
     P->last_jmixed = jmixed;
     const bool prof = P->opts.profile && !concurrent;
-    int nl = 0;
     auto jlaunch = [&](int X, int Y, int tier, cudaStream_t ls) -> int {
       const int lab = kClassL1[X] + kClassL2[X], lcd = kClassL1[Y] + kClassL2[Y];
       ja.counter = P->d_counters2 + ((tier ? 3 : 0) * NPAIRCLASS * NPAIRCLASS + X * NPAIRCLASS + Y) * 3;
@@ -1451,11 +1488,20 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       }
       return ERI_OK;
     };
+    std::vector<ClassLaunch> order;
     for (int X = 0; X < NPAIRCLASS; ++X)
       for (int Y = 0; Y < NPAIRCLASS; ++Y) {
+        const int64_t tot = P->h_jtot[X * NPAIRCLASS + Y];
+        if (tot > 0) order.push_back({X, Y, jengine_flops(X, Y, (double)tot * P->h_maxnp[X] * P->h_maxnp[Y]), 0});
+      }
+    assign_branches(order, nbranch);
+    if (concurrent) {
+      const int rc = P->fork(s, nbranch);
+      if (rc != ERI_OK) return rc;
+    }
+    for (const ClassLaunch& l : order) {
+        const int X = l.X, Y = l.Y, b = l.branch;
         const WorkList full = P->jlist(X, Y);
-        if (full.total == 0) continue;
-        const int b = concurrent ? nl++ % nbranch : 0;
         const cudaStream_t ls = concurrent ? P->branch[b] : s;
         if (!jmixed) {
           ja.wl = full;
@@ -1487,12 +1533,11 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
         }
         ja.items = nullptr;
         ja.nitems = nullptr;
-      }
-    if (concurrent)
-      for (int b = 0; b < nbranch; ++b) {
-        CK(cudaEventRecord(P->join_ev[b], P->branch[b]));
-        CK(cudaStreamWaitEvent(s, P->join_ev[b], 0));
-      }
+    }
+    if (concurrent) {
+      const int rc = P->join(s, nbranch);
+      if (rc != ERI_OK) return rc;
+    }
     CK(cudaMemsetAsync(J, 0, sizeof(double) * nn, s));
     k_post_j<<<grid1((int64_t)P->npair * 100, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_pnp, P->d_ppoff,
                                                                  P->d_phoff, P->d_sh_l, P->d_pao1, P->d_pao2,
@@ -1529,25 +1574,22 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
     P->last_mixed = mixed;
     P->last_do_j = J != nullptr;
     P->last_do_k = K != nullptr;
-    // class pairs in decreasing order of estimated work (primitive quartets x class cost)
-    struct L { int X, Y; double cost; };
-    std::vector<L> order;
+    std::vector<ClassLaunch> order;  // cost: primitive quartets x class cost
     for (int X = 0; X < NPAIRCLASS; ++X)
       for (int Y = 0; Y <= X; ++Y) {
         const int64_t tot = P->h_ktot[X * NPAIRCLASS + Y];
         if (tot == 0) continue;
         order.push_back({X, Y, class_flops(X, Y, (double)tot, (double)P->h_kprim[X * NPAIRCLASS + Y], 0.0,
-                                           J != nullptr, K != nullptr)});
+                                           J != nullptr, K != nullptr), 0});
       }
-    if (split && !concurrent) {
-      const int rc = P->ensure_tier_bufs(1);
+    if (split) {
+      const int rc = P->ensure_tier_bufs(std::max(1, nbranch));  // (a graph capture has them already)
       if (rc != ERI_OK) return rc;
     }
-    if (split && P->tier_nb < (concurrent ? nbranch : 1)) return ERI_EINVAL;
+    assign_branches(order, nbranch);
     if (concurrent) {
-      std::stable_sort(order.begin(), order.end(), [](const L& a, const L& b) { return a.cost > b.cost; });
-      CK(cudaEventRecord(P->fork_ev, s));
-      for (int b = 0; b < nbranch; ++b) CK(cudaStreamWaitEvent(P->branch[b], P->fork_ev, 0));
+      const int rc = P->fork(s, nbranch);
+      if (rc != ERI_OK) return rc;
     }
     const bool prof = P->opts.profile && !concurrent;
     auto launch = [&](int X, int Y, int tier, cudaStream_t ls) -> int {
@@ -1566,15 +1608,9 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       }
       return ERI_OK;
     };
-    double load[eri_plan_impl::kBranches] = {};
-    for (const L& l : order) {
-      cudaStream_t ls = s;
-      int b = 0;
-      if (concurrent) {  // least-loaded branch
-        b = (int)(std::min_element(load, load + nbranch) - load);
-        load[b] += l.cost;
-        ls = P->branch[b];
-      }
+    for (const ClassLaunch& l : order) {
+      const int b = l.branch;
+      const cudaStream_t ls = concurrent ? P->branch[b] : s;
       ka.same_class = l.X == l.Y;
       if (!split) {
         ka.wl = P->klist(l.X, l.Y);
@@ -1613,11 +1649,10 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       ka.items = nullptr;
       ka.nitems = nullptr;
     }
-    if (concurrent)
-      for (int b = 0; b < nbranch; ++b) {
-        CK(cudaEventRecord(P->join_ev[b], P->branch[b]));
-        CK(cudaStreamWaitEvent(s, P->join_ev[b], 0));
-      }
+    if (concurrent) {
+      const int rc = P->join(s, nbranch);
+      if (rc != ERI_OK) return rc;
+    }
     P->prof_builds += P->opts.profile ? 1 : 0;
     if (K) {
       k_post_k<<<P->mat_grid(256), 256, 0, s>>>(mm, P->d_Kh, P->d_f, K, ka.det, P->d_status);
@@ -1642,7 +1677,7 @@ extern "C" int eri_build_jk(eri_plan_t* plan, const double* D, double* J, double
     int rc = P->build_lists(thresh, s);
     if (rc != ERI_OK) return rc;
   }
-  return build_impl(P, D, J, K, precision, s, 0);
+  return build_impl(P, D, J, K, precision, s, P->eager_branches());
 }
 
 extern "C" int eri_build_jk_graph(eri_plan_t* plan, const double* D, double* J, double* K, int32_t precision,
@@ -2016,7 +2051,7 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
     k_dmax<<<grid1(P->npair, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_sh_l, P->d_pao1, P->d_pao2,
                                                 P->d_pmol, P->d_mat_off, P->d_mat_n, P->d_Dp, P->d_dmax);
     CK(cudaGetLastError());
-    const int rc = P->ensure_tier_bufs(1);
+    const int rc = P->ensure_tier_bufs(std::max(1, P->eager_branches()));
     if (rc != ERI_OK) return rc;
   }
   GradArgs ga{};
@@ -2036,54 +2071,69 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
   ka.tau = (float)P->opts.mixed_tau; ka.pmax32 = (float)kPmax32; ka.mixed = 1;
   unsigned long long* gcnt = P->d_counters2 + NPAIRCLASS * NPAIRCLASS * 3;  // kinds 1 (FP64) and 2 (FP32)
   CK(cudaMemsetAsync(gcnt, 0, sizeof(unsigned long long) * 2 * NPAIRCLASS * NPAIRCLASS * 3, s));
-  auto launch = [&](int X, int Y, int tier) -> int {
+  auto launch = [&](int X, int Y, int tier, cudaStream_t ls) -> int {
     ga.counter = gcnt + ((tier * NPAIRCLASS + X) * NPAIRCLASS + Y) * 3;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (P->opts.profile) {
       CK(P->prof_event_pair(&e0, &e1));
-      CK(cudaEventRecord(e0, s));
+      CK(cudaEventRecord(e0, ls));
     }
-    CK(launch_grad_class(X, Y, tier, ga, s, P->nsm));
+    CK(launch_grad_class(X, Y, tier, ga, ls, P->nsm));
     if (P->opts.profile) {
-      CK(cudaEventRecord(e1, s));
+      CK(cudaEventRecord(e1, ls));
       P->prof_log.push_back({X, Y, tier ? 4 : 2, P->prof_ev_used - 2});
     }
     return ERI_OK;
   };
+  const int nbranch = P->eager_branches();
+  std::vector<ClassLaunch> order;
   for (int X = 0; X < NPAIRCLASS; ++X)
     for (int Y = 0; Y < NPAIRCLASS; ++Y) {
-      const WorkList full = P->jlist(X, Y);
-      if (full.total == 0) continue;
-      if (!mixed) {
+      const double tot = (double)P->h_jtot[X * NPAIRCLASS + Y], mb = P->h_maxnp[X], mk = P->h_maxnp[Y];
+      if (tot > 0.0) order.push_back({X, Y, grad_flops(X, Y, tot, tot * mb * mk, tot * mb), 0});
+    }
+  assign_branches(order, nbranch);
+  if (nbranch > 0) {
+    const int rc = P->fork(s, nbranch);
+    if (rc != ERI_OK) return rc;
+  }
+  for (const ClassLaunch& l : order) {
+    const WorkList full = P->jlist(l.X, l.Y);
+    const cudaStream_t ls = nbranch > 0 ? P->branch[l.branch] : s;
+    if (!mixed) {
+      ga.wl = full;
+      ga.items = nullptr;
+      ga.nitems = nullptr;
+      const int rc = launch(l.X, l.Y, 0, ls);
+      if (rc != ERI_OK) return rc;
+      continue;
+    }
+    int2* buf = P->tbuf[l.branch];
+    unsigned int* cnt = P->tcnt + 2 * l.branch;
+    for (int64_t f = 0; f < full.total; f += P->tier_cap) {
+      ka.wl = full;
+      ka.wl.first = f;
+      ka.wl.total = std::min<int64_t>(full.total, f + P->tier_cap);
+      CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned int), ls));
+      const int64_t nch = (ka.wl.total - f + 31) / 32;
+      k_tier_split<<<(int)std::max<int64_t>(1, std::min<int64_t>((nch + 7) / 8, (int64_t)P->nsm * 8)), 256, 0, ls>>>(
+          ka, buf, buf + P->tier_cap, cnt);
+      CK(cudaGetLastError());
+      for (int tier = 0; tier < 2; ++tier) {
         ga.wl = full;
-        ga.items = nullptr;
-        ga.nitems = nullptr;
-        const int rc = launch(X, Y, 0);
+        ga.wl.first = 0;
+        ga.wl.total = ka.wl.total - f;  // upper bound of the tier's count (grid sizing)
+        ga.items = buf + (tier ? P->tier_cap : 0);
+        ga.nitems = cnt + tier;
+        const int rc = launch(l.X, l.Y, tier, ls);
         if (rc != ERI_OK) return rc;
-        continue;
-      }
-      int2* buf = P->tbuf[0];
-      unsigned int* cnt = P->tcnt;
-      for (int64_t f = 0; f < full.total; f += P->tier_cap) {
-        ka.wl = full;
-        ka.wl.first = f;
-        ka.wl.total = std::min<int64_t>(full.total, f + P->tier_cap);
-        CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned int), s));
-        const int64_t nch = (ka.wl.total - f + 31) / 32;
-        k_tier_split<<<(int)std::max<int64_t>(1, std::min<int64_t>((nch + 7) / 8, (int64_t)P->nsm * 8)), 256, 0,
-                       s>>>(ka, buf, buf + P->tier_cap, cnt);
-        CK(cudaGetLastError());
-        for (int tier = 0; tier < 2; ++tier) {
-          ga.wl = full;
-          ga.wl.first = 0;
-          ga.wl.total = ka.wl.total - f;  // upper bound of the tier's count (grid sizing)
-          ga.items = buf + (tier ? P->tier_cap : 0);
-          ga.nitems = cnt + tier;
-          const int rc = launch(X, Y, tier);
-          if (rc != ERI_OK) return rc;
-        }
       }
     }
+  }
+  if (nbranch > 0) {
+    const int rc = P->join(s, nbranch);
+    if (rc != ERI_OK) return rc;
+  }
   if (ga.det) {
     k_fix_to_double<<<grid1(3 * P->natom, 128), 128, 0, s>>>(3 * P->natom, dEdR, P->d_status);
     CK(cudaGetLastError());

@@ -46,6 +46,7 @@ struct eri_plan_impl {
   int64_t kpre_cap = 0, jpre_cap = 0;
   int64_t* d_cumnp = nullptr;
   int h_ccount[eri::NPAIRCLASS] = {}, h_coff[eri::NPAIRCLASS] = {};
+  int h_maxnp[eri::NPAIRCLASS] = {};  // most primitive pairs of a shell pair, per class
   int64_t h_koff[eri::NPAIRCLASS * eri::NPAIRCLASS] = {}, h_joff[eri::NPAIRCLASS * eri::NPAIRCLASS] = {};
   int64_t h_ktot[eri::NPAIRCLASS * eri::NPAIRCLASS] = {}, h_jtot[eri::NPAIRCLASS * eri::NPAIRCLASS] = {};
   int64_t h_kprim[eri::NPAIRCLASS * eri::NPAIRCLASS] = {};
@@ -77,16 +78,22 @@ struct eri_plan_impl {
   // the class launches forked onto kBranches side streams so that independent
   // classes overlap (their tails, and small launches, fill idle SMs)
   static constexpr int kBranches = 4;
+  // eager builds and gradients fork their class launches over the same side
+  // streams, kStreams of them, and join them before they return
+  static constexpr int kStreams = 8;
   cudaStream_t cap_stream = nullptr;
-  cudaStream_t branch[kBranches] = {};
-  cudaEvent_t fork_ev = nullptr, join_ev[kBranches] = {};
+  cudaStream_t branch[kStreams] = {};
+  cudaEvent_t fork_ev = nullptr, join_ev[kStreams] = {};
   cudaGraphExec_t gexec = nullptr;
   const void* gkey[3] = {};
   int gprec = -1;
   int gbranches = 0;  // branches of the kept graph (1: serial chain, kBranches: forked)
   int ensure_streams();
+  int fork(cudaStream_t s, int n);  // branch[0 .. n) continue from s
+  int join(cudaStream_t s, int n);  // s continues after branch[0 .. n)
+  int eager_branches() const;       // streams an eager call forks over (0: none, one launch after another on s)
   // compacted tier lists of mixed builds (per branch), see ensure_tier_bufs
-  int2* tbuf[kBranches] = {};
+  int2* tbuf[kStreams] = {};
   unsigned int* tcnt = nullptr;
   int64_t tier_cap = 0;
   int tier_nb = 0;
