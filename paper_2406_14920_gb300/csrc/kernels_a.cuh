@@ -106,9 +106,9 @@ __device__ __forceinline__ void eri_block_reg_pq(const KArgs& a, int offb, int p
       kp.load(a.pd, offk + pk);
       T ek[3 * S::NEK];
       load_or_build_e<LC, LD, T>(a.pd, ek0 + pk * 3 * S::NEK, kp, ek);
-      const T ps = bp.p + kp.p;
-      T rho = bp.p * kp.p / ps;
-      T pref = bp.pref * kp.pref * rsqrt_t(ps);
+      T rho, rs;
+      quartet_rho(bp.p, kp.p, rho, rs);
+      T pref = bp.pref * kp.pref * rs;
       attenuate(om2<T>(a), rho, pref);
       const T PQx = bp.P[0] - kp.P[0], PQy = bp.P[1] - kp.P[1], PQz = bp.P[2] - kp.P[2];
       T F[L + 1];
@@ -164,9 +164,9 @@ __device__ __forceinline__ void eri_block_reg(const KArgs& a, int offb, int pb0,
       kp.load(a.pd, offk + pk);
       T ek[3 * S::NEK];
       load_or_build_e<LC, LD, T>(a.pd, ek0 + pk * 3 * S::NEK, kp, ek);
-      const T ps = bp.p + kp.p;
-      T rho = bp.p * kp.p / ps;
-      T pref = bp.pref * kp.pref * rsqrt_t(ps);
+      T rho, rs;
+      quartet_rho(bp.p, kp.p, rho, rs);
+      T pref = bp.pref * kp.pref * rs;
       attenuate(om2<T>(a), rho, pref);
       const T PQx = bp.P[0] - kp.P[0], PQy = bp.P[1] - kp.P[1], PQz = bp.P[2] - kp.P[2];
       T F[L + 1];

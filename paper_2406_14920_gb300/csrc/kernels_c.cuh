@@ -95,9 +95,9 @@ __device__ __forceinline__ void quartet_scalars(const A& a, int q0, int nq, int 
     const int pb = (q0 + t) / npk, pk = q0 + t - pb * npk;
     const int ib = offb + pb, ik = offk + pk;
     const T bp = pdv<T>(a.pd.p, a.pd.pf, ib), kp = pdv<T>(a.pd.p, a.pd.pf, ik);
-    const T ps = bp + kp;
-    T rho = bp * kp / ps;
-    T pref = pdv<T>(a.pd.pref, a.pd.preff, ib) * pdv<T>(a.pd.pref, a.pd.preff, ik) * rsqrt_t(ps);
+    T rho, rs;
+    quartet_rho(bp, kp, rho, rs);
+    T pref = pdv<T>(a.pd.pref, a.pd.preff, ib) * pdv<T>(a.pd.pref, a.pd.preff, ik) * rs;
     attenuate(om2<T>(a), rho, pref);
     const T X = pdv<T>(a.pd.P, a.pd.Pf, ib) - pdv<T>(a.pd.P, a.pd.Pf, ik);
     const T Y = pdv<T>(a.pd.P, a.pd.Pf, a.pd.n + ib) - pdv<T>(a.pd.P, a.pd.Pf, a.pd.n + ik);

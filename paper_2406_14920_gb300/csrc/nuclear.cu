@@ -305,8 +305,8 @@ extern "C" int eri_nuclear(eri_plan_t* plan, int32_t ncharge, const double* q, c
   NCK(launch_herm<6>(P, ncharge, q, xyz, s));
   const MolMats mm = molmats(P);
   k_post_j<<<(int)(((int64_t)P->npair * 100 + 127) / 128), 128, 0, s>>>(
-      P->npair, P->d_ps1, P->d_ps2, P->d_pnp, P->d_ppoff, P->d_phoff, P->d_sh_l, P->d_pao1, P->d_pao2, P->d_pmol, mm,
-      nullptr, P->pairdata(), P->d_Jherm, P->d_f, V, 0, P->d_status);
+      P->npair, P->d_ps1, P->d_ps2, P->d_pnp, P->d_phoff, P->d_peoff, P->d_sh_l, P->d_pao1, P->d_pao2, P->d_pmol, mm,
+      nullptr, P->d_E, P->d_Jherm, P->d_f, V, 0, P->d_status);
   NCK(cudaGetLastError());
   return ERI_OK;
 }

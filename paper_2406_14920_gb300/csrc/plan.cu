@@ -245,88 +245,224 @@ __global__ void k_etab(int npair, const int* __restrict__ s1, const int* __restr
 }
 
 // Schwarz bound per shell pair: Q = sqrt(max_{mu,nu} |(mu nu|mu nu)|) in FP64, rounded up to float32.
-__global__ void k_schwarz(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
-                          const int* __restrict__ poff, const int* __restrict__ sh_l, const int* __restrict__ ao,
-                          const double* __restrict__ f, PairData pd, BoysTabs bt,
-                          const RStep* __restrict__ st, float* __restrict__ Q) {
-  int ip = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ip >= npair) return;
+// One warp per pair: R of a primitive quartet level by level over the lanes, then
+// a lane per component pair (a thread per pair kept E and R in local memory and
+// took 2 ms for one (ff|ff) diagonal, the longest kernel of a small molecule's
+// geometry step).  The E tables are those of k_etab; primitive quartets (i, j)
+// and (j, i) are equal, so j <= i with weight 2.
+constexpr int kSchwarzWarps = 4;
+constexpr int kSchwarzR = nherm(4 * LMAX);
+__global__ void __launch_bounds__(32 * kSchwarzWarps)
+    k_schwarz(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
+              const int* __restrict__ poff, const int* __restrict__ eoff, const int* __restrict__ sh_l,
+              const int* __restrict__ ao, const double* __restrict__ f, PairData pd, BoysTabs bt,
+              const RStep* __restrict__ st, float* __restrict__ Q) {
+  __shared__ double Rs[kSchwarzWarps][2][kSchwarzR], Fs[kSchwarzWarps][4 * LMAX + 1];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int ip = blockIdx.x * kSchwarzWarps + w;
+  if (ip >= npair) return;  // uniform over the warp; nothing below syncs the block
   const int l1 = sh_l[s1[ip]], l2 = sh_l[s2[ip]], lp = l1 + l2, L = 2 * lp;
-  const int n1 = ncart(l1), n2 = ncart(l2);
-  double diag[100];
-  for (int x = 0; x < n1 * n2; ++x) diag[x] = 0.0;
-  double E1[3][225], E2[3][225], Ra[455], Rb[455], F[13];
+  const int n2 = ncart(l2), nc = ncart(l1) * n2, ne = (l1 + 1) * (l2 + 1) * (lp + 1);
+  double* F = Fs[w];
+  double diag[4] = {0.0, 0.0, 0.0, 0.0};  // component pairs lane + 32 k (at most 100)
   for (int i = 0; i < np[ip]; ++i) {
     const int pi = poff[ip] + i;
-    for (int d = 0; d < 3; ++d) md_e_rt(l1, l2, pd.PA[d * pd.n + pi], pd.PB[d * pd.n + pi], 0.5 / pd.p[pi], E1[d]);
-    for (int j = 0; j < np[ip]; ++j) {
+    for (int j = 0; j <= i; ++j) {
       const int pj = poff[ip] + j;
-      for (int d = 0; d < 3; ++d) md_e_rt(l1, l2, pd.PA[d * pd.n + pj], pd.PB[d * pd.n + pj], 0.5 / pd.p[pj], E2[d]);
       const double p = pd.p[pi], q = pd.p[pj], rho = p * q / (p + q);
-      double X = pd.P[pi] - pd.P[pj], Y = pd.P[pd.n + pi] - pd.P[pd.n + pj], Z = pd.P[2 * pd.n + pi] - pd.P[2 * pd.n + pj];
+      const double X = pd.P[pi] - pd.P[pj], Y = pd.P[pd.n + pi] - pd.P[pd.n + pj],
+                   Z = pd.P[2 * pd.n + pi] - pd.P[2 * pd.n + pj];
       const double T = rho * (X * X + Y * Y + Z * Z);
       // generic Boys (runtime order): Taylor at the top order then downward
+      double fm;
       if (T < BOYS_TMAX) {
-        int k = __double2int_rn(T * BOYS_INV_H);
+        const int k = __double2int_rn(T * BOYS_INV_H);
         const double* c = bt.c64 + ((size_t)k * (BOYS_MMAX + 1) + L) * BOYS_J64;
-        double dd = k * BOYS_H - T, acc = c[BOYS_J64 - 1];
-        for (int jj = BOYS_J64 - 2; jj >= 0; --jj) acc = acc * dd + c[jj];
-        F[L] = acc;
-        double e = exp(-T);
-        for (int m = L - 1; m >= 0; --m) F[m] = (2 * T * F[m + 1] + e) / (2 * m + 1);
-      } else {
-        double e = exp(-T);
-        F[0] = 0.5 * sqrt(3.14159265358979323846 / T);
-        for (int m = 0; m < L; ++m) F[m + 1] = ((2 * m + 1) * F[m] - e) / (2 * T);
-      }
-      const double pref = pd.pref[pi] * pd.pref[pj] / sqrt(p + q);
-      // R into Ra (ping-pong with Rb), result lands in Ra if L even else Rb
-      double* cur = Ra;
-      double* nxt = Rb;
-      cur[0] = pref * F[L];
-      for (int m = L - 1; m >= 0; --m) {
-        int ne = nherm(L - m);
-        for (int e = 0; e < ne; ++e) {
-          if (e == 0) { nxt[0] = pref * F[m]; continue; }
-          RStep s = st[e];
-          double pq = s.dir == 0 ? X : (s.dir == 1 ? Y : Z);
-          double v = pq * cur[s.dep1];
-          if (s.dep2 >= 0) v += s.k * cur[s.dep2];
-          nxt[e] = -2.0 * rho * v;
+        const double dd = k * BOYS_H - T;
+        fm = c[BOYS_J64 - 1];
+        for (int jj = BOYS_J64 - 2; jj >= 0; --jj) fm = fm * dd + c[jj];
+        if (lane == 0) F[L] = fm;
+        const double e = exp(-T);
+        for (int m = L - 1; m >= 0; --m) {
+          fm = (2 * T * fm + e) / (2 * m + 1);
+          if (lane == 0) F[m] = fm;
         }
+      } else {
+        const double e = exp(-T);
+        fm = 0.5 * sqrt(3.14159265358979323846 / T);
+        if (lane == 0) F[0] = fm;
+        for (int m = 0; m < L; ++m) {
+          fm = ((2 * m + 1) * fm - e) / (2 * T);
+          if (lane == 0) F[m + 1] = fm;
+        }
+      }
+      __syncwarp();
+      const double pref = (i == j ? 1.0 : 2.0) * pd.pref[pi] * pd.pref[pj] / sqrt(p + q);
+      double* cur = Rs[w][0];
+      double* nxt = Rs[w][1];
+      if (lane == 0) cur[0] = pref * F[L];
+      __syncwarp();
+      for (int m = L - 1; m >= 0; --m) {
+        const int nr = nherm(L - m);
+        for (int e = lane; e < nr; e += 32) {
+          double v;
+          if (e == 0) {
+            v = pref * F[m];
+          } else {
+            const RStep s = st[e];
+            v = (s.dir == 0 ? X : (s.dir == 1 ? Y : Z)) * cur[s.dep1];
+            if (s.dep2 >= 0) v += s.k * cur[s.dep2];
+            v *= -2.0 * rho;
+          }
+          nxt[e] = v;
+        }
+        __syncwarp();
         double* t = cur; cur = nxt; nxt = t;
       }
-      const double* R = cur;
-      for (int mu = 0; mu < n1; ++mu) {
-        int ix, iy, iz;
-        cart_xyz(l1, mu, ix, iy, iz);
-        for (int nu = 0; nu < n2; ++nu) {
-          int jx, jy, jz;
-          cart_xyz(l2, nu, jx, jy, jz);
-          double v = 0.0;
-          for (int tx = 0; tx <= ix + jx; ++tx)
-            for (int ty = 0; ty <= iy + jy; ++ty)
-              for (int tz = 0; tz <= iz + jz; ++tz) {
-                const double ep = E1[0][(ix * 5 + jx) * 9 + tx] * E1[1][(iy * 5 + jy) * 9 + ty] * E1[2][(iz * 5 + jz) * 9 + tz];
-                for (int sx = 0; sx <= ix + jx; ++sx)
-                  for (int sy = 0; sy <= iy + jy; ++sy)
-                    for (int sz = 0; sz <= iz + jz; ++sz) {
-                      const double eq = E2[0][(ix * 5 + jx) * 9 + sx] * E2[1][(iy * 5 + jy) * 9 + sy] *
-                                        E2[2][(iz * 5 + jz) * 9 + sz];
-                      const double sg = ((sx + sy + sz) & 1) ? -1.0 : 1.0;
-                      v += ep * eq * sg * R[herm_index(tx + sx, ty + sy, tz + sz)];
-                    }
-              }
-          const double fn = f[ao[s1[ip]] + mu] * f[ao[s2[ip]] + nu];
-          diag[mu * n2 + nu] += v * fn * fn;
-        }
+      const double* E1 = pd.E + eoff[ip] + (size_t)i * 3 * ne;
+      const double* E2 = pd.E + eoff[ip] + (size_t)j * 3 * ne;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int c = lane + 32 * k;
+        if (c >= nc) break;
+        int ix, iy, iz, jx, jy, jz;
+        cart_xyz(l1, c / n2, ix, iy, iz);
+        cart_xyz(l2, c % n2, jx, jy, jz);
+        const int ox = (ix * (l2 + 1) + jx) * (lp + 1), oy = ne + (iy * (l2 + 1) + jy) * (lp + 1),
+                  oz = 2 * ne + (iz * (l2 + 1) + jz) * (lp + 1);
+        double v = 0.0;
+        for (int tx = 0; tx <= ix + jx; ++tx)
+          for (int ty = 0; ty <= iy + jy; ++ty)
+            for (int tz = 0; tz <= iz + jz; ++tz) {
+              double u = 0.0;
+              for (int sx = 0; sx <= ix + jx; ++sx)
+                for (int sy = 0; sy <= iy + jy; ++sy) {
+                  double uz = 0.0;
+                  for (int sz = 0; sz <= iz + jz; ++sz)
+                    uz = fma((sx + sy + sz) & 1 ? -E2[oz + sz] : E2[oz + sz],
+                             cur[herm_index(tx + sx, ty + sy, tz + sz)], uz);
+                  u = fma(E2[ox + sx] * E2[oy + sy], uz, u);
+                }
+              v = fma(E1[ox + tx] * E1[oy + ty] * E1[oz + tz], u, v);
+            }
+        diag[k] += v;
       }
+      __syncwarp();
     }
   }
   double mx = 0.0;
-  for (int x = 0; x < n1 * n2; ++x) mx = fmax(mx, fabs(diag[x]));
-  (void)lp;
-  Q[ip] = __double2float_ru(sqrt(mx));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int c = lane + 32 * k;
+    if (c < nc) {
+      const double fn = f[ao[s1[ip]] + c / n2] * f[ao[s2[ip]] + c % n2];
+      mx = fmax(mx, fabs(diag[k] * fn * fn));
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) Q[ip] = __double2float_ru(sqrt(mx));
+}
+
+// Primitive screening.  A contracted pair holds primitive pairs whose prefactor
+// exp(-ab/p |AB|^2) is far below anything a quartet of the lists contributes
+// (tight exponents on two centres).  In the Coulomb metric ||x|| = (x|x)^(1/2)
+// the triangle inequality bounds a primitive pair by its Hermite functions,
+//   q = |pref| (2p)^(-1/4) max_{mu nu} prod_d sum_t |E_t| ((2t-1)!! p^t)^(1/2)
+// (||Lambda_tuv||^2 = (2p)^(-1/2) p^n (2t-1)!! (2u-1)!! (2v-1)!! / (2n+1) in the
+// units of pref), and |(ab|cd)| <= q_ab q_cd for every primitive quartet.
+// k_primpack moves the primitive pairs with q qmax >= kPrimEps thresh to the
+// front of their shell pair and counts them; the J/K, J-engine and gradient
+// kernels run over those.  Each dropped primitive quartet is below 1e-8 of the
+// quartet threshold (thresh = 0 drops none).
+constexpr double kPrimEps = 1e-8;
+__global__ void k_primq(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
+                        const int* __restrict__ poff, const int* __restrict__ eoff, const int* __restrict__ sh_l,
+                        const int* __restrict__ ao, const double* __restrict__ f, const int* __restrict__ pmol,
+                        PairData pd, double* __restrict__ pq, unsigned int* __restrict__ pqmax) {
+  const int ip = blockIdx.x * blockDim.x + threadIdx.x;
+  if (ip >= npair) return;
+  const int a = s1[ip], b = s2[ip], l1 = sh_l[a], l2 = sh_l[b], lp = l1 + l2;
+  const int ne = (l1 + 1) * (l2 + 1) * (lp + 1);
+  double fm = 0.0, fn = 0.0;
+  for (int c = 0; c < ncart(l1); ++c) fm = fmax(fm, f[ao[a] + c]);
+  for (int c = 0; c < ncart(l2); ++c) fn = fmax(fn, f[ao[b] + c]);
+  double top = 0.0;
+  for (int k = 0; k < np[ip]; ++k) {
+    const int pi = poff[ip] + k;
+    const double p = pd.p[pi], rp = sqrt(p);
+    double S[3][(LMAX + 1) * (LMAX + 1)];
+    for (int d = 0; d < 3; ++d)
+      for (int r = 0; r < (l1 + 1) * (l2 + 1); ++r) {
+        const double* E = pd.E + eoff[ip] + ((size_t)k * 3 + d) * ne + (size_t)r * (lp + 1);
+        double w = 1.0, v = 0.0;  // w = (p^t (2t-1)!!)^(1/2)
+        for (int t = 0; t <= lp; ++t) {
+          v += fabs(E[t]) * w;
+          w *= rp * sqrt(2.0 * t + 1.0);
+        }
+        S[d][r] = v;
+      }
+    double mx = 0.0;
+    for (int mu = 0; mu < ncart(l1); ++mu)
+      for (int nu = 0; nu < ncart(l2); ++nu) {
+        int ix, iy, iz, jx, jy, jz;
+        cart_xyz(l1, mu, ix, iy, iz);
+        cart_xyz(l2, nu, jx, jy, jz);
+        mx = fmax(mx, S[0][ix * (l2 + 1) + jx] * S[1][iy * (l2 + 1) + jy] * S[2][iz * (l2 + 1) + jz]);
+      }
+    const double q = fabs(pd.pref[pi]) * rsqrt(sqrt(2.0 * p)) * mx * fm * fn;
+    pq[pi] = q;
+    top = fmax(top, q);
+  }
+  atomicMax(pqmax + pmol[ip], __float_as_uint(__double2float_ru(fmin(top, 1e38))));
+}
+
+template <typename T>
+__device__ __forceinline__ void dswap(T& x, T& y) {
+  const T t = x;
+  x = y;
+  y = t;
+}
+__global__ void k_primpack(int npair, const int* __restrict__ s1, const int* __restrict__ s2,
+                           const int* __restrict__ np, const int* __restrict__ poff, const int* __restrict__ eoff,
+                           const int* __restrict__ sh_l, const int* __restrict__ pmol,
+                           const unsigned int* __restrict__ pqmax, double limit, int n, double* pq, double* p,
+                           double* P, double* PA, double* PB, double* pref, double* ea, float* pf, float* Pf,
+                           float* PAf, float* PBf, float* preff, float4* q4, double* E, float* Ef,
+                           int* __restrict__ nkeep) {
+  const int ip = blockIdx.x * blockDim.x + threadIdx.x;
+  if (ip >= npair) return;
+  const int l1 = sh_l[s1[ip]], l2 = sh_l[s2[ip]], ne3 = 3 * (l1 + 1) * (l2 + 1) * (l1 + l2 + 1);
+  const int o = poff[ip];
+  const double qmax = (double)__uint_as_float(pqmax[pmol[ip]]);
+  int m = 0;
+  for (int k = 0; k < np[ip]; ++k) {
+    if (pq[o + k] * qmax < limit) continue;  // (a NaN bound is kept)
+    if (k != m) {
+      const int x = o + k, y = o + m;
+      dswap(pq[x], pq[y]);
+      dswap(p[x], p[y]);
+      dswap(pref[x], pref[y]);
+      dswap(ea[x], ea[y]);
+      dswap(pf[x], pf[y]);
+      dswap(preff[x], preff[y]);
+      for (int d = 0; d < 3; ++d) {
+        dswap(P[d * n + x], P[d * n + y]);
+        dswap(PA[d * n + x], PA[d * n + y]);
+        dswap(PB[d * n + x], PB[d * n + y]);
+        dswap(Pf[d * n + x], Pf[d * n + y]);
+        dswap(PAf[d * n + x], PAf[d * n + y]);
+        dswap(PBf[d * n + x], PBf[d * n + y]);
+        dswap(q4[3 * (size_t)x + d], q4[3 * (size_t)y + d]);
+      }
+      const size_t ex = (size_t)eoff[ip] + (size_t)k * ne3, ey = (size_t)eoff[ip] + (size_t)m * ne3;
+      for (int e = 0; e < ne3; ++e) {
+        dswap(E[ex + e], E[ey + e]);
+        dswap(Ef[ex + e], Ef[ey + e]);
+      }
+    }
+    ++m;
+  }
+  nkeep[ip] = m;
 }
 
 // Per-molecule Schwarz maximum (pairs never cross molecules).  Q >= 0, so
@@ -521,74 +657,74 @@ __global__ void k_scale_d(MolMats mm, const double* __restrict__ D, const double
 // Hermite density per primitive pair (Eq. j_formula, first sub-step):
 // D_Q = (-1)^|Q| s sum_{l in s1, s in s2} E_Q^{ls} D'_ls, s = 2 for s1 != s2
 // (the pair stands for both orders), 1 for a diagonal pair.
-__global__ void k_hermite_density(int npair, const int* __restrict__ s1, const int* __restrict__ s2,
-                                  const int* __restrict__ np, const int* __restrict__ poff, const int* __restrict__ hoff,
-                                  const int* __restrict__ sh_l, const int* __restrict__ pao1,
-                                  const int* __restrict__ pao2, const int* __restrict__ pmol, MolMats mm,
-                                  const int* __restrict__ sig, PairData pd, const double* __restrict__ Dp,
-                                  double* __restrict__ Dh, float* __restrict__ Dhf) {
-  int ip = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per shell pair, a lane per Hermite index (E is zero outside t <= i + j).
+__global__ void __launch_bounds__(128)
+    k_hermite_density(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
+                      const int* __restrict__ poff, const int* __restrict__ hoff, const int* __restrict__ eoff,
+                      const int* __restrict__ sh_l, const int* __restrict__ pao1, const int* __restrict__ pao2,
+                      const int* __restrict__ pmol, MolMats mm, const int* __restrict__ sig, PairData pd,
+                      const double* __restrict__ Dp, double* __restrict__ Dh, float* __restrict__ Dhf) {
+  const int ip = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (ip >= npair || !sig[ip]) return;
-  const int a = s1[ip], b = s2[ip], la = sh_l[a], lb = sh_l[b], H = nherm(la + lb);
+  const int a = s1[ip], b = s2[ip], la = sh_l[a], lb = sh_l[b], lp = la + lb, H = nherm(lp);
+  const int ne = (la + 1) * (lb + 1) * (lp + 1);
   const int m = pmol[ip], nbf = mm.n[m];
   const double* Dm = Dp + mm.off[m];
   const double sc = a == b ? 1.0 : 2.0;
-  double E[3][225];
   for (int k = 0; k < np[ip]; ++k) {
-    const int pi = poff[ip] + k;
-    for (int d = 0; d < 3; ++d) md_e_rt(la, lb, pd.PA[d * pd.n + pi], pd.PB[d * pd.n + pi], 0.5 / pd.p[pi], E[d]);
-    double* out = Dh + hoff[ip] + (size_t)k * H;
-    for (int q = 0; q < H; ++q) out[q] = 0.0;
-    for (int mu = 0; mu < ncart(la); ++mu) {
-      int ix, iy, iz;
-      cart_xyz(la, mu, ix, iy, iz);
-      for (int nu = 0; nu < ncart(lb); ++nu) {
-        int jx, jy, jz;
-        cart_xyz(lb, nu, jx, jy, jz);
-        const double dv = sc * Dm[(size_t)(pao1[ip] + mu) * nbf + pao2[ip] + nu];
-        for (int tx = 0; tx <= ix + jx; ++tx)
-          for (int ty = 0; ty <= iy + jy; ++ty)
-            for (int tz = 0; tz <= iz + jz; ++tz) {
-              const double sg = ((tx + ty + tz) & 1) ? -1.0 : 1.0;
-              out[herm_index(tx, ty, tz)] +=
-                  sg * dv * E[0][(ix * 5 + jx) * 9 + tx] * E[1][(iy * 5 + jy) * 9 + ty] * E[2][(iz * 5 + jz) * 9 + tz];
-            }
+    const double* E = pd.E + eoff[ip] + (size_t)k * 3 * ne;
+    for (int q = lane; q < H; q += 32) {
+      const int t = herm_t(q), u = herm_u(q), v = herm_v(q);
+      double acc = 0.0;
+      for (int mu = 0; mu < ncart(la); ++mu) {
+        int ix, iy, iz;
+        cart_xyz(la, mu, ix, iy, iz);
+        for (int nu = 0; nu < ncart(lb); ++nu) {
+          int jx, jy, jz;
+          cart_xyz(lb, nu, jx, jy, jz);
+          const double e = E[(ix * (lb + 1) + jx) * (lp + 1) + t] * E[ne + (iy * (lb + 1) + jy) * (lp + 1) + u] *
+                           E[2 * ne + (iz * (lb + 1) + jz) * (lp + 1) + v];
+          acc = fma(Dm[(size_t)(pao1[ip] + mu) * nbf + pao2[ip] + nu], e, acc);
+        }
       }
+      acc *= (t + u + v) & 1 ? -sc : sc;
+      const size_t o = hoff[ip] + (size_t)k * H + q;
+      Dh[o] = acc;
+      if (Dhf) Dhf[o] = (float)acc;  // FP32 copy for the FP32 tier of a mixed J-engine build
     }
-    if (Dhf)  // FP32 copy for the FP32 tier of a mixed J-engine build
-      for (int q = 0; q < H; ++q) Dhf[hoff[ip] + (size_t)k * H + q] = (float)out[q];
   }
 }
 
 // Cartesian J from Hermite J (Eq. j_formula, last sub-step): thread per (pair, mu, nu)
 __global__ void k_post_j(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
-                         const int* __restrict__ poff, const int* __restrict__ hoff, const int* __restrict__ sh_l,
+                         const int* __restrict__ hoff, const int* __restrict__ eoff, const int* __restrict__ sh_l,
                          const int* __restrict__ pao1, const int* __restrict__ pao2, const int* __restrict__ pmol,
-                         MolMats mm, const int* __restrict__ sig, PairData pd, const double* __restrict__ Jh,
-                         const double* __restrict__ f, double* __restrict__ J, int det, int* __restrict__ status) {
+                         MolMats mm, const int* __restrict__ sig, const double* __restrict__ E,
+                         const double* __restrict__ Jh, const double* __restrict__ f, double* __restrict__ J, int det,
+                         int* __restrict__ status) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= npair * 100) return;
   const int ip = t / 100, c = t % 100;
   if (sig && !sig[ip]) return;
-  const int a = s1[ip], b = s2[ip], la = sh_l[a], lb = sh_l[b];
+  const int a = s1[ip], b = s2[ip], la = sh_l[a], lb = sh_l[b], lp = la + lb;
   const int mu = c / 10, nu = c % 10;
   if (mu >= ncart(la) || nu >= ncart(lb)) return;
   int ix, iy, iz, jx, jy, jz;
   cart_xyz(la, mu, ix, iy, iz);
   cart_xyz(lb, nu, jx, jy, jz);
-  const int H = nherm(la + lb);
-  double E[3][225];
+  const int H = nherm(lp), ne = (la + 1) * (lb + 1) * (lp + 1);
   double v = 0.0;
   for (int k = 0; k < np[ip]; ++k) {
-    const int pi = poff[ip] + k;
-    for (int d = 0; d < 3; ++d) md_e_rt(la, lb, pd.PA[d * pd.n + pi], pd.PB[d * pd.n + pi], 0.5 / pd.p[pi], E[d]);
+    const double* e = E + eoff[ip] + (size_t)k * 3 * ne;  // the tables of k_etab
+    const double *ex = e + (ix * (lb + 1) + jx) * (lp + 1), *ey = e + ne + (iy * (lb + 1) + jy) * (lp + 1),
+                 *ez = e + 2 * ne + (iz * (lb + 1) + jz) * (lp + 1);
     const double* jh = Jh + hoff[ip] + (size_t)k * H;
     for (int tx = 0; tx <= ix + jx; ++tx)
       for (int ty = 0; ty <= iy + jy; ++ty)
         for (int tz = 0; tz <= iz + jz; ++tz) {
           const double hv = acc_value(jh + herm_index(tx, ty, tz), det);
           if (det && fabs(hv) > kFixLimit) atomicOr(status, DEV_RANGE);
-          v += E[0][(ix * 5 + jx) * 9 + tx] * E[1][(iy * 5 + jy) * 9 + ty] * E[2][(iz * 5 + jz) * 9 + tz] * hv;
+          v += ex[tx] * ey[ty] * ez[tz] * hv;
         }
   }
   const int m = pmol[ip], nbf = mm.n[m], a0 = mm.aobase[m];
@@ -728,7 +864,7 @@ BoysTabs eri_plan_impl::boystabs() const {
 
 ShellPairInfo eri_plan_impl::spinfo() const {
   ShellPairInfo sp;
-  sp.s1 = d_ps1; sp.s2 = d_ps2; sp.np = d_pnp; sp.poff = d_ppoff; sp.ao1 = d_pao1; sp.ao2 = d_pao2; sp.hoff = d_phoff; sp.eoff = d_peoff;
+  sp.s1 = d_ps1; sp.s2 = d_ps2; sp.np = d_pnk; sp.poff = d_ppoff; sp.ao1 = d_pao1; sp.ao2 = d_pao2; sp.hoff = d_phoff; sp.eoff = d_peoff;
   sp.pmol = d_pmol; sp.mat_off = d_mat_off; sp.mat_n = d_mat_n;
   return sp;
 }
@@ -757,11 +893,23 @@ int eri_plan_impl::geometry(cudaStream_t s, bool rebuild_q) {
   k_etab<<<grid1(npair, 64), 64, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff, d_sh_l, pairdata(), d_E, d_Ef);
   CK(cudaGetLastError());
   if (rebuild_q) {
-    k_schwarz<<<grid1(npair, 64), 64, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_sh_l, d_sh_ao, d_f, pairdata(), boystabs(),
-                                              d_rsteps, d_Q);
+    k_schwarz<<<grid1(npair, kSchwarzWarps), 32 * kSchwarzWarps, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff,
+                                                                         d_sh_l, d_sh_ao, d_f, pairdata(), boystabs(),
+                                                                         d_rsteps, d_Q);
     CK(cudaGetLastError());
-    return build_lists(thresh, s);
   }
+  CK(cudaMemsetAsync(d_pqmax, 0, sizeof(unsigned int) * nmol, s));
+  k_primq<<<grid1(npair, 64), 64, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff, d_sh_l, d_sh_ao, d_f, d_pmol,
+                                          pairdata(), d_pq, d_pqmax);
+  CK(cudaGetLastError());
+  return rebuild_q ? build_lists(thresh, s) : pack_primitives(s);
+}
+
+int eri_plan_impl::pack_primitives(cudaStream_t s) {
+  k_primpack<<<grid1(npair, 64), 64, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff, d_sh_l, d_pmol, d_pqmax,
+                                             kPrimEps * thresh, nprimpair, d_pq, d_p, d_P, d_PA, d_PB, d_pref, d_ea,
+                                             d_pf, d_Pf, d_PAf, d_PBf, d_preff, d_q4, d_E, d_Ef, d_pnk);
+  CK(cudaGetLastError());
   return ERI_OK;
 }
 
@@ -772,6 +920,8 @@ int eri_plan_impl::build_lists(double th, cudaStream_t s) {
     CK(cudaGraphExecDestroy(gexec));
     gexec = nullptr;
   }
+  int rc = pack_primitives(s);
+  if (rc != ERI_OK) return rc;
   const int nm10 = nmol * NPAIRCLASS;
   CK(cudaMemsetAsync(d_qmax, 0, sizeof(unsigned int) * nmol, s));
   CK(cudaMemsetAsync(d_ccm, 0, sizeof(int) * nm10, s));
@@ -876,7 +1026,7 @@ void eri_plan_impl::release() {
                   d_kpre, d_jpre, d_ktot, d_jtot, d_kprim, d_boys64, d_boys32, d_rsteps, d_Dp, d_Kh, d_Jh, d_Dherm,
                   d_Jherm, d_status, d_bexp64, d_bexp32, d_peoff, d_E, d_Ef, d_pmaxp, d_dmax, d_counters, d_cumnp, d_prefmaxp, d_ea,
                   d_mat_off, d_mat_n, d_aobase, d_pbase, d_pmol, d_shloc, d_ccm, d_segloc, d_Dpf,
-                  d_nuc_list, d_nuc_goff, d_nuc_dens, d_counters2, d_q4, d_Dhermf};
+                  d_nuc_list, d_nuc_goff, d_nuc_dens, d_counters2, d_q4, d_Dhermf, d_pq, d_pqmax, d_pnk};
   xc_release();
   for (auto& e : prof_events) cudaEventDestroy(e);
   prof_events.clear();
@@ -1322,6 +1472,7 @@ static int plan_create(int nmol, const eri_basis_t* const* bases, const double* 
     CKP(dalloc(&P->d_boys64, (size_t)BOYS_NT * (BOYS_MMAX + 1) * BOYS_J64));
     CKP(dalloc(&P->d_boys32, (size_t)BOYS_NT * (BOYS_MMAX + 1) * BOYS_J32));
     CKP(dalloc(&P->d_bexp64, BOYS_NT)); CKP(dalloc(&P->d_bexp32, BOYS_NT));
+    CKP(dalloc(&P->d_pq, nprimpair)); CKP(dalloc(&P->d_pqmax, nmol)); CKP(dalloc(&P->d_pnk, npair));
     CKP(dalloc(&P->d_peoff, npair)); CKP(dalloc(&P->d_E, ne_tot)); CKP(dalloc(&P->d_Ef, ne_tot));
     CKP(dalloc(&P->d_pmaxp, npair)); CKP(dalloc(&P->d_prefmaxp, npair)); CKP(dalloc(&P->d_ea, nprimpair));
     CKP(dalloc(&P->d_dmax, npair));
@@ -1433,10 +1584,10 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
     // both add into the FP64 Hermite J.
     const bool jmixed = precision == ERI_MIXED;
     CK(cudaMemsetAsync(P->d_Jherm, 0, sizeof(double) * (size_t)P->nherm_tot, s));
-    k_hermite_density<<<grid1(P->npair, 64), 64, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_pnp, P->d_ppoff,
-                                                          P->d_phoff, P->d_sh_l, P->d_pao1, P->d_pao2, P->d_pmol, mm,
-                                                          P->d_sig, P->pairdata(), P->d_Dp, P->d_Dherm,
-                                                          jmixed ? P->d_Dhermf : nullptr);
+    k_hermite_density<<<grid1(P->npair, 4), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_pnk, P->d_ppoff,
+                                                         P->d_phoff, P->d_peoff, P->d_sh_l, P->d_pao1, P->d_pao2,
+                                                         P->d_pmol, mm, P->d_sig, P->pairdata(), P->d_Dp, P->d_Dherm,
+                                                         jmixed ? P->d_Dhermf : nullptr);
     CK(cudaGetLastError());
     if (jmixed) {
       k_dmax<<<grid1(P->npair, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_sh_l, P->d_pao1, P->d_pao2,
@@ -1539,10 +1690,10 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       if (rc != ERI_OK) return rc;
     }
     CK(cudaMemsetAsync(J, 0, sizeof(double) * nn, s));
-    k_post_j<<<grid1((int64_t)P->npair * 100, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_pnp, P->d_ppoff,
-                                                                 P->d_phoff, P->d_sh_l, P->d_pao1, P->d_pao2,
-                                                                 P->d_pmol, mm, P->d_sig, P->pairdata(), P->d_Jherm,
-                                                                 P->d_f, J, ja.det, P->d_status);
+    k_post_j<<<grid1((int64_t)P->npair * 100, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_pnk, P->d_phoff,
+                                                                 P->d_peoff, P->d_sh_l, P->d_pao1, P->d_pao2,
+                                                                 P->d_pmol, mm, P->d_sig, P->d_E, P->d_Jherm, P->d_f,
+                                                                 J, ja.det, P->d_status);
     CK(cudaGetLastError());
   } else {
     // J and/or K from contracted Cartesian ERIs over canonical quartets

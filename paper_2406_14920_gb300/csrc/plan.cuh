@@ -35,6 +35,9 @@ struct eri_plan_impl {
   // primitive pairs
   double *d_p = nullptr, *d_P = nullptr, *d_PA = nullptr, *d_PB = nullptr, *d_pref = nullptr;
   float *d_pf = nullptr, *d_Pf = nullptr, *d_PAf = nullptr, *d_PBf = nullptr, *d_preff = nullptr;
+  double* d_pq = nullptr;           // Schwarz-type bound per primitive pair
+  unsigned int* d_pqmax = nullptr;  // its maximum per molecule (float bits)
+  int* d_pnk = nullptr;             // primitive pairs kept per shell pair (the first ones)
   float4* d_q4 = nullptr;  // packed FP32 shadows, 3 float4 per primitive pair (PairData::q4)
   // screening and lists
   float* d_Q = nullptr;
@@ -126,6 +129,7 @@ struct eri_plan_impl {
   int alloc_pairs();
   int geometry(cudaStream_t s, bool rebuild_q);
   int build_lists(double th, cudaStream_t s);
+  int pack_primitives(cudaStream_t s);  // primitive screening at the plan's threshold
   eri::PairData pairdata() const;
   eri::BoysTabs boystabs() const;
   eri::ShellPairInfo spinfo() const;
@@ -167,7 +171,8 @@ __device__ __forceinline__ void md_e_rt(int li, int lj, double PA, double PB, do
 
 // Cartesian J from Hermite J per primitive pair (plan.cu); sig == nullptr takes every pair
 __global__ void k_post_j(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
-                         const int* __restrict__ poff, const int* __restrict__ hoff, const int* __restrict__ sh_l,
+                         const int* __restrict__ hoff, const int* __restrict__ eoff, const int* __restrict__ sh_l,
                          const int* __restrict__ pao1, const int* __restrict__ pao2, const int* __restrict__ pmol,
-                         MolMats mm, const int* __restrict__ sig, eri::PairData pd, const double* __restrict__ Jh,
-                         const double* __restrict__ f, double* __restrict__ J, int det, int* __restrict__ status);
+                         MolMats mm, const int* __restrict__ sig, const double* __restrict__ E,
+                         const double* __restrict__ Jh, const double* __restrict__ f, double* __restrict__ J, int det,
+                         int* __restrict__ status);
