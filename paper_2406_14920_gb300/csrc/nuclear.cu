@@ -9,17 +9,21 @@
 // then one Hermite-to-Cartesian pass (the J-engine's k_post_j) gives V.
 //
 // Gradient of E_V = sum_mn D_mn V_mn with D fixed (SI Sec. 1.3,
-// Eq. si_v1e_derivative_A / _B / _C): with the Hermite densities of each
+// Eq. si_v1e_derivative_A / _B / _C).  With the Hermite densities of each
 // primitive pair (sign-free, the pair counted in both orders)
-//   d_P      = s sum_mn D'_mn E_P^{mn},                          P <= l1 + l2
-//   dA_{t,P} = s sum_mn D'_mn [2a E_P^{(m+1_t) n} - m_t E_P^{(m-1_t) n}],  P <= l1 + l2 + 1
-// (the raising/lowering rule on the centre A of the first shell), each term
-// (pair, charge C) contributes
-//   dE/dA_t = sum_P dA_{t,P} R_P,   dE/dC_t = -sum_P d_P R_{P+1_t}  (dR/dC = -R_{P+1_t}),
-//   dE/dB_t = -(dE/dA_t + dE/dC_t)  (the term depends on A, B, C through differences only).
-// One kernel runs per primitive pair over the charges (A and B), one per
-// charge over the primitive pairs (C); both evaluate R up to l1 + l2 + 1 in
-// registers with compile-time indices, one specialisation per l1 + l2.
+//   d_P      = s sum_mn D'_mn E_P^{mn},     dR_{t,P} = s sum_mn D'_mn E_P^{(1_t) mn}
+// (E^{(1_t)}: the derivative of E with respect to (A-B)_t at fixed P, in closed
+// form from E, see kernels_g.cuh), the pair moves as a whole with P:
+//   dE/dP_t = sum_C q_C sum_P d_P R_{P+1_t},   dE/dA = (a/p) dE/dP + g_R,
+//   dE/dB = (b/p) dE/dP - g_R,   g_{R,t} = sum_P dR_{t,P} sum_C q_C R_P,
+//   dE/dC_t = -q_C sum_pairs sum_P d_P R_{P+1_t}.
+// The sums over charges commute with the densities, so A and B need only
+// h_P = sum_C q_C R_P to order l1 + l2 + 1, like V itself; per (pair, charge) the
+// work is one R table, its addition to h and the 3 nherm(l1 + l2) products of
+// dE/dC.  One kernel does all three (a kernel per pair and one per charge built R
+// twice and contracted six densities per term); dE/dC is transposed through
+// shared memory so that a lane sums one charge over the warp's 32 pairs (3
+// additions per charge instead of 15 shuffles).
 #include <algorithm>
 #include <vector>
 
@@ -39,6 +43,12 @@ constexpr int kChunk = 256;                    // charges (or primitive pairs) p
     cudaError_t e_ = (x);                                                        \
     if (e_ != cudaSuccess) return e_ == cudaErrorMemoryAllocation ? ERI_ENOMEM : ERI_ECUDA; \
   } while (0)
+
+__device__ __forceinline__ double warp_add(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 
 // h_P of one list entry (primitive pair) summed over one chunk of charges
 template <int L>
@@ -69,150 +79,169 @@ __global__ void __launch_bounds__(128) k_nuc_herm(const int4* __restrict__ list,
   for (int x = 0; x < NH; ++x) atomicAdd(Vh + e.y + x, h[x]);
 }
 
-// Hermite densities d_P and dA_{t,P} of every primitive pair (thread per shell pair)
-__global__ void k_nuc_dens(int npair, const int* __restrict__ s1, const int* __restrict__ s2,
-                           const int* __restrict__ np, const int* __restrict__ poff, const int* __restrict__ goff,
-                           const int* __restrict__ sh_l, const int* __restrict__ pao1, const int* __restrict__ pao2,
-                           const int* __restrict__ pmol, MolMats mm, PairData pd, const double* __restrict__ Dp,
-                           double* __restrict__ G) {
-  const int ip = blockIdx.x * blockDim.x + threadIdx.x;
+// Layout of a primitive pair's gradient block: d_P [H], dR_x, dR_y, dR_z [H each],
+// h [H1], H = nherm(l1 + l2), H1 = nherm(l1 + l2 + 1)
+__host__ __device__ constexpr int grad_block(int L) { return 4 * nherm(L) + nherm(L + 1); }
+
+// d_P and dR_{t,P} of every primitive pair, h = 0 (one warp per shell pair, a
+// lane per Hermite index; E is zero outside t <= i + j)
+__global__ void __launch_bounds__(128)
+    k_nuc_dens(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
+               const int* __restrict__ poff, const int* __restrict__ goff, const int* __restrict__ eoff,
+               const int* __restrict__ sh_l, const int* __restrict__ pao1, const int* __restrict__ pao2,
+               const int* __restrict__ pmol, MolMats mm, PairData pd, const double* __restrict__ Dp,
+               double* __restrict__ G) {
+  const int ip = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (ip >= npair) return;
   const int a = s1[ip], b = s2[ip], la = sh_l[a], lb = sh_l[b], L = la + lb;
-  const int H = nherm(L), H1 = nherm(L + 1), stride = H + 3 * H1;
+  const int H = nherm(L), H1 = nherm(L + 1), stride = grad_block(L), ne = (la + 1) * (lb + 1) * (L + 1);
   const int m = pmol[ip], nbf = mm.n[m];
   const double* Dm = Dp + mm.off[m];
   const double sc = a == b ? 1.0 : 2.0;
-  double E[3][225];
   for (int k = 0; k < np[ip]; ++k) {
     const int pi = poff[ip] + k;
-    const double a2 = 2.0 * pd.ea[pi];
-    for (int d = 0; d < 3; ++d) md_e_rt(la + 1, lb, pd.PA[d * pd.n + pi], pd.PB[d * pd.n + pi], 0.5 / pd.p[pi], E[d]);
+    const double ea = pd.ea[pi], aop = ea / pd.p[pi], bop = 1.0 - aop;
+    const double* E = pd.E + eoff[ip] + (size_t)k * 3 * ne;
     double* out = G + goff[ip] + (size_t)k * stride;
-    for (int x = 0; x < stride; ++x) out[x] = 0.0;
-    for (int mu = 0; mu < ncart(la); ++mu) {
-      int i3[3];
-      cart_xyz(la, mu, i3[0], i3[1], i3[2]);
-      for (int nu = 0; nu < ncart(lb); ++nu) {
-        int j3[3];
-        cart_xyz(lb, nu, j3[0], j3[1], j3[2]);
-        const double dv = sc * Dm[(size_t)(pao1[ip] + mu) * nbf + pao2[ip] + nu];
-        for (int tx = 0; tx <= i3[0] + j3[0]; ++tx)
-          for (int ty = 0; ty <= i3[1] + j3[1]; ++ty)
-            for (int tz = 0; tz <= i3[2] + j3[2]; ++tz)
-              out[herm_index(tx, ty, tz)] += dv * E[0][(i3[0] * 5 + j3[0]) * 9 + tx] *
-                                             E[1][(i3[1] * 5 + j3[1]) * 9 + ty] * E[2][(i3[2] * 5 + j3[2]) * 9 + tz];
-        // derivative densities: direction t raised (2a) and lowered (-i_t)
-        for (int t = 0; t < 3; ++t) {
-          double* o = out + H + t * H1;
-          for (int sgn = 0; sgn < 2; ++sgn) {
-            int ii[3] = {i3[0], i3[1], i3[2]};
-            double w;
-            if (sgn == 0) {
-              ii[t] += 1;
-              w = a2 * dv;
-            } else {
-              if (i3[t] == 0) continue;
-              ii[t] -= 1;
-              w = -i3[t] * dv;
-            }
-            for (int tx = 0; tx <= ii[0] + j3[0]; ++tx)
-              for (int ty = 0; ty <= ii[1] + j3[1]; ++ty)
-                for (int tz = 0; tz <= ii[2] + j3[2]; ++tz)
-                  o[herm_index(tx, ty, tz)] += w * E[0][(ii[0] * 5 + j3[0]) * 9 + tx] *
-                                               E[1][(ii[1] * 5 + j3[1]) * 9 + ty] *
-                                               E[2][(ii[2] * 5 + j3[2]) * 9 + tz];
+    for (int q = lane; q < H; q += 32) {
+      const int t[3] = {herm_t(q), herm_u(q), herm_v(q)};
+      double s0 = 0.0, sr[3] = {0.0, 0.0, 0.0};
+      for (int mu = 0; mu < ncart(la); ++mu) {
+        int i3[3];
+        cart_xyz(la, mu, i3[0], i3[1], i3[2]);
+        for (int nu = 0; nu < ncart(lb); ++nu) {
+          int j3[3];
+          cart_xyz(lb, nu, j3[0], j3[1], j3[2]);
+          const double dv = sc * Dm[(size_t)(pao1[ip] + mu) * nbf + pao2[ip] + nu];
+          double e[3], e1[3];
+          for (int d = 0; d < 3; ++d) {
+            const double* r = E + d * ne + (i3[d] * (lb + 1) + j3[d]) * (L + 1) + t[d];
+            e[d] = *r;
+            double v = 2.0 * ea * pd.PA[d * pd.n + pi] * e[d];
+            if (i3[d] > 0) v = fma(-bop * i3[d], r[-(lb + 1) * (L + 1)], v);
+            if (j3[d] > 0) v = fma(aop * j3[d], r[-(L + 1)], v);
+            e1[d] = v;
           }
+          s0 = fma(dv, e[0] * e[1] * e[2], s0);
+          sr[0] = fma(dv, e1[0] * e[1] * e[2], sr[0]);
+          sr[1] = fma(dv, e[0] * e1[1] * e[2], sr[1]);
+          sr[2] = fma(dv, e[0] * e[1] * e1[2], sr[2]);
         }
       }
+      out[q] = s0;
+      for (int d = 0; d < 3; ++d) out[(1 + d) * H + q] = sr[d];
     }
+    for (int q = lane; q < H1; q += 32) out[4 * H + q] = 0.0;
   }
 }
 
-// d/dA and d/dB of one primitive pair, summed over one chunk of charges
+// h_P of one primitive pair over one chunk of charges, and dE/dC of the chunk
+// (dEdC may be null) over the block's pairs
+constexpr int kTr = 16;  // charges transposed at a time
 template <int L>
-__global__ void __launch_bounds__(128) k_nuc_grad_pair(const int4* __restrict__ list, int n, PairData pd,
-                                                       BoysTabs bt, const int* __restrict__ s1,
-                                                       const int* __restrict__ s2, const int* __restrict__ sh_atom,
-                                                       const double* __restrict__ G, int nc,
-                                                       const double* __restrict__ q, const double* __restrict__ xyz,
-                                                       double* __restrict__ dEdR) {
+__global__ void __launch_bounds__(128) k_nuc_grad(const int4* __restrict__ list, int n, PairData pd, BoysTabs bt,
+                                                  double* __restrict__ G, int nc, const double* __restrict__ q,
+                                                  const double* __restrict__ xyz, double* __restrict__ dEdC) {
   constexpr int H = nherm(L), H1 = nherm(L + 1);
+  __shared__ double tr[4][3 * kTr][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int4 e = __ldg(list + i);
+  const bool ok = i < n;  // lanes past the list repeat its last entry with weight 0
+  const int4 e = __ldg(list + (ok ? i : n - 1));
   const int pi = e.x;
-  const double p = __ldg(pd.p + pi), pref = __ldg(pd.pref + pi) * kVfac;
+  const double p = __ldg(pd.p + pi), pref = ok ? __ldg(pd.pref + pi) * kVfac : 0.0;
   const double Px = __ldg(pd.P + pi), Py = __ldg(pd.P + pd.n + pi), Pz = __ldg(pd.P + 2 * pd.n + pi);
   const double* g = G + e.z;
-  double gA[3] = {0.0, 0.0, 0.0}, gC[3] = {0.0, 0.0, 0.0};
-  const int c0 = blockIdx.y * kChunk, c1 = min(nc, c0 + kChunk);
-  for (int c = c0; c < c1; ++c) {
-    const double X = Px - __ldg(xyz + 3 * c), Y = Py - __ldg(xyz + 3 * c + 1), Z = Pz - __ldg(xyz + 3 * c + 2);
-    double F[L + 2];
-    boys_f64<L + 1>(p * (X * X + Y * Y + Z * Z), bt, F);
-    double R[H1];
-    r_build_reg<L + 1, double>(F, pref * __ldg(q + c), X, Y, Z, -2.0 * p, R);
-    sfor<3>([&](auto t_) {
-      constexpr int t = ERI_CI(t_);
-      double sa = 0.0, sc = 0.0;
-      for_herm<L + 1>([&](auto x, auto y, auto z) {
-        constexpr int P = herm_index(ERI_CI(x), ERI_CI(y), ERI_CI(z));
-        sa = fma(__ldg(g + H + t * H1 + P), R[P], sa);
-      });
-      for_herm<L>([&](auto x, auto y, auto z) {
-        constexpr int P = herm_index(ERI_CI(x), ERI_CI(y), ERI_CI(z));
-        constexpr int P1 = herm_index(ERI_CI(x) + (t == 0), ERI_CI(y) + (t == 1), ERI_CI(z) + (t == 2));
-        sc = fma(__ldg(g + P), R[P1], sc);
-      });
-      gA[t] += sa;
-      gC[t] -= sc;
-    });
-  }
-  const int ip = e.w;
-  const int atA = __ldg(sh_atom + __ldg(s1 + ip)), atB = __ldg(sh_atom + __ldg(s2 + ip));
+  double h[H1];
 #pragma unroll
-  for (int t = 0; t < 3; ++t) {
-    atomicAdd(dEdR + 3 * atA + t, gA[t]);
-    atomicAdd(dEdR + 3 * atB + t, -(gA[t] + gC[t]));
+  for (int x = 0; x < H1; ++x) h[x] = 0.0;
+  const int c0 = blockIdx.y * kChunk, c1 = min(nc, c0 + kChunk);
+  for (int cb = c0; cb < c1; cb += kTr) {
+    const int ce = min(c1, cb + kTr);
+    for (int c = cb; c < ce; ++c) {
+      const double X = Px - __ldg(xyz + 3 * c), Y = Py - __ldg(xyz + 3 * c + 1), Z = Pz - __ldg(xyz + 3 * c + 2);
+      double F[L + 2];
+      boys_f64<L + 1>(p * (X * X + Y * Y + Z * Z), bt, F);
+      double R[H1];
+      r_build_reg<L + 1, double>(F, pref * __ldg(q + c), X, Y, Z, -2.0 * p, R);
+#pragma unroll
+      for (int x = 0; x < H1; ++x) h[x] += R[x];
+      if (dEdC) {
+        double s[3] = {0.0, 0.0, 0.0};
+        for_herm<L>([&](auto x, auto y, auto z) {
+          const double d = __ldg(g + herm_index(ERI_CI(x), ERI_CI(y), ERI_CI(z)));
+          s[0] = fma(d, R[herm_index(ERI_CI(x) + 1, ERI_CI(y), ERI_CI(z))], s[0]);
+          s[1] = fma(d, R[herm_index(ERI_CI(x), ERI_CI(y) + 1, ERI_CI(z))], s[1]);
+          s[2] = fma(d, R[herm_index(ERI_CI(x), ERI_CI(y), ERI_CI(z) + 1)], s[2]);
+        });
+#pragma unroll
+        for (int t = 0; t < 3; ++t) tr[w][3 * (c - cb) + t][lane] = s[t];
+      }
+    }
+    if (dEdC) {
+      __syncwarp();
+      for (int r = lane; r < 3 * (ce - cb); r += 32) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int x = 0; x < 32; ++x) s += tr[w][r][x];
+        atomicAdd(dEdC + 3 * cb + r, -s);
+      }
+      __syncwarp();
+    }
+  }
+  if (ok) {
+    double* hg = G + e.z + 4 * H;
+#pragma unroll
+    for (int x = 0; x < H1; ++x) atomicAdd(hg + x, h[x]);
   }
 }
 
-// d/dC of one charge, summed over one chunk of primitive pairs of list L
-template <int L>
-__global__ void __launch_bounds__(128) k_nuc_grad_charge(const int4* __restrict__ list, int n, PairData pd,
-                                                         BoysTabs bt, const double* __restrict__ G, int nc,
-                                                         const double* __restrict__ q,
-                                                         const double* __restrict__ xyz, double* __restrict__ dEdC) {
-  constexpr int H = nherm(L), H1 = nherm(L + 1);
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nc) return;
-  const double Cx = __ldg(xyz + 3 * c), Cy = __ldg(xyz + 3 * c + 1), Cz = __ldg(xyz + 3 * c + 2), qc = __ldg(q + c);
-  double gC[3] = {0.0, 0.0, 0.0};
-  const int i0 = blockIdx.y * kChunk, i1 = min(n, i0 + kChunk);
-  for (int i = i0; i < i1; ++i) {  // every thread reads the same entry: broadcast loads
+// dE/dA and dE/dB of every primitive pair from its densities and h
+__global__ void __launch_bounds__(128)
+    k_nuc_atoms(const int4* __restrict__ list, int n, int L, PairData pd, const int* __restrict__ s1,
+                const int* __restrict__ s2, const int* __restrict__ sh_atom, const double* __restrict__ G,
+                double* __restrict__ dEdR) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  const bool ok = i < n;
+  double gA[3] = {0.0, 0.0, 0.0}, gB[3] = {0.0, 0.0, 0.0};
+  int atA = -1, atB = -1;
+  if (ok) {
     const int4 e = __ldg(list + i);
-    const int pi = e.x;
-    const double p = __ldg(pd.p + pi), pref = __ldg(pd.pref + pi) * kVfac;
-    const double X = __ldg(pd.P + pi) - Cx, Y = __ldg(pd.P + pd.n + pi) - Cy, Z = __ldg(pd.P + 2 * pd.n + pi) - Cz;
-    double F[L + 2];
-    boys_f64<L + 1>(p * (X * X + Y * Y + Z * Z), bt, F);
-    double R[H1];
-    r_build_reg<L + 1, double>(F, pref * qc, X, Y, Z, -2.0 * p, R);
+    const int H = nherm(L);
     const double* g = G + e.z;
-    sfor<3>([&](auto t_) {
-      constexpr int t = ERI_CI(t_);
-      double sc = 0.0;
-      for_herm<L>([&](auto x, auto y, auto z) {
-        constexpr int P = herm_index(ERI_CI(x), ERI_CI(y), ERI_CI(z));
-        constexpr int P1 = herm_index(ERI_CI(x) + (t == 0), ERI_CI(y) + (t == 1), ERI_CI(z) + (t == 2));
-        sc = fma(__ldg(g + P), R[P1], sc);
-      });
-      gC[t] -= sc;
-    });
+    const double* h = g + 4 * H;
+    double gP[3] = {0.0, 0.0, 0.0}, gR[3] = {0.0, 0.0, 0.0};
+    for (int q = 0; q < H; ++q) {
+      const int t = herm_t(q), u = herm_u(q), v = herm_v(q);
+      gP[0] = fma(g[q], h[herm_index(t + 1, u, v)], gP[0]);
+      gP[1] = fma(g[q], h[herm_index(t, u + 1, v)], gP[1]);
+      gP[2] = fma(g[q], h[herm_index(t, u, v + 1)], gP[2]);
+      for (int d = 0; d < 3; ++d) gR[d] = fma(g[(1 + d) * H + q], h[q], gR[d]);
+    }
+    const double aop = __ldg(pd.ea + e.x) / __ldg(pd.p + e.x), bop = 1.0 - aop;
+    atA = __ldg(sh_atom + __ldg(s1 + e.w));
+    atB = __ldg(sh_atom + __ldg(s2 + e.w));
+    for (int d = 0; d < 3; ++d) {
+      gA[d] = fma(aop, gP[d], gR[d]);
+      gB[d] = fma(bop, gP[d], -gR[d]);
+    }
   }
-#pragma unroll
-  for (int t = 0; t < 3; ++t) atomicAdd(dEdC + 3 * c + t, gC[t]);
-  (void)H;
+  const int a0 = __shfl_sync(0xffffffffu, atA, 0), b0 = __shfl_sync(0xffffffffu, atB, 0);
+  if (__all_sync(0xffffffffu, !ok || (atA == a0 && atB == b0))) {  // the warp's pairs share their atoms
+    if (a0 < 0) return;
+    for (int d = 0; d < 3; ++d) {
+      const double x = warp_add(gA[d]), y = warp_add(gB[d]);
+      if (lane == 0) {
+        atomicAdd(dEdR + 3 * a0 + d, x);
+        atomicAdd(dEdR + 3 * b0 + d, y);
+      }
+    }
+  } else if (ok) {
+    for (int d = 0; d < 3; ++d) {
+      atomicAdd(dEdR + 3 * atA + d, gA[d]);
+      atomicAdd(dEdR + 3 * atB + d, gB[d]);
+    }
+  }
 }
 
 template <int L>
@@ -231,13 +260,12 @@ cudaError_t launch_grad(const eri_plan_impl* P, int nc, const double* q, const d
   const int n = P->nuc_cnt[L];
   if (n == 0 || nc == 0) return cudaSuccess;
   const int4* list = P->d_nuc_list + P->nuc_first[L];
-  const dim3 gp((n + 127) / 128, (nc + kChunk - 1) / kChunk);
-  k_nuc_grad_pair<L><<<gp, 128, 0, s>>>(list, n, P->pairdata(), P->boystabs(), P->d_ps1, P->d_ps2, P->d_sh_atom,
-                                        P->d_nuc_dens, nc, q, xyz, dEdR);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || !dEdC) return e;
-  const dim3 gc((nc + 127) / 128, (n + kChunk - 1) / kChunk);
-  k_nuc_grad_charge<L><<<gc, 128, 0, s>>>(list, n, P->pairdata(), P->boystabs(), P->d_nuc_dens, nc, q, xyz, dEdC);
+  const dim3 grid((n + 127) / 128, (nc + kChunk - 1) / kChunk);
+  k_nuc_grad<L><<<grid, 128, 0, s>>>(list, n, P->pairdata(), P->boystabs(), P->d_nuc_dens, nc, q, xyz, dEdC);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_nuc_atoms<<<(n + 127) / 128, 128, 0, s>>>(list, n, L, P->pairdata(), P->d_ps1, P->d_ps2, P->d_sh_atom,
+                                              P->d_nuc_dens, dEdR);
   return cudaGetLastError();
 }
 
@@ -258,7 +286,7 @@ int ensure_nuc(eri_plan_impl* P) {
   std::vector<int> goff(npair);
   int64_t g = 0;
   for (int ip = 0; ip < npair; ++ip) {
-    const int L = shl[s1[ip]] + shl[s2[ip]], H = nherm(L), G = H + 3 * nherm(L + 1);
+    const int L = shl[s1[ip]] + shl[s2[ip]], H = nherm(L), G = grad_block(L);
     goff[ip] = (int)g;
     for (int k = 0; k < np[ip]; ++k) lists[L].push_back(make_int4(poff[ip] + k, hoff[ip] + k * H, (int)(g + (int64_t)k * G), ip));
     g += (int64_t)np[ip] * G;
@@ -322,9 +350,9 @@ extern "C" int eri_nuclear_grad(eri_plan_t* plan, const double* D, int32_t nchar
   const MolMats mm = molmats(P);
   k_scale_d_launch(P, D, s);
   NCK(cudaGetLastError());
-  k_nuc_dens<<<(P->npair + 63) / 64, 64, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_pnp, P->d_ppoff, P->d_nuc_goff,
-                                                 P->d_sh_l, P->d_pao1, P->d_pao2, P->d_pmol, mm, P->pairdata(),
-                                                 P->d_Dp, P->d_nuc_dens);
+  k_nuc_dens<<<(P->npair + 3) / 4, 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_pnp, P->d_ppoff, P->d_nuc_goff,
+                                                P->d_peoff, P->d_sh_l, P->d_pao1, P->d_pao2, P->d_pmol, mm,
+                                                P->pairdata(), P->d_Dp, P->d_nuc_dens);
   NCK(cudaGetLastError());
   NCK(cudaMemsetAsync(dEdR, 0, sizeof(double) * 3 * (size_t)P->natom, s));
   if (dEdC && ncharge > 0) NCK(cudaMemsetAsync(dEdC, 0, sizeof(double) * 3 * (size_t)ncharge, s));
