@@ -22,12 +22,12 @@
 // once per geometry and kept in HBM ([block][component c = phi, d/dx, d/dy,
 // d/dz][function][point]); above the workspace cap they are recomputed per
 // chunk of blocks instead.  The density is one dense product X = D_b Phi_b per
-// block (thread = grid point, rows of D_b staged in shared memory, then
-// rho = sum_m phi_m X_m and grad rho = 2 sum_m grad phi_m X_m); the matrix is
-// the block-sparse product V = sum_b (Z_b Phi_b^T + Phi_b Z_b^T) with
-// Z = w (v_rho phi / 2 + v_grad . grad phi), computed output-stationary: a CTA
-// owns a 32 x 32 tile of V and walks the blocks of its share, so V receives
-// one atomic per element per share.  All arithmetic is FP64.
+// block, then rho = sum_m phi_m X_m and grad rho = 2 sum_m grad phi_m X_m; the
+// matrix is V = sum_b (Z_b Phi_b^T + Phi_b Z_b^T) with
+// Z = w (v_rho phi / 2 + v_grad . grad phi), one product A_b = Z_b Phi_b^T per
+// block added to a half matrix by atomics, V = Vh + Vh^T at the end.  Both
+// products run on the tensor cores as exact digit sums (xc_mma.cuh); everything
+// else is FP64.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -35,6 +35,7 @@
 
 #include "../../include/eri.h"
 #include "plan.cuh"
+#include "xc_mma.cuh"
 
 using namespace eri;
 
@@ -42,12 +43,10 @@ namespace {
 
 constexpr int kBP = 32;           // points per block (at most) = threads of the per-block kernels
 constexpr int kWarps = kBP / 32;
-constexpr int kRT = 16;           // rows of D_b per register tile (k_xc_rho)
-constexpr int kNC = 64;           // columns of D_b per staged chunk (k_xc_rho)
-constexpr int kVT = 64;           // V tile edge (basis functions), k_xc_vmat
-constexpr int kVP = 16;           // points per staged chunk, k_xc_vmat
-constexpr int kVThreads = 256;    // k_xc_vmat block
-constexpr int kVOut = kVT * kVT / kVThreads;  // outputs per thread and block (at most)
+constexpr int kRhoWarps = 4;      // k_xc_rho: warps per block, 16 rows of D_b each at a time
+constexpr int kKC = 128;          // k_xc_rho: functions of Phi_b staged at a time
+constexpr int kVWarps = 8;        // k_xc_vmat: warps per block, 16 rows of Z_b each at a time
+constexpr int kVC = 128;          // k_xc_vmat: functions of Phi_b staged at a time
 constexpr int kSlots = 5;         // workspace rows per function: phi, d/dx, d/dy, d/dz, Z
 constexpr double kAoEps = 1e-15;  // shell extent: every |phi| and |grad phi| below this beyond it
 constexpr double kRhoMin = 1e-14; // points with a smaller density contribute nothing
@@ -304,10 +303,12 @@ __global__ void __launch_bounds__(kBP) k_xc_ao(int b0, const int* __restrict__ p
                                                const int* __restrict__ sh_np, const int* __restrict__ sh_po,
                                                const int* __restrict__ sh_ao, const double* __restrict__ ex,
                                                const double* __restrict__ cn, const double* __restrict__ f,
-                                               const double* __restrict__ xyz, double* __restrict__ work) {
+                                               const double* __restrict__ xyz, double* __restrict__ work,
+                                               int* __restrict__ pexp) {
   const int b = b0 + blockIdx.x, t = threadIdx.x;
   const int g = perm[(int64_t)b * kBP + t];
   const int n = nbfb[b], ns = nsh[b];
+  int emax = 0;  // largest exponent of phi at this point
   double* W = work + woff[b];
   double px = 0.0, py = 0.0, pz = 0.0;
   if (g >= 0) {
@@ -342,64 +343,174 @@ __global__ void __launch_bounds__(kBP) k_xc_ao(int b0, const int* __restrict__ p
       }
       const double fc = f[ao + k];
       const int row = o + k;
-      W[(int64_t)row * kBP + t] = fc * pw[0] * pw[1] * pw[2] * e0;
+      const double phi = fc * pw[0] * pw[1] * pw[2] * e0;
+      emax = max(emax, exponent_of(phi));
+      W[(int64_t)row * kBP + t] = phi;
       W[((int64_t)n + row) * kBP + t] = fc * (pl[0] * e0 - 2.0 * pu[0] * e1) * pw[1] * pw[2];
       W[((int64_t)2 * n + row) * kBP + t] = fc * (pl[1] * e0 - 2.0 * pu[1] * e1) * pw[0] * pw[2];
       W[((int64_t)3 * n + row) * kBP + t] = fc * (pl[2] * e0 - 2.0 * pu[2] * e1) * pw[0] * pw[1];
     }
   }
+  pexp[(int64_t)b * kBP + t] = emax;
+}
+
+// Digits of D, 8 bf16 per element (one 16-byte row), row by row under the row's
+// exponent, and each row's scale; a row with an infinity or NaN is marked bad
+__global__ void __launch_bounds__(256) k_xc_ddigits(int nbf, const double* __restrict__ D, uint4* __restrict__ Dd,
+                                                    double* __restrict__ scale, int* __restrict__ bad) {
+  __shared__ int red[8];
+  const int r = blockIdx.x, t = threadIdx.x;
+  const double* row = D + (int64_t)r * nbf;
+  int E = 0;
+  for (int c = t; c < nbf; c += blockDim.x) E = max(E, exponent_of(row[c]));
+  E = __reduce_max_sync(0xffffffffu, E);
+  if ((t & 31) == 0) red[t >> 5] = E;
+  __syncthreads();
+#pragma unroll
+  for (int x = 0; x < 8; ++x) E = max(E, red[x]);
+  if (t == 0) {
+    scale[r] = digit_scale(E);
+    bad[r] = E == 2047;
+  }
+  for (int c = t; c < nbf; c += blockDim.x) {
+    uint32_t d[kDigits];
+    digits_of(row[c], E, d);
+    Dd[(int64_t)r * nbf + c] = make_uint4(bf16_pair(d[0], d[1]), bf16_pair(d[2], d[3]), bf16_pair(d[4], d[5]),
+                                          bf16_pair(d[6], d[7]));
+  }
 }
 
 // Step (2): X_m = sum_n D_mn phi_n at every point of the block, then
-// rho = sum_m phi_m X_m, grad rho = 2 sum_m grad phi_m X_m (D symmetric)
-__global__ void __launch_bounds__(kBP) k_xc_rho(int b0, int nbf, const int* __restrict__ perm,
-                                                const int* __restrict__ nbfb, const int* __restrict__ bfl,
-                                                const int64_t* __restrict__ woff, const double* __restrict__ work,
-                                                const double* __restrict__ D, double* __restrict__ rho,
-                                                double* __restrict__ grad) {
-  __shared__ double Ds[kRT][kNC];
-  const int b = b0 + blockIdx.x, t = threadIdx.x;
-  const int g = perm[(int64_t)b * kBP + t];
+// rho = sum_m phi_m X_m, grad rho = 2 sum_m grad phi_m X_m (D symmetric).
+// A warp owns 16 rows of X x the 32 points (nine accumulators of 16 values per
+// lane) and gathers the digit rows of D at the block's functions straight into
+// its operand registers (16 B per element, from L2); the digits of kKC functions
+// of Phi_b are staged in shared memory in operand order.  X goes through shared
+// memory to a lane per point for the sums with phi and grad phi.  A block that
+// holds a function with an infinity or NaN in its row of D takes the plain sums.
+struct RhoSmem {
+  uint2 B[kKC / 16][kBP / 8][kDigits][32];
+  double X[kRhoWarps][16][kBP];
+  double sum[kRhoWarps][4][kBP];
+  double pscale[kBP];
+};
+__global__ void __launch_bounds__(32 * kRhoWarps, 2)
+    k_xc_rho(int b0, int nbf, const int* __restrict__ perm, const int* __restrict__ nbfb, const int* __restrict__ bfl,
+             const int64_t* __restrict__ woff, const double* __restrict__ work, const int* __restrict__ pexp,
+             const double* __restrict__ D, const uint4* __restrict__ Dd, const double* __restrict__ dscale,
+             const int* __restrict__ dbad, double* __restrict__ rho, double* __restrict__ grad) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  RhoSmem& S = *reinterpret_cast<RhoSmem*>(smraw);
+  const int b = b0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   const int n = nbfb[b];
   const int* L = bfl + (int64_t)b * nbf;
   const double* W = work + woff[b];
-  double r = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
-  for (int m0 = 0; m0 < n; m0 += kRT) {
-    const int nr = min(kRT, n - m0);
-    double acc[kRT];
+  int isbad = 0;
+  for (int i = tid; i < n; i += 32 * kRhoWarps) isbad |= dbad[L[i]];
+  isbad = __syncthreads_or(isbad);
+  double sum[4] = {0.0, 0.0, 0.0, 0.0};  // rho, grad rho / 2 of point `lane` over this warp's rows
+  auto add_row = [&](int row, double x) {
 #pragma unroll
-    for (int i = 0; i < kRT; ++i) acc[i] = 0.0;
-    for (int n0 = 0; n0 < n; n0 += kNC) {
-      const int nc = min(kNC, n - n0);
-      __syncthreads();
-      for (int e = t; e < kRT * kNC; e += kBP) {
-        const int i = e / kNC, c = e % kNC;
-        Ds[i][c] = (i < nr && c < nc) ? __ldg(D + (int64_t)L[m0 + i] * nbf + L[n0 + c]) : 0.0;
-      }
-      __syncthreads();
-      for (int c = 0; c < nc; ++c) {
-        const double ph = W[(int64_t)(n0 + c) * kBP + t];
-#pragma unroll
-        for (int i = 0; i < kRT; ++i) acc[i] = fma(Ds[i][c], ph, acc[i]);
-      }
+    for (int c = 0; c < 4; ++c) sum[c] = fma(W[((int64_t)c * n + row) * kBP + lane], x, sum[c]);
+  };
+  if (isbad) {
+    for (int m = wp; m < n; m += kRhoWarps) {
+      double x = 0.0;
+      for (int c = 0; c < n; ++c) x = fma(D[(int64_t)L[m] * nbf + L[c]], W[(int64_t)c * kBP + lane], x);
+      add_row(m, x);
     }
+  } else {
+    const int g = lane >> 2, t = lane & 3;  // operand row and column pair of this lane
+    if (tid < kBP) S.pscale[tid] = digit_scale(pexp[(int64_t)b * kBP + tid]);
+    for (int mg = 0; mg < n; mg += 16 * kRhoWarps) {
+      const int m0 = mg + 16 * wp;
+      const int64_t r0 = (int64_t)L[min(m0 + g, n - 1)] * nbf, r1 = (int64_t)L[min(m0 + g + 8, n - 1)] * nbf;
+      for (int seg = 0; seg < n; seg += kExactTerms) {
+        const int send = min(n, seg + kExactTerms);
+        float acc[kBP / 8][kWeights][4];
 #pragma unroll
-    for (int i = 0; i < kRT; ++i) {
-      if (i < nr) {
-        const int row = m0 + i;
-        r = fma(W[(int64_t)row * kBP + t], acc[i], r);
-        gx = fma(W[((int64_t)n + row) * kBP + t], acc[i], gx);
-        gy = fma(W[((int64_t)2 * n + row) * kBP + t], acc[i], gy);
-        gz = fma(W[((int64_t)3 * n + row) * kBP + t], acc[i], gz);
+        for (int x = 0; x < kBP / 8; ++x)
+#pragma unroll
+          for (int k = 0; k < kWeights; ++k)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[x][k][c] = 0.0f;
+        for (int kc = seg; kc < send; kc += kKC) {
+          const int nks = (min(send - kc, kKC) + 15) / 16;
+          __syncthreads();  // the previous chunk has been read
+          // one pair of functions (k, k + 1) at one point per step, both halves of a 16-step
+          for (int e = tid; e < nks * (kBP / 8) * 64; e += 32 * kRhoWarps) {
+            const int el = e & 31, h = (e >> 5) & 1, nt = (e >> 6) & (kBP / 8 - 1), ks = e >> 8;
+            const int k = kc + 16 * ks + 2 * (el & 3) + 8 * h, p = 8 * nt + (el >> 2);
+            const int E = pexp[(int64_t)b * kBP + p];
+            uint32_t d0[kDigits], d1[kDigits];
+            digits_of(k < n ? W[(int64_t)k * kBP + p] : 0.0, E, d0);
+            digits_of(k + 1 < n ? W[(int64_t)(k + 1) * kBP + p] : 0.0, E, d1);
+#pragma unroll
+            for (int x = 0; x < kDigits; ++x) (&S.B[ks][nt][x][el].x)[h] = bf16_pair(d0[x], d1[x]);
+          }
+          __syncthreads();
+          if (m0 < n) {
+            for (int ks = 0; ks < nks; ++ks) {
+              uint32_t a[kDigits][4];
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {  // columns 2t, 2t+1 and 2t+8, 2t+9 of rows g and g + 8
+                const int k = kc + 16 * ks + 2 * t + 8 * h;
+                const int c0 = __ldg(L + min(k, n - 1)), c1 = __ldg(L + min(k + 1, n - 1));
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                  const uint4 u = __ldg(Dd + (y ? r1 : r0) + c0), v = __ldg(Dd + (y ? r1 : r0) + c1);
+                  const uint32_t uu[4] = {u.x, u.y, u.z, u.w}, vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                  for (int x = 0; x < 4; ++x) {
+                    a[2 * x][2 * h + y] = __byte_perm(uu[x], vv[x], 0x5410);
+                    a[2 * x + 1][2 * h + y] = __byte_perm(uu[x], vv[x], 0x7632);
+                  }
+                }
+              }
+#pragma unroll
+              for (int nt = 0; nt < kBP / 8; ++nt)
+#pragma unroll
+                for (int y = 0; y < kDigits; ++y) {
+                  const uint2 bb = S.B[ks][nt][y][lane];
+#pragma unroll
+                  for (int x = 0; x < kDigits; ++x)
+                    if (x + y < kWeights) mma_bf16(acc[nt][x + y], a[x], bb);
+                }
+            }
+          }
+        }
+        if (m0 < n) {
+          const double s0 = dscale[L[min(m0 + g, n - 1)]], s1 = dscale[L[min(m0 + g + 8, n - 1)]];
+          __syncwarp();
+#pragma unroll
+          for (int nt = 0; nt < kBP / 8; ++nt)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const int p = 8 * nt + 2 * t + (c & 1);
+              S.X[wp][g + 8 * (c >> 1)][p] = combine(acc[nt], c) * (c < 2 ? s0 : s1) * S.pscale[p];
+            }
+          __syncwarp();
+          const int nr = min(16, n - m0);
+          for (int r = 0; r < nr; ++r) add_row(m0 + r, S.X[wp][r][lane]);
+        }
       }
     }
   }
-  if (g >= 0) {
-    rho[g] = r;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) S.sum[wp][c][lane] = sum[c];
+  __syncthreads();
+  if (wp == 0) {
+    const int g = perm[(int64_t)b * kBP + lane];
+    if (g < 0) return;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int x = 0; x < kRhoWarps; ++x)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] += S.sum[x][c][lane];
+    rho[g] = v[0];
     if (grad) {
-      grad[3 * (int64_t)g] = 2.0 * gx;
-      grad[3 * (int64_t)g + 1] = 2.0 * gy;
-      grad[3 * (int64_t)g + 2] = 2.0 * gz;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) grad[3 * (int64_t)g + c] = 2.0 * v[1 + c];
     }
   }
 }
@@ -454,26 +565,18 @@ __global__ void k_xc_func(int64_t G, int kind, const double* __restrict__ w, con
   }
 }
 
-__device__ __forceinline__ int lower_bound_i(const int* __restrict__ a, int n, int v) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] < v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
 // Step (4a): Z_m(g) = w_g (v_rho,g phi_m(g) / 2 + v_grad,g . grad phi_m(g)) for
 // every significant function of the block (workspace slot 4)
 __global__ void __launch_bounds__(kBP) k_xc_z(int b0, const int* __restrict__ perm, const int* __restrict__ nbfb,
                                               const int64_t* __restrict__ woff, const double* __restrict__ w,
                                               const double* __restrict__ vrho, const double* __restrict__ vgrad,
-                                              double* __restrict__ work) {
+                                              double* __restrict__ work, int* __restrict__ bad) {
   const int b = b0 + blockIdx.x, t = threadIdx.x;
   const int g = perm[(int64_t)b * kBP + t];
   const int n = nbfb[b];
   double* W = work + woff[b];
   double pw = 0.0, pv = 0.0, g0 = 0.0, g1 = 0.0, g2 = 0.0;
+  int inf = 0;
   if (g >= 0) {
     pw = w[g];
     pv = 0.5 * vrho[g];
@@ -484,115 +587,153 @@ __global__ void __launch_bounds__(kBP) k_xc_z(int b0, const int* __restrict__ pe
   for (int m = 0; m < n; ++m) {
     const double phi = W[(int64_t)m * kBP + t], dx = W[((int64_t)n + m) * kBP + t],
                  dy = W[((int64_t)2 * n + m) * kBP + t], dz = W[((int64_t)3 * n + m) * kBP + t];
-    W[((int64_t)4 * n + m) * kBP + t] = pw * (pv * phi + g0 * dx + g1 * dy + g2 * dz);
+    const double z = pw * (pv * phi + g0 * dx + g1 * dy + g2 * dz);
+    W[((int64_t)4 * n + m) * kBP + t] = z;
+    inf |= exponent_of(z) == 2047;
+  }
+  inf = __any_sync(0xffffffffu, inf);
+  if (t == 0) bad[b] = inf;  // an infinity or NaN among the block's Z
+}
+
+// The digits of one function's 32 values that a lane holds as an operand (row or
+// column `lane >> 2`, steps 16 s + 2t, +1, +8, +9): d[s][h][digit], h the half of
+// the step; returns the function's exponent.  Whole warp; `row` may differ per lane.
+__device__ __forceinline__ int operand_digits(const double* row, int t, uint32_t (&d)[2][2][kDigits]) {
+  double2 v[2][2];
+  int E = 0;
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      v[s][h] = *reinterpret_cast<const double2*>(row + 16 * s + 2 * t + 8 * h);
+      E = max(E, max(exponent_of(v[s][h].x), exponent_of(v[s][h].y)));
+    }
+  E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));  // the four lanes of the function
+  E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t lo[kDigits], hi[kDigits];
+      digits_of(v[s][h].x, E, lo);
+      digits_of(v[s][h].y, E, hi);
+#pragma unroll
+      for (int x = 0; x < kDigits; ++x) d[s][h][x] = bf16_pair(lo[x], hi[x]);
+    }
+  return E;
+}
+
+// Step (4b): A_ij = sum_g Z_i(g) phi_j(g) of one block over its functions, added
+// to the half matrix Vh.  A warp holds the digits of 16 functions of Z over the
+// block's 32 points in registers and walks the staged functions of Phi, 8 at a
+// time; the 32 points are one exact accumulation.  (Tiles of V that walk every
+// block waste products on functions a block does not hold, 2.8 times as many on
+// workload 1 at 32 x 32.)
+struct VmatSmem {
+  uint2 B[kVC / 8][2][kDigits][32];
+  double scale[kVC];
+  int ao[kVC];
+};
+__global__ void __launch_bounds__(32 * kVWarps, 2)
+    k_xc_vmat(int b0, int nbf, const int* __restrict__ nbfb, const int* __restrict__ bfl,
+              const int64_t* __restrict__ woff, const double* __restrict__ work, const int* __restrict__ bad,
+              double* __restrict__ Vh) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  VmatSmem& S = *reinterpret_cast<VmatSmem*>(smraw);
+  const int b = b0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int n = nbfb[b];
+  const int* L = bfl + (int64_t)b * nbf;
+  const double* phi = work + woff[b];
+  const double* Z = phi + (int64_t)4 * n * kBP;
+  if (bad[b]) {  // an infinity or NaN: plain sums
+    for (int64_t o = tid; o < (int64_t)n * n; o += 32 * kVWarps) {
+      const int i = (int)(o / n), j = (int)(o - (int64_t)i * n);
+      double v = 0.0;
+      for (int p = 0; p < kBP; ++p) v = fma(Z[(int64_t)i * kBP + p], phi[(int64_t)j * kBP + p], v);
+      atomicAdd(Vh + (int64_t)L[i] * nbf + L[j], v);
+    }
+    return;
+  }
+  const int g = lane >> 2, t = lane & 3;
+  for (int j0 = 0; j0 < n; j0 += kVC) {
+    const int nj = min(kVC, n - j0), njt = (nj + 7) / 8;
+    __syncthreads();  // the previous chunk has been read
+    for (int nt = wp; nt < njt; nt += kVWarps) {
+      const int j = min(j0 + 8 * nt + g, n - 1);
+      uint32_t d[2][2][kDigits];
+      const int E = operand_digits(phi + (int64_t)j * kBP, t, d);
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int x = 0; x < kDigits; ++x) S.B[nt][s][x][lane] = make_uint2(d[s][0][x], d[s][1][x]);
+      if (t == 0) {
+        S.scale[8 * nt + g] = digit_scale(E);
+        S.ao[8 * nt + g] = L[j];
+      }
+    }
+    __syncthreads();
+    for (int m0 = 16 * wp; m0 < n; m0 += 16 * kVWarps) {
+      const int i0 = min(m0 + g, n - 1), i1 = min(m0 + g + 8, n - 1);
+      uint32_t a[2][kDigits][4];
+      double s0, s1;
+      {
+        uint32_t d[2][2][kDigits];
+        s0 = digit_scale(operand_digits(Z + (int64_t)i0 * kBP, t, d));
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+          for (int x = 0; x < kDigits; ++x) {
+            a[s][x][0] = d[s][0][x];
+            a[s][x][2] = d[s][1][x];
+          }
+        s1 = digit_scale(operand_digits(Z + (int64_t)i1 * kBP, t, d));
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+          for (int x = 0; x < kDigits; ++x) {
+            a[s][x][1] = d[s][0][x];
+            a[s][x][3] = d[s][1][x];
+          }
+      }
+      double* v0 = Vh + (int64_t)L[i0] * nbf;
+      double* v1 = Vh + (int64_t)L[i1] * nbf;
+      const bool ok0 = m0 + g < n, ok1 = m0 + g + 8 < n;
+      for (int nt = 0; nt < njt; ++nt) {
+        float acc[kWeights][4];
+#pragma unroll
+        for (int k = 0; k < kWeights; ++k)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[k][c] = 0.0f;
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+          for (int y = 0; y < kDigits; ++y) {
+            const uint2 bb = S.B[nt][s][y][lane];
+#pragma unroll
+            for (int x = 0; x < kDigits; ++x)
+              if (x + y < kWeights) mma_bf16(acc[x + y], a[s][x], bb);
+          }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int jl = 8 * nt + 2 * t + (c & 1);
+          if (jl >= nj || !(c < 2 ? ok0 : ok1)) continue;
+          const double v = combine(acc, c) * (c < 2 ? s0 : s1) * S.scale[jl];
+          if (v != 0.0) atomicAdd((c < 2 ? v0 : v1) + S.ao[jl], v);
+        }
+      }
+    }
   }
 }
 
-// Step (4b): tile (I, J), I >= J, of V over the blocks of this CTA's share:
-// V_ij += sum_g Z_i(g) phi_j(g) + phi_i(g) Z_j(g).  Per block only the
-// functions it holds take part: the block's rows inside the tile's function
-// range (contiguous in its list) form an nI x nJ product (nI (nI+1)/2 on the
-// diagonal), spread flat over the threads, so no lane works on an absent
-// function.  Each product element is added to a shared-memory accumulator at
-// its tile position; the tile goes to V with one atomic per element at the end.
-__global__ void __launch_bounds__(kVThreads) k_xc_vmat(int b0, int b1, int nsplit, int nbf,
-                                                       const int* __restrict__ nbfb, const int* __restrict__ bfl,
-                                                       const int64_t* __restrict__ woff,
-                                                       const double* __restrict__ work, double* __restrict__ V) {
-  extern __shared__ double xs[];
-  double* accs = xs;                          // [kVT][kVT + 1]
-  double* zI = accs + kVT * (kVT + 1);        // [kVT][kVP + 1] each
-  double* pI = zI + kVT * (kVP + 1);
-  double* zJ = pI + kVT * (kVP + 1);
-  double* pJ = zJ + kVT * (kVP + 1);
-  int* posI = (int*)(pJ + kVT * (kVP + 1));   // [kVT]
-  int* posJ = posI + kVT;
-  const int tix = blockIdx.x;
-  int I = (int)((sqrt(8.0 * tix + 1.0) - 1.0) * 0.5);
-  while ((I + 1) * (I + 2) / 2 <= tix) ++I;
-  while (I * (I + 1) / 2 > tix) --I;
-  const int J = tix - I * (I + 1) / 2;
-  const bool diag = I == J;
-  const int t = threadIdx.x;
-  for (int e = t; e < kVT * (kVT + 1); e += kVThreads) accs[e] = 0.0;
-  const int nb = b1 - b0, per = (nb + nsplit - 1) / nsplit;
-  const int bs = b0 + blockIdx.y * per, be = min(b1, bs + per);
-  for (int b = bs; b < be; ++b) {
-    const int n = nbfb[b];
-    const int* L = bfl + (int64_t)b * nbf;
-    const int iI0 = lower_bound_i(L, n, I * kVT), iI1 = lower_bound_i(L, n, I * kVT + kVT);
-    const int iJ0 = diag ? iI0 : lower_bound_i(L, n, J * kVT), iJ1 = diag ? iI1 : lower_bound_i(L, n, J * kVT + kVT);
-    const int nI = iI1 - iI0, nJ = iJ1 - iJ0;
-    if (nI == 0 || nJ == 0) continue;  // uniform over the CTA
-    const int nout = diag ? nI * (nI + 1) / 2 : nI * nJ;
-    const double* W = work + woff[b];
-    __syncthreads();  // the previous block's accumulator updates and positions are done
-    if (t < nI) posI[t] = L[iI0 + t] - I * kVT;
-    if (t < nJ) posJ[t] = L[iJ0 + t] - J * kVT;
-    int rc[kVOut];  // row | col << 8 of each of this thread's outputs (-1: none)
-    double acc[kVOut];
-#pragma unroll
-    for (int k = 0; k < kVOut; ++k) {
-      const int o = t + k * kVThreads;
-      acc[k] = 0.0;
-      rc[k] = -1;
-      if (o < nout) {
-        int r, c;
-        if (diag) {
-          r = (int)((sqrtf(8.0f * o + 1.0f) - 1.0f) * 0.5f);
-          while ((r + 1) * (r + 2) / 2 <= o) ++r;
-          while (r * (r + 1) / 2 > o) --r;
-          c = o - r * (r + 1) / 2;
-        } else {
-          r = o / nJ;
-          c = o - r * nJ;
-        }
-        rc[k] = r | (c << 8);
-      }
-    }
-    const double* zJs = diag ? zI : zJ;
-    const double* pJs = diag ? pI : pJ;
-    for (int p0 = 0; p0 < kBP; p0 += kVP) {
-      __syncthreads();
-      for (int e = t; e < kVT * kVP; e += kVThreads) {
-        const int r = e / kVP, q = e - r * kVP, col = p0 + q;
-        if (r < nI) {
-          zI[r * (kVP + 1) + q] = W[((int64_t)4 * n + iI0 + r) * kBP + col];
-          pI[r * (kVP + 1) + q] = W[(int64_t)(iI0 + r) * kBP + col];
-        }
-        if (!diag && r < nJ) {
-          zJ[r * (kVP + 1) + q] = W[((int64_t)4 * n + iJ0 + r) * kBP + col];
-          pJ[r * (kVP + 1) + q] = W[(int64_t)(iJ0 + r) * kBP + col];
-        }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < kVOut; ++k) {
-        if (rc[k] < 0) continue;
-        const int oi = (rc[k] & 255) * (kVP + 1), oj = (rc[k] >> 8) * (kVP + 1);
-        double a = acc[k];
-#pragma unroll
-        for (int q = 0; q < kVP; ++q) a = fma(zI[oi + q], pJs[oj + q], fma(pI[oi + q], zJs[oj + q], a));
-        acc[k] = a;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < kVOut; ++k)
-      if (rc[k] >= 0) accs[posI[rc[k] & 255] * (kVT + 1) + posJ[rc[k] >> 8]] += acc[k];
-  }
-  __syncthreads();
-  for (int e = t; e < kVT * kVT; e += kVThreads) {
-    const int i = e / kVT, j = e - i * kVT;
-    const int gi = I * kVT + i, gj = J * kVT + j;
-    if (gi >= nbf || gj >= nbf || (diag && j > i)) continue;
-    const double v = accs[i * (kVT + 1) + j];
-    if (v == 0.0) continue;
-    atomicAdd(V + (int64_t)gi * nbf + gj, v);
-    if (gi != gj) atomicAdd(V + (int64_t)gj * nbf + gi, v);
+// V = Vh + Vh^T in place
+__global__ void k_xc_symm(int nbf, double* __restrict__ V) {
+  const int i = blockIdx.x, j0 = threadIdx.x;
+  for (int j = j0; j <= i; j += blockDim.x) {
+    const double v = V[(int64_t)i * nbf + j] + V[(int64_t)j * nbf + i];
+    V[(int64_t)i * nbf + j] = v;
+    V[(int64_t)j * nbf + i] = v;
   }
 }
-
-constexpr size_t kVmatSmem = sizeof(double) * (kVT * (kVT + 1) + 4 * kVT * (kVP + 1)) + sizeof(int) * 2 * kVT;
 
 }  // namespace
 
@@ -603,7 +744,7 @@ constexpr size_t kVmatSmem = sizeof(double) * (kVT * (kVT + 1) + 4 * kVT * (kVP 
 void eri_plan_impl::xc_release() {
   void* ptrs[] = {xc.d_pts, xc.d_w, xc.d_rad, xc.d_ang, xc.d_invab, xc.d_perm, xc.d_bsph, xc.d_ext, xc.d_nsh,
                   xc.d_shl, xc.d_shoff, xc.d_nbfb, xc.d_bfl, xc.d_woff, xc.d_work, xc.d_rho, xc.d_grad,
-                  xc.d_vrho, xc.d_vgrad};
+                  xc.d_vrho, xc.d_vgrad, xc.d_pexp, xc.d_ddig, xc.d_dscale, xc.d_dbad, xc.d_zbad};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   xc = XcState{};
@@ -656,6 +797,11 @@ static int xc_build(eri_plan_impl* P, cudaStream_t s) {
   XCK(xalloc(&X.d_grad, 3 * (size_t)X.npts));
   XCK(xalloc(&X.d_vrho, (size_t)X.npts));
   XCK(xalloc(&X.d_vgrad, 3 * (size_t)X.npts));
+  XCK(xalloc(&X.d_pexp, (size_t)nb * kBP));
+  XCK(xalloc(&X.d_ddig, (size_t)nbf * nbf));
+  XCK(xalloc(&X.d_dscale, (size_t)nbf));
+  XCK(xalloc(&X.d_dbad, (size_t)nbf));
+  XCK(xalloc(&X.d_zbad, (size_t)nb));
   XCK(cudaMemcpyAsync(X.d_perm, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice, s));
   const int nt = std::max(nrad, nth);
   k_xc_nodes<<<(nt + 127) / 128, 128, 0, s>>>(nrad, nth, X.radius, X.d_rad, X.d_ang);
@@ -702,7 +848,7 @@ static int xc_build(eri_plan_impl* P, cudaStream_t s) {
   if (X.resident) {
     k_xc_ao<<<nb, kBP, 0, s>>>(0, X.d_perm, X.d_pts, X.d_nsh, X.d_shl, X.d_shoff, X.d_nbfb, ns, X.d_woff,
                                P->d_sh_atom, P->d_sh_l, P->d_sh_np, P->d_sh_po, P->d_sh_ao, P->d_exps, P->d_cn,
-                               P->d_f, P->d_coords, X.d_work);
+                               P->d_f, P->d_coords, X.d_work, X.d_pexp);
     XCK(cudaGetLastError());
   }
   X.built_serial = P->geom_serial;
@@ -739,16 +885,21 @@ static void xc_launch_ao(eri_plan_impl* P, int b0, int b1, cudaStream_t s) {
   XcState& X = P->xc;
   k_xc_ao<<<b1 - b0, kBP, 0, s>>>(b0, X.d_perm, X.d_pts, X.d_nsh, X.d_shl, X.d_shoff, X.d_nbfb, P->nshell, X.d_woff,
                                   P->d_sh_atom, P->d_sh_l, P->d_sh_np, P->d_sh_po, P->d_sh_ao, P->d_exps, P->d_cn,
-                                  P->d_f, P->d_coords, X.d_work);
+                                  P->d_f, P->d_coords, X.d_work, X.d_pexp);
 }
 
 static int xc_density_impl(eri_plan_impl* P, const double* D, double* rho, double* grad, cudaStream_t s) {
   XcState& X = P->xc;
+  const int nbf = P->nbf;
+  XCK(cudaFuncSetAttribute(k_xc_rho, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RhoSmem)));
+  k_xc_ddigits<<<nbf, 256, 0, s>>>(nbf, D, X.d_ddig, X.d_dscale, X.d_dbad);
+  XCK(cudaGetLastError());
   for (size_t c = 0; c + 1 < X.chunk.size(); ++c) {
     const int b0 = X.chunk[c], b1 = X.chunk[c + 1];
     if (b1 <= b0) continue;
     if (!X.resident) xc_launch_ao(P, b0, b1, s);
-    k_xc_rho<<<b1 - b0, kBP, 0, s>>>(b0, P->nbf, X.d_perm, X.d_nbfb, X.d_bfl, X.d_woff, X.d_work, D, rho, grad);
+    k_xc_rho<<<b1 - b0, 32 * kRhoWarps, sizeof(RhoSmem), s>>>(b0, nbf, X.d_perm, X.d_nbfb, X.d_bfl, X.d_woff, X.d_work,
+                                                             X.d_pexp, D, X.d_ddig, X.d_dscale, X.d_dbad, rho, grad);
     XCK(cudaGetLastError());
   }
   return ERI_OK;
@@ -756,19 +907,20 @@ static int xc_density_impl(eri_plan_impl* P, const double* D, double* rho, doubl
 
 static int xc_matrix_impl(eri_plan_impl* P, const double* vrho, const double* vgrad, double* V, cudaStream_t s) {
   XcState& X = P->xc;
-  const int nbf = P->nbf, T = (nbf + kVT - 1) / kVT, npairs = T * (T + 1) / 2;
+  const int nbf = P->nbf;
   XCK(cudaMemsetAsync(V, 0, sizeof(double) * (size_t)nbf * nbf, s));
-  XCK(cudaFuncSetAttribute(k_xc_vmat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVmatSmem));
+  XCK(cudaFuncSetAttribute(k_xc_vmat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(VmatSmem)));
   for (size_t c = 0; c + 1 < X.chunk.size(); ++c) {
     const int b0 = X.chunk[c], b1 = X.chunk[c + 1];
     if (b1 <= b0) continue;
     if (!X.resident) xc_launch_ao(P, b0, b1, s);
-    k_xc_z<<<b1 - b0, kBP, 0, s>>>(b0, X.d_perm, X.d_nbfb, X.d_woff, X.d_w, vrho, vgrad, X.d_work);
-    const int nsplit = std::max(1, std::min(b1 - b0, (24 * P->nsm + npairs - 1) / npairs));
-    k_xc_vmat<<<dim3(npairs, nsplit), kVThreads, kVmatSmem, s>>>(b0, b1, nsplit, nbf, X.d_nbfb, X.d_bfl, X.d_woff,
-                                                                 X.d_work, V);
+    k_xc_z<<<b1 - b0, kBP, 0, s>>>(b0, X.d_perm, X.d_nbfb, X.d_woff, X.d_w, vrho, vgrad, X.d_work, X.d_zbad);
+    k_xc_vmat<<<b1 - b0, 32 * kVWarps, sizeof(VmatSmem), s>>>(b0, nbf, X.d_nbfb, X.d_bfl, X.d_woff, X.d_work, X.d_zbad,
+                                                             V);
     XCK(cudaGetLastError());
   }
+  k_xc_symm<<<nbf, 128, 0, s>>>(nbf, V);
+  XCK(cudaGetLastError());
   return ERI_OK;
 }
 
