@@ -354,10 +354,10 @@ __global__ void __launch_bounds__(kBP) k_xc_ao(int b0, const int* __restrict__ p
   pexp[(int64_t)b * kBP + t] = emax;
 }
 
-// Digits of D, 8 bf16 per element (one 16-byte row), row by row under the row's
-// exponent, and each row's scale; a row with an infinity or NaN is marked bad
+// Digits of D, 8 f16 per element (16 bytes), row by row under the row's exponent,
+// which is kept (2047: the row holds an infinity or NaN)
 __global__ void __launch_bounds__(256) k_xc_ddigits(int nbf, const double* __restrict__ D, uint4* __restrict__ Dd,
-                                                    double* __restrict__ scale, int* __restrict__ bad) {
+                                                    int* __restrict__ dexp) {
   __shared__ int red[8];
   const int r = blockIdx.x, t = threadIdx.x;
   const double* row = D + (int64_t)r * nbf;
@@ -368,15 +368,10 @@ __global__ void __launch_bounds__(256) k_xc_ddigits(int nbf, const double* __res
   __syncthreads();
 #pragma unroll
   for (int x = 0; x < 8; ++x) E = max(E, red[x]);
-  if (t == 0) {
-    scale[r] = digit_scale(E);
-    bad[r] = E == 2047;
-  }
+  if (t == 0) dexp[r] = E;
   for (int c = t; c < nbf; c += blockDim.x) {
-    uint32_t d[kDigits];
-    digits_of(row[c], E, d);
-    Dd[(int64_t)r * nbf + c] = make_uint4(bf16_pair(d[0], d[1]), bf16_pair(d[2], d[3]), bf16_pair(d[4], d[5]),
-                                          bf16_pair(d[6], d[7]));
+    const unsigned long long u = digits_of(row[c], E);
+    Dd[(int64_t)r * nbf + c] = make_uint4(digit_two(u, 0), digit_two(u, 2), digit_two(u, 4), digit_two(u, 6));
   }
 }
 
@@ -392,13 +387,13 @@ struct RhoSmem {
   uint2 B[kKC / 16][kBP / 8][kDigits][32];
   double X[kRhoWarps][16][kBP];
   double sum[kRhoWarps][4][kBP];
-  double pscale[kBP];
+  int pexp[kBP];
 };
 __global__ void __launch_bounds__(32 * kRhoWarps, 2)
     k_xc_rho(int b0, int nbf, const int* __restrict__ perm, const int* __restrict__ nbfb, const int* __restrict__ bfl,
              const int64_t* __restrict__ woff, const double* __restrict__ work, const int* __restrict__ pexp,
-             const double* __restrict__ D, const uint4* __restrict__ Dd, const double* __restrict__ dscale,
-             const int* __restrict__ dbad, double* __restrict__ rho, double* __restrict__ grad) {
+             const double* __restrict__ D, const uint4* __restrict__ Dd, const int* __restrict__ dexp,
+             double* __restrict__ rho, double* __restrict__ grad) {
   extern __shared__ __align__(16) unsigned char smraw[];
   RhoSmem& S = *reinterpret_cast<RhoSmem*>(smraw);
   const int b = b0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
@@ -406,7 +401,7 @@ __global__ void __launch_bounds__(32 * kRhoWarps, 2)
   const int* L = bfl + (int64_t)b * nbf;
   const double* W = work + woff[b];
   int isbad = 0;
-  for (int i = tid; i < n; i += 32 * kRhoWarps) isbad |= dbad[L[i]];
+  for (int i = tid; i < n; i += 32 * kRhoWarps) isbad |= dexp[L[i]] == 2047;
   isbad = __syncthreads_or(isbad);
   double sum[4] = {0.0, 0.0, 0.0, 0.0};  // rho, grad rho / 2 of point `lane` over this warp's rows
   auto add_row = [&](int row, double x) {
@@ -421,7 +416,7 @@ __global__ void __launch_bounds__(32 * kRhoWarps, 2)
     }
   } else {
     const int g = lane >> 2, t = lane & 3;  // operand row and column pair of this lane
-    if (tid < kBP) S.pscale[tid] = digit_scale(pexp[(int64_t)b * kBP + tid]);
+    if (tid < kBP) S.pexp[tid] = pexp[(int64_t)b * kBP + tid];
     for (int mg = 0; mg < n; mg += 16 * kRhoWarps) {
       const int m0 = mg + 16 * wp;
       const int64_t r0 = (int64_t)L[min(m0 + g, n - 1)] * nbf, r1 = (int64_t)L[min(m0 + g + 8, n - 1)] * nbf;
@@ -441,12 +436,11 @@ __global__ void __launch_bounds__(32 * kRhoWarps, 2)
           for (int e = tid; e < nks * (kBP / 8) * 64; e += 32 * kRhoWarps) {
             const int el = e & 31, h = (e >> 5) & 1, nt = (e >> 6) & (kBP / 8 - 1), ks = e >> 8;
             const int k = kc + 16 * ks + 2 * (el & 3) + 8 * h, p = 8 * nt + (el >> 2);
-            const int E = pexp[(int64_t)b * kBP + p];
-            uint32_t d0[kDigits], d1[kDigits];
-            digits_of(k < n ? W[(int64_t)k * kBP + p] : 0.0, E, d0);
-            digits_of(k + 1 < n ? W[(int64_t)(k + 1) * kBP + p] : 0.0, E, d1);
+            const int E = S.pexp[p];
+            const unsigned long long u0 = digits_of(k < n ? W[(int64_t)k * kBP + p] : 0.0, E);
+            const unsigned long long u1 = digits_of(k + 1 < n ? W[(int64_t)(k + 1) * kBP + p] : 0.0, E);
 #pragma unroll
-            for (int x = 0; x < kDigits; ++x) (&S.B[ks][nt][x][el].x)[h] = bf16_pair(d0[x], d1[x]);
+            for (int x = 0; x < kDigits; ++x) (&S.B[ks][nt][x][el].x)[h] = digit_pair(u0, u1, x);
           }
           __syncthreads();
           if (m0 < n) {
@@ -474,20 +468,20 @@ __global__ void __launch_bounds__(32 * kRhoWarps, 2)
                   const uint2 bb = S.B[ks][nt][y][lane];
 #pragma unroll
                   for (int x = 0; x < kDigits; ++x)
-                    if (x + y < kWeights) mma_bf16(acc[nt][x + y], a[x], bb);
+                    if (x + y < kWeights) mma_f16(acc[nt][x + y], a[x], bb);
                 }
             }
           }
         }
         if (m0 < n) {
-          const double s0 = dscale[L[min(m0 + g, n - 1)]], s1 = dscale[L[min(m0 + g + 8, n - 1)]];
+          const int e0 = dexp[L[min(m0 + g, n - 1)]], e1 = dexp[L[min(m0 + g + 8, n - 1)]];
           __syncwarp();
 #pragma unroll
           for (int nt = 0; nt < kBP / 8; ++nt)
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
               const int p = 8 * nt + 2 * t + (c & 1);
-              S.X[wp][g + 8 * (c >> 1)][p] = combine(acc[nt], c) * (c < 2 ? s0 : s1) * S.pscale[p];
+              S.X[wp][g + 8 * (c >> 1)][p] = combine<false>(acc[nt], c, c < 2 ? e0 : e1, S.pexp[p]);
             }
           __syncwarp();
           const int nr = min(16, n - m0);
@@ -614,11 +608,9 @@ __device__ __forceinline__ int operand_digits(const double* row, int t, uint32_t
   for (int s = 0; s < 2; ++s)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      uint32_t lo[kDigits], hi[kDigits];
-      digits_of(v[s][h].x, E, lo);
-      digits_of(v[s][h].y, E, hi);
+      const unsigned long long lo = digits_of(v[s][h].x, E), hi = digits_of(v[s][h].y, E);
 #pragma unroll
-      for (int x = 0; x < kDigits; ++x) d[s][h][x] = bf16_pair(lo[x], hi[x]);
+      for (int x = 0; x < kDigits; ++x) d[s][h][x] = digit_pair(lo, hi, x);
     }
   return E;
 }
@@ -631,8 +623,7 @@ __device__ __forceinline__ int operand_digits(const double* row, int t, uint32_t
 // workload 1 at 32 x 32.)
 struct VmatSmem {
   uint2 B[kVC / 8][2][kDigits][32];
-  double scale[kVC];
-  int ao[kVC];
+  int exp[kVC], ao[kVC];
 };
 __global__ void __launch_bounds__(32 * kVWarps, 2)
     k_xc_vmat(int b0, int nbf, const int* __restrict__ nbfb, const int* __restrict__ bfl,
@@ -667,7 +658,7 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
 #pragma unroll
         for (int x = 0; x < kDigits; ++x) S.B[nt][s][x][lane] = make_uint2(d[s][0][x], d[s][1][x]);
       if (t == 0) {
-        S.scale[8 * nt + g] = digit_scale(E);
+        S.exp[8 * nt + g] = E;
         S.ao[8 * nt + g] = L[j];
       }
     }
@@ -675,10 +666,10 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
     for (int m0 = 16 * wp; m0 < n; m0 += 16 * kVWarps) {
       const int i0 = min(m0 + g, n - 1), i1 = min(m0 + g + 8, n - 1);
       uint32_t a[2][kDigits][4];
-      double s0, s1;
+      int e0, e1;
       {
         uint32_t d[2][2][kDigits];
-        s0 = digit_scale(operand_digits(Z + (int64_t)i0 * kBP, t, d));
+        e0 = operand_digits(Z + (int64_t)i0 * kBP, t, d);
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -686,7 +677,7 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
             a[s][x][0] = d[s][0][x];
             a[s][x][2] = d[s][1][x];
           }
-        s1 = digit_scale(operand_digits(Z + (int64_t)i1 * kBP, t, d));
+        e1 = operand_digits(Z + (int64_t)i1 * kBP, t, d);
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -703,7 +694,7 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
 #pragma unroll
         for (int k = 0; k < kWeights; ++k)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) acc[k][c] = 0.0f;
+          for (int c = 0; c < 4; ++c) acc[k][c] = kMagic;
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -711,13 +702,13 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
             const uint2 bb = S.B[nt][s][y][lane];
 #pragma unroll
             for (int x = 0; x < kDigits; ++x)
-              if (x + y < kWeights) mma_bf16(acc[x + y], a[s][x], bb);
+              if (x + y < kWeights) mma_f16(acc[x + y], a[s][x], bb);
           }
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const int jl = 8 * nt + 2 * t + (c & 1);
           if (jl >= nj || !(c < 2 ? ok0 : ok1)) continue;
-          const double v = combine(acc, c) * (c < 2 ? s0 : s1) * S.scale[jl];
+          const double v = combine<true>(acc, c, c < 2 ? e0 : e1, S.exp[jl]);
           if (v != 0.0) atomicAdd((c < 2 ? v0 : v1) + S.ao[jl], v);
         }
       }
@@ -744,7 +735,7 @@ __global__ void k_xc_symm(int nbf, double* __restrict__ V) {
 void eri_plan_impl::xc_release() {
   void* ptrs[] = {xc.d_pts, xc.d_w, xc.d_rad, xc.d_ang, xc.d_invab, xc.d_perm, xc.d_bsph, xc.d_ext, xc.d_nsh,
                   xc.d_shl, xc.d_shoff, xc.d_nbfb, xc.d_bfl, xc.d_woff, xc.d_work, xc.d_rho, xc.d_grad,
-                  xc.d_vrho, xc.d_vgrad, xc.d_pexp, xc.d_ddig, xc.d_dscale, xc.d_dbad, xc.d_zbad};
+                  xc.d_vrho, xc.d_vgrad, xc.d_pexp, xc.d_ddig, xc.d_dexp, xc.d_zbad};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   xc = XcState{};
@@ -799,8 +790,7 @@ static int xc_build(eri_plan_impl* P, cudaStream_t s) {
   XCK(xalloc(&X.d_vgrad, 3 * (size_t)X.npts));
   XCK(xalloc(&X.d_pexp, (size_t)nb * kBP));
   XCK(xalloc(&X.d_ddig, (size_t)nbf * nbf));
-  XCK(xalloc(&X.d_dscale, (size_t)nbf));
-  XCK(xalloc(&X.d_dbad, (size_t)nbf));
+  XCK(xalloc(&X.d_dexp, (size_t)nbf));
   XCK(xalloc(&X.d_zbad, (size_t)nb));
   XCK(cudaMemcpyAsync(X.d_perm, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice, s));
   const int nt = std::max(nrad, nth);
@@ -892,14 +882,14 @@ static int xc_density_impl(eri_plan_impl* P, const double* D, double* rho, doubl
   XcState& X = P->xc;
   const int nbf = P->nbf;
   XCK(cudaFuncSetAttribute(k_xc_rho, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RhoSmem)));
-  k_xc_ddigits<<<nbf, 256, 0, s>>>(nbf, D, X.d_ddig, X.d_dscale, X.d_dbad);
+  k_xc_ddigits<<<nbf, 256, 0, s>>>(nbf, D, X.d_ddig, X.d_dexp);
   XCK(cudaGetLastError());
   for (size_t c = 0; c + 1 < X.chunk.size(); ++c) {
     const int b0 = X.chunk[c], b1 = X.chunk[c + 1];
     if (b1 <= b0) continue;
     if (!X.resident) xc_launch_ao(P, b0, b1, s);
     k_xc_rho<<<b1 - b0, 32 * kRhoWarps, sizeof(RhoSmem), s>>>(b0, nbf, X.d_perm, X.d_nbfb, X.d_bfl, X.d_woff, X.d_work,
-                                                             X.d_pexp, D, X.d_ddig, X.d_dscale, X.d_dbad, rho, grad);
+                                                             X.d_pexp, D, X.d_ddig, X.d_dexp, rho, grad);
     XCK(cudaGetLastError());
   }
   return ERI_OK;

@@ -1,14 +1,14 @@
 // FP64 products on the tensor cores for the exchange-correlation contractions.
 //
 // What bounds them otherwise: GB300's FP64 pipe, 1.06 TFLOP/s, against 0.6
-// PFLOP/s of mma.sync bf16 (both measured).  A row of operands is written as
+// PFLOP/s of mma.sync f16 (both measured).  A row of operands is written as
 // integers q = rint(v 2^(55 - e)) under the row's common power of two 2^e >
-// max |v|, and q as 8 signed digits of 7 bits, |digit| <= 64, which bf16 holds
+// max |v|, and q as 8 signed digits of 7 bits, |digit| <= 64, which f16 holds
 // exactly.  A product of two digits is at most 2^12, so the FP32 accumulator of
 // the tensor core holds the sum of the up to 8 digit products of one weight
 // (i + j = k) over 512 terms exactly (8 x 512 x 2^12 = 2^24): no rounding
-// happens before the nine sums of weights k = 0..8 are put together, in 64-bit
-// integers and one FP64 FMA.  43 bf16 products replace one FP64 product; the
+// happens before the nine sums of weights k = 0..8 are put together, in
+// integers and rounded once.  43 f16 products replace one FP64 product; the
 // pairs left out (k > 8) are below 2^-63 of 2^(e_a + e_b) per term, and the
 // digits represent an operand to 2^-56 of its row's maximum, where a plain FP64
 // sum rounds every step to 2^-53 of its partial sum.
@@ -18,6 +18,7 @@
 // gathered (digit rows of D at the block's functions) or converted (Z).
 #pragma once
 #include <cstdint>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 namespace eri {
@@ -31,49 +32,84 @@ __device__ __forceinline__ int exponent_of(double v) {
   return (int)((unsigned)__double2hiint(v) >> 20 & 0x7ffu);
 }
 
-// The digits of v under the row exponent E = max exponent_of: bf16 of the digits
-// in the high halves of d[0] (most significant) .. d[7]
-__device__ __forceinline__ void digits_of(double v, int E, uint32_t* d) {
+// v as an integer under the row exponent E = max exponent_of, 64 added to every
+// digit: digit i (0: most significant) + 64 = bits 7 (7 - i) .., 7 bits each, the
+// top one 8 (0..128)
+__device__ __forceinline__ unsigned long long digits_of(double v, int E) {
   const long long bits = __double_as_longlong(v);
   const int ex = (int)(bits >> 52) & 0x7ff, r = E - ex - 2;  // q = mantissa 2^-r
   long long m = ex ? ((bits & 0xfffffffffffffLL) | 0x10000000000000LL) : 0LL;
   if (r <= 0) m <<= -r;
   else m = r < 56 ? (m + (1LL << (r - 1))) >> r : 0LL;
-  // + 64 in every digit: unsigned digits 0..127 (the top one 0..128)
-  constexpr long long kBias = 64LL * 0x2040810204081LL;  // 64 (128^8 - 1) / 127, top digit included
-  const unsigned long long u = (unsigned long long)((bits < 0 ? -m : m) + kBias);
-#pragma unroll
-  for (int i = 0; i < kDigits; ++i) {
-    const unsigned x = (unsigned)(u >> (7 * (kDigits - 1 - i))) & (i == 0 ? 0xffu : 0x7fu);
-    d[i] = __float_as_uint(__uint_as_float(0x4b000000u | x) - 8388672.0f);  // x - 64, exact in bf16
-  }
+  constexpr long long kBias = 64LL * 0x2040810204081LL;  // 64 (128^8 - 1) / 127
+  return (unsigned long long)((bits < 0 ? -m : m) + kBias);
 }
-// bf16 pair (k, k + 1) of one digit from two such words
-__device__ __forceinline__ uint32_t bf16_pair(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }
-
-// scale of a row with exponent E, so that value = combine() * scale_a * scale_b;
-// rows below 2^-960 count as zero
-__device__ __forceinline__ double digit_scale(int E) {
-  return E > 63 ? __longlong_as_double((long long)(E - 33) << 52) : 0.0;
+// (x + 1024) halves -> x - 64, both exact
+__device__ __forceinline__ uint32_t unbias(uint32_t w) {
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), __half2half2(__ushort_as_half(0x6440)));
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+// digit i of two values as an f16 pair (u0 in the low half)
+__device__ __forceinline__ uint32_t digit_pair(unsigned long long u0, unsigned long long u1, int i) {
+  const int s = 7 * (kDigits - 1 - i);
+  const uint32_t mask = i == 0 ? 0xffu : 0x7fu;
+  return unbias(((uint32_t)(u0 >> s) & mask) | (((uint32_t)(u1 >> s) & mask) << 16) | 0x64006400u);
+}
+// digits i and i + 1 of one value as an f16 pair
+__device__ __forceinline__ uint32_t digit_two(unsigned long long u, int i) {
+  const int s = 7 * (kDigits - 1 - i);
+  const uint32_t mask = i == 0 ? 0xffu : 0x7fu;
+  return unbias(((uint32_t)(u >> s) & mask) | (((uint32_t)(u >> (s - 7)) & 0x7fu) << 16) | 0x64006400u);
 }
 
-// D[16 x 8] += A[16 x 16] B[16 x 8], bf16 operands, FP32 accumulators
-__device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint2& b) {
+// D[16 x 8] += A[16 x 16] B[16 x 8], f16 operands, FP32 accumulators
+__device__ __forceinline__ void mma_f16(float* c, const uint32_t* a, const uint2& b) {
   asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
 }
 
-// the nine exact sums of element c of a tile -> sum 2^(-7 k) s_k, times 2^56
-template <int N>
-__device__ __forceinline__ double combine(const float (&acc)[kWeights][N], int c) {
-  long long hi = 0, lo = 0;
+// Accumulators of products with at most kShortTerms terms may start at kMagic =
+// 1.5 2^23: a sum below 2^22 is then the low bits of the FP32 word, which saves
+// the conversions.
+constexpr int kShortTerms = 128;
+constexpr float kMagic = 12582912.0f;
+constexpr int kMagicBits = 0x4b400000;
+
+// value of element c of a tile whose rows have the exponents Ea (operand a) and Eb:
+// the nine exact sums s_k are put together as (hi 2^35 + lo) 2^-56 and rounded
+// once, in integers (the FP64 pipe is 30 times slower); values below 2^-1022
+// count as zero
+template <bool MAGIC>
+__device__ __forceinline__ double combine(const float (&acc)[kWeights][4], int c, int Ea, int Eb) {
+  int s[kWeights];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) hi = hi * 128 + __float2int_rn(acc[k][c]);
-#pragma unroll
-  for (int k = 4; k < kWeights; ++k) lo = lo * 128 + __float2int_rn(acc[k][c]);
-  return fma((double)hi, 34359738368.0 /* 2^35 */, (double)lo);
+  for (int k = 0; k < kWeights; ++k)
+    s[k] = MAGIC ? __float_as_int(acc[k][c]) - kMagicBits : __float2int_rn(acc[k][c]);
+  const long long hi = (long long)(s[0] * 128 + s[1]) * 16384 + (s[2] * 128LL + s[3]);
+  const long long lo = ((long long)(s[4] * 128LL + s[5]) * 16384 + (s[6] * 128LL + s[7])) * 128 + s[8];
+  unsigned long long l = ((unsigned long long)hi << 35) + (unsigned long long)lo;
+  long long h = (hi >> 29) + (lo >> 63) + (l < (unsigned long long)lo ? 1 : 0);
+  const bool neg = h < 0;
+  if (neg) {
+    l = 0ULL - l;
+    h = ~h + (l == 0 ? 1 : 0);
+  }
+  unsigned long long top = (unsigned long long)h, low = l;
+  int e = 127 + Ea + Eb - 1089;  // biased exponent of a leading one in bit 127
+  if (top == 0) {
+    top = low;
+    low = 0;
+    e -= 64;
+  }
+  const int n = __clzll((long long)top);
+  e -= n;
+  const unsigned long long m = n ? top << n | low >> (64 - n) : top;
+  if (m == 0 || e <= 0) return 0.0;
+  if (e >= 2047) return neg ? -__longlong_as_double(0x7ff0000000000000LL) : __longlong_as_double(0x7ff0000000000000LL);
+  const unsigned long long r = ((unsigned long long)(e - 1) << 52) + (m >> 11) + (m >> 10 & 1);
+  return __longlong_as_double((long long)(r | (neg ? 1ULL << 63 : 0ULL)));
 }
 
 }  // namespace eri

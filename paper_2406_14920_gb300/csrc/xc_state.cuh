@@ -27,9 +27,8 @@ struct XcState {
   size_t work_doubles = 0;
   std::vector<int> chunk;  // block boundaries of the workspace chunks
   int* d_pexp = nullptr;      // largest exponent of phi per block slot (xc_mma.cuh)
-  uint4* d_ddig = nullptr;    // digits of D, its row scales and rows with an infinity or NaN (per call)
-  double* d_dscale = nullptr;
-  int *d_dbad = nullptr, *d_zbad = nullptr;  // d_zbad: blocks with an infinity or NaN in Z
+  uint4* d_ddig = nullptr;    // digits of D and its row exponents (written by each call)
+  int *d_dexp = nullptr, *d_zbad = nullptr;  // d_zbad: blocks with an infinity or NaN in Z
   double *d_rho = nullptr, *d_grad = nullptr, *d_vrho = nullptr, *d_vgrad = nullptr;
   double sum_nb = 0.0, sum_nb2 = 0.0;  // sum over blocks of n_b and n_b^2 (significant functions)
   double sum_nbp = 0.0, sum_nb2p = 0.0;  // the same weighted by each block's number of points
