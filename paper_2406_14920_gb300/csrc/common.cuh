@@ -19,6 +19,7 @@ namespace eri {
 constexpr int LMAX = 3;              // basis functions up to f
 constexpr int LMAX_PAIR = 2 * LMAX;  // Hermite order of a pair
 constexpr int LMAX_QUARTET = 4 * LMAX + 1;  // +1: gradient raises one bra index
+constexpr int kKetGroup = 128;       // kets ordered by their primitive pairs at a time (ket_pos)
 constexpr int NPAIRCLASS = 10;       // ss ps pp ds dp dd fs fp fd ff
 
 // Boys tables on the grid T_k = k * BOYS_H, k = 0..BOYS_NT-1:
@@ -62,20 +63,26 @@ __device__ __forceinline__ void sfor(F&& f) {
 }
 #define ERI_CI(x) decltype(x)::value
 
-// sum_{x <= NX, y <= NY, z <= NZ} cx[x] cy[y] cz[z] v(x, y, z), factored as
+// init + sum_{x <= NX, y <= NY, z <= NZ} cx[x] cy[y] cz[z] v(x, y, z), factored as
 // sum_x cx[x] (sum_y cy[y] (sum_z cz[z] v)).  A direction with N = 0 has the
 // single Hermite coefficient E^{00}_0 = 1 (the exponential factor lives in the
 // pair prefactor), so it contributes no multiplication.  ALT: coefficient of
-// index s carries (-1)^s (the ket sign of Eq. eri_formula).
+// index s carries (-1)^s (the ket sign of Eq. eri_formula).  `init` starts the
+// outermost open direction's chain, so that a sum added to an accumulator costs
+// no separate addition (a seventh of the operations of the (pp|ps) kernel).
 template <int NX, int NY, int NZ, bool ALT, typename T, typename V>
-__device__ __forceinline__ T tsum(const T* cx, const T* cy, const T* cz, V&& v) {
-  T acc = T(0);
+__device__ __forceinline__ T tsum(const T* cx, const T* cy, const T* cz, V&& v, T init = T(0)) {
+  if constexpr (NX == 0 && NY == 0 && NZ == 0) {
+    using Z = std::integral_constant<int, 0>;
+    return init + v(Z{}, Z{}, Z{});
+  }
+  T acc = NX > 0 ? init : T(0);
   sfor<NX + 1>([&](auto ix) {
     constexpr int x = ERI_CI(ix);
-    T accy = T(0);
+    T accy = NX == 0 && NY > 0 ? init : T(0);
     sfor<NY + 1>([&](auto iy) {
       constexpr int y = ERI_CI(iy);
-      T accz = T(0);
+      T accz = NX == 0 && NY == 0 ? init : T(0);
       sfor<NZ + 1>([&](auto iz) {
         constexpr int z = ERI_CI(iz);
         const T val = v(std::integral_constant<int, x>{}, std::integral_constant<int, y>{},
@@ -211,6 +218,7 @@ struct WorkList {
   int64_t first;           // items [first, total) are processed (0 except in tuning trials)
   int tile;                // consecutive items per worker tile (warp kernels: per warp; thread kernel: per lane)
   int shard, nshard;       // this launch takes the tiles t with t % nshard == shard (work split over GPUs)
+  const int32_t* korder;   // ket positions inside their segment in visiting order (parallel to `ket`, see ket_pos)
   int mpb, mpk;            // most primitive pairs of a shell pair in the bra and in the ket class
 };
 

@@ -71,8 +71,8 @@ cudaError_t launch_over(const Args& a, int64_t workers, int per_block, int threa
 // work items of a thread kernel over a list of n items (with the parts of a
 // short list, see prim_split; longer lists fill the grid by themselves)
 template <typename T>
-inline int64_t split_items(const WorkList& wl, int64_t n) {
-  return sizeof(T) == 4 || wl.nshard > 1 ? n : n * wl.mpb * wl.mpk;
+inline int64_t split_items(const WorkList& wl, int64_t n, bool kets = true) {
+  return sizeof(T) == 4 || wl.nshard > 1 ? n : n * wl.mpb * (kets ? wl.mpk : 1);
 }
 
 template <int LA, int LB, int LC, int LD, typename T>
@@ -80,11 +80,16 @@ cudaError_t launch_jk_t(const JKArgs& a, cudaStream_t s, int nsm) {
   const int64_t n = a.k.wl.total - a.k.wl.first;
   if (n <= 0) return cudaSuccess;
   if constexpr (use_thread_kernel(LA, LB, LC, LD, sizeof(T) == 4)) {
+    if constexpr (block_when_short<LA, LB, LC, LD, T>()) {
+      using S = CShape<LA, LB, LC, LD, T>;
+      if (n <= (int64_t)kShortList * nsm)
+        return launch_over<jk_block_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.k.wl, n, false), 1, S::NT, S::smem(), s, nsm);
+    }
     return launch_over<jk_thread_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.k.wl, n), 128, 128, 0, s, nsm);
   } else if constexpr (use_block_kernel<LA, LB, LC, LD, T>()) {
     using S = CShape<LA, LB, LC, LD, T>;
     static_assert(S::smem() <= 227 * 1024, "block kernel exceeds 227 KB");
-    return launch_over<jk_block_kernel<LA, LB, LC, LD, T>>(a, n, 1, S::NT, S::smem(), s, nsm);
+    return launch_over<jk_block_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.k.wl, n, false), 1, S::NT, S::smem(), s, nsm);
   } else {
     using S = BShape<LA, LB, LC, LD, T>;
     constexpr int WPB = 4;
@@ -127,7 +132,7 @@ cudaError_t launch_grad_unit(int y, const GradArgs& a, cudaStream_t s, int nsm) 
       } else {
         using S = GShape<LA, LB, LC, LD, T>;
         static_assert(S::smem() <= 227 * 1024, "gradient block exceeds 227 KB");
-        return launch_over<grad_block_kernel<LA, LB, LC, LD, T>>(a, n, 1, S::NT, S::smem(), s, nsm);
+        return launch_over<grad_block_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.wl, n, false), 1, S::NT, S::smem(), s, nsm);
       }
     }
     return launch_grad_unit<X, P, Y + 1>(y, a, s, nsm);

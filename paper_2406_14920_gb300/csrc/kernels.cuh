@@ -173,23 +173,44 @@ struct PrimSplit {
     k1 = npk * (pk + 1) / sk;
   }
 };
+// (kets = false: bra primitives only, for the block kernels.)
 template <typename T>
-__device__ __forceinline__ PrimSplit prim_split(const WorkList& wl, int64_t items, int64_t lanes) {
+__device__ __forceinline__ PrimSplit prim_split(const WorkList& wl, int64_t items, int64_t lanes, bool kets = true) {
   PrimSplit s{1, 1, 1};
   if (sizeof(T) == 4 || wl.nshard > 1 || items <= 0 || 2 * items > lanes) return s;
   const int64_t room = lanes / items;
   s.sb = (int)(room < wl.mpb ? room : wl.mpb);
   const int64_t rk = room / s.sb;
-  s.sk = (int)(rk < wl.mpk ? rk : wl.mpk);
+  s.sk = kets ? (int)(rk < wl.mpk ? rk : wl.mpk) : 1;
   s.n = s.sb * s.sk;
   return s;
 }
 
-// Items per tile of a block kernel: wl.tile, fewer when that would leave blocks idle
-__device__ __forceinline__ int64_t block_tile(const WorkList& wl, int64_t items) {
+// Rounds of 32 items per tile of a thread kernel over the ordered lists: wl.tile
+// (long runs share a bra pair, whose sums go out together), fewer on lists that
+// would leave warps idle (185 functions, J-engine (ps|ps): 9.4 -> 6.0 ms)
+__device__ __forceinline__ int64_t thread_tile(const WorkList& wl, int64_t items, int64_t warps) {
   if (wl.nshard > 1) return wl.tile;
-  const int64_t t = items / (2 * (int64_t)gridDim.x);
+  const int64_t t = items / (64 * warps);
   return t < 1 ? 1 : (t < wl.tile ? t : wl.tile);
+}
+
+// Items per tile of a kernel whose `workers` warps or blocks take one item at a
+// time: wl.tile, fewer when that would leave workers idle
+__device__ __forceinline__ int64_t item_tile(const WorkList& wl, int64_t items, int64_t workers) {
+  if (wl.nshard > 1) return wl.tile;
+  const int64_t t = items / (2 * workers);
+  return t < 1 ? 1 : (t < wl.tile ? t : wl.tile);
+}
+
+// Ket position of list item ik of a bra pair with `count` kets.  Primitive
+// screening leaves the shell pairs of a class with different numbers of primitive
+// pairs, and a warp of a thread kernel takes as long as its longest item: every
+// full group of kKetGroup kets (in the order of the lists, Q descending) is
+// visited by decreasing number of primitive pairs (k_ketorder), so that the 32
+// lanes have about as many.
+__device__ __forceinline__ int ket_pos(const WorkList& wl, int seg, int ik, int64_t count) {
+  return (ik | (kKetGroup - 1)) < count ? __ldg(wl.korder + seg + ik) : ik;
 }
 
 template <typename T> __device__ __forceinline__ T ldT(const double* p) { return (T)__ldg(p); }
@@ -323,7 +344,7 @@ __global__ void __launch_bounds__(128) j_warp_kernel(JArgs a) {
   const int64_t first = compact ? 0 : a.wl.first;
   const int nshard = compact ? 1 : a.wl.nshard, shard = compact ? 0 : a.wl.shard;
   unsigned long long done = 0, doneq = 0, doneb = 0;
-  const int64_t tile = a.wl.tile, ntiles = (total - first + tile - 1) / tile;
+  const int64_t tile = item_tile(a.wl, total - first, nwarps), ntiles = (total - first + tile - 1) / tile;
   for (int64_t tl = ((int64_t)blockIdx.x * (blockDim.x >> 5) + wib) * nshard + shard; tl < ntiles;
        tl += nwarps * nshard) {
   const int64_t i0 = first + tl * tile, i1 = i0 + tile < total ? i0 + tile : total;
@@ -421,8 +442,8 @@ __global__ void __launch_bounds__(128) j_thread_kernel(JArgs a) {
   const int64_t total = compact ? (int64_t)__ldg(a.nitems) : a.wl.total;
   const int64_t first = compact ? 0 : a.wl.first;
   const int nshard = compact ? 1 : a.wl.nshard, shard = compact ? 0 : a.wl.shard;
-  const int64_t span = 32 * (int64_t)a.wl.tile, ntiles = (total - first + span - 1) / span;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int64_t span = 32 * thread_tile(a.wl, total - first, nwarps), ntiles = (total - first + span - 1) / span;
   unsigned long long done = 0, doneq = 0, doneb = 0;
   const PrimSplit sp = prim_split<T>(a.wl, total - first, 32 * nwarps);
   for (int64_t tl = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * nshard + shard;
@@ -447,7 +468,9 @@ __global__ void __launch_bounds__(128) j_thread_kernel(JArgs a) {
         }
         pb_id = __ldg(a.wl.bra + ib);
         const int mol = __ldg(a.sp.pmol + pb_id);
-        const int pk_id = __ldg(a.wl.ket + __ldg(a.wl.kseg + mol * NPAIRCLASS) + ik);
+        const int seg = __ldg(a.wl.kseg + mol * NPAIRCLASS);
+        if (!compact) ik = ket_pos(a.wl, seg, ik, cur.be - cur.bs);
+        const int pk_id = __ldg(a.wl.ket + seg + ik);
         npb = __ldg(a.sp.np + pb_id);
         offb = __ldg(a.sp.poff + pb_id);
         hb = __ldg(a.sp.hoff + pb_id);

@@ -81,10 +81,10 @@ __device__ __forceinline__ void load_or_build_e(const PairData& pd, int e0, cons
 // exponents), one bra Hermite index P = (t, u, v):
 //   sum_Q (-1)^|Q| E_Q^{cd} R_{P+Q}
 template <int L, int KX, int KY, int KZ, int T_, int U_, int V_, typename T>
-__device__ __forceinline__ T ket_term(const T* ex, const T* ey, const T* ez, const T* R) {
+__device__ __forceinline__ T ket_term(const T* ex, const T* ey, const T* ez, const T* R, T init = T(0)) {
   return tsum<KX, KY, KZ, true>(ex, ey, ez, [&](auto sx, auto sy, auto sz) {
     return R[herm_index(T_ + ERI_CI(sx), U_ + ERI_CI(sy), V_ + ERI_CI(sz))];
-  });
+  }, init);
 }
 
 // Variant for classes whose W (all ket pairs) does not fit in registers: the
@@ -136,8 +136,9 @@ __device__ __forceinline__ void eri_block_reg_pq(const KArgs& a, int offb, int p
               const T* fx = eb + 0 * S::NEB + (IX * (LB + 1) + JX) * (LAB + 1);
               const T* fy = eb + 1 * S::NEB + (IY * (LB + 1) + JY) * (LAB + 1);
               const T* fz = eb + 2 * S::NEB + (IZ * (LB + 1) + JZ) * (LAB + 1);
-              X[iab * S::NCD + icd] += tsum<IX + JX, IY + JY, IZ + JZ, false>(
-                  fx, fy, fz, [&](auto tx, auto ty, auto tz) { return W[herm_index(ERI_CI(tx), ERI_CI(ty), ERI_CI(tz))]; });
+              X[iab * S::NCD + icd] = tsum<IX + JX, IY + JY, IZ + JZ, false>(
+                  fx, fy, fz, [&](auto tx, auto ty, auto tz) { return W[herm_index(ERI_CI(tx), ERI_CI(ty), ERI_CI(tz))]; },
+                  X[iab * S::NCD + icd]);
             });
           });
         });
@@ -182,8 +183,8 @@ __device__ __forceinline__ void eri_block_reg(const KArgs& a, int offb, int pb0,
           const T* ey = ek + 1 * S::NEK + (KY * (LD + 1) + LY) * (LCD + 1);
           const T* ez = ek + 2 * S::NEK + (KZ * (LD + 1) + LZ) * (LCD + 1);
           for_herm<LAB>([&](auto t, auto u, auto v) {
-            W[icd * S::HAB + herm_index(ERI_CI(t), ERI_CI(u), ERI_CI(v))] +=
-                ket_term<L, KX + LX, KY + LY, KZ + LZ, ERI_CI(t), ERI_CI(u), ERI_CI(v)>(ex, ey, ez, R);
+            T& w = W[icd * S::HAB + herm_index(ERI_CI(t), ERI_CI(u), ERI_CI(v))];
+            w = ket_term<L, KX + LX, KY + LY, KZ + LZ, ERI_CI(t), ERI_CI(u), ERI_CI(v)>(ex, ey, ez, R, w);
           });
         });
       });
@@ -200,9 +201,10 @@ __device__ __forceinline__ void eri_block_reg(const KArgs& a, int offb, int pb0,
           const T* fx = eb + 0 * S::NEB + (IX * (LB + 1) + JX) * (LAB + 1);
           const T* fy = eb + 1 * S::NEB + (IY * (LB + 1) + JY) * (LAB + 1);
           const T* fz = eb + 2 * S::NEB + (IZ * (LB + 1) + JZ) * (LAB + 1);
-          X[iab * S::NCD + icd] += tsum<IX + JX, IY + JY, IZ + JZ, false>(
+          X[iab * S::NCD + icd] = tsum<IX + JX, IY + JY, IZ + JZ, false>(
               fx, fy, fz,
-              [&](auto tx, auto ty, auto tz) { return W[icd * S::HAB + herm_index(ERI_CI(tx), ERI_CI(ty), ERI_CI(tz))]; });
+              [&](auto tx, auto ty, auto tz) { return W[icd * S::HAB + herm_index(ERI_CI(tx), ERI_CI(ty), ERI_CI(tz))]; },
+              X[iab * S::NCD + icd]);
         });
       });
     });
@@ -290,14 +292,15 @@ __device__ __forceinline__ void contract_block(const JKArgs& A, const T* X, T w,
 
 // One quartet (bra position ib, ket position ik of the work list) of a thread-kernel class.
 template <int LA, int LB, int LC, int LD, typename T>
-__device__ __forceinline__ void thread_item(const JKArgs& A, int ib, int ik, const PrimSplit& sp, int part,
+__device__ __forceinline__ void thread_item(const JKArgs& A, int ib, int ik, int64_t nket, const PrimSplit& sp, int part,
                                             unsigned long long& done, unsigned long long& doneq,
                                             unsigned long long& doneb) {
   using S = AShape<LA, LB, LC, LD>;
   const KArgs& a = A.k;
   const int pb_id = __ldg(a.wl.bra + ib);
   const int mol = __ldg(a.sp.pmol + pb_id);
-  const int pk_id = __ldg(a.wl.ket + __ldg(a.wl.kseg + mol * NPAIRCLASS) + ik);
+  const int seg = __ldg(a.wl.kseg + mol * NPAIRCLASS);
+  const int pk_id = __ldg(a.wl.ket + seg + ket_pos(a.wl, seg, ik, nket));  // nket = 0: ik is a position already
   const int s1 = __ldg(a.sp.s1 + pb_id), s2 = __ldg(a.sp.s2 + pb_id);
   const int s3 = __ldg(a.sp.s1 + pk_id), s4 = __ldg(a.sp.s2 + pk_id);
   const int npb_ = __ldg(a.sp.np + pb_id), npk_ = __ldg(a.sp.np + pk_id);
@@ -350,13 +353,13 @@ __global__ void __launch_bounds__(128) jk_thread_kernel(JKArgs A) {
     if (compact) {
       for (int64_t item = i0; item < i1; item += 32) {
         const int2 v = __ldg(a.items + item);
-        thread_item<LA, LB, LC, LD, T>(A, v.x, v.y, sp, part, done, doneq, doneb);
+        thread_item<LA, LB, LC, LD, T>(A, v.x, v.y, 0, sp, part, done, doneq, doneb);
       }
     } else {
       BraCursor cur(a.wl, i0);
       for (int64_t item = i0; item < i1; item += 32) {
         const int ik = cur.at(a.wl, item);
-        thread_item<LA, LB, LC, LD, T>(A, cur.ib, ik, sp, part, done, doneq, doneb);
+        thread_item<LA, LB, LC, LD, T>(A, cur.ib, ik, cur.be - cur.bs, sp, part, done, doneq, doneb);
       }
     }
   }

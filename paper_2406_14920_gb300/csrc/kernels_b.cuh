@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
   const int64_t first = compact ? 0 : a.wl.first;
   const int nshard = compact ? 1 : a.wl.nshard, shard = compact ? 0 : a.wl.shard;
   unsigned long long done = 0, doneq = 0, doneb = 0;
-  const int64_t tile = a.wl.tile, ntiles = (total - first + tile - 1) / tile;
+  const int64_t tile = item_tile(a.wl, total - first, nwarps), ntiles = (total - first + tile - 1) / tile;
   for (int64_t tl = ((int64_t)blockIdx.x * (blockDim.x >> 5) + wib) * nshard + shard; tl < ntiles;
        tl += nwarps * nshard) {
   const int64_t t0 = first + tl * tile, i1 = t0 + tile < total ? t0 + tile : total;
@@ -349,10 +349,10 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
                     constexpr int j = ERI_CI(j_);
                     if (j * 32 + 32 <= HAB || lane + 32 * j < HAB) {
                       const T* r = rbox + pslot[j];
-                      wreg[j * NCD + icd] += tsum<KX + LX, KY + LY, KZ + LZ, false>(
+                      wreg[j * NCD + icd] = tsum<KX + LX, KY + LY, KZ + LZ, false>(
                           ex, ey, ez, [&](auto sx, auto sy, auto sz) {
                             return r[(ERI_CI(sx) * B + ERI_CI(sy)) * B + ERI_CI(sz)];
-                          });
+                          }, wreg[j * NCD + icd]);
                     }
                   });
                 });
@@ -411,10 +411,10 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
                   const T* fx = Eb + (IX * (LB + 1) + JX) * (LAB + 1);
                   const T* fy = Eb + NEB + (IY * (LB + 1) + JY) * (LAB + 1);
                   const T* fz = Eb + 2 * NEB + (IZ * (LB + 1) + JZ) * (LAB + 1);
-                  xreg[j * NAB + iab] += tsum<IX + JX, IY + JY, IZ + JZ, false>(
+                  xreg[j * NAB + iab] = tsum<IX + JX, IY + JY, IZ + JZ, false>(
                       fx, fy, fz, [&](auto tx, auto ty, auto tz) {
                         return wc[lex_base(LAB, ERI_CI(tx), ERI_CI(ty)) + ERI_CI(tz)];
-                      });
+                      }, xreg[j * NAB + iab]);
                 });
               });
             }

@@ -207,9 +207,11 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
   const int64_t first = compact ? 0 : a.wl.first;
   const int nshard = compact ? 1 : a.wl.nshard, shard = compact ? 0 : a.wl.shard;
   unsigned long long done = 0, doneq = 0, doneb = 0;
-  const int64_t tile = block_tile(a.wl, total - first), ntiles = (total - first + tile - 1) / tile;
-  for (int64_t tl = (int64_t)blockIdx.x * nshard + shard; tl < ntiles; tl += (int64_t)gridDim.x * nshard) {
-    const int64_t t0 = first + tl * tile, t1 = t0 + tile < total ? t0 + tile : total;
+  const int64_t tile = item_tile(a.wl, total - first, gridDim.x), ntiles = (total - first + tile - 1) / tile;
+  const PrimSplit sp = prim_split<T>(a.wl, total - first, gridDim.x, false);
+  for (int64_t tl = (int64_t)blockIdx.x * nshard + shard; tl < ntiles * sp.n; tl += (int64_t)gridDim.x * nshard) {
+    const int part = (int)(tl / ntiles);
+    const int64_t t0 = first + (tl - part * ntiles) * tile, t1 = t0 + tile < total ? t0 + tile : total;
     BraCursor cur;
     if (!compact) cur.seek(a.wl, t0);
     for (int64_t item = t0; item < t1; ++item) {
@@ -231,9 +233,14 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
       const int ao3 = __ldg(a.sp.ao1 + pk_id), ao4 = __ldg(a.sp.ao2 + pk_id);
       const int64_t mbase = __ldg(a.sp.mat_off + mol);
       const int n = __ldg(a.sp.mat_n + mol);
-      ++done;
-      doneq += (unsigned long long)npb * npk;
-      doneb += npb;
+      if (part == 0) {
+        ++done;
+        doneq += (unsigned long long)npb * npk;
+        doneb += npb;
+      }
+      int pb0, pb1, pk0, pk1;
+      sp.range(part, npb, npk, pb0, pb1, pk0, pk1);
+      if (pb0 >= pb1) continue;  // uniform over the block
       __syncthreads();  // the previous item's shared memory (first item: the tables) is done with
       const T* Dp = dens<T>(a) + mbase;
       for (int x = tid; x < S::NDB; x += NT) {
@@ -253,9 +260,9 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
         }
         db[x] = __ldg(Dp + (size_t)r * n + c);
       }
-      const int nq = npb * npk;
+      const int nq = pb1 * npk;
       int win = 0, wend = 0;  // primitive quartets whose scalars are in `scal`
-      for (int pb = 0; pb < npb; ++pb) {
+      for (int pb = pb0; pb < pb1; ++pb) {
         auto bra_terms = [&]() {
           for (int x = tid; x < S::TB; x += NT) {
             const unsigned w = btm[x];
@@ -332,7 +339,7 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
             x1 = fma(c, w1[o], x1);
           }
           T* x = Xs + iab * NCDP;
-          if (pb == 0) {
+          if (pb == pb0) {
             x[c0] = x0;
             if (c1 != c0) x[c1] = x1;
           } else {
@@ -391,6 +398,16 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
     atomicAdd(a.counter + 1, doneq);
     atomicAdd(a.counter + 2, doneb);
   }
+}
+
+// FP64 classes of the register kernel whose unrolled code is long run a block per
+// quartet while the list is short (at most kShortList quartets per SM): a warp
+// that passes once through some hundred kilobytes of straight-line code waits on
+// instruction fetches (6 (pp|pp) quartets: 0.36 ms).
+constexpr int kShortList = 8;
+template <int LA, int LB, int LC, int LD, typename T>
+__host__ __device__ constexpr bool block_when_short() {
+  return sizeof(T) == 8 && ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD) >= 36;
 }
 
 // Which J+K classes outside the register kernel run a block per quartet: every

@@ -80,7 +80,9 @@ __host__ __device__ constexpr int grad_footprint(int la, int lb, int lc, int ld)
 #define ERI_GRAD_THREAD32 330
 #endif
 __host__ __device__ constexpr bool use_grad_thread(int la, int lb, int lc, int ld, bool fp32) {
-  return grad_footprint(la, lb, lc, ld) <= (fp32 ? ERI_GRAD_THREAD32 : ERI_GRAD_THREAD64);
+  // (a large bra against (ss|: little work per thread and long code; a block is faster)
+  return grad_footprint(la, lb, lc, ld) <= (fp32 ? ERI_GRAD_THREAD32 : ERI_GRAD_THREAD64) &&
+         !(lc + ld == 0 && ncart(la) * ncart(lb) > 18);
 }
 
 // dE/dA and dE/dB of one item, bra primitives [pb0, pb1) and ket primitives [pk0, pk1)
@@ -148,8 +150,8 @@ __device__ __forceinline__ void grad_item(const GradArgs& a, int pb_id, int pk_i
           const T* ey = ek + 1 * NEK + (KY * (LD + 1) + LY) * (LCD + 1);
           const T* ez = ek + 2 * NEK + (KZ * (LD + 1) + LZ) * (LCD + 1);
           for_herm<LAB + 1>([&](auto t, auto u, auto v) {
-            W[icd * HAB + herm_index(ERI_CI(t), ERI_CI(u), ERI_CI(v))] +=
-                ket_term<L, KX + LX, KY + LY, KZ + LZ, ERI_CI(t), ERI_CI(u), ERI_CI(v)>(ex, ey, ez, R);
+            T& w = W[icd * HAB + herm_index(ERI_CI(t), ERI_CI(u), ERI_CI(v))];
+            w = ket_term<L, KX + LX, KY + LY, KZ + LZ, ERI_CI(t), ERI_CI(u), ERI_CI(v)>(ex, ey, ez, R, w);
           });
         });
       });
@@ -235,7 +237,7 @@ __global__ void __launch_bounds__(128) grad_thread_kernel(GradArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const PrimSplit sp = prim_split<T>(a.wl, total - first, 32 * nwarps);
-  const int64_t span = 32 * (int64_t)a.wl.tile, ntiles = (total - first + span - 1) / span;
+  const int64_t span = 32 * thread_tile(a.wl, total - first, nwarps), ntiles = (total - first + span - 1) / span;
   unsigned long long done = 0, doneq = 0, doneb = 0;
   for (int64_t tl = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * nshard + shard; tl < ntiles * sp.n;
        tl += nwarps * nshard) {
@@ -259,7 +261,9 @@ __global__ void __launch_bounds__(128) grad_thread_kernel(GradArgs a) {
           ib = cur.ib;
         }
         const int pb_id = __ldg(a.wl.bra + ib), mol = __ldg(a.sp.pmol + pb_id);
-        const int pk_id = __ldg(a.wl.ket + __ldg(a.wl.kseg + mol * NPAIRCLASS) + ik);
+        const int seg = __ldg(a.wl.kseg + mol * NPAIRCLASS);
+        if (!compact) ik = ket_pos(a.wl, seg, ik, cur.be - cur.bs);
+        const int pk_id = __ldg(a.wl.ket + seg + ik);
         const int npb = __ldg(a.sp.np + pb_id), npk = __ldg(a.sp.np + pk_id);
         if (part == 0) {
           ++done;
@@ -406,7 +410,7 @@ __global__ void __launch_bounds__(GShape<LA, LB, LC, LD, T>::NT) grad_block_kern
   const int64_t first = compact ? 0 : a.wl.first;
   const int nshard = compact ? 1 : a.wl.nshard, shard = compact ? 0 : a.wl.shard;
   unsigned long long done = 0, doneq = 0, doneb = 0;
-  const int64_t tile = block_tile(a.wl, total - first), ntiles = (total - first + tile - 1) / tile;
+  const int64_t tile = item_tile(a.wl, total - first, gridDim.x), ntiles = (total - first + tile - 1) / tile;
   T gA[3] = {T(0), T(0), T(0)}, gB[3] = {T(0), T(0), T(0)};
   int atA = -1, atB = -1;
   // sum the threads' gA, gB and add them to the two atoms (whole block)
@@ -428,8 +432,10 @@ __global__ void __launch_bounds__(GShape<LA, LB, LC, LD, T>::NT) grad_block_kern
 #pragma unroll
     for (int d = 0; d < 3; ++d) gA[d] = gB[d] = T(0);
   };
-  for (int64_t tl = (int64_t)blockIdx.x * nshard + shard; tl < ntiles; tl += (int64_t)gridDim.x * nshard) {
-    const int64_t t0 = first + tl * tile, t1 = t0 + tile < total ? t0 + tile : total;
+  const PrimSplit sp = prim_split<T>(a.wl, total - first, gridDim.x, false);
+  for (int64_t tl = (int64_t)blockIdx.x * nshard + shard; tl < ntiles * sp.n; tl += (int64_t)gridDim.x * nshard) {
+    const int part = (int)(tl / ntiles);
+    const int64_t t0 = first + (tl - part * ntiles) * tile, t1 = t0 + tile < total ? t0 + tile : total;
     BraCursor cur;
     if (!compact) cur.seek(a.wl, t0);
     for (int64_t item = t0; item < t1; ++item) {
@@ -450,9 +456,14 @@ __global__ void __launch_bounds__(GShape<LA, LB, LC, LD, T>::NT) grad_block_kern
       const int npk = __ldg(a.sp.np + pk_id), offk = __ldg(a.sp.poff + pk_id), ek0 = __ldg(a.sp.eoff + pk_id);
       const int ao1 = __ldg(a.sp.ao1 + pb_id), ao2 = __ldg(a.sp.ao2 + pb_id);
       const int ao3 = __ldg(a.sp.ao1 + pk_id), ao4 = __ldg(a.sp.ao2 + pk_id);
-      ++done;
-      doneq += (unsigned long long)npb * npk;
-      doneb += npb;
+      if (part == 0) {
+        ++done;
+        doneq += (unsigned long long)npb * npk;
+        doneb += npb;
+      }
+      int pb0, pb1, pk0, pk1;
+      sp.range(part, npb, npk, pb0, pb1, pk0, pk1);
+      if (pb0 >= pb1) continue;  // uniform over the block
       // items of a tile usually share the bra atoms: their sums go out together
       // (FP32 sums and deterministic builds: once per item)
       const int nA = __ldg(a.sh_atom + s1), nB = __ldg(a.sh_atom + s2);
@@ -500,9 +511,9 @@ __global__ void __launch_bounds__(GShape<LA, LB, LC, LD, T>::NT) grad_block_kern
         __syncthreads();
         density(0);
       }
-      const int nq = npb * npk;
+      const int nq = pb1 * npk;
       int win = 0, wend = 0;
-      for (int pb = 0; pb < npb; ++pb) {
+      for (int pb = pb0; pb < pb1; ++pb) {
         const int ipb = offb + pb;
         const T ea = (T)__ldg(a.ea + ipb), aop = ea / pdv<T>(a.pd.p, a.pd.pf, ipb), bop = T(1) - aop;
         for (int x = tid; x < 3 * S::NER; x += NT) {  // E and E1 rows, zero-padded

@@ -117,18 +117,18 @@ __global__ void k_pairs(int npair, const int* __restrict__ s1, const int* __rest
                         const double* __restrict__ coords, int nprimpair, double* p_, double* P_, double* PA_,
                         double* PB_, double* pref_, float* pf, float* Pf, float* PAf, float* PBf, float* preff,
                         float* pmaxp, float* prefmaxp, double* ea_, float4* q4) {
-  int ip = blockIdx.x * blockDim.x + threadIdx.x;
+  const int ip = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;  // one warp per pair
   if (ip >= npair) return;
   const int a = s1[ip], b = s2[ip];
   const double* A = coords + 3 * sh_atom[a];
   const double* Bc = coords + 3 * sh_atom[b];
   double AB2 = 0.0;
   for (int d = 0; d < 3; ++d) AB2 += (A[d] - Bc[d]) * (A[d] - Bc[d]);
-  int o = poff[ip];
+  const int nb = sh_np[b];
   double pmx = 0.0, prmx = 0.0;
   const double s2pi52 = 5.9149671727956129;  // sqrt(2 pi^(5/2))
-  for (int i = 0; i < sh_np[a]; ++i)
-    for (int j = 0; j < sh_np[b]; ++j, ++o) {
+  for (int k = lane; k < sh_np[a] * nb; k += 32) {
+      const int i = k / nb, j = k - i * nb, o = poff[ip] + k;
       const double ea = ex[sh_po[a] + i], eb = ex[sh_po[b] + j];
       const double p = ea + eb;
       const double pr = cn[sh_po[a] + i] * cn[sh_po[b] + j] * exp(-ea * eb / p * AB2) * s2pi52 / p;
@@ -156,6 +156,11 @@ __global__ void k_pairs(int npair, const int* __restrict__ s1, const int* __rest
       q4[3 * (size_t)o + 1] = make_float4(fA[0], fA[1], fA[2], (float)pr);
       q4[3 * (size_t)o + 2] = make_float4(fB[0], fB[1], fB[2], 0.0f);
     }
+  for (int o = 16; o > 0; o >>= 1) {
+    pmx = fmax(pmx, __shfl_xor_sync(0xffffffffu, pmx, o));
+    prmx = fmax(prmx, __shfl_xor_sync(0xffffffffu, prmx, o));
+  }
+  if (lane != 0) return;
   pmaxp[ip] = (float)pmx;
   prefmaxp[ip] = (float)fmin(prmx, 1.0e30);
 }
@@ -178,7 +183,9 @@ __global__ void __launch_bounds__(256) k_tier_split(KArgs a, int2* __restrict__ 
       ik = (int)(item - __ldg(a.wl.prefix + ib));
       const int pb_id = __ldg(a.wl.bra + ib);
       const int mol = __ldg(a.sp.pmol + pb_id);
-      const int pk_id = __ldg(a.wl.ket + __ldg(a.wl.kseg + mol * NPAIRCLASS) + ik);
+      const int seg = __ldg(a.wl.kseg + mol * NPAIRCLASS);
+      ik = ket_pos(a.wl, seg, ik, __ldg(a.wl.prefix + ib + 1) - __ldg(a.wl.prefix + ib));
+      const int pk_id = __ldg(a.wl.ket + seg + ik);
       tier = quartet_tier(a, mol, pb_id, pk_id, __ldg(a.sp.s1 + pb_id), __ldg(a.sp.s2 + pb_id),
                           __ldg(a.sp.s1 + pk_id), __ldg(a.sp.s2 + pk_id));
     }
@@ -223,34 +230,32 @@ __global__ void k_dmax(int npair, const int* __restrict__ s1, const int* __restr
 __global__ void k_etab(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
                        const int* __restrict__ poff, const int* __restrict__ eoff, const int* __restrict__ sh_l,
                        PairData pd, double* __restrict__ E, float* __restrict__ Ef) {
-  int ip = blockIdx.x * blockDim.x + threadIdx.x;
+  const int ip = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (ip >= npair) return;
   const int l1 = sh_l[s1[ip]], l2 = sh_l[s2[ip]];
   const int ne = (l1 + 1) * (l2 + 1) * (l1 + l2 + 1);
   double tmp[225];
-  for (int k = 0; k < np[ip]; ++k) {
-    const int pi = poff[ip] + k;
-    for (int d = 0; d < 3; ++d) {
-      md_e_rt(l1, l2, pd.PA[d * pd.n + pi], pd.PB[d * pd.n + pi], 0.5 / pd.p[pi], tmp);
-      const size_t o = (size_t)eoff[ip] + ((size_t)k * 3 + d) * ne;
-      for (int i = 0; i <= l1; ++i)
-        for (int j = 0; j <= l2; ++j)
-          for (int t = 0; t <= l1 + l2; ++t) {
-            const double v = tmp[(i * 5 + j) * 9 + t];
-            E[o + (i * (l2 + 1) + j) * (l1 + l2 + 1) + t] = v;
-            Ef[o + (i * (l2 + 1) + j) * (l1 + l2 + 1) + t] = (float)v;
-          }
-    }
+  for (int x = lane; x < 3 * np[ip]; x += 32) {  // one warp per pair, a lane per (primitive pair, direction)
+    const int k = x / 3, d = x - 3 * k, pi = poff[ip] + k;
+    md_e_rt(l1, l2, pd.PA[d * pd.n + pi], pd.PB[d * pd.n + pi], 0.5 / pd.p[pi], tmp);
+    const size_t o = (size_t)eoff[ip] + (size_t)x * ne;
+    for (int i = 0; i <= l1; ++i)
+      for (int j = 0; j <= l2; ++j)
+        for (int t = 0; t <= l1 + l2; ++t) {
+          const double v = t <= i + j ? tmp[(i * 5 + j) * 9 + t] : 0.0;
+          E[o + (i * (l2 + 1) + j) * (l1 + l2 + 1) + t] = v;
+          Ef[o + (i * (l2 + 1) + j) * (l1 + l2 + 1) + t] = (float)v;
+        }
   }
 }
 
 // Schwarz bound per shell pair: Q = sqrt(max_{mu,nu} |(mu nu|mu nu)|) in FP64, rounded up to float32.
-// One warp per pair: R of a primitive quartet level by level over the lanes, then
-// a lane per component pair (a thread per pair kept E and R in local memory and
+// One block per pair, a warp per primitive quartet: R level by level over the
+// lanes, then a lane per component pair (a thread per pair kept E and R in local memory and
 // took 2 ms for one (ff|ff) diagonal, the longest kernel of a small molecule's
 // geometry step).  The E tables are those of k_etab; primitive quartets (i, j)
 // and (j, i) are equal, so j <= i with weight 2.
-constexpr int kSchwarzWarps = 4;
+constexpr int kSchwarzWarps = 6;  // 44 KB of shared memory
 constexpr int kSchwarzR = nherm(4 * LMAX);
 __global__ void __launch_bounds__(32 * kSchwarzWarps)
     k_schwarz(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
@@ -258,16 +263,16 @@ __global__ void __launch_bounds__(32 * kSchwarzWarps)
               const int* __restrict__ ao, const double* __restrict__ f, PairData pd, BoysTabs bt,
               const RStep* __restrict__ st, float* __restrict__ Q) {
   __shared__ double Rs[kSchwarzWarps][2][kSchwarzR], Fs[kSchwarzWarps][4 * LMAX + 1];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int ip = blockIdx.x * kSchwarzWarps + w;
-  if (ip >= npair) return;  // uniform over the warp; nothing below syncs the block
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, ip = blockIdx.x;
   const int l1 = sh_l[s1[ip]], l2 = sh_l[s2[ip]], lp = l1 + l2, L = 2 * lp;
   const int n2 = ncart(l2), nc = ncart(l1) * n2, ne = (l1 + 1) * (l2 + 1) * (lp + 1);
   double* F = Fs[w];
   double diag[4] = {0.0, 0.0, 0.0, 0.0};  // component pairs lane + 32 k (at most 100)
+  int turn = 0;
   for (int i = 0; i < np[ip]; ++i) {
     const int pi = poff[ip] + i;
     for (int j = 0; j <= i; ++j) {
+      if (turn++ % kSchwarzWarps != w) continue;
       const int pj = poff[ip] + j;
       const double p = pd.p[pi], q = pd.p[pj], rho = p * q / (p + q);
       const double X = pd.P[pi] - pd.P[pj], Y = pd.P[pd.n + pi] - pd.P[pd.n + pj],
@@ -350,11 +355,17 @@ __global__ void __launch_bounds__(32 * kSchwarzWarps)
       __syncwarp();
     }
   }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) Rs[w][0][lane + 32 * k] = diag[k];
+  __syncthreads();
+  if (w != 0) return;
   double mx = 0.0;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int c = lane + 32 * k;
     if (c < nc) {
+      for (int x = 1; x < kSchwarzWarps; ++x) diag[k] += Rs[x][0][c];
       const double fn = f[ao[s1[ip]] + c / n2] * f[ao[s2[ip]] + c % n2];
       mx = fmax(mx, fabs(diag[k] * fn * fn));
     }
@@ -379,7 +390,7 @@ __global__ void k_primq(int npair, const int* __restrict__ s1, const int* __rest
                         const int* __restrict__ poff, const int* __restrict__ eoff, const int* __restrict__ sh_l,
                         const int* __restrict__ ao, const double* __restrict__ f, const int* __restrict__ pmol,
                         PairData pd, double* __restrict__ pq, unsigned int* __restrict__ pqmax) {
-  const int ip = blockIdx.x * blockDim.x + threadIdx.x;
+  const int ip = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;  // one warp per pair
   if (ip >= npair) return;
   const int a = s1[ip], b = s2[ip], l1 = sh_l[a], l2 = sh_l[b], lp = l1 + l2;
   const int ne = (l1 + 1) * (l2 + 1) * (lp + 1);
@@ -387,7 +398,7 @@ __global__ void k_primq(int npair, const int* __restrict__ s1, const int* __rest
   for (int c = 0; c < ncart(l1); ++c) fm = fmax(fm, f[ao[a] + c]);
   for (int c = 0; c < ncart(l2); ++c) fn = fmax(fn, f[ao[b] + c]);
   double top = 0.0;
-  for (int k = 0; k < np[ip]; ++k) {
+  for (int k = lane; k < np[ip]; k += 32) {
     const int pi = poff[ip] + k;
     const double p = pd.p[pi], rp = sqrt(p);
     double S[3][(LMAX + 1) * (LMAX + 1)];
@@ -413,7 +424,8 @@ __global__ void k_primq(int npair, const int* __restrict__ s1, const int* __rest
     pq[pi] = q;
     top = fmax(top, q);
   }
-  atomicMax(pqmax + pmol[ip], __float_as_uint(__double2float_ru(fmin(top, 1e38))));
+  for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if (lane == 0) atomicMax(pqmax + pmol[ip], __float_as_uint(__double2float_ru(fmin(top, 1e38))));
 }
 
 template <typename T>
@@ -429,7 +441,7 @@ __global__ void k_primpack(int npair, const int* __restrict__ s1, const int* __r
                            double* P, double* PA, double* PB, double* pref, double* ea, float* pf, float* Pf,
                            float* PAf, float* PBf, float* preff, float4* q4, double* E, float* Ef,
                            int* __restrict__ nkeep) {
-  const int ip = blockIdx.x * blockDim.x + threadIdx.x;
+  const int ip = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;  // one warp per pair
   if (ip >= npair) return;
   const int l1 = sh_l[s1[ip]], l2 = sh_l[s2[ip]], ne3 = 3 * (l1 + 1) * (l2 + 1) * (l1 + l2 + 1);
   const int o = poff[ip];
@@ -439,13 +451,16 @@ __global__ void k_primpack(int npair, const int* __restrict__ s1, const int* __r
     if (pq[o + k] * qmax < limit) continue;  // (a NaN bound is kept)
     if (k != m) {
       const int x = o + k, y = o + m;
-      dswap(pq[x], pq[y]);
-      dswap(p[x], p[y]);
-      dswap(pref[x], pref[y]);
-      dswap(ea[x], ea[y]);
-      dswap(pf[x], pf[y]);
-      dswap(preff[x], preff[y]);
-      for (int d = 0; d < 3; ++d) {
+      __syncwarp();  // every lane has read pq[o + k]
+      if (lane == 0) {
+        dswap(pq[x], pq[y]);
+        dswap(p[x], p[y]);
+        dswap(pref[x], pref[y]);
+        dswap(ea[x], ea[y]);
+        dswap(pf[x], pf[y]);
+        dswap(preff[x], preff[y]);
+      } else if (lane <= 3) {
+        const int d = lane - 1;
         dswap(P[d * n + x], P[d * n + y]);
         dswap(PA[d * n + x], PA[d * n + y]);
         dswap(PB[d * n + x], PB[d * n + y]);
@@ -455,14 +470,15 @@ __global__ void k_primpack(int npair, const int* __restrict__ s1, const int* __r
         dswap(q4[3 * (size_t)x + d], q4[3 * (size_t)y + d]);
       }
       const size_t ex = (size_t)eoff[ip] + (size_t)k * ne3, ey = (size_t)eoff[ip] + (size_t)m * ne3;
-      for (int e = 0; e < ne3; ++e) {
+      for (int e = lane; e < ne3; e += 32) {
         dswap(E[ex + e], E[ey + e]);
         dswap(Ef[ex + e], Ef[ey + e]);
       }
+      __syncwarp();
     }
     ++m;
   }
-  nkeep[ip] = m;
+  if (lane == 0) nkeep[ip] = m;
 }
 
 // Per-molecule Schwarz maximum (pairs never cross molecules).  Q >= 0, so
@@ -533,6 +549,31 @@ __global__ void k_counts(int npair, const float* __restrict__ Q, const int* __re
     if (qi * (double)Q[lst[mid]] >= thresh) lo = mid + 1; else hi = mid;
   }
   counts[t] = lo;
+}
+
+// Visiting order of the kets of one (molecule, class) segment: inside each full
+// group of kKetGroup positions by decreasing number of primitive pairs (ties by
+// position).  One block of kKetGroup threads per group; grid (segment, group).
+__global__ void __launch_bounds__(kKetGroup)
+    k_ketorder(const int* __restrict__ sorted, const int* __restrict__ coff, const int* __restrict__ segloc,
+               const int* __restrict__ ccm, const int* __restrict__ np, int* __restrict__ korder) {
+  __shared__ int key[kKetGroup];
+  const int s = blockIdx.x, X = s % NPAIRCLASS, n = ccm[s], t = threadIdx.x;
+  const int64_t base = (int64_t)coff[X] + segloc[s];
+  for (int g = blockIdx.y * kKetGroup; g < n; g += gridDim.y * kKetGroup) {
+    const int i = g + t;
+    if (g + kKetGroup > n) {  // a partial group keeps the order of the list
+      if (i < n) korder[base + i] = i;
+      return;
+    }
+    const int k = np[sorted[base + i]];
+    key[t] = k;
+    __syncthreads();
+    int r = 0;
+    for (int j = 0; j < kKetGroup; ++j) r += key[j] > k || (key[j] == k && j < t);
+    korder[base + g + r] = i;
+    __syncthreads();
+  }
 }
 
 // Exclusive scan of one int64 per thread over the block (blockDim.x a multiple
@@ -886,27 +927,27 @@ MolMats molmats(const eri_plan_impl* P) {
 
 // pair data + Schwarz + lists for the current device coordinates
 int eri_plan_impl::geometry(cudaStream_t s, bool rebuild_q) {
-  k_pairs<<<grid1(npair, 128), 128, 0, s>>>(npair, d_ps1, d_ps2, d_ppoff, d_sh_atom, d_sh_np, d_sh_po, d_exps, d_cn,
+  k_pairs<<<grid1(npair, 4), 128, 0, s>>>(npair, d_ps1, d_ps2, d_ppoff, d_sh_atom, d_sh_np, d_sh_po, d_exps, d_cn,
                                         d_coords, nprimpair, d_p, d_P, d_PA, d_PB, d_pref, d_pf, d_Pf, d_PAf, d_PBf,
                                         d_preff, d_pmaxp, d_prefmaxp, d_ea, d_q4);
   CK(cudaGetLastError());
-  k_etab<<<grid1(npair, 64), 64, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff, d_sh_l, pairdata(), d_E, d_Ef);
+  k_etab<<<grid1(npair, 4), 128, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff, d_sh_l, pairdata(), d_E, d_Ef);
   CK(cudaGetLastError());
   if (rebuild_q) {
-    k_schwarz<<<grid1(npair, kSchwarzWarps), 32 * kSchwarzWarps, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff,
+    k_schwarz<<<npair, 32 * kSchwarzWarps, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff,
                                                                          d_sh_l, d_sh_ao, d_f, pairdata(), boystabs(),
                                                                          d_rsteps, d_Q);
     CK(cudaGetLastError());
   }
   CK(cudaMemsetAsync(d_pqmax, 0, sizeof(unsigned int) * nmol, s));
-  k_primq<<<grid1(npair, 64), 64, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff, d_sh_l, d_sh_ao, d_f, d_pmol,
+  k_primq<<<grid1(npair, 4), 128, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff, d_sh_l, d_sh_ao, d_f, d_pmol,
                                           pairdata(), d_pq, d_pqmax);
   CK(cudaGetLastError());
   return rebuild_q ? build_lists(thresh, s) : pack_primitives(s);
 }
 
 int eri_plan_impl::pack_primitives(cudaStream_t s) {
-  k_primpack<<<grid1(npair, 64), 64, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff, d_sh_l, d_pmol, d_pqmax,
+  k_primpack<<<grid1(npair, 4), 128, 0, s>>>(npair, d_ps1, d_ps2, d_pnp, d_ppoff, d_peoff, d_sh_l, d_pmol, d_pqmax,
                                              kPrimEps * thresh, nprimpair, d_pq, d_p, d_P, d_PA, d_PB, d_pref, d_ea,
                                              d_pf, d_Pf, d_PAf, d_PBf, d_preff, d_q4, d_E, d_Ef, d_pnk);
   CK(cudaGetLastError());
@@ -952,6 +993,7 @@ int eri_plan_impl::build_lists(double th, cudaStream_t s) {
                                            d_pos);
   k_counts<<<grid1((int64_t)npair * NPAIRCLASS, 256), 256, 0, s>>>(npair, d_Q, d_sig, d_pmol, d_sorted, d_coff,
                                                                    d_segloc, d_ccm, th, d_counts);
+  k_ketorder<<<dim3(nm10, 16), kKetGroup, 0, s>>>(d_sorted, d_coff, d_segloc, d_ccm, d_pnk, d_korder);
   CK(cudaGetLastError());
   int64_t ko = 0, jo = 0;
   for (int X = 0; X < NPAIRCLASS; ++X)
@@ -994,6 +1036,7 @@ WorkList eri_plan_impl::klist(int X, int Y) const {
   w.bra = d_sorted + h_coff[X];
   w.ket = d_sorted + h_coff[Y];
   w.kseg = d_segloc + Y;
+  w.korder = d_korder + h_coff[Y];
   w.prefix = d_kpre + h_koff[X * NPAIRCLASS + Y];
   w.nbra = h_ccount[X];
   w.total = h_ktot[X * NPAIRCLASS + Y];
@@ -1011,6 +1054,7 @@ WorkList eri_plan_impl::jlist(int X, int Y) const {
   w.bra = d_sorted + h_coff[X];
   w.ket = d_sorted + h_coff[Y];
   w.kseg = d_segloc + Y;
+  w.korder = d_korder + h_coff[Y];
   w.prefix = d_jpre + h_joff[X * NPAIRCLASS + Y];
   w.nbra = h_ccount[X];
   w.total = h_jtot[X * NPAIRCLASS + Y];
@@ -1026,7 +1070,7 @@ void eri_plan_impl::release() {
                   d_kpre, d_jpre, d_ktot, d_jtot, d_kprim, d_boys64, d_boys32, d_rsteps, d_Dp, d_Kh, d_Jh, d_Dherm,
                   d_Jherm, d_status, d_bexp64, d_bexp32, d_peoff, d_E, d_Ef, d_pmaxp, d_dmax, d_counters, d_cumnp, d_prefmaxp, d_ea,
                   d_mat_off, d_mat_n, d_aobase, d_pbase, d_pmol, d_shloc, d_ccm, d_segloc, d_Dpf,
-                  d_nuc_list, d_nuc_goff, d_nuc_dens, d_counters2, d_q4, d_Dhermf, d_pq, d_pqmax, d_pnk};
+                  d_nuc_list, d_nuc_goff, d_nuc_dens, d_counters2, d_q4, d_Dhermf, d_pq, d_pqmax, d_pnk, d_korder};
   xc_release();
   for (auto& e : prof_events) cudaEventDestroy(e);
   prof_events.clear();
@@ -1195,7 +1239,8 @@ static double grad_flops(int X, int Y, double nq, double npq, double nbp) {
 }
 
 // Default work-tile length: the thread kernel's lanes already take adjacent
-// items; a warp kernel takes 4 consecutive quartets (mostly one bra) per tile.
+// items; a warp or block takes 4 consecutive quartets (mostly one bra) per tile,
+// fewer on short lists (item_tile).
 static int default_tile(int X, int Y, int tier) {
   return use_thread_kernel(kClassL1[X], kClassL2[X], kClassL1[Y], kClassL2[Y], tier == 1) ? 1 : 4;
 }
@@ -1472,7 +1517,7 @@ static int plan_create(int nmol, const eri_basis_t* const* bases, const double* 
     CKP(dalloc(&P->d_boys64, (size_t)BOYS_NT * (BOYS_MMAX + 1) * BOYS_J64));
     CKP(dalloc(&P->d_boys32, (size_t)BOYS_NT * (BOYS_MMAX + 1) * BOYS_J32));
     CKP(dalloc(&P->d_bexp64, BOYS_NT)); CKP(dalloc(&P->d_bexp32, BOYS_NT));
-    CKP(dalloc(&P->d_pq, nprimpair)); CKP(dalloc(&P->d_pqmax, nmol)); CKP(dalloc(&P->d_pnk, npair));
+    CKP(dalloc(&P->d_pq, nprimpair)); CKP(dalloc(&P->d_pqmax, nmol)); CKP(dalloc(&P->d_pnk, npair)); CKP(dalloc(&P->d_korder, npair));
     CKP(dalloc(&P->d_peoff, npair)); CKP(dalloc(&P->d_E, ne_tot)); CKP(dalloc(&P->d_Ef, ne_tot));
     CKP(dalloc(&P->d_pmaxp, npair)); CKP(dalloc(&P->d_prefmaxp, npair)); CKP(dalloc(&P->d_ea, nprimpair));
     CKP(dalloc(&P->d_dmax, npair));

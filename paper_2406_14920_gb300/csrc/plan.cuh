@@ -38,6 +38,7 @@ struct eri_plan_impl {
   double* d_pq = nullptr;           // Schwarz-type bound per primitive pair
   unsigned int* d_pqmax = nullptr;  // its maximum per molecule (float bits)
   int* d_pnk = nullptr;             // primitive pairs kept per shell pair (the first ones)
+  int* d_korder = nullptr;          // visiting order of the kets (ket_pos)
   float4* d_q4 = nullptr;  // packed FP32 shadows, 3 float4 per primitive pair (PairData::q4)
   // screening and lists
   float* d_Q = nullptr;
@@ -83,7 +84,7 @@ struct eri_plan_impl {
   static constexpr int kBranches = 4;
   // eager builds and gradients fork their class launches over the same side
   // streams, kStreams of them, and join them before they return
-  static constexpr int kStreams = 8;
+  static constexpr int kStreams = 16;
   cudaStream_t cap_stream = nullptr;
   cudaStream_t branch[kStreams] = {};
   cudaEvent_t fork_ev = nullptr, join_ev[kStreams] = {};
