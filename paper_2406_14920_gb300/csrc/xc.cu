@@ -378,14 +378,21 @@ __global__ void __launch_bounds__(256) k_xc_ddigits(int nbf, const double* __res
 // Step (2): X_m = sum_n D_mn phi_n at every point of the block, then
 // rho = sum_m phi_m X_m, grad rho = 2 sum_m grad phi_m X_m (D symmetric).
 // A warp owns 16 rows of X x the 32 points (nine accumulators of 16 values per
-// lane) and gathers the digit rows of D at the block's functions straight into
-// its operand registers (16 B per element, from L2); the digits of kKC functions
-// of Phi_b are staged in shared memory in operand order.  X goes through shared
+// lane).  It gathers the digit rows of D at the block's functions (16 B per
+// element, from L2) one step of 16 ahead with cp.async, so that the L2 latency
+// runs under the 172 products of a step (read straight into registers, 2.7 of 8.5
+// issue slots waited on it); the digits of kKC functions of Phi_b are staged in
+// shared memory in operand order.  X goes through shared
 // memory to a lane per point for the sums with phi and grad phi.  A block that
 // holds a function with an infinity or NaN in its row of D takes the plain sums.
 struct RhoSmem {
   uint2 B[kKC / 16][kBP / 8][kDigits][32];
-  double X[kRhoWarps][16][kBP];
+  // two steps of a warp's operand A, 16 B per element of D, rows 17 elements apart
+  // (no bank conflicts); X, the warp's 16 x 32 sums, takes their place at the end
+  union {
+    uint4 A[2][16][17];
+    double X[16][kBP];
+  } w[kRhoWarps];
   double sum[kRhoWarps][4][kBP];
   int pexp[kBP];
 };
@@ -419,7 +426,21 @@ __global__ void __launch_bounds__(32 * kRhoWarps, 2)
     if (tid < kBP) S.pexp[tid] = pexp[(int64_t)b * kBP + tid];
     for (int mg = 0; mg < n; mg += 16 * kRhoWarps) {
       const int m0 = mg + 16 * wp;
-      const int64_t r0 = (int64_t)L[min(m0 + g, n - 1)] * nbf, r1 = (int64_t)L[min(m0 + g + 8, n - 1)] * nbf;
+      // step of 16 functions from k on: lane l copies column l % 16 of rows l / 16 + 2 i
+      int arow[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) arow[i] = L[min(m0 + 2 * i + (lane >> 4), n - 1)];
+      auto fetch = [&](int k, int stage) {
+        if (m0 < n && k < n) {
+          const uint4* col = Dd + __ldg(L + min(k + (lane & 15), n - 1));
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            copy16(&S.w[wp].A[stage][2 * i + (lane >> 4)][lane & 15], col + (int64_t)arow[i] * nbf);
+        }
+        copy_commit();
+      };
+      __syncwarp();  // X of the previous rows has been read
+      fetch(0, 0);
       for (int seg = 0; seg < n; seg += kExactTerms) {
         const int send = min(n, seg + kExactTerms);
         float acc[kBP / 8][kWeights][4];
@@ -433,26 +454,44 @@ __global__ void __launch_bounds__(32 * kRhoWarps, 2)
           const int nks = (min(send - kc, kKC) + 15) / 16;
           __syncthreads();  // the previous chunk has been read
           // one pair of functions (k, k + 1) at one point per step, both halves of a 16-step
-          for (int e = tid; e < nks * (kBP / 8) * 64; e += 32 * kRhoWarps) {
-            const int el = e & 31, h = (e >> 5) & 1, nt = (e >> 6) & (kBP / 8 - 1), ks = e >> 8;
-            const int k = kc + 16 * ks + 2 * (el & 3) + 8 * h, p = 8 * nt + (el >> 2);
-            const int E = S.pexp[p];
-            const unsigned long long u0 = digits_of(k < n ? W[(int64_t)k * kBP + p] : 0.0, E);
-            const unsigned long long u1 = digits_of(k + 1 < n ? W[(int64_t)(k + 1) * kBP + p] : 0.0, E);
+          // (four at a time: their loads are in flight together)
+          const int ntask = nks * (kBP / 8) * 64;
+#pragma unroll 1
+          for (int e0 = tid; e0 < ntask; e0 += 4 * 32 * kRhoWarps) {
+            double v[4][2];
 #pragma unroll
-            for (int x = 0; x < kDigits; ++x) (&S.B[ks][nt][x][el].x)[h] = digit_pair(u0, u1, x);
+            for (int i = 0; i < 4; ++i) {
+              const int e = e0 + i * 32 * kRhoWarps, el = e & 31, h = (e >> 5) & 1, nt = (e >> 6) & (kBP / 8 - 1);
+              const int k = kc + 16 * (e >> 8) + 2 * (el & 3) + 8 * h, p = 8 * nt + (el >> 2);
+              v[i][0] = e < ntask && k < n ? W[(int64_t)k * kBP + p] : 0.0;
+              v[i][1] = e < ntask && k + 1 < n ? W[(int64_t)(k + 1) * kBP + p] : 0.0;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int e = e0 + i * 32 * kRhoWarps, el = e & 31, h = (e >> 5) & 1, nt = (e >> 6) & (kBP / 8 - 1);
+              if (e < ntask) {
+                const int E = S.pexp[8 * nt + (el >> 2)];
+                const unsigned long long u0 = digits_of(v[i][0], E), u1 = digits_of(v[i][1], E);
+#pragma unroll
+                for (int x = 0; x < kDigits; ++x) (&S.B[e >> 8][nt][x][el].x)[h] = digit_pair(u0, u1, x);
+              }
+            }
           }
           __syncthreads();
           if (m0 < n) {
             for (int ks = 0; ks < nks; ++ks) {
+              const int k = kc + 16 * ks, stage = (k >> 4) & 1;
+              if (k + 16 < send) fetch(k + 16, stage ^ 1);  // (X is in the way of the next segment's first step)
+              else copy_commit();
+              copy_wait<1>();
+              __syncwarp();
               uint32_t a[kDigits][4];
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {  // columns 2t, 2t+1 and 2t+8, 2t+9 of rows g and g + 8
-                const int k = kc + 16 * ks + 2 * t + 8 * h;
-                const int c0 = __ldg(L + min(k, n - 1)), c1 = __ldg(L + min(k + 1, n - 1));
+              for (int h = 0; h < 2; ++h)  // columns 2t, 2t+1 and 2t+8, 2t+9 of rows g and g + 8
 #pragma unroll
                 for (int y = 0; y < 2; ++y) {
-                  const uint4 u = __ldg(Dd + (y ? r1 : r0) + c0), v = __ldg(Dd + (y ? r1 : r0) + c1);
+                  const uint4* e = &S.w[wp].A[stage][g + 8 * y][2 * t + 8 * h];
+                  const uint4 u = e[0], v = e[1];
                   const uint32_t uu[4] = {u.x, u.y, u.z, u.w}, vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                   for (int x = 0; x < 4; ++x) {
@@ -460,7 +499,7 @@ __global__ void __launch_bounds__(32 * kRhoWarps, 2)
                     a[2 * x + 1][2 * h + y] = __byte_perm(uu[x], vv[x], 0x7632);
                   }
                 }
-              }
+              __syncwarp();  // the step has been read; its place may be refilled
 #pragma unroll
               for (int nt = 0; nt < kBP / 8; ++nt)
 #pragma unroll
@@ -481,11 +520,28 @@ __global__ void __launch_bounds__(32 * kRhoWarps, 2)
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
               const int p = 8 * nt + 2 * t + (c & 1);
-              S.X[wp][g + 8 * (c >> 1)][p] = combine<false>(acc[nt], c, c < 2 ? e0 : e1, S.pexp[p]);
+              S.w[wp].X[g + 8 * (c >> 1)][p] = combine<false>(acc[nt], c, c < 2 ? e0 : e1, S.pexp[p]);
             }
           __syncwarp();
-          const int nr = min(16, n - m0);
-          for (int r = 0; r < nr; ++r) add_row(m0 + r, S.X[wp][r][lane]);
+          // four rows at a time: their 16 values of phi and grad phi are in flight together
+#pragma unroll 1
+          for (int r = 0; r < 16; r += 4) {
+            double v[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int c = 0; c < 4; ++c) v[i][c] = W[((int64_t)c * n + min(m0 + r + i, n - 1)) * kBP + lane];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const double x = m0 + r + i < n ? S.w[wp].X[r + i][lane] : 0.0;
+#pragma unroll
+              for (int c = 0; c < 4; ++c) sum[c] = fma(v[i][c], x, sum[c]);
+            }
+          }
+          if (send < n) {
+            __syncwarp();
+            fetch(send, 0);
+          }
         }
       }
     }
@@ -618,7 +674,9 @@ __device__ __forceinline__ int operand_digits(const double* row, int t, uint32_t
 // Step (4b): A_ij = sum_g Z_i(g) phi_j(g) of one block over its functions, added
 // to the half matrix Vh.  A warp holds the digits of 16 functions of Z over the
 // block's 32 points in registers and walks the staged functions of Phi, 8 at a
-// time; the 32 points are one exact accumulation.  (Tiles of V that walk every
+// time; the 32 points are one exact accumulation.  Half of the sums are put
+// together in integers and half on the FP64 pipe (combine_fp64), so that neither
+// pipe outlasts the tensor work of a tile.  (Tiles of V that walk every
 // block waste products on functions a block does not hold, 2.8 times as many on
 // workload 1 at 32 x 32.)
 struct VmatSmem {
@@ -708,7 +766,8 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
         for (int c = 0; c < 4; ++c) {
           const int jl = 8 * nt + 2 * t + (c & 1);
           if (jl >= nj || !(c < 2 ? ok0 : ok1)) continue;
-          const double v = combine<true>(acc, c, c < 2 ? e0 : e1, S.exp[jl]);
+          const double v = c & 1 ? combine_fp64(acc, c, c < 2 ? e0 : e1, S.exp[jl])
+                                 : combine<true>(acc, c, c < 2 ? e0 : e1, S.exp[jl]);
           if (v != 0.0) atomicAdd((c < 2 ? v0 : v1) + S.ao[jl], v);
         }
       }

@@ -112,4 +112,34 @@ __device__ __forceinline__ double combine(const float (&acc)[kWeights][4], int c
   return __longlong_as_double((long long)(r | (neg ? 1ULL << 63 : 0ULL)));
 }
 
+// The same value (accumulators started at kMagic, sums below 2^20) with three FP64
+// operations: hi and lo become doubles as the low bits of 1.5 2^52, the sum is
+// rounded once, and the exponents are added to the word.
+__device__ __forceinline__ double combine_fp64(const float (&acc)[kWeights][4], int c, int Ea, int Eb) {
+  int s[kWeights];
+#pragma unroll
+  for (int k = 0; k < kWeights; ++k) s[k] = __float_as_int(acc[k][c]) - kMagicBits;
+  const long long hi = (long long)(s[0] * 128 + s[1]) * 16384 + (s[2] * 128 + s[3]);
+  const long long lo = ((long long)(s[4] * 128 + s[5]) * 16384 + (s[6] * 128 + s[7])) * 128 + s[8];
+  constexpr long long kOne = 0x4338000000000000LL;  // 1.5 2^52
+  constexpr double kBase = 6755399441055744.0, kTop = kBase * 34359738368.0;
+  const double h = fma(__longlong_as_double(kOne + hi), 34359738368.0, -kTop);  // hi 2^35, exact
+  const double v = h + (__longlong_as_double(kOne + lo) - kBase);
+  const int e = exponent_of(v), f = e + Ea + Eb - 2112;
+  if (e == 0 || f <= 0) return 0.0;
+  if (f >= 2047) return __longlong_as_double((long long)(v < 0.0 ? 0xfff0000000000000ULL : 0x7ff0000000000000ULL));
+  return __hiloint2double(__double2hiint(v) + (f - e) * 1048576, __double2loint(v));
+}
+
+// 16-byte copies from global to shared memory, one group per commit
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {  // at most N groups still in flight
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 }  // namespace eri
