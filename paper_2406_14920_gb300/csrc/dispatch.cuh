@@ -128,6 +128,12 @@ cudaError_t launch_grad_unit(int y, const GradArgs& a, cudaStream_t s, int nsm) 
       using T = std::conditional_t<P == 1, float, double>;
       const int64_t n = a.wl.total - a.wl.first;
       if constexpr (use_grad_thread(LA, LB, LC, LD, P == 1)) {
+        if constexpr (grad_block_when_short<LA, LB, LC, LD, T>()) {
+          using S = GShape<LA, LB, LC, LD, T>;
+          if (n <= (int64_t)kShortList * nsm)
+            return launch_over<grad_block_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.wl, n, false), 1, S::NT,
+                                                                     S::smem(), s, nsm);
+        }
         return launch_over<grad_thread_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.wl, n), 128, 128, 0, s, nsm);
       } else {
         using S = GShape<LA, LB, LC, LD, T>;

@@ -203,6 +203,11 @@ __device__ __forceinline__ int64_t item_tile(const WorkList& wl, int64_t items, 
   return t < 1 ? 1 : (t < wl.tile ? t : wl.tile);
 }
 
+// an item's primitive quartets in 16 steps of its class pair's largest
+__device__ __forceinline__ int work_bucket(const WorkList& wl, int npb, int npk) {
+  return (int)((int64_t)(npb * npk - 1) * 16 / ((int64_t)wl.mpb * wl.mpk));
+}
+
 // Ket position of list item ik of a bra pair with `count` kets.  Primitive
 // screening leaves the shell pairs of a class with different numbers of primitive
 // pairs, and a warp of a thread kernel takes as long as its longest item: every

@@ -16,7 +16,7 @@
 #define ERI_THREAD64_LMAX 6
 #endif
 #ifndef ERI_THREAD64_FOOT
-#define ERI_THREAD64_FOOT 200
+#define ERI_THREAD64_FOOT 190
 #endif
 
 namespace eri {

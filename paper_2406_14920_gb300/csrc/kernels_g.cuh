@@ -74,7 +74,7 @@ __host__ __device__ constexpr int grad_footprint(int la, int lb, int lc, int ld)
   return ncd * nherm(la + lb + 1) + ncart(la) * ncart(lb) * ncd + nherm(la + lb + lc + ld + 1);
 }
 #ifndef ERI_GRAD_THREAD64
-#define ERI_GRAD_THREAD64 155
+#define ERI_GRAD_THREAD64 235
 #endif
 #ifndef ERI_GRAD_THREAD32
 #define ERI_GRAD_THREAD32 330
@@ -83,6 +83,13 @@ __host__ __device__ constexpr bool use_grad_thread(int la, int lb, int lc, int l
   // (a large bra against (ss|: little work per thread and long code; a block is faster)
   return grad_footprint(la, lb, lc, ld) <= (fp32 ? ERI_GRAD_THREAD32 : ERI_GRAD_THREAD64) &&
          !(lc + ld == 0 && ncart(la) * ncart(lb) > 18);
+}
+
+// FP64 thread classes with long code run a block per item while the list is short
+// (see block_when_short)
+template <int LA, int LB, int LC, int LD, typename T>
+__host__ __device__ constexpr bool grad_block_when_short() {
+  return sizeof(T) == 8 && grad_footprint(LA, LB, LC, LD) >= 100;
 }
 
 // dE/dA and dE/dB of one item, bra primitives [pb0, pb1) and ket primitives [pk0, pk1)

@@ -166,43 +166,71 @@ __global__ void k_pairs(int npair, const int* __restrict__ s1, const int* __rest
 }
 
 // Mixed-precision tier split of the items [wl.first, wl.total) of one class
-// pair: one warp per chunk of 32 items (chunks t with t % nshard == shard), each
-// lane locates and tests one item; the FP64-tier and FP32-tier quartets are
-// appended to out0 / out1 (warp-aggregated atomics on cnt[0], cnt[1]).
-__global__ void __launch_bounds__(256) k_tier_split(KArgs a, int2* __restrict__ out0, int2* __restrict__ out1,
-                                                    unsigned int* __restrict__ cnt) {
+// pair: one warp per run of `rounds` x 32 items (runs t with t % nshard == shard;
+// the host takes one round per run where the work is shared over GPUs or the list
+// is short), each lane locates and tests one item per round; the FP64-tier and
+// FP32-tier quartets are appended to out0 / out1 (one atomic per run on cnt[0],
+// cnt[1]).  Inside a run the items of a tier are written by increasing number of
+// primitive quartets, so that the 32 lanes of a thread kernel's warp have about as
+// many (runs of 32 in list order: the FP32 (fp|pp) kernel of 900 functions took
+// 38.6 ms, its lanes waiting for the longest).
+constexpr int kSplitRounds = 8;
+__global__ void __launch_bounds__(256) k_tier_split(KArgs a, int rounds, int2* __restrict__ out0,
+                                                    int2* __restrict__ out1, unsigned int* __restrict__ cnt) {
+  __shared__ unsigned slots[8][32];  // per warp: [tier][work bucket] counts, then positions
   const int lane = threadIdx.x & 31;
+  unsigned* slot = slots[threadIdx.x >> 5];
   const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  const int64_t nch = (a.wl.total - a.wl.first + 31) / 32;
-  for (int64_t ch = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * a.wl.nshard + a.wl.shard;
-       ch < nch; ch += nwarps * a.wl.nshard) {
-    const int64_t item = a.wl.first + ch * 32 + lane;
-    int tier = -1, ib = 0, ik = 0;
-    if (item < a.wl.total) {
-      ib = find_bra(a.wl.prefix, a.wl.nbra, item);
-      ik = (int)(item - __ldg(a.wl.prefix + ib));
-      const int pb_id = __ldg(a.wl.bra + ib);
+  const int64_t nrun = (a.wl.total - a.wl.first + 32 * rounds - 1) / (32 * rounds);
+  for (int64_t run = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * a.wl.nshard + a.wl.shard;
+       run < nrun; run += nwarps * a.wl.nshard) {
+    int ib[kSplitRounds], ik[kSplitRounds], key[kSplitRounds];
+    int guard = 0, dropped = 0;
+    __syncwarp();
+    slot[lane] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < kSplitRounds; ++r) {
+      key[r] = -1;
+      const int64_t item = a.wl.first + (run * rounds + r) * 32 + lane;
+      if (r >= rounds || item >= a.wl.total) continue;
+      ib[r] = find_bra(a.wl.prefix, a.wl.nbra, item);
+      ik[r] = (int)(item - __ldg(a.wl.prefix + ib[r]));
+      const int pb_id = __ldg(a.wl.bra + ib[r]);
       const int mol = __ldg(a.sp.pmol + pb_id);
       const int seg = __ldg(a.wl.kseg + mol * NPAIRCLASS);
-      ik = ket_pos(a.wl, seg, ik, __ldg(a.wl.prefix + ib + 1) - __ldg(a.wl.prefix + ib));
-      const int pk_id = __ldg(a.wl.ket + seg + ik);
-      tier = quartet_tier(a, mol, pb_id, pk_id, __ldg(a.sp.s1 + pb_id), __ldg(a.sp.s2 + pb_id),
-                          __ldg(a.sp.s1 + pk_id), __ldg(a.sp.s2 + pk_id));
+      ik[r] = ket_pos(a.wl, seg, ik[r], __ldg(a.wl.prefix + ib[r] + 1) - __ldg(a.wl.prefix + ib[r]));
+      const int pk_id = __ldg(a.wl.ket + seg + ik[r]);
+      const int tier = a.mixed || a.screen > 0.0f
+                           ? quartet_tier(a, mol, pb_id, pk_id, __ldg(a.sp.s1 + pb_id), __ldg(a.sp.s2 + pb_id),
+                                          __ldg(a.sp.s1 + pk_id), __ldg(a.sp.s2 + pk_id))
+                           : 0;  // plain FP64 builds: the order only
+      guard += tier == 2;
+      dropped += tier == 3;
+      if (tier == 3) continue;
+      key[r] = (tier == 1 ? 16 : 0) + work_bucket(a.wl, __ldg(a.sp.np + pb_id), __ldg(a.sp.np + pk_id));
+      atomicAdd(slot + key[r], 1u);
     }
-    const unsigned gm = __ballot_sync(0xffffffffu, tier == 2);
-    if (gm && lane == 0 && a.guard) atomicAdd(a.guard, (unsigned long long)__popc(gm));
-    const unsigned sm = __ballot_sync(0xffffffffu, tier == 3);
-    if (sm && lane == 0 && a.screened) atomicAdd(a.screened, (unsigned long long)__popc(sm));
-    if (tier == 2) tier = 0;
+    guard = __reduce_add_sync(0xffffffffu, guard);
+    dropped = __reduce_add_sync(0xffffffffu, dropped);
+    if (lane == 0 && guard && a.guard) atomicAdd(a.guard, (unsigned long long)guard);
+    if (lane == 0 && dropped && a.screened) atomicAdd(a.screened, (unsigned long long)dropped);
+    __syncwarp();
+    const unsigned v = slot[lane];
+    unsigned x = v;  // inclusive sum over the buckets of the lane's tier
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const unsigned m = __ballot_sync(0xffffffffu, tier == t);
-      if (!m) continue;
-      unsigned base = 0;
-      if (lane == __ffs(m) - 1) base = atomicAdd(cnt + t, (unsigned)__popc(m));
-      base = __shfl_sync(0xffffffffu, base, __ffs(m) - 1);
-      if (tier == t) (t == 0 ? out0 : out1)[base + __popc(m & ((1u << lane) - 1u))] = make_int2(ib, ik);
+    for (int d = 1; d < 16; d <<= 1) {
+      const unsigned y = __shfl_up_sync(0xffffffffu, x, d, 16);
+      if ((lane & 15) >= d) x += y;
     }
+    unsigned base = 0;
+    if ((lane & 15) == 15 && x) base = atomicAdd(cnt + (lane >> 4), x);
+    base = __shfl_sync(0xffffffffu, base, 15, 16);
+    slot[lane] = base + x - v;
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < kSplitRounds; ++r)
+      if (key[r] >= 0) (key[r] < 16 ? out0 : out1)[atomicAdd(slot + key[r], 1u)] = make_int2(ib[r], ik[r]);
   }
 }
 
@@ -250,11 +278,14 @@ __global__ void k_etab(int npair, const int* __restrict__ s1, const int* __restr
 }
 
 // Schwarz bound per shell pair: Q = sqrt(max_{mu,nu} |(mu nu|mu nu)|) in FP64, rounded up to float32.
-// One block per pair, a warp per primitive quartet: R level by level over the
-// lanes, then a lane per component pair (a thread per pair kept E and R in local memory and
-// took 2 ms for one (ff|ff) diagonal, the longest kernel of a small molecule's
-// geometry step).  The E tables are those of k_etab; primitive quartets (i, j)
-// and (j, i) are equal, so j <= i with weight 2.
+// One block per pair.  Contracted pairs: a warp per primitive quartet; single
+// primitive pairs: the warps share the component pairs.  R goes level by level
+// over the lanes; then component pair by component pair (uniform loops) a lane
+// per bra Hermite index, summed over the warp in a fixed order.  (A lane per
+// component pair ran the union of the lanes' nested loops: 1.2 ms for the (ff|ff)
+// diagonal; a thread per pair with local arrays 2 ms; now 0.1 ms.)  The E tables
+// are those of k_etab; primitive quartets (i, j) and (j, i) are equal, so j <= i
+// with weight 2.
 constexpr int kSchwarzWarps = 6;  // 44 KB of shared memory
 constexpr int kSchwarzR = nherm(4 * LMAX);
 __global__ void __launch_bounds__(32 * kSchwarzWarps)
@@ -262,17 +293,19 @@ __global__ void __launch_bounds__(32 * kSchwarzWarps)
               const int* __restrict__ poff, const int* __restrict__ eoff, const int* __restrict__ sh_l,
               const int* __restrict__ ao, const double* __restrict__ f, PairData pd, BoysTabs bt,
               const RStep* __restrict__ st, float* __restrict__ Q) {
-  __shared__ double Rs[kSchwarzWarps][2][kSchwarzR], Fs[kSchwarzWarps][4 * LMAX + 1];
+  __shared__ double Rs[kSchwarzWarps][2][kSchwarzR], Fs[kSchwarzWarps][4 * LMAX + 1], dsum[kSchwarzWarps][100];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, ip = blockIdx.x;
   const int l1 = sh_l[s1[ip]], l2 = sh_l[s2[ip]], lp = l1 + l2, L = 2 * lp;
   const int n2 = ncart(l2), nc = ncart(l1) * n2, ne = (l1 + 1) * (l2 + 1) * (lp + 1);
+  const bool shared_quartet = np[ip] == 1;
   double* F = Fs[w];
-  double diag[4] = {0.0, 0.0, 0.0, 0.0};  // component pairs lane + 32 k (at most 100)
+  for (int c = lane; c < nc; c += 32) dsum[w][c] = 0.0;
+  __syncwarp();
   int turn = 0;
   for (int i = 0; i < np[ip]; ++i) {
     const int pi = poff[ip] + i;
     for (int j = 0; j <= i; ++j) {
-      if (turn++ % kSchwarzWarps != w) continue;
+      if (!shared_quartet && turn++ % kSchwarzWarps != w) continue;
       const int pj = poff[ip] + j;
       const double p = pd.p[pi], q = pd.p[pj], rho = p * q / (p + q);
       const double X = pd.P[pi] - pd.P[pj], Y = pd.P[pd.n + pi] - pd.P[pd.n + pj],
@@ -326,49 +359,40 @@ __global__ void __launch_bounds__(32 * kSchwarzWarps)
       }
       const double* E1 = pd.E + eoff[ip] + (size_t)i * 3 * ne;
       const double* E2 = pd.E + eoff[ip] + (size_t)j * 3 * ne;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int c = lane + 32 * k;
-        if (c >= nc) break;
+      for (int c = shared_quartet ? w : 0; c < nc; c += shared_quartet ? kSchwarzWarps : 1) {  // uniform over the warp
         int ix, iy, iz, jx, jy, jz;
         cart_xyz(l1, c / n2, ix, iy, iz);
         cart_xyz(l2, c % n2, jx, jy, jz);
+        const int mx = ix + jx + 1, my = iy + jy + 1, mz = iz + jz + 1;
         const int ox = (ix * (l2 + 1) + jx) * (lp + 1), oy = ne + (iy * (l2 + 1) + jy) * (lp + 1),
                   oz = 2 * ne + (iz * (l2 + 1) + jz) * (lp + 1);
         double v = 0.0;
-        for (int tx = 0; tx <= ix + jx; ++tx)
-          for (int ty = 0; ty <= iy + jy; ++ty)
-            for (int tz = 0; tz <= iz + jz; ++tz) {
-              double u = 0.0;
-              for (int sx = 0; sx <= ix + jx; ++sx)
-                for (int sy = 0; sy <= iy + jy; ++sy) {
-                  double uz = 0.0;
-                  for (int sz = 0; sz <= iz + jz; ++sz)
-                    uz = fma((sx + sy + sz) & 1 ? -E2[oz + sz] : E2[oz + sz],
-                             cur[herm_index(tx + sx, ty + sy, tz + sz)], uz);
-                  u = fma(E2[ox + sx] * E2[oy + sy], uz, u);
-                }
-              v = fma(E1[ox + tx] * E1[oy + ty] * E1[oz + tz], u, v);
+        for (int t = lane; t < mx * my * mz; t += 32) {
+          const int tx = t / (my * mz), ty = t / mz % my, tz = t % mz;
+          double u = 0.0;
+          for (int sx = 0; sx < mx; ++sx)
+            for (int sy = 0; sy < my; ++sy) {
+              double uz = 0.0;
+              for (int sz = 0; sz < mz; ++sz)
+                uz = fma((sx + sy + sz) & 1 ? -E2[oz + sz] : E2[oz + sz], cur[herm_index(tx + sx, ty + sy, tz + sz)], uz);
+              u = fma(E2[ox + sx] * E2[oy + sy], uz, u);
             }
-        diag[k] += v;
+          v = fma(E1[ox + tx] * E1[oy + ty] * E1[oz + tz], u, v);
+        }
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) dsum[w][c] += v;
       }
       __syncwarp();
     }
   }
   __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 4; ++k) Rs[w][0][lane + 32 * k] = diag[k];
-  __syncthreads();
   if (w != 0) return;
   double mx = 0.0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int c = lane + 32 * k;
-    if (c < nc) {
-      for (int x = 1; x < kSchwarzWarps; ++x) diag[k] += Rs[x][0][c];
-      const double fn = f[ao[s1[ip]] + c / n2] * f[ao[s2[ip]] + c % n2];
-      mx = fmax(mx, fabs(diag[k] * fn * fn));
-    }
+  for (int c = lane; c < nc; c += 32) {
+    double v = 0.0;
+    for (int x = 0; x < kSchwarzWarps; ++x) v += dsum[x][c];
+    const double fn = f[ao[s1[ip]] + c / n2] * f[ao[s2[ip]] + c % n2];
+    mx = fmax(mx, fabs(v * fn * fn));
   }
   for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if (lane == 0) Q[ip] = __double2float_ru(sqrt(mx));
@@ -386,45 +410,48 @@ __global__ void __launch_bounds__(32 * kSchwarzWarps)
 // kernels run over those.  Each dropped primitive quartet is below 1e-8 of the
 // quartet threshold (thresh = 0 drops none).
 constexpr double kPrimEps = 1e-8;
-__global__ void k_primq(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
-                        const int* __restrict__ poff, const int* __restrict__ eoff, const int* __restrict__ sh_l,
-                        const int* __restrict__ ao, const double* __restrict__ f, const int* __restrict__ pmol,
-                        PairData pd, double* __restrict__ pq, unsigned int* __restrict__ pqmax) {
+__global__ void __launch_bounds__(128)
+    k_primq(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
+            const int* __restrict__ poff, const int* __restrict__ eoff, const int* __restrict__ sh_l,
+            const int* __restrict__ ao, const double* __restrict__ f, const int* __restrict__ pmol, PairData pd,
+            double* __restrict__ pq, unsigned int* __restrict__ pqmax) {
+  __shared__ double Ss[4][3 * (LMAX + 1) * (LMAX + 1)];
   const int ip = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;  // one warp per pair
   if (ip >= npair) return;
+  double* S = Ss[threadIdx.x >> 5];
   const int a = s1[ip], b = s2[ip], l1 = sh_l[a], l2 = sh_l[b], lp = l1 + l2;
-  const int ne = (l1 + 1) * (l2 + 1) * (lp + 1);
+  const int rows = (l1 + 1) * (l2 + 1), n2 = ncart(l2), nc = ncart(l1) * n2;
   double fm = 0.0, fn = 0.0;
   for (int c = 0; c < ncart(l1); ++c) fm = fmax(fm, f[ao[a] + c]);
-  for (int c = 0; c < ncart(l2); ++c) fn = fmax(fn, f[ao[b] + c]);
+  for (int c = 0; c < n2; ++c) fn = fmax(fn, f[ao[b] + c]);
+  const double df[2 * LMAX + 1] = {1.0, 1.0, 3.0, 15.0, 105.0, 945.0, 10395.0};  // (2t-1)!!
   double top = 0.0;
-  for (int k = lane; k < np[ip]; k += 32) {
+  for (int k = 0; k < np[ip]; ++k) {
     const int pi = poff[ip] + k;
-    const double p = pd.p[pi], rp = sqrt(p);
-    double S[3][(LMAX + 1) * (LMAX + 1)];
-    for (int d = 0; d < 3; ++d)
-      for (int r = 0; r < (l1 + 1) * (l2 + 1); ++r) {
-        const double* E = pd.E + eoff[ip] + ((size_t)k * 3 + d) * ne + (size_t)r * (lp + 1);
-        double w = 1.0, v = 0.0;  // w = (p^t (2t-1)!!)^(1/2)
-        for (int t = 0; t <= lp; ++t) {
-          v += fabs(E[t]) * w;
-          w *= rp * sqrt(2.0 * t + 1.0);
-        }
-        S[d][r] = v;
+    const double p = pd.p[pi];
+    for (int r = lane; r < 3 * rows; r += 32) {
+      const double* E = pd.E + eoff[ip] + ((size_t)k * 3 * rows + r) * (lp + 1);
+      double v = 0.0, pt = 1.0;
+      for (int t = 0; t <= lp; ++t) {
+        v += fabs(E[t]) * sqrt(pt * df[t]);
+        pt *= p;
       }
+      S[r] = v;
+    }
+    __syncwarp();
     double mx = 0.0;
-    for (int mu = 0; mu < ncart(l1); ++mu)
-      for (int nu = 0; nu < ncart(l2); ++nu) {
-        int ix, iy, iz, jx, jy, jz;
-        cart_xyz(l1, mu, ix, iy, iz);
-        cart_xyz(l2, nu, jx, jy, jz);
-        mx = fmax(mx, S[0][ix * (l2 + 1) + jx] * S[1][iy * (l2 + 1) + jy] * S[2][iz * (l2 + 1) + jz]);
-      }
+    for (int c = lane; c < nc; c += 32) {
+      int ix, iy, iz, jx, jy, jz;
+      cart_xyz(l1, c / n2, ix, iy, iz);
+      cart_xyz(l2, c % n2, jx, jy, jz);
+      mx = fmax(mx, S[ix * (l2 + 1) + jx] * S[rows + iy * (l2 + 1) + jy] * S[2 * rows + iz * (l2 + 1) + jz]);
+    }
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     const double q = fabs(pd.pref[pi]) * rsqrt(sqrt(2.0 * p)) * mx * fm * fn;
-    pq[pi] = q;
+    if (lane == 0) pq[pi] = q;
     top = fmax(top, q);
+    __syncwarp();
   }
-  for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
   if (lane == 0) atomicMax(pqmax + pmol[ip], __float_as_uint(__double2float_ru(fmin(top, 1e38))));
 }
 
@@ -1113,6 +1140,9 @@ int eri_plan_impl::ensure_streams() {
   return ERI_OK;
 }
 
+// longest compacted tier list (items); longer class-pair lists are split in windows
+static const int64_t kTierCap = 1 << 23;
+
 int eri_plan_impl::fork(cudaStream_t s, int n) {
   CK(cudaEventRecord(fork_ev, s));
   for (int b = 0; b < n; ++b) CK(cudaStreamWaitEvent(branch[b], fork_ev, 0));
@@ -1132,14 +1162,22 @@ int eri_plan_impl::join(cudaStream_t s, int n) {
 // hold a few blocks each, and one after another they leave most SMs idle.
 // Profiled calls run in order on the caller's stream, so that an event pair
 // times one launch.
-int eri_plan_impl::eager_branches() const {
-  return opts.profile ? 0 : kStreams;
+// With tier lists the streams are as many (4 to kStreams) as keep the lists
+// within 512 MB.
+int eri_plan_impl::eager_branches(bool lists) const {
+  if (opts.profile) return 0;
+  int n = kStreams;
+  if (lists) {
+    int64_t mx = 1;
+    for (int64_t t : h_jtot) mx = std::max(mx, t);
+    while (n > kBranches && n * std::min(mx, kTierCap) > (int64_t)1 << 25) n /= 2;
+  }
+  return n;
 }
 
 // Compacted tier lists of mixed-precision builds: per branch, two lists of
 // tier_cap items (int2 bra / ket positions) and two counters.  tier_cap is the
 // longest class-pair list, at most kTierCap; longer lists are split in windows.
-static const int64_t kTierCap = 1 << 23;
 
 int eri_plan_impl::ensure_tier_bufs(int nb) {
   int64_t mx = 1;
@@ -1159,6 +1197,19 @@ int eri_plan_impl::ensure_tier_bufs(int nb) {
   for (int b = tier_nb; b < nb; ++b) CK(dalloc(&tbuf[b], 2 * (size_t)tier_cap));
   tier_nb = std::max(tier_nb, nb);
   return ERI_OK;
+}
+
+// tier split of the window ka.wl into buf (FP64 tier) and buf + tier_cap (FP32 tier)
+static cudaError_t launch_tier_split(const eri_plan_impl* P, const KArgs& ka, int2* buf, unsigned int* cnt,
+                                     cudaStream_t s) {
+  const int64_t items = ka.wl.total - ka.wl.first, warps = (int64_t)P->nsm * 64;
+  // long runs sort better; they may leave this kernel short of warps (8 per SM), not the tiers' kernels
+  const int rounds =
+      ka.wl.nshard > 1 ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(kSplitRounds, items / (4 * warps)));
+  const int64_t runs = (items + 32 * rounds - 1) / (32 * rounds);
+  k_tier_split<<<(int)std::max<int64_t>(1, std::min<int64_t>((runs + 7) / 8, warps / 8)), 256, 0, s>>>(
+      ka, rounds, buf, buf + P->tier_cap, cnt);
+  return cudaGetLastError();
 }
 
 cudaError_t eri_plan_impl::prof_event_pair(cudaEvent_t* a, cudaEvent_t* b) {
@@ -1611,6 +1662,15 @@ static void assign_branches(std::vector<ClassLaunch>& v, int nbranch) {
   }
 }
 
+// Whether a plain FP64 build orders this class pair's list by work first: a thread
+// kernel, contracted pairs, and some quartets per lane (225 functions: (pp|ps) 6.5
+// ms in list order, of which a third is lanes waiting for the longest).
+static bool order_first(const eri_plan_impl* P, int X, int Y) {
+  return use_thread_kernel(kClassL1[X], kClassL2[X], kClassL1[Y], kClassL2[Y], false) &&
+         P->h_maxnp[X] * P->h_maxnp[Y] > 1 && P->nshard == 1 &&
+         P->h_ktot[X * NPAIRCLASS + Y] >= (int64_t)256 * P->nsm;
+}
+
 // One J/K build on stream s, lists as they stand.  nbranch > 0: the class
 // launches are spread over that many of the plan's side streams (fork / join by
 // events); 0: they run in order on s (profiled builds).
@@ -1713,10 +1773,7 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
           sa.wl.first = f;
           sa.wl.total = std::min<int64_t>(full.total, f + P->tier_cap);
           CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned int), ls));
-          const int64_t nch = (sa.wl.total - f + 31) / 32;
-          k_tier_split<<<(int)std::max<int64_t>(1, std::min<int64_t>((nch + 7) / 8, (int64_t)P->nsm * 8)), 256, 0,
-                         ls>>>(sa, buf, buf + P->tier_cap, cnt);
-          CK(cudaGetLastError());
+          CK(launch_tier_split(P, sa, buf, cnt, ls));
           for (int tier = 0; tier < 2; ++tier) {
             ja.wl = full;
             ja.wl.first = 0;
@@ -1782,6 +1839,19 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       const int rc = P->ensure_tier_bufs(std::max(1, nbranch));  // (a graph capture has them already)
       if (rc != ERI_OK) return rc;
     }
+    // Plain FP64 builds order the long lists of the thread kernels the same way
+    // (every quartet in one list, see k_tier_split); without room for the lists, or
+    // while the caller captures before the first build, they run in list order.
+    bool ordered = false;
+    if (!split) {
+      for (const ClassLaunch& l : order) ordered = ordered || order_first(P, l.X, l.Y);
+      if (ordered && P->tier_nb < std::max(1, nbranch)) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(s, &st));
+        ordered = st == cudaStreamCaptureStatusNone && P->ensure_tier_bufs(std::max(1, nbranch)) == ERI_OK;
+        if (!ordered) cudaGetLastError();
+      }
+    }
     assign_branches(order, nbranch);
     if (concurrent) {
       const int rc = P->fork(s, nbranch);
@@ -1808,7 +1878,7 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       const int b = l.branch;
       const cudaStream_t ls = concurrent ? P->branch[b] : s;
       ka.same_class = l.X == l.Y;
-      if (!split) {
+      if (!split && !(ordered && order_first(P, l.X, l.Y))) {
         ka.wl = P->klist(l.X, l.Y);
         ka.items = nullptr;
         ka.nitems = nullptr;
@@ -1828,10 +1898,7 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
         sa.wl.first = f;
         sa.wl.total = std::min<int64_t>(full.total, f + P->tier_cap);
         CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned int), ls));
-        const int64_t nch = (sa.wl.total - f + 31) / 32;
-        k_tier_split<<<(int)std::max<int64_t>(1, std::min<int64_t>((nch + 7) / 8, (int64_t)P->nsm * 8)), 256, 0,
-                       ls>>>(sa, buf, buf + P->tier_cap, cnt);
-        CK(cudaGetLastError());
+        CK(launch_tier_split(P, sa, buf, cnt, ls));
         for (int tier = 0; tier < (mixed ? 2 : 1); ++tier) {
           ka.wl = full;
           ka.wl.first = 0;
@@ -1873,7 +1940,7 @@ extern "C" int eri_build_jk(eri_plan_t* plan, const double* D, double* J, double
     int rc = P->build_lists(thresh, s);
     if (rc != ERI_OK) return rc;
   }
-  return build_impl(P, D, J, K, precision, s, P->eager_branches());
+  return build_impl(P, D, J, K, precision, s, P->eager_branches(true));
 }
 
 extern "C" int eri_build_jk_graph(eri_plan_t* plan, const double* D, double* J, double* K, int32_t precision,
@@ -1886,9 +1953,11 @@ extern "C" int eri_build_jk_graph(eri_plan_t* plan, const double* D, double* J, 
   if (!P->gexec || P->gkey[0] != D || P->gkey[1] != J || P->gkey[2] != K || P->gprec != precision) {
     int rc = P->ensure_streams();
     if (rc != ERI_OK) return rc;
-    if (precision == ERI_MIXED || P->opts.density_screen) {
-      rc = P->ensure_tier_bufs(eri_plan_impl::kBranches);
-      if (rc != ERI_OK) return rc;
+    rc = P->ensure_tier_bufs(eri_plan_impl::kBranches);
+    if (rc != ERI_OK) {
+      if (precision == ERI_MIXED || P->opts.density_screen) return rc;
+      rc = ERI_OK;  // a plain FP64 build runs without them
+      cudaGetLastError();
     }
     if (P->gexec) {
       CK(cudaStreamSynchronize(s));
@@ -2022,9 +2091,7 @@ extern "C" int eri_autotune(eri_plan_t* plan, const double* D, int32_t precision
         ka.nitems = nullptr;
         if (mixed) {
           if (cudaMemsetAsync(P->tcnt, 0, 2 * sizeof(unsigned int), s) != cudaSuccess) return -1.0;
-          const int64_t nch = (last - f + 31) / 32;
-          k_tier_split<<<(int)std::max<int64_t>(1, std::min<int64_t>((nch + 7) / 8, (int64_t)P->nsm * 8)), 256, 0,
-                         s>>>(ka, P->tbuf[0], P->tbuf[0] + P->tier_cap, P->tcnt);
+          if (launch_tier_split(P, ka, P->tbuf[0], P->tcnt, s) != cudaSuccess) return -1.0;
           ka.wl.first = 0;
           ka.wl.total = last - f;
           ka.items = P->tbuf[0] + (tier ? P->tier_cap : 0);
@@ -2247,7 +2314,7 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
     k_dmax<<<grid1(P->npair, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_sh_l, P->d_pao1, P->d_pao2,
                                                 P->d_pmol, P->d_mat_off, P->d_mat_n, P->d_Dp, P->d_dmax);
     CK(cudaGetLastError());
-    const int rc = P->ensure_tier_bufs(std::max(1, P->eager_branches()));
+    const int rc = P->ensure_tier_bufs(std::max(1, P->eager_branches(true)));
     if (rc != ERI_OK) return rc;
   }
   GradArgs ga{};
@@ -2281,7 +2348,7 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
     }
     return ERI_OK;
   };
-  const int nbranch = P->eager_branches();
+  const int nbranch = P->eager_branches(mixed);
   std::vector<ClassLaunch> order;
   for (int X = 0; X < NPAIRCLASS; ++X)
     for (int Y = 0; Y < NPAIRCLASS; ++Y) {
@@ -2311,10 +2378,7 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
       ka.wl.first = f;
       ka.wl.total = std::min<int64_t>(full.total, f + P->tier_cap);
       CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned int), ls));
-      const int64_t nch = (ka.wl.total - f + 31) / 32;
-      k_tier_split<<<(int)std::max<int64_t>(1, std::min<int64_t>((nch + 7) / 8, (int64_t)P->nsm * 8)), 256, 0, ls>>>(
-          ka, buf, buf + P->tier_cap, cnt);
-      CK(cudaGetLastError());
+      CK(launch_tier_split(P, ka, buf, cnt, ls));
       for (int tier = 0; tier < 2; ++tier) {
         ga.wl = full;
         ga.wl.first = 0;
