@@ -35,8 +35,26 @@ using namespace eri;
 
 namespace {
 
+static_assert(2 * LMAX + 1 <= eri_plan_impl::kStreams, "one stream per pair order");
 constexpr double kVfac = 1.0622519320271968;  // (2 pi / p) / (sqrt(2 pi^(5/2)) / p): pair prefactor of V from the ERI one
-constexpr int kChunk = 256;                    // charges (or primitive pairs) per block row
+constexpr int kChunk = 256;  // charges per warp at most
+constexpr int kTr = 16;      // at least (and the charges whose gradients are transposed at a time)
+
+// A warp takes 32 primitive pairs and a chunk of the charges.  The chunks are as
+// long as leave 16 warps per SM: the lists of f pairs are short, and in fixed
+// chunks of 256 charges ten (ff) pairs were 12 warps with 2 ms each.
+struct NucGrid {
+  int groups, chunk, blocks;
+};
+inline NucGrid nuc_grid(const eri_plan_impl* P, int n, int nc) {
+  NucGrid g;
+  g.groups = (n + 31) / 32;
+  const int64_t c = (int64_t)nc * g.groups / (16 * (int64_t)P->nsm);
+  g.chunk = (int)std::max<int64_t>(kTr, std::min<int64_t>(kChunk, c / kTr * kTr));
+  const int64_t warps = (int64_t)g.groups * ((nc + g.chunk - 1) / g.chunk);
+  g.blocks = (int)((warps + 3) / 4);
+  return g;
+}
 
 #define NCK(x)                                                                   \
   do {                                                                           \
@@ -52,12 +70,14 @@ __device__ __forceinline__ double warp_add(double v) {
 
 // h_P of one list entry (primitive pair) summed over one chunk of charges
 template <int L>
-__global__ void __launch_bounds__(128) k_nuc_herm(const int4* __restrict__ list, int n, PairData pd, BoysTabs bt,
-                                                  int nc, const double* __restrict__ q, const double* __restrict__ xyz,
-                                                  double* __restrict__ Vh) {
+__global__ void __launch_bounds__(128) k_nuc_herm(const int4* __restrict__ list, int n, NucGrid ng, PairData pd,
+                                                  BoysTabs bt, int nc, const double* __restrict__ q,
+                                                  const double* __restrict__ xyz, double* __restrict__ Vh) {
   constexpr int NH = nherm(L);
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  const int64_t warp = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int i = (int)(warp % ng.groups) * 32 + (threadIdx.x & 31);
+  const int64_t c0 = warp / ng.groups * ng.chunk;
+  if (i >= n || c0 >= nc) return;
   const int4 e = __ldg(list + i);
   const int pi = e.x;
   const double p = __ldg(pd.p + pi), pref = __ldg(pd.pref + pi) * kVfac;
@@ -65,8 +85,8 @@ __global__ void __launch_bounds__(128) k_nuc_herm(const int4* __restrict__ list,
   double h[NH];
 #pragma unroll
   for (int x = 0; x < NH; ++x) h[x] = 0.0;
-  const int c0 = blockIdx.y * kChunk, c1 = min(nc, c0 + kChunk);
-  for (int c = c0; c < c1; ++c) {
+  const int c1 = (int)min((int64_t)nc, c0 + ng.chunk);
+  for (int c = (int)c0; c < c1; ++c) {
     const double X = Px - __ldg(xyz + 3 * c), Y = Py - __ldg(xyz + 3 * c + 1), Z = Pz - __ldg(xyz + 3 * c + 2);
     double F[L + 1];
     boys_f64<L>(p * (X * X + Y * Y + Z * Z), bt, F);
@@ -137,15 +157,17 @@ __global__ void __launch_bounds__(128)
 
 // h_P of one primitive pair over one chunk of charges, and dE/dC of the chunk
 // (dEdC may be null) over the block's pairs
-constexpr int kTr = 16;  // charges transposed at a time
 template <int L>
-__global__ void __launch_bounds__(128) k_nuc_grad(const int4* __restrict__ list, int n, PairData pd, BoysTabs bt,
-                                                  double* __restrict__ G, int nc, const double* __restrict__ q,
+__global__ void __launch_bounds__(128) k_nuc_grad(const int4* __restrict__ list, int n, NucGrid ng, PairData pd,
+                                                  BoysTabs bt, double* __restrict__ G, int nc, const double* __restrict__ q,
                                                   const double* __restrict__ xyz, double* __restrict__ dEdC) {
   constexpr int H = nherm(L), H1 = nherm(L + 1);
   __shared__ double tr[4][3 * kTr][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t warp = (int64_t)blockIdx.x * 4 + w;
+  const int i = (int)(warp % ng.groups) * 32 + lane;
+  const int64_t c0 = warp / ng.groups * ng.chunk;
+  if (c0 >= nc) return;   // whole warp; nothing syncs the block
   const bool ok = i < n;  // lanes past the list repeat its last entry with weight 0
   const int4 e = __ldg(list + (ok ? i : n - 1));
   const int pi = e.x;
@@ -155,8 +177,8 @@ __global__ void __launch_bounds__(128) k_nuc_grad(const int4* __restrict__ list,
   double h[H1];
 #pragma unroll
   for (int x = 0; x < H1; ++x) h[x] = 0.0;
-  const int c0 = blockIdx.y * kChunk, c1 = min(nc, c0 + kChunk);
-  for (int cb = c0; cb < c1; cb += kTr) {
+  const int c1 = (int)min((int64_t)nc, c0 + ng.chunk);
+  for (int cb = (int)c0; cb < c1; cb += kTr) {
     const int ce = min(c1, cb + kTr);
     for (int c = cb; c < ce; ++c) {
       const double X = Px - __ldg(xyz + 3 * c), Y = Py - __ldg(xyz + 3 * c + 1), Z = Pz - __ldg(xyz + 3 * c + 2);
@@ -248,9 +270,9 @@ template <int L>
 cudaError_t launch_herm(const eri_plan_impl* P, int nc, const double* q, const double* xyz, cudaStream_t s) {
   const int n = P->nuc_cnt[L];
   if (n == 0 || nc == 0) return cudaSuccess;
-  const dim3 grid((n + 127) / 128, (nc + kChunk - 1) / kChunk);
-  k_nuc_herm<L><<<grid, 128, 0, s>>>(P->d_nuc_list + P->nuc_first[L], n, P->pairdata(), P->boystabs(), nc, q, xyz,
-                                     P->d_Jherm);
+  const NucGrid ng = nuc_grid(P, n, nc);
+  k_nuc_herm<L><<<ng.blocks, 128, 0, s>>>(P->d_nuc_list + P->nuc_first[L], n, ng, P->pairdata(), P->boystabs(), nc, q,
+                                          xyz, P->d_Jherm);
   return cudaGetLastError();
 }
 
@@ -260,8 +282,8 @@ cudaError_t launch_grad(const eri_plan_impl* P, int nc, const double* q, const d
   const int n = P->nuc_cnt[L];
   if (n == 0 || nc == 0) return cudaSuccess;
   const int4* list = P->d_nuc_list + P->nuc_first[L];
-  const dim3 grid((n + 127) / 128, (nc + kChunk - 1) / kChunk);
-  k_nuc_grad<L><<<grid, 128, 0, s>>>(list, n, P->pairdata(), P->boystabs(), P->d_nuc_dens, nc, q, xyz, dEdC);
+  const NucGrid ng = nuc_grid(P, n, nc);
+  k_nuc_grad<L><<<ng.blocks, 128, 0, s>>>(list, n, ng, P->pairdata(), P->boystabs(), P->d_nuc_dens, nc, q, xyz, dEdC);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_nuc_atoms<<<(n + 127) / 128, 128, 0, s>>>(list, n, L, P->pairdata(), P->d_ps1, P->d_ps2, P->d_sh_atom,
@@ -324,13 +346,16 @@ extern "C" int eri_nuclear(eri_plan_t* plan, int32_t ncharge, const double* q, c
   NCK(cudaSetDevice(P->device));
   if ((rc = ensure_nuc(P)) != ERI_OK) return rc;
   NCK(cudaMemsetAsync(P->d_Jherm, 0, sizeof(double) * (size_t)P->nherm_tot, s));
-  NCK(launch_herm<0>(P, ncharge, q, xyz, s));
-  NCK(launch_herm<1>(P, ncharge, q, xyz, s));
-  NCK(launch_herm<2>(P, ncharge, q, xyz, s));
-  NCK(launch_herm<3>(P, ncharge, q, xyz, s));
-  NCK(launch_herm<4>(P, ncharge, q, xyz, s));
-  NCK(launch_herm<5>(P, ncharge, q, xyz, s));
-  NCK(launch_herm<6>(P, ncharge, q, xyz, s));
+  // independent sums (atomics), one of the plan's streams each
+  if ((rc = P->fork(s, 2 * LMAX + 1)) != ERI_OK) return rc;
+  NCK(launch_herm<6>(P, ncharge, q, xyz, P->branch[0]));
+  NCK(launch_herm<5>(P, ncharge, q, xyz, P->branch[1]));
+  NCK(launch_herm<4>(P, ncharge, q, xyz, P->branch[2]));
+  NCK(launch_herm<3>(P, ncharge, q, xyz, P->branch[3]));
+  NCK(launch_herm<2>(P, ncharge, q, xyz, P->branch[4]));
+  NCK(launch_herm<1>(P, ncharge, q, xyz, P->branch[5]));
+  NCK(launch_herm<0>(P, ncharge, q, xyz, P->branch[6]));
+  if ((rc = P->join(s, 2 * LMAX + 1)) != ERI_OK) return rc;
   const MolMats mm = molmats(P);
   k_post_j<<<(int)(((int64_t)P->npair * 100 + 127) / 128), 128, 0, s>>>(
       P->npair, P->d_ps1, P->d_ps2, P->d_pnp, P->d_phoff, P->d_peoff, P->d_sh_l, P->d_pao1, P->d_pao2, P->d_pmol, mm,
@@ -356,12 +381,15 @@ extern "C" int eri_nuclear_grad(eri_plan_t* plan, const double* D, int32_t nchar
   NCK(cudaGetLastError());
   NCK(cudaMemsetAsync(dEdR, 0, sizeof(double) * 3 * (size_t)P->natom, s));
   if (dEdC && ncharge > 0) NCK(cudaMemsetAsync(dEdC, 0, sizeof(double) * 3 * (size_t)ncharge, s));
-  NCK(launch_grad<0>(P, ncharge, q, xyz, dEdR, dEdC, s));
-  NCK(launch_grad<1>(P, ncharge, q, xyz, dEdR, dEdC, s));
-  NCK(launch_grad<2>(P, ncharge, q, xyz, dEdR, dEdC, s));
-  NCK(launch_grad<3>(P, ncharge, q, xyz, dEdR, dEdC, s));
-  NCK(launch_grad<4>(P, ncharge, q, xyz, dEdR, dEdC, s));
-  NCK(launch_grad<5>(P, ncharge, q, xyz, dEdR, dEdC, s));
-  NCK(launch_grad<6>(P, ncharge, q, xyz, dEdR, dEdC, s));
+  // independent sums (atomics), one of the plan's streams each
+  if ((rc = P->fork(s, 2 * LMAX + 1)) != ERI_OK) return rc;
+  NCK(launch_grad<6>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[0]));
+  NCK(launch_grad<5>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[1]));
+  NCK(launch_grad<4>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[2]));
+  NCK(launch_grad<3>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[3]));
+  NCK(launch_grad<2>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[4]));
+  NCK(launch_grad<1>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[5]));
+  NCK(launch_grad<0>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[6]));
+  if ((rc = P->join(s, 2 * LMAX + 1)) != ERI_OK) return rc;
   return ERI_OK;
 }
