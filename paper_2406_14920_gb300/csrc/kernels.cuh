@@ -186,6 +186,13 @@ __device__ __forceinline__ PrimSplit prim_split(const WorkList& wl, int64_t item
   return s;
 }
 
+// Tile of a warp's turn: turns of nwarps tiles, the warps shifted by three from
+// turn to turn.  Lists are ordered by work inside runs of 8 rounds, and nwarps is
+// a multiple of 8: unshifted, a warp would meet the same place of every run.
+__device__ __forceinline__ int64_t warp_tile(int64_t turn, int64_t warp, int64_t nwarps) {
+  return turn * nwarps + (warp + 3 * turn) % nwarps;
+}
+
 // Rounds of 32 items per tile of a thread kernel over the ordered lists: wl.tile
 // (long runs share a bra pair, whose sums go out together), fewer on lists that
 // would leave warps idle (185 functions, J-engine (ps|ps): 9.4 -> 6.0 ms)
@@ -451,8 +458,10 @@ __global__ void __launch_bounds__(128) j_thread_kernel(JArgs a) {
   const int64_t span = 32 * thread_tile(a.wl, total - first, nwarps), ntiles = (total - first + span - 1) / span;
   unsigned long long done = 0, doneq = 0, doneb = 0;
   const PrimSplit sp = prim_split<T>(a.wl, total - first, 32 * nwarps);
-  for (int64_t tl = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * nshard + shard;
-       tl < ntiles * sp.n; tl += nwarps * nshard) {
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  for (int64_t turn = 0; turn * nwarps * nshard < ntiles * sp.n; ++turn) {
+    const int64_t tl = warp_tile(turn, warp, nwarps) * nshard + shard;
+    if (tl >= ntiles * sp.n) continue;
     const int part = (int)(tl / ntiles);
     const int64_t t0 = first + (tl - part * ntiles) * span, i1 = t0 + span < total ? t0 + span : total;
     BraCursor cur;

@@ -343,8 +343,10 @@ __global__ void __launch_bounds__(128) jk_thread_kernel(JKArgs A) {
   const int64_t span = 32 * (int64_t)a.wl.tile, ntiles = (total - first + span - 1) / span;
   const int lane = threadIdx.x & 31;
   const PrimSplit sp = prim_split<T>(a.wl, total - first, stride);
-  for (int64_t tl = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * nshard + shard; tl < ntiles * sp.n;
-       tl += (stride >> 5) * nshard) {
+  const int64_t nwarps = stride >> 5, warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  for (int64_t turn = 0; turn * nwarps * nshard < ntiles * sp.n; ++turn) {
+    const int64_t tl = warp_tile(turn, warp, nwarps) * nshard + shard;
+    if (tl >= ntiles * sp.n) continue;
     const int part = (int)(tl / ntiles);
     const int64_t t0 = first + (tl - part * ntiles) * span;
     const int64_t i1 = t0 + span < total ? t0 + span : total;

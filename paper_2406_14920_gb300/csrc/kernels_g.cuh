@@ -246,8 +246,10 @@ __global__ void __launch_bounds__(128) grad_thread_kernel(GradArgs a) {
   const PrimSplit sp = prim_split<T>(a.wl, total - first, 32 * nwarps);
   const int64_t span = 32 * thread_tile(a.wl, total - first, nwarps), ntiles = (total - first + span - 1) / span;
   unsigned long long done = 0, doneq = 0, doneb = 0;
-  for (int64_t tl = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * nshard + shard; tl < ntiles * sp.n;
-       tl += nwarps * nshard) {
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  for (int64_t turn = 0; turn * nwarps * nshard < ntiles * sp.n; ++turn) {
+    const int64_t tl = warp_tile(turn, warp, nwarps) * nshard + shard;
+    if (tl >= ntiles * sp.n) continue;
     const int part = (int)(tl / ntiles);
     const int64_t t0 = first + (tl - part * ntiles) * span, i1 = t0 + span < total ? t0 + span : total;
     BraCursor cur;

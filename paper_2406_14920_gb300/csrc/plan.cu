@@ -1652,14 +1652,18 @@ struct ClassLaunch {
   double cost;
   int branch;
 };
-static void assign_branches(std::vector<ClassLaunch>& v, int nbranch) {
-  if (nbranch <= 0) return;
+// Returns the number of streams used (no more than there are launches: a fork and
+// join costs the host about 1 us per stream).
+static int assign_branches(std::vector<ClassLaunch>& v, int nbranch) {
+  nbranch = std::min(nbranch, (int)v.size());
+  if (nbranch <= 0) return 0;
   std::stable_sort(v.begin(), v.end(), [](const ClassLaunch& a, const ClassLaunch& b) { return a.cost > b.cost; });
   double load[eri_plan_impl::kStreams] = {};
   for (ClassLaunch& l : v) {
     l.branch = (int)(std::min_element(load, load + nbranch) - load);
     load[l.branch] += l.cost;
   }
+  return nbranch;
 }
 
 // Whether a plain FP64 build orders this class pair's list by work first: a thread
@@ -1750,7 +1754,7 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
         const int64_t tot = P->h_jtot[X * NPAIRCLASS + Y];
         if (tot > 0) order.push_back({X, Y, jengine_flops(X, Y, (double)tot * P->h_maxnp[X] * P->h_maxnp[Y]), 0});
       }
-    assign_branches(order, nbranch);
+    nbranch = assign_branches(order, nbranch);
     if (concurrent) {
       const int rc = P->fork(s, nbranch);
       if (rc != ERI_OK) return rc;
@@ -1852,7 +1856,7 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
         if (!ordered) cudaGetLastError();
       }
     }
-    assign_branches(order, nbranch);
+    nbranch = assign_branches(order, nbranch);
     if (concurrent) {
       const int rc = P->fork(s, nbranch);
       if (rc != ERI_OK) return rc;
@@ -2348,14 +2352,14 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
     }
     return ERI_OK;
   };
-  const int nbranch = P->eager_branches(mixed);
+  int nbranch = P->eager_branches(mixed);
   std::vector<ClassLaunch> order;
   for (int X = 0; X < NPAIRCLASS; ++X)
     for (int Y = 0; Y < NPAIRCLASS; ++Y) {
       const double tot = (double)P->h_jtot[X * NPAIRCLASS + Y], mb = P->h_maxnp[X], mk = P->h_maxnp[Y];
       if (tot > 0.0) order.push_back({X, Y, grad_flops(X, Y, tot, tot * mb * mk, tot * mb), 0});
     }
-  assign_branches(order, nbranch);
+  nbranch = assign_branches(order, nbranch);
   if (nbranch > 0) {
     const int rc = P->fork(s, nbranch);
     if (rc != ERI_OK) return rc;

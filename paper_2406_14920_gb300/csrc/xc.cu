@@ -47,6 +47,13 @@ constexpr int kRhoWarps = 4;      // k_xc_rho: warps per block, 16 rows of D_b e
 constexpr int kKC = 128;          // k_xc_rho: functions of Phi_b staged at a time
 constexpr int kVWarps = 8;        // k_xc_vmat: warps per block, 16 rows of Z_b each at a time
 constexpr int kVC = 128;          // k_xc_vmat: functions of Phi_b staged at a time
+// V is summed in up to kParts half matrices, 2^kPartShift consecutive blocks to
+// one (two or three are in L2 at a time), and these are added at the end: one sum
+// over the thousands of blocks of an element loses sqrt(blocks) roundings (60
+// atoms: 5.7e-15 of V against 1.6e-15).  The parts take at most kPartBytes, but
+// are four or more.
+constexpr int kParts = 16, kPartShift = 8;
+constexpr size_t kPartBytes = size_t(1) << 30;
 constexpr int kSlots = 5;         // workspace rows per function: phi, d/dx, d/dy, d/dz, Z
 constexpr double kAoEps = 1e-15;  // shell extent: every |phi| and |grad phi| below this beyond it
 constexpr double kRhoMin = 1e-14; // points with a smaller density contribute nothing
@@ -685,8 +692,8 @@ struct VmatSmem {
 };
 __global__ void __launch_bounds__(32 * kVWarps, 2)
     k_xc_vmat(int b0, int nbf, const int* __restrict__ nbfb, const int* __restrict__ bfl,
-              const int64_t* __restrict__ woff, const double* __restrict__ work, const int* __restrict__ bad,
-              double* __restrict__ Vh) {
+              const int64_t* __restrict__ woff, const double* __restrict__ work, const int* __restrict__ bad, int parts,
+              double* __restrict__ Vparts) {
   extern __shared__ __align__(16) unsigned char smraw[];
   VmatSmem& S = *reinterpret_cast<VmatSmem*>(smraw);
   const int b = b0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
@@ -694,6 +701,7 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
   const int* L = bfl + (int64_t)b * nbf;
   const double* phi = work + woff[b];
   const double* Z = phi + (int64_t)4 * n * kBP;
+  double* Vh = Vparts + (int64_t)((b >> kPartShift) % parts) * nbf * nbf;
   if (bad[b]) {  // an infinity or NaN: plain sums
     for (int64_t o = tid; o < (int64_t)n * n; o += 32 * kVWarps) {
       const int i = (int)(o / n), j = (int)(o - (int64_t)i * n);
@@ -762,24 +770,28 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
             for (int x = 0; x < kDigits; ++x)
               if (x + y < kWeights) mma_f16(acc[x + y], a[s][x], bb);
           }
+        const int jl = 8 * nt + 2 * t, ej[2] = {S.exp[jl], S.exp[jl + 1]}, aj[2] = {S.ao[jl], S.ao[jl + 1]};
+        double v[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int jl = 8 * nt + 2 * t + (c & 1);
-          if (jl >= nj || !(c < 2 ? ok0 : ok1)) continue;
-          const double v = c & 1 ? combine_fp64(acc, c, c < 2 ? e0 : e1, S.exp[jl])
-                                 : combine<true>(acc, c, c < 2 ? e0 : e1, S.exp[jl]);
-          if (v != 0.0) atomicAdd((c < 2 ? v0 : v1) + S.ao[jl], v);
-        }
+        for (int c = 0; c < 4; ++c)
+          v[c] = c & 1 ? combine_fp64(acc, c, c < 2 ? e0 : e1, ej[c & 1]) : combine<true>(acc, c, c < 2 ? e0 : e1, ej[c & 1]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (jl + (c & 1) < nj && (c < 2 ? ok0 : ok1) && v[c] != 0.0) atomicAdd((c < 2 ? v0 : v1) + aj[c & 1], v[c]);
       }
     }
   }
 }
 
-// V = Vh + Vh^T in place
-__global__ void k_xc_symm(int nbf, double* __restrict__ V) {
-  const int i = blockIdx.x, j0 = threadIdx.x;
-  for (int j = j0; j <= i; j += blockDim.x) {
-    const double v = V[(int64_t)i * nbf + j] + V[(int64_t)j * nbf + i];
+// V = Vh + Vh^T, Vh = sum of the parts
+__global__ void k_xc_symm(int nbf, int parts, const double* __restrict__ Vparts, double* __restrict__ V) {
+  const int i = blockIdx.x;
+  for (int j = threadIdx.x; j <= i; j += blockDim.x) {
+    double v = 0.0;
+    for (int p = 0; p < parts; ++p) {
+      const double* Vh = Vparts + (int64_t)p * nbf * nbf;
+      v += Vh[(int64_t)i * nbf + j] + Vh[(int64_t)j * nbf + i];
+    }
     V[(int64_t)i * nbf + j] = v;
     V[(int64_t)j * nbf + i] = v;
   }
@@ -794,7 +806,7 @@ __global__ void k_xc_symm(int nbf, double* __restrict__ V) {
 void eri_plan_impl::xc_release() {
   void* ptrs[] = {xc.d_pts, xc.d_w, xc.d_rad, xc.d_ang, xc.d_invab, xc.d_perm, xc.d_bsph, xc.d_ext, xc.d_nsh,
                   xc.d_shl, xc.d_shoff, xc.d_nbfb, xc.d_bfl, xc.d_woff, xc.d_work, xc.d_rho, xc.d_grad,
-                  xc.d_vrho, xc.d_vgrad, xc.d_pexp, xc.d_ddig, xc.d_dexp, xc.d_zbad};
+                  xc.d_vrho, xc.d_vgrad, xc.d_pexp, xc.d_ddig, xc.d_dexp, xc.d_zbad, xc.d_vpart};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   xc = XcState{};
@@ -851,6 +863,9 @@ static int xc_build(eri_plan_impl* P, cudaStream_t s) {
   XCK(xalloc(&X.d_ddig, (size_t)nbf * nbf));
   XCK(xalloc(&X.d_dexp, (size_t)nbf));
   XCK(xalloc(&X.d_zbad, (size_t)nb));
+  const size_t nn8 = sizeof(double) * (size_t)nbf * nbf;
+  X.parts = (int)std::min<size_t>({(size_t)kParts, std::max<size_t>(4, kPartBytes / nn8), (size_t)(nb >> kPartShift) + 1});
+  XCK(xalloc(&X.d_vpart, (size_t)X.parts * nbf * nbf));
   XCK(cudaMemcpyAsync(X.d_perm, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice, s));
   const int nt = std::max(nrad, nth);
   k_xc_nodes<<<(nt + 127) / 128, 128, 0, s>>>(nrad, nth, X.radius, X.d_rad, X.d_ang);
@@ -957,7 +972,7 @@ static int xc_density_impl(eri_plan_impl* P, const double* D, double* rho, doubl
 static int xc_matrix_impl(eri_plan_impl* P, const double* vrho, const double* vgrad, double* V, cudaStream_t s) {
   XcState& X = P->xc;
   const int nbf = P->nbf;
-  XCK(cudaMemsetAsync(V, 0, sizeof(double) * (size_t)nbf * nbf, s));
+  XCK(cudaMemsetAsync(X.d_vpart, 0, sizeof(double) * (size_t)X.parts * nbf * nbf, s));
   XCK(cudaFuncSetAttribute(k_xc_vmat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(VmatSmem)));
   for (size_t c = 0; c + 1 < X.chunk.size(); ++c) {
     const int b0 = X.chunk[c], b1 = X.chunk[c + 1];
@@ -965,10 +980,10 @@ static int xc_matrix_impl(eri_plan_impl* P, const double* vrho, const double* vg
     if (!X.resident) xc_launch_ao(P, b0, b1, s);
     k_xc_z<<<b1 - b0, kBP, 0, s>>>(b0, X.d_perm, X.d_nbfb, X.d_woff, X.d_w, vrho, vgrad, X.d_work, X.d_zbad);
     k_xc_vmat<<<b1 - b0, 32 * kVWarps, sizeof(VmatSmem), s>>>(b0, nbf, X.d_nbfb, X.d_bfl, X.d_woff, X.d_work, X.d_zbad,
-                                                             V);
+                                                             X.parts, X.d_vpart);
     XCK(cudaGetLastError());
   }
-  k_xc_symm<<<nbf, 128, 0, s>>>(nbf, V);
+  k_xc_symm<<<nbf, 128, 0, s>>>(nbf, X.parts, X.d_vpart, V);
   XCK(cudaGetLastError());
   return ERI_OK;
 }

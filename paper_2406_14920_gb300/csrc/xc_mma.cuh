@@ -90,26 +90,23 @@ __device__ __forceinline__ double combine(const float (&acc)[kWeights][4], int c
   const long long hi = (long long)(s[0] * 128 + s[1]) * 16384 + (s[2] * 128LL + s[3]);
   const long long lo = ((long long)(s[4] * 128LL + s[5]) * 16384 + (s[6] * 128LL + s[7])) * 128 + s[8];
   unsigned long long l = ((unsigned long long)hi << 35) + (unsigned long long)lo;
-  long long h = (hi >> 29) + (lo >> 63) + (l < (unsigned long long)lo ? 1 : 0);
-  const bool neg = h < 0;
-  if (neg) {
-    l = 0ULL - l;
-    h = ~h + (l == 0 ? 1 : 0);
-  }
-  unsigned long long top = (unsigned long long)h, low = l;
-  int e = 127 + Ea + Eb - 1089;  // biased exponent of a leading one in bit 127
-  if (top == 0) {
-    top = low;
-    low = 0;
-    e -= 64;
-  }
+  unsigned long long h = (unsigned long long)((hi >> 29) + (lo >> 63)) + (l < (unsigned long long)lo ? 1 : 0);
+  // magnitude: two's complement of (h, l) where negative (no branches below: the
+  // sums of a tile are put together side by side)
+  const unsigned long long sg = (unsigned long long)((long long)h >> 63);
+  l ^= sg;
+  h ^= sg;
+  l -= sg;
+  h += (sg & 1) & (l == 0 ? 1ULL : 0ULL);
+  const bool up = h != 0;
+  const unsigned long long top = up ? h : l, low = up ? l : 0;
   const int n = __clzll((long long)top);
-  e -= n;
-  const unsigned long long m = n ? top << n | low >> (64 - n) : top;
-  if (m == 0 || e <= 0) return 0.0;
-  if (e >= 2047) return neg ? -__longlong_as_double(0x7ff0000000000000LL) : __longlong_as_double(0x7ff0000000000000LL);
-  const unsigned long long r = ((unsigned long long)(e - 1) << 52) + (m >> 11) + (m >> 10 & 1);
-  return __longlong_as_double((long long)(r | (neg ? 1ULL << 63 : 0ULL)));
+  const int e = (up ? 127 : 63) + Ea + Eb - 1089 - n;  // biased exponent of the leading one
+  const unsigned long long m = (top << (n & 63)) | (low >> 1 >> (63 - (n & 63)));
+  unsigned long long r = ((unsigned long long)(unsigned)(e - 1) << 52) + (m >> 11) + (m >> 10 & 1);
+  r = e >= 2047 ? 0x7ff0000000000000ULL : r;
+  r = top == 0 || e <= 0 ? 0ULL : r | (sg & (1ULL << 63));
+  return __longlong_as_double((long long)r);
 }
 
 // The same value (accumulators started at kMagic, sums below 2^20) with three FP64
@@ -126,9 +123,9 @@ __device__ __forceinline__ double combine_fp64(const float (&acc)[kWeights][4], 
   const double h = fma(__longlong_as_double(kOne + hi), 34359738368.0, -kTop);  // hi 2^35, exact
   const double v = h + (__longlong_as_double(kOne + lo) - kBase);
   const int e = exponent_of(v), f = e + Ea + Eb - 2112;
-  if (e == 0 || f <= 0) return 0.0;
-  if (f >= 2047) return __longlong_as_double((long long)(v < 0.0 ? 0xfff0000000000000ULL : 0x7ff0000000000000ULL));
-  return __hiloint2double(__double2hiint(v) + (f - e) * 1048576, __double2loint(v));
+  const bool zero = e == 0 || f <= 0, inf = f >= 2047;
+  const int word = __double2hiint(v), hw = inf ? (word & (int)0x80000000) | 0x7ff00000 : word + (f - e) * 1048576;
+  return __hiloint2double(zero ? 0 : hw, zero || inf ? 0 : __double2loint(v));
 }
 
 // 16-byte copies from global to shared memory, one group per commit
