@@ -27,8 +27,14 @@ constexpr int NPAIRCLASS = 10;       // ss ps pp ds dp dd fs fp fd ff
 //   FP32: [k][m][j], j < 4;  plus exp(-T_k) in both precisions.
 constexpr double BOYS_H = 0.05;
 constexpr double BOYS_INV_H = 20.0;
-constexpr double BOYS_TMAX = 36.0;   // Taylor + downward recursion below, asymptote + upward above
-constexpr int BOYS_NT = 722;         // covers T < 36 + h/2
+// Taylor + downward recursion below, asymptote + upward recursion above.  FP64: the
+// line for order M is where exp(-T) falls below 2^-55 of (2m+1) F_m for every
+// m < M, so that the branch above needs no exp (about 20 FP64 operations, which a
+// warp paid whenever one lane lay a little above the line; 36 for every order and
+// exp above it: (ps|ss) of 225 functions 4.5 ms, now 3.7).
+__host__ __device__ constexpr double boys_tmax(int M) { return M == 0 ? 36.0 : 42.0 + 3.0 * M; }
+constexpr double BOYS_TMAX32 = 36.0;  // FP32
+constexpr int BOYS_NT = 1624;         // covers T < boys_tmax(13) + h/2
 constexpr int BOYS_J64 = 8;          // |dT| <= 0.025: truncation ~ dT^8/8! ~ 4e-18 relative
 constexpr int BOYS_J32 = 4;          // dT^4/4! ~ 1.6e-8 relative
 constexpr int BOYS_MMAX = LMAX_QUARTET;  // 13
@@ -222,12 +228,13 @@ struct WorkList {
   int mpb, mpk;            // most primitive pairs of a shell pair in the bra and in the ket class
 };
 
-// Boys F_0..F_M at T.  Below BOYS_TMAX: Taylor expansion of F_M around the
+// Boys F_0..F_M at T.  Below boys_tmax(M): Taylor expansion of F_M around the
 // nearest grid point, F_M(T) = sum_j F_{M+j}(T_k) (T_k - T)^j / j!  (from
 // dF_m/dT = -F_{m+1}), exp(-T) = exp(-T_k) exp(T_k - T) with a short Taylor
 // series, then the downward recursion F_m = (2T F_{m+1} + exp(-T)) / (2m+1).
 // Above: F_0 = sqrt(pi/T)/2 (erf(sqrt T) = 1 to double precision) and the upward
-// recursion F_{m+1} = ((2m+1) F_m - exp(-T)) / (2T).  Our own construction
+// recursion F_{m+1} = ((2m+1) F_m - exp(-T)) / (2T), in FP64 without the
+// exponential, which no longer counts there.  Our own construction
 // ("interpolation and downward recursion", Sec. 2.3); CUDA's exp/rsqrt are
 // called where needed, not reproduced.
 struct BoysTabs {
@@ -239,7 +246,7 @@ struct BoysTabs {
 
 template <int M>
 __device__ __forceinline__ void boys_f64(double T, const BoysTabs& bt, double* F) {
-  if (T < BOYS_TMAX) {
+  if (T < boys_tmax(M)) {
     const int k = __double2int_rn(T * BOYS_INV_H);
     const double d = k * BOYS_H - T;
     // the 8 Taylor coefficients of (k, M) are one 64-byte row: four 16-byte loads
@@ -280,20 +287,17 @@ __device__ __forceinline__ void boys_f64(double T, const BoysTabs& bt, double* F
       for (int m = M - 1; m >= 0; --m) F[m] = fma(t2, F[m + 1], e) * (1.0 / (2 * m + 1));
     }
   } else {
-    // exp(-T) falls below 2^-55 of (2m+1) F_m for every m < M beyond T = 42 + 3 M
-    // (F_m >= (2m-1)!!/(2T)^m F_0), where subtracting it changes nothing
-    const double e = M > 0 && T < 42.0 + 3.0 * M ? exp(-T) : 0.0;
     const double rt = rsqrt(T);
     F[0] = 0.88622692545275801365 * rt;  // sqrt(pi)/2
     const double inv2t = 0.5 * rt * rt;
 #pragma unroll
-    for (int m = 0; m < M; ++m) F[m + 1] = fma((double)(2 * m + 1), F[m], -e) * inv2t;
+    for (int m = 0; m < M; ++m) F[m + 1] = (2 * m + 1) * inv2t * F[m];
   }
 }
 
 template <int M>
 __device__ __forceinline__ void boys_f32(float T, const BoysTabs& bt, float* F) {
-  if (T < (float)BOYS_TMAX) {
+  if (T < (float)BOYS_TMAX32) {
     const int k = __float2int_rn(T * (float)BOYS_INV_H);
     const float d = k * (float)BOYS_H - T;
     // the 4 Taylor coefficients of (k, M) are one 16-byte row: one load

@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(32 * kSchwarzWarps)
       const double T = rho * (X * X + Y * Y + Z * Z);
       // generic Boys (runtime order): Taylor at the top order then downward
       double fm;
-      if (T < BOYS_TMAX) {
+      if (T < boys_tmax(4 * LMAX)) {
         const int k = __double2int_rn(T * BOYS_INV_H);
         const double* c = bt.c64 + ((size_t)k * (BOYS_MMAX + 1) + L) * BOYS_J64;
         const double dd = k * BOYS_H - T;
