@@ -56,6 +56,22 @@ __device__ __forceinline__ void block_starts(int* start, F&& count) {
   __syncthreads();
 }
 
+// order[0 .. N) = the component pairs by decreasing number of terms: the lanes of
+// a warp take neighbours of this order and run loops of the same length
+template <int N>
+__device__ __forceinline__ void order_by_terms(const int* start, uint8_t* order) {
+  const int m = threadIdx.x;
+  if (m < N) {
+    const int k = start[m + 1] - start[m];
+    int r = 0;
+    for (int c = 0; c < N; ++c) {
+      const int kc = start[c + 1] - start[c];
+      r += kc > k || (kc == k && c < m);
+    }
+    order[r] = (uint8_t)m;
+  }
+}
+
 // Term table of a shell pair (la, lb), built once per block: component pair m
 // owns terms [start[m], start[m+1]); term k is the product of the 1D
 // coefficients at element offsets te[k] & 1023, (te[k] >> 10) & 1023, te[k] >> 20
@@ -171,7 +187,7 @@ struct CShape {
   static constexpr int NT = NAB * NCD >= 1500 ? 256 : 128;
   static constexpr int TOTAL = FIXED + G * PER_G;
   static constexpr size_t smem() {
-    return sizeof(T) * ((TOTAL + 3) / 4 * 4) + 4 * (TB + TK + NAB + NCD + 2) + 2 * (TB + TK + HAB + 3);
+    return sizeof(T) * ((TOTAL + 3) / 4 * 4) + 4 * (TB + TK + NAB + NCD + 2) + 2 * (TB + TK + HAB + 3) + NAB + NCD;
   }
 };
 
@@ -201,6 +217,10 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
   build_terms<LC, LD, LCD + 1>(ks, kt, ko, [](int t, int u, int v) { return (t * B + u) * B + v; });
   build_terms<LA, LB, LAB + 1>(bs, btm, bo, [](int t, int u, int v) { return herm_index(t, u, v); });
   for (int i = tid; i < HAB; i += NT) pbox[i] = (uint16_t)((herm_t(i) * B + herm_u(i)) * B + herm_v(i));
+  uint8_t* cdo = reinterpret_cast<uint8_t*>(pbox + HAB);  // [NCD], [NAB]: order of the tasks
+  uint8_t* abo = cdo + NCD;
+  order_by_terms<NCD>(ks, cdo);
+  order_by_terms<NAB>(bs, abo);
 
   const bool compact = a.items != nullptr;
   const int64_t total = compact ? (int64_t)__ldg(a.nitems) : a.wl.total;
@@ -292,7 +312,7 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
           // C: two Hermite indices per task share the coefficients
           constexpr int HH = (HAB + 1) / 2;
           for (int it = tid; it < NCD * HH; it += NT) {
-            const int cd = it / HH, P = it - cd * HH, P2 = P + HH < HAB ? P + HH : P;
+            const int row = it / HH, cd = cdo[row], P = it - row * HH, P2 = P + HH < HAB ? P + HH : P;
             const int s0 = ks[cd], s1 = ks[cd + 1];
             T x0 = T(0), x1 = T(0);
             for (int g = 0; g < ng; ++g) {
@@ -326,7 +346,7 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
         // D: two ket pairs per task
         constexpr int CH = (NCD + 1) / 2;
         for (int it = tid; it < NAB * CH; it += NT) {
-          const int iab = it / CH, c0 = it - iab * CH, c1 = c0 + CH < NCD ? c0 + CH : c0;
+          const int row = it / CH, iab = abo[row], c0 = it - row * CH, c1 = c0 + CH < NCD ? c0 + CH : c0;
           const int s0 = bs[iab], s1 = bs[iab + 1];
           const T* w0 = Ws + c0 * HABP;
           const T* w1 = Ws + c1 * HABP;

@@ -353,7 +353,7 @@ struct GShape {
   static constexpr int PER_G = BOX + 2 * NP + TK;
   // G is held whole, or (where that would not fit) in NH parts of the bra pairs
   static constexpr int REST = NCD * HABP + 6 * NER + kWin * NSC + NDB + 48;
-  static constexpr size_t TABLES = 4 * (size_t)(TK + NV + NCD + 1 + 2 * NAB + 1) + 2 * (TK + HAB + 2);
+  static constexpr size_t TABLES = 4 * (size_t)(TK + NV + NCD + 1 + 2 * NAB + 1) + 2 * (TK + HAB + 2) + NCD;
   static constexpr int NH = sizeof(T) * (size_t)(REST + PER_G + NAB * NCD + 4) + TABLES <= 226 * 1024 ? 1 : 2;
   static constexpr int NABH = (NAB + NH - 1) / NH;
   static constexpr int FIXED = REST + NABH * NCD;
@@ -390,6 +390,8 @@ __global__ void __launch_bounds__(GShape<LA, LB, LC, LD, T>::NT) grad_block_kern
   uint16_t* pbox = ko + S::TK;          // [HAB]
   build_terms<LC, LD, LCD + 1>(ks, kt, ko, [](int t, int u, int v) { return (t * B + u) * B + v; });
   for (int i = tid; i < HAB; i += NT) pbox[i] = (uint16_t)((herm_t(i) * B + herm_u(i)) * B + herm_v(i));
+  uint8_t* cdo = reinterpret_cast<uint8_t*>(pbox + HAB);  // [NCD]: order of the tasks
+  order_by_terms<NCD>(ks, cdo);
   auto powers = [](int m, int* x, int* y) {
     cart_xyz(LA, m / NB, x[0], x[1], x[2]);
     cart_xyz(LB, m % NB, y[0], y[1], y[2]);
@@ -561,7 +563,7 @@ __global__ void __launch_bounds__(GShape<LA, LB, LC, LD, T>::NT) grad_block_kern
           __syncthreads();
           constexpr int HH = (HAB + 1) / 2;
           for (int it = tid; it < NCD * HH; it += NT) {
-            const int cd = it / HH, P = it - cd * HH, P2 = P + HH < HAB ? P + HH : P;
+            const int row = it / HH, cd = cdo[row], P = it - row * HH, P2 = P + HH < HAB ? P + HH : P;
             const int s0 = ks[cd], s1k = ks[cd + 1];
             T x0 = T(0), x1 = T(0);
             for (int g = 0; g < ng; ++g) {
