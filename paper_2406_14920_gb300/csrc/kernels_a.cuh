@@ -7,11 +7,12 @@
 #include "kernels.cuh"
 
 // FP64 register kernel beyond the tiny classes: largest L and footprint
-// (doubles).  GB300 issues about 3.4 FP64 FMAs per clock per SM, so every warp
-// instruction with idle lanes is expensive; one quartet per lane keeps all 32
-// lanes busy (measured: (pp|pp) 31 -> 9.8 ms, (ds|pp) 16 -> 5.1 ms, (fp|ps)
-// 12 -> 4.9 ms on workload 1; raising the limits from L 5 / 200 to L 6 / 300
-// took (dp|pp) 16.5 -> 13.6 ms and (fs|fs) 2.5 -> 1.5 ms).
+// (doubles).  GB300 issues about 1.8 FP64 FMAs per clock per SM, one warp
+// instruction every 17 clocks however many lanes are active; one quartet per
+// lane keeps all 32 busy as long as the lanes' contraction lengths are alike
+// (the lists are ordered for that, see k_tier_split).  Above the footprint the
+// block kernel (kernels_c.cuh) is faster: it spills nothing and its lanes share
+// one quartet.
 #ifndef ERI_THREAD64_LMAX
 #define ERI_THREAD64_LMAX 6
 #endif
@@ -42,15 +43,15 @@ struct AShape {
   static constexpr bool WACC = REG_WACC <= 260;
 };
 
-// Which classes run one quartet per thread (registers) rather than one per warp.
-// FP64: classes with L <= 5 whose per-primitive-quartet footprint is at most
-// 200 doubles.  FP32: every class of L <= 7 whose per-primitive-quartet register
-// footprint is at most 460 values.  Measured on GB300 (workload 1, FP32 tier):
-// the register kernel runs these classes 2.2x to 9.6x faster than the
-// shared-memory warp kernel even where ptxas spills up to ~6 KB per thread
-// (spills are lane-interleaved local memory, served by L1), because every
-// index is a compile-time constant and all 32 lanes do useful work; the warp
-// kernel stays for the classes with larger ERI blocks.
+// Which classes run one quartet per thread (registers).  FP64: classes with
+// L <= 6 whose per-primitive-quartet footprint is at most 190 doubles; the
+// others take a block per quartet.  FP32: every class of L <= 7 whose footprint
+// is at most 460 values.  Measured on GB300 (900 functions, FP32 tier): the
+// register kernel runs these classes 2.2x to 9.6x faster than the shared-memory
+// warp kernel even where ptxas spills up to ~6 KB per thread (spills are
+// lane-interleaved local memory, served by L1), because every index is a
+// compile-time constant and all 32 lanes do useful work; the warp kernel and the
+// block kernel take the classes with larger ERI blocks.
 __host__ __device__ constexpr bool use_thread_kernel(int la, int lb, int lc, int ld, bool fp32) {
   const int L = la + lb + lc + ld;
   const int nab = ncart(la) * ncart(lb), ncd = ncart(lc) * ncart(ld);

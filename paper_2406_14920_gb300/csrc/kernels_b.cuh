@@ -1,54 +1,41 @@
-// General J+K kernel: one warp per canonical shell quartet, contracted ERI block
-// staged in shared memory.  Used for every class that does not fit the
-// register kernel (kernels_a.cuh).
+// FP32 J+K kernel of the middle classes: one warp per canonical shell quartet,
+// contracted ERI block staged in shared memory, both transforms written out at
+// compile time.  Used for the FP32 classes that do not fit the register kernel
+// (kernels_a.cuh) and whose transforms do (use_block_kernel); the larger ones
+// and FP64 run a block per quartet (kernels_c.cuh).
 //
-// Per quartet, per chunk of CH ket Cartesian pairs cd, per bra primitive pair,
-// the ket primitive pairs are taken G at a time:
+// Per quartet, per bra primitive pair, the ket primitive pairs are taken G at a
+// time:
 //   step A  (lane g): quartet scalars for ket primitive g -- rho, P-Q, prefactor,
 //           Boys F_0..F_L (Eq. boys_function); all lanes: ket E tables to smem
 //           with (-1)^|Q| folded in;
-//   step B  items (g, e), level by level: R^0 of the G primitive quartets
-//           (Eq. R_recursion);
-//   step C  items (cd, P): W[cd][P] += sum_g sum_Q E'_Q^{cd}(g) R_{P+Q}(g);
+//   step B  R^0 of the G primitive quartets (Eq. R_recursion), a lane per quartet
+//           in registers up to L = 6, level by level over the warp above;
+//   step C  lane-owned bra Hermite index P: W[cd][P] += sum_g sum_Q E'_Q^{cd}(g) R_{P+Q}(g);
 // then for the bra primitive:
-//   step D  items (ab, cd): X[ab][cd] += sum_P E_P^{ab} W[cd][P]        (Eq. eri_formula)
-// and per chunk the contraction, one lane per output element:
+//   step D  lane-owned ket pair cd: X[ab][cd] += sum_P E_P^{ab} W[cd][P]   (Eq. eri_formula)
+// and the contraction, one lane per output element:
 //   Kh_ac, Kh_ad, Kh_bc, Kh_bd (Eq. k_definition), Jh_ab, Jh_cd (Eq. j_definition),
 //   one atomic per element.
-// Every per-primitive-quartet scalar is computed by one lane, not redundantly
-// by the warp (GB300's FP64 pipe charges a full warp issue per instruction
-// whatever the number of active lanes).
 #pragma once
 #include "kernels_a.cuh"
 
-// base shared memory per warp (KB) of the warp kernel, per precision: FP64
-// keeps 8 warps per SM (two resident 4-warp blocks), FP32 about 16-20
-#ifndef ERI_WARP_SMEM64_KB
-#define ERI_WARP_SMEM64_KB 22
-#endif
+// base shared memory per warp (KB), about 16-20 warps per SM, and the upper limit
+// when a larger ket-primitive batch saves a batch
 #ifndef ERI_WARP_SMEM32_KB
 #define ERI_WARP_SMEM32_KB 12
-#endif
-// upper limits when a larger ket-primitive batch saves a batch (FP64: two
-// 4-warp blocks still fit in an SM's 228 KB)
-#ifndef ERI_WARP_SMEM64_MAX_KB
-#define ERI_WARP_SMEM64_MAX_KB 27
 #endif
 #ifndef ERI_WARP_SMEM32_MAX_KB
 #define ERI_WARP_SMEM32_MAX_KB 16
 #endif
-// FP32 compile-time bra transform: largest X slice per lane, and the shared
-// memory per warp a class may take to get there (measured on GB300: (fd|fp)
-// 58 -> 9.9 ms with the 24 KB budget, (ff|dp) 35 -> 4.8 ms with 100-value slices)
+// compile-time bra transform: largest X slice per lane, and the shared memory per
+// warp a class may take to get there (measured on GB300: (fd|fp) 58 -> 9.9 ms with
+// the 24 KB budget, (ff|dp) 35 -> 4.8 ms with 100-value slices)
 #ifndef ERI_REGD32_MAX
 #define ERI_REGD32_MAX 100
 #endif
 #ifndef ERI_WARP_SMEM32_FULL_KB
 #define ERI_WARP_SMEM32_FULL_KB 24
-#endif
-// FP64 also takes the lane-owned-P ket transform where W fits in registers
-#ifndef ERI_REGW64
-#define ERI_REGW64 1
 #endif
 
 namespace eri {
@@ -69,8 +56,8 @@ struct BShape {
   static constexpr int FIXED = 3 * NEB;
   static constexpr int PER_G = BOX + 2 * NPING + NSC + 3 * NEK;
   static constexpr int PER_C = HABP + NAB;
-  static constexpr int BASE = sizeof(T) == 8 ? (ERI_WARP_SMEM64_KB * 1024) / 8 : (ERI_WARP_SMEM32_KB * 1024) / 4;
-  static constexpr int MAXB = sizeof(T) == 8 ? (ERI_WARP_SMEM64_MAX_KB * 1024) / 8 : (ERI_WARP_SMEM32_MAX_KB * 1024) / 4;
+  static constexpr int BASE = (ERI_WARP_SMEM32_KB * 1024) / 4;
+  static constexpr int MAXB = (ERI_WARP_SMEM32_MAX_KB * 1024) / 4;
   static constexpr int GTARGET = (LC <= 1 && LD <= 1) ? 9 : 3;
   static constexpr int fit_g(int budget) { return (budget - FIXED - NCD * PER_C) / PER_G; }
   static constexpr int GMAXB = fit_g(MAXB) < 1 ? 1 : fit_g(MAXB);
@@ -78,21 +65,21 @@ struct BShape {
   static constexpr int GWANT = (GTARGET + NBATCH - 1) / NBATCH;
   static constexpr int NEED = FIXED + NCD * PER_C + GWANT * PER_G;
   static constexpr int BUDGET0 = NEED <= BASE ? BASE : (NEED <= MAXB ? NEED : MAXB);
-  // FP32 classes with many ket components take a larger budget when that is
-  // what lets the whole ket range sit in one chunk (one ket primitive per
+  // classes with many ket components take a larger budget when that is
+  // what lets the whole ket range sit in one pass (one ket primitive per
   // batch), the condition of the compile-time bra transform below
   static constexpr int NEED_FULL = FIXED + NCD * PER_C + PER_G;
-  static constexpr bool WANT_FULL = sizeof(T) == 4 && NCD >= 8 && NAB * ((NCD + 31) / 32) <= ERI_REGD32_MAX &&
+  static constexpr bool WANT_FULL = NCD >= 8 && NAB * ((NCD + 31) / 32) <= ERI_REGD32_MAX &&
                                     NEED_FULL <= (ERI_WARP_SMEM32_FULL_KB * 1024) / 4;
   static constexpr int BUDGET = (WANT_FULL && BUDGET0 < NEED_FULL) ? NEED_FULL : BUDGET0;
   static constexpr int G0 = (BUDGET - FIXED - NCD * PER_C) / PER_G;
   static constexpr int G = G0 >= 1 ? (G0 > 16 ? 16 : G0) : 1;
   static constexpr int CHMAX = (BUDGET - FIXED - G * PER_G) / PER_C;
-  static constexpr int CH = CHMAX >= NCD ? NCD : (CHMAX < 1 ? 1 : CHMAX);
-  // FP32 register path for step C: lane j-slot P = lane + 32 j holds W[cd][P]
+  static constexpr bool FITS = CHMAX >= NCD;  // the whole ket range in one pass
+  // step C: lane j-slot P = lane + 32 j holds W[cd][P]
   // for every ket pair cd in registers, the cd loop unrolled at compile time
   static constexpr int NPS = (HAB + 31) / 32;
-  static constexpr bool REGW = CH == NCD && (sizeof(T) == 4 ? NCD * NPS <= 64 : (ERI_REGW64 && NCD * NPS <= 32));
+  static constexpr bool REGW = FITS && NCD * NPS <= 64;
   // step D with compile-time indices: lane owns ket pair cd = lane + 32 j, the
   // bra pairs ab are a compile-time loop (E broadcast, W row at a per-lane
   // base), X[ab][cd] stays in registers over the bra primitives.  Worth it
@@ -100,15 +87,13 @@ struct BShape {
   // workload 1, FP32: (ff|pp) 17.9 -> 9.6 ms, (fd|fs) 15.8 -> 9.4 ms, against
   // the (ab, cd) item loop).
   static constexpr int NCS = (NCD + 31) / 32;
-  static constexpr bool REGD = CH == NCD && NCD >= 8 && NAB * NCS <= (sizeof(T) == 4 ? ERI_REGD32_MAX : 48);
+  static constexpr bool REGD = FITS && NCD >= 8 && NAB * NCS <= ERI_REGD32_MAX;
   static constexpr int SM_BOX = 0, SM_PING = SM_BOX + G * BOX, SM_SC = SM_PING + G * 2 * NPING,
                        SM_EK = SM_SC + G * NSC, SM_EB = SM_EK + G * 3 * NEK, SM_W = SM_EB + 3 * NEB,
-                       SM_X = SM_W + CH * HABP, SM_TOTAL = SM_X + NAB * CH;
+                       SM_X = SM_W + NCD * HABP, SM_TOTAL = SM_X + NAB * NCD;
   __host__ __device__ static constexpr size_t smem_per_warp() { return sizeof(T) * SM_TOTAL; }
-  // block-shared index tables (ints): cd table, ab table, P table, W row bases
-  static constexpr int LEXB = (LAB + 1) * (LAB + 1);
-  static constexpr int TAB_INTS = 2 * NCD + 2 * NAB + HAB + LEXB;
-  static constexpr int TABLE_BYTES = ((4 * TAB_INTS + 15) / 16) * 16;
+  // block-shared index table (ints): per bra Hermite index P its box offset and W slot
+  static constexpr int TABLE_BYTES = ((4 * HAB + 15) / 16) * 16;
   __host__ __device__ static constexpr size_t table_bytes() { return TABLE_BYTES; }
 };
 
@@ -121,47 +106,20 @@ __host__ __device__ constexpr int lex_base(int lmax, int t, int u) {
   return b;
 }
 
-// FP64: two resident blocks per SM are the target (the register budget follows);
-// FP32: left to the compiler
 template <int LA, int LB, int LC, int LD, typename T>
-__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JKArgs A) {
+__global__ void __launch_bounds__(128) jk_warp_kernel(JKArgs A) {
   using S = BShape<LA, LB, LC, LD, T>;
+  static_assert(sizeof(T) == 4 && S::REGW && S::REGD);
   constexpr int LAB = S::LAB, LCD = S::LCD, L = S::L, B = S::B, BOX = S::BOX, NSC = S::NSC;
-  constexpr int NA = S::NA, NB = S::NB, ND = S::ND, NAB = S::NAB, NCD = S::NCD, HAB = S::HAB, HABP = S::HABP,
-                CH = S::CH, G = S::G, NEB = S::NEB, NEK = S::NEK, NPING = S::NPING;
+  constexpr int NA = S::NA, NB = S::NB, NC = S::NC, ND = S::ND, NAB = S::NAB, NCD = S::NCD, HAB = S::HAB, HABP = S::HABP,
+                G = S::G, NEB = S::NEB, NEK = S::NEK, NPING = S::NPING;
   const KArgs& a = A.k;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  // index tables shared by the block: per ket pair cd the E offsets and term
-  // counts, the same per bra pair ab, per bra Hermite index P its box offset
-  // and its W slot, and the W row bases for step D
-  int* tab_cd = reinterpret_cast<int*>(smraw);
-  int* tab_ab = tab_cd + 2 * NCD;
-  int* tab_p = tab_ab + 2 * NAB;
-  int* tab_lex = tab_p + HAB;
-  for (int i = threadIdx.x; i < NCD; i += blockDim.x) {
-    int kx, ky, kz, lx, ly, lz;
-    cart_xyz(LC, i / ND, kx, ky, kz);
-    cart_xyz(LD, i % ND, lx, ly, lz);
-    tab_cd[2 * i] = ((kx * (LD + 1) + lx) * (LCD + 1)) | ((NEK + (ky * (LD + 1) + ly) * (LCD + 1)) << 10) |
-                    ((2 * NEK + (kz * (LD + 1) + lz) * (LCD + 1)) << 20);
-    tab_cd[2 * i + 1] = (kx + lx) | ((ky + ly) << 4) | ((kz + lz) << 8);
-  }
-  for (int i = threadIdx.x; i < NAB; i += blockDim.x) {
-    int ix, iy, iz, jx, jy, jz;
-    cart_xyz(LA, i / NB, ix, iy, iz);
-    cart_xyz(LB, i % NB, jx, jy, jz);
-    tab_ab[2 * i] = ((ix * (LB + 1) + jx) * (LAB + 1)) | ((NEB + (iy * (LB + 1) + jy) * (LAB + 1)) << 10) |
-                    ((2 * NEB + (iz * (LB + 1) + jz) * (LAB + 1)) << 20);
-    tab_ab[2 * i + 1] = (ix + jx) | ((iy + jy) << 4) | ((iz + jz) << 8);
-  }
+  int* tab_p = reinterpret_cast<int*>(smraw);
   for (int i = threadIdx.x; i < HAB; i += blockDim.x) {
     const int t = herm_t(i), u = herm_u(i), v = herm_v(i);
     tab_p[i] = ((t * B + u) * B + v) | ((lex_base(LAB, t, u) + v) << 16);
-  }
-  for (int i = threadIdx.x; i < S::LEXB; i += blockDim.x) {
-    const int t = i / (LAB + 1), u = i % (LAB + 1);
-    tab_lex[i] = (t + u <= LAB) ? lex_base(LAB, t, u) : 0;
   }
   __syncthreads();
   int pslot[S::NPS];  // box offset of this lane's bra Hermite indices P = lane + 32 j
@@ -229,23 +187,15 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
     double* Kh = a.Kh ? a.Kh + mbase : nullptr;
     double* Jh = A.Jh ? A.Jh + mbase : nullptr;
 
-    for (int c0 = 0; c0 < NCD; c0 += CH) {
-      const int nci = NCD - c0 < CH ? NCD - c0 : CH;
-      for (int x = lane; x < NAB * CH; x += 32) Xs[x] = T(0);
-      T xreg[S::REGD ? S::NCS * NAB : 1];
-      if constexpr (S::REGD) {
+    {
+      T xreg[S::NCS * NAB];
 #pragma unroll
-        for (int x = 0; x < S::NCS * NAB; ++x) xreg[x] = T(0);
-      }
+      for (int x = 0; x < S::NCS * NAB; ++x) xreg[x] = T(0);
       for (int pb = 0; pb < npb; ++pb) {
         for (int x = lane; x < 3 * NEB; x += 32) Eb[x] = ldE<T>(a.pd, eb0 + pb * 3 * NEB + x);
-        T wreg[S::REGW ? S::NPS * NCD : 1];
-        if constexpr (S::REGW) {
+        T wreg[S::NPS * NCD];
 #pragma unroll
-          for (int x = 0; x < S::NPS * NCD; ++x) wreg[x] = T(0);
-        } else {
-          for (int x = lane; x < CH * HABP; x += 32) Ws[x] = T(0);
-        }
+        for (int x = 0; x < S::NPS * NCD; ++x) wreg[x] = T(0);
         const int ipb = offb + pb;
         const T bp_p = pdv<T>(a.pd.p, a.pd.pf, ipb), bp_pref = pdv<T>(a.pd.pref, a.pd.preff, ipb);
         const T bPx = pdv<T>(a.pd.P, a.pd.Pf, ipb), bPy = pdv<T>(a.pd.P, a.pd.Pf, a.pd.n + ipb),
@@ -279,11 +229,11 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
             sc[L + 4] = T(-2) * rho;
           }
           __syncwarp();
-          // step B: R^0 for the ng primitive quartets.  FP32 and L <= 6: each lane
+          // step B: R^0 for the ng primitive quartets.  L <= 6: each lane
           // builds its own quartet's table in registers (compile-time indices) and
           // stores it in its box.  Otherwise the warp builds all of them level by
           // level (scaled form, see r_build_warp).
-          if constexpr (sizeof(T) == 4 && L <= 6) {
+          if constexpr (L <= 6) {
             if (lane < ng) {
               const T* sc = scal + lane * NSC;
               T Fl[L + 1];
@@ -299,8 +249,6 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
 #pragma unroll
                   for (int v = 0; v <= L - t - u; ++v) bx[(t * B + u) * B + v] = R[herm_index(t, u, v)];
             }
-          } else if (L == 0) {
-            if (lane < ng) boxes[lane * BOX] = scal[lane * NSC];
           } else {
             if (lane < ng) pings[lane * 2 * NPING] = scal[lane * NSC + L];
             __syncwarp();
@@ -330,10 +278,9 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
             }
           }
           __syncwarp();
-          // step C: ket transform
-          if constexpr (S::REGW) {
-            // lane-owned P, every cd unrolled: R read at a per-lane base plus
-            // compile-time offsets, E' broadcast, W accumulated in registers
+          // step C: ket transform; lane-owned P, every cd unrolled: R read at a
+          // per-lane base plus compile-time offsets, E' broadcast, W in registers
+          {
             for (int g = 0; g < ng; ++g) {
               const T* ek = Ek + g * 3 * NEK;
               const T* rbox = boxes + g * BOX;
@@ -358,46 +305,19 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
                 });
               });
             }
-          } else {
-          for (int it = lane; it < nci * HAB; it += 32) {
-            const int ci = it / HAB, P = it - ci * HAB;
-            const int c0w = tab_cd[2 * (c0 + ci)], c1w = tab_cd[2 * (c0 + ci) + 1];
-            const int ox = c0w & 1023, oy = (c0w >> 10) & 1023, oz = c0w >> 20;
-            const int nx = c1w & 15, ny = (c1w >> 4) & 15, nz = c1w >> 8;
-            const int pw = tab_p[P];
-            const int base = pw & 0xffff;
-            T acc = T(0);
-            for (int g = 0; g < ng; ++g) {
-              const T* ek = Ek + g * 3 * NEK;
-              const T* rb = boxes + g * BOX + base;
-              for (int sx = 0; sx <= nx; ++sx) {
-                T accy = T(0);
-                for (int sy = 0; sy <= ny; ++sy) {
-                  const T* r = rb + sx * B * B + sy * B;
-                  T accz = T(0);
-                  for (int sz = 0; sz <= nz; ++sz) accz = fma(ek[oz + sz], r[sz], accz);
-                  accy = fma(ek[oy + sy], accz, accy);
-                }
-                acc = fma(ek[ox + sx], accy, acc);
-              }
-            }
-            Ws[ci * HABP + (pw >> 16)] += acc;
-          }
           }
           __syncwarp();
         }
-        if constexpr (S::REGW) {
 #pragma unroll
-          for (int j = 0; j < S::NPS; ++j)
-            if (lane + 32 * j < HAB) {
-              const int slot = tab_p[lane + 32 * j] >> 16;
+        for (int j = 0; j < S::NPS; ++j)
+          if (lane + 32 * j < HAB) {
+            const int slot = tab_p[lane + 32 * j] >> 16;
 #pragma unroll
-              for (int icd = 0; icd < NCD; ++icd) Ws[icd * HABP + slot] = wreg[j * NCD + icd];
-            }
-          __syncwarp();
-        }
+            for (int icd = 0; icd < NCD; ++icd) Ws[icd * HABP + slot] = wreg[j * NCD + icd];
+          }
+        __syncwarp();
         // step D: bra transform
-        if constexpr (S::REGD) {
+        {
           sfor<S::NCS>([&](auto j_) {
             constexpr int j = ERI_CI(j_);
             const int cd = lane + 32 * j;
@@ -419,78 +339,51 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
               });
             }
           });
-        } else {
-        // items (ab, ci)
-        for (int it = lane; it < NAB * nci; it += 32) {
-          const int iab = it / nci, ci = it - iab * nci;
-          const int a0w = tab_ab[2 * iab], a1w = tab_ab[2 * iab + 1];
-          const T* fx = Eb + (a0w & 1023);
-          const T* fy = Eb + ((a0w >> 10) & 1023);
-          const T* fz = Eb + (a0w >> 20);
-          const int nx = a1w & 15, ny = (a1w >> 4) & 15, nz = a1w >> 8;
-          const T* wc = Ws + ci * HABP;
-          T acc = T(0);
-          for (int tx = 0; tx <= nx; ++tx) {
-            T accy = T(0);
-            for (int ty = 0; ty <= ny; ++ty) {
-              const T* wr = wc + tab_lex[tx * (LAB + 1) + ty];
-              T accz = T(0);
-              for (int tz = 0; tz <= nz; ++tz) accz = fma(fz[tz], wr[tz], accz);
-              accy = fma(fy[ty], accz, accy);
-            }
-            acc = fma(fx[tx], accy, acc);
-          }
-          Xs[iab * CH + ci] += acc;
-        }
         }
         __syncwarp();
       }
-      if constexpr (S::REGD) {  // X to shared memory for the contraction
+      {  // X to shared memory for the contraction
         sfor<S::NCS>([&](auto j_) {
           constexpr int j = ERI_CI(j_);
           const int cd = lane + 32 * j;
           if (j * 32 + 32 <= NCD || cd < NCD) {
 #pragma unroll
-            for (int iab = 0; iab < NAB; ++iab) Xs[iab * CH + cd] = xreg[j * NAB + iab];
+            for (int iab = 0; iab < NAB; ++iab) Xs[iab * NCD + cd] = xreg[j * NAB + iab];
           }
         });
         __syncwarp();
       }
-      // contraction of the chunk; one lane per output element
-      const int cfirst = c0 / ND, clast = (c0 + nci - 1) / ND;
-      const int ncr = clast - cfirst + 1;
+      // contraction; one lane per output element
       if (Kh) {
-        // Kh_ac[a][c] += w sum_{b, d: (c,d) in chunk} X D_bd ; Kh_bc[b][c] += w sum_{a,d} X D_ad
-        for (int o = lane; o < (NA + NB) * ncr; o += 32) {
-          const bool isA = o < NA * ncr;
-          const int oo = isA ? o : o - NA * ncr;
-          const int r = oo / ncr, c = cfirst + oo % ncr;
+        // Kh_ac[a][c] += w sum_{b, d} X D_bd ; Kh_bc[b][c] += w sum_{a, d} X D_ad
+        for (int o = lane; o < (NA + NB) * NC; o += 32) {
+          const bool isA = o < NA * NC;
+          const int oo = isA ? o : o - NA * NC;
+          const int r = oo / NC, c = oo % NC;
           T s = T(0);
           for (int d = 0; d < ND; ++d) {
-            const int ci = c * ND + d - c0;
-            if (ci < 0 || ci >= nci) continue;
+            const int ci = c * ND + d;
             if (isA) {
-              for (int b = 0; b < NB; ++b) s = fma(Xs[(r * NB + b) * CH + ci], __ldg(Dp + (size_t)(ao2 + b) * n + ao4 + d), s);
+              for (int b = 0; b < NB; ++b) s = fma(Xs[(r * NB + b) * NCD + ci], __ldg(Dp + (size_t)(ao2 + b) * n + ao4 + d), s);
             } else {
-              for (int x = 0; x < NA; ++x) s = fma(Xs[(x * NB + r) * CH + ci], __ldg(Dp + (size_t)(ao1 + x) * n + ao4 + d), s);
+              for (int x = 0; x < NA; ++x) s = fma(Xs[(x * NB + r) * NCD + ci], __ldg(Dp + (size_t)(ao1 + x) * n + ao4 + d), s);
             }
           }
           const int row = isA ? ao1 + r : ao2 + r;
           acc_add(Kh + (size_t)row * n + ao3 + c, (double)(w * s), a.det);
         }
-        // Kh_ad[a][d] += w sum_{b, c in chunk} X D_bc ; Kh_bd[b][d] += w sum_{a, c} X D_ac
+        // Kh_ad[a][d] += w sum_{b, c} X D_bc ; Kh_bd[b][d] += w sum_{a, c} X D_ac
         for (int o = lane; o < (NA + NB) * ND; o += 32) {
           const bool isA = o < NA * ND;
           const int oo = isA ? o : o - NA * ND;
           const int r = oo / ND, d = oo % ND;
           T s = T(0);
-          for (int c = cfirst; c <= clast; ++c) {
-            const int ci = c * ND + d - c0;
-            if (ci < 0 || ci >= nci) continue;
+          for (int c = 0; c < NC; ++c) {
+            const int ci = c * ND + d;
             if (isA) {
-              for (int b = 0; b < NB; ++b) s = fma(Xs[(r * NB + b) * CH + ci], __ldg(Dp + (size_t)(ao2 + b) * n + ao3 + c), s);
+              for (int b = 0; b < NB; ++b) s = fma(Xs[(r * NB + b) * NCD + ci], __ldg(Dp + (size_t)(ao2 + b) * n + ao3 + c), s);
             } else {
-              for (int x = 0; x < NA; ++x) s = fma(Xs[(x * NB + r) * CH + ci], __ldg(Dp + (size_t)(ao1 + x) * n + ao3 + c), s);
+              for (int x = 0; x < NA; ++x) s = fma(Xs[(x * NB + r) * NCD + ci], __ldg(Dp + (size_t)(ao1 + x) * n + ao3 + c), s);
             }
           }
           const int row = isA ? ao1 + r : ao2 + r;
@@ -499,19 +392,16 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 0) jk_warp_kernel(JK
       }
       if (Jh) {
         const T w2 = T(2) * w;
-        for (int iab = lane; iab < NAB; iab += 32) {  // Jh_ab += 2w sum_cd X D_cd (chunk part)
+        for (int iab = lane; iab < NAB; iab += 32) {  // Jh_ab += 2w sum_cd X D_cd
           T s = T(0);
-          for (int ci = 0; ci < nci; ++ci) {
-            const int cd = c0 + ci;
-            s = fma(Xs[iab * CH + ci], __ldg(Dp + (size_t)(ao3 + cd / ND) * n + ao4 + cd % ND), s);
-          }
+          for (int cd = 0; cd < NCD; ++cd)
+            s = fma(Xs[iab * NCD + cd], __ldg(Dp + (size_t)(ao3 + cd / ND) * n + ao4 + cd % ND), s);
           acc_add(Jh + (size_t)(ao1 + iab / NB) * n + ao2 + iab % NB, (double)(w2 * s), a.det);
         }
-        for (int ci = lane; ci < nci; ci += 32) {  // Jh_cd += 2w sum_ab X D_ab
+        for (int cd = lane; cd < NCD; cd += 32) {  // Jh_cd += 2w sum_ab X D_ab
           T s = T(0);
           for (int iab = 0; iab < NAB; ++iab)
-            s = fma(Xs[iab * CH + ci], __ldg(Dp + (size_t)(ao1 + iab / NB) * n + ao2 + iab % NB), s);
-          const int cd = c0 + ci;
+            s = fma(Xs[iab * NCD + cd], __ldg(Dp + (size_t)(ao1 + iab / NB) * n + ao2 + iab % NB), s);
           acc_add(Jh + (size_t)(ao3 + cd / ND) * n + ao4 + cd % ND, (double)(w2 * s), a.det);
         }
       }

@@ -24,6 +24,9 @@
 // twice and contracted six densities per term); dE/dC is transposed through
 // shared memory so that a lane sums one charge over the warp's 32 pairs (3
 // additions per charge instead of 15 shuffles).
+// Bound by the FP64 pipe.  12 atoms and 3001 charges on GB300, V plus gradient:
+// 64.7 ms with a kernel per pair and one per charge, 37.7 ms with this one, 10.7 ms
+// with chunks sized to the lists and the pair orders side by side.
 #include <algorithm>
 #include <vector>
 
