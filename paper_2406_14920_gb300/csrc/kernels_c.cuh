@@ -22,6 +22,10 @@
 //   D  X[ab][cd] += sum_P E_P^{ab} W[cd][P], once per bra primitive
 //   contraction: a thread per output element of Kh and Jh, D' blocks staged in
 //   shared memory, one atomic per element.
+// Measured on GB300: one (ff|ff) quartet 5.4 ms with a warp per quartet; FP64 J/K
+// of 225 functions 184 ms then, 104 ms with this kernel, 53 ms now.  Component
+// pairs ordered by their number of terms (lanes of a warp then run equally long
+// sums; 22 of 32 lanes were active): (dp|pp) of it 4.05 -> 3.31 ms.
 #pragma once
 #include "kernels_b.cuh"
 
@@ -423,8 +427,11 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
 // FP64 classes of the register kernel whose unrolled code is long run a block per
 // quartet while the list is short (at most kShortList quartets per SM): a warp
 // that passes once through some hundred kilobytes of straight-line code waits on
-// instruction fetches (6 (pp|pp) quartets: 0.36 ms).
-constexpr int kShortList = 8;
+// instruction fetches (6 (pp|pp) quartets: 0.36 ms).  The line lies above the lists
+// of a small molecule and below those of a medium one: 45 functions 1.64 ms at 8 per
+// SM, 1.54 ms at 256; 225 functions 52.9 ms at 8, 55.2 ms at 256 ((pp|pp) 3.0 against
+// 4.0 ms).
+constexpr int kShortList = 16;
 template <int LA, int LB, int LC, int LD, typename T>
 __host__ __device__ constexpr bool block_when_short() {
   return sizeof(T) == 8 && ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD) >= 36;
