@@ -1129,6 +1129,8 @@ static const double kPmax32 = 1.0e3;
 static const int kClassL1[NPAIRCLASS] = {0, 1, 1, 2, 2, 2, 3, 3, 3, 3};
 static const int kClassL2[NPAIRCLASS] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3};
 
+static void ensure_order_bufs(eri_plan_impl* P);
+
 int eri_plan_impl::ensure_streams() {
   if (cap_stream) return ERI_OK;
   CK(cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking));
@@ -1194,7 +1196,8 @@ int eri_plan_impl::ensure_tier_bufs(int nb) {
     tier_cap = cap;
   }
   if (!tcnt) CK(dalloc(&tcnt, 2 * kStreams));
-  for (int b = tier_nb; b < nb; ++b) CK(dalloc(&tbuf[b], 2 * (size_t)tier_cap));
+  for (int b = tier_nb; b < nb; ++b)
+    if (!tbuf[b]) CK(dalloc(&tbuf[b], 2 * (size_t)tier_cap));
   tier_nb = std::max(tier_nb, nb);
   return ERI_OK;
 }
@@ -1601,6 +1604,7 @@ static int plan_create(int nmol, const eri_basis_t* const* bases, const double* 
     rc = P->geometry(s, true);
     if (rc != ERI_OK) goto fail;
     CKP(cudaDeviceSynchronize());
+    ensure_order_bufs(P);
   }
 #undef CKP
   tune_cache_load(P, o.precision);
@@ -1673,6 +1677,15 @@ static bool order_first(const eri_plan_impl* P, int X, int Y) {
   return use_thread_kernel(kClassL1[X], kClassL2[X], kClassL1[Y], kClassL2[Y], false) &&
          P->h_maxnp[X] * P->h_maxnp[Y] > 1 && P->nshard == 1 &&
          P->h_ktot[X * NPAIRCLASS + Y] >= (int64_t)256 * P->nsm;
+}
+
+// The lists that order FP64 builds, taken when the plan is made (a build allocates
+// nothing); a plan without room for them builds in list order.
+static void ensure_order_bufs(eri_plan_impl* P) {
+  bool any = false;
+  for (int X = 0; X < NPAIRCLASS; ++X)
+    for (int Y = 0; Y <= X; ++Y) any = any || order_first(P, X, Y);
+  if (any && P->ensure_tier_bufs(std::max(1, P->eager_branches(true))) != ERI_OK) cudaGetLastError();
 }
 
 // One J/K build on stream s, lists as they stand.  nbranch > 0: the class
@@ -1844,18 +1857,12 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       if (rc != ERI_OK) return rc;
     }
     // Plain FP64 builds order the long lists of the thread kernels the same way
-    // (every quartet in one list, see k_tier_split); without room for the lists, or
-    // while the caller captures before the first build, they run in list order.
+    // (every quartet in one list, see k_tier_split) where the plan holds the lists
+    // (see ensure_order_bufs); without them they run in list order.
     bool ordered = false;
-    if (!split) {
+    if (!split && P->tier_nb >= std::max(1, std::min(nbranch, eri_plan_impl::kBranches)))
       for (const ClassLaunch& l : order) ordered = ordered || order_first(P, l.X, l.Y);
-      if (ordered && P->tier_nb < std::max(1, nbranch)) {
-        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-        CK(cudaStreamIsCapturing(s, &st));
-        ordered = st == cudaStreamCaptureStatusNone && P->ensure_tier_bufs(std::max(1, nbranch)) == ERI_OK;
-        if (!ordered) cudaGetLastError();
-      }
-    }
+    if (ordered) nbranch = std::min(nbranch, P->tier_nb);
     nbranch = assign_branches(order, nbranch);
     if (concurrent) {
       const int rc = P->fork(s, nbranch);

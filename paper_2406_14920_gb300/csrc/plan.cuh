@@ -96,7 +96,8 @@ struct eri_plan_impl {
   int fork(cudaStream_t s, int n);  // branch[0 .. n) continue from s
   int join(cudaStream_t s, int n);  // s continues after branch[0 .. n)
   int eager_branches(bool lists) const;  // streams an eager call forks over (0: none, one launch after another on s)
-  // compacted tier lists of mixed builds (per branch), see ensure_tier_bufs
+  // compacted tier lists of mixed builds (per branch), see ensure_tier_bufs; FP64
+  // builds order their long lists in them
   int2* tbuf[kStreams] = {};
   unsigned int* tcnt = nullptr;
   int64_t tier_cap = 0;
