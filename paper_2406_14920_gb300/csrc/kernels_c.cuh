@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
 // quartet while the list is short (at most kShortList quartets per SM): a warp
 // that passes once through some hundred kilobytes of straight-line code waits on
 // instruction fetches (6 (pp|pp) quartets: 0.36 ms).  The line lies above the lists
-// of a small molecule and below those of a medium one: 45 functions 1.64 ms at 8 per
+// of a small molecule and below those of a medium one: 75 functions 1.64 ms at 8 per
 // SM, 1.54 ms at 256; 225 functions 52.9 ms at 8, 55.2 ms at 256 ((pp|pp) 3.0 against
 // 4.0 ms).
 constexpr int kShortList = 16;
