@@ -149,8 +149,13 @@ template <int LAB, int LCD, typename T>
 cudaError_t launch_j_t(const JArgs& a, cudaStream_t s, int nsm) {
   const int64_t n = a.wl.total - a.wl.first;
   if (n <= 0) return cudaSuccess;
+  constexpr bool small = j_footprint(LAB, LCD) <= kJAlways;
   if constexpr (use_j_thread(LAB, LCD)) {
-    return launch_over<j_thread_kernel<LAB, LCD, T>>(a, split_items<T>(a.wl, n), 128, 128, 0, s, nsm);
+    if (small || n > (int64_t)kJLong * nsm)
+      return launch_over<j_thread_kernel<LAB, LCD, T>>(a, split_items<T>(a.wl, n), 128, 128, 0, s, nsm);
+  }
+  if constexpr (small) {
+    return cudaErrorInvalidValue;  // (not reached)
   } else {
     constexpr int WPB = 4;
     constexpr size_t smem = WPB * JShape<LAB, LCD, T>::smem_per_warp();

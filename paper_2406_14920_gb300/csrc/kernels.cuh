@@ -432,11 +432,22 @@ __global__ void __launch_bounds__(128) j_warp_kernel(JArgs a) {
   }
 }
 
-// Which J-engine classes run one ordered item per thread (R, the item's
-// Hermite J and the ket's Hermite density in registers) instead of one per warp.
-__host__ __device__ constexpr bool use_j_thread(int lab, int lcd) {
-  return nherm(lab + lcd) + nherm(lab) + nherm(lcd) <= 130;
+// Values per thread of the J-engine's register form: R, the item's Hermite J and
+// the ket's Hermite density.
+__host__ __device__ constexpr int j_footprint(int lab, int lcd) {
+  return nherm(lab + lcd) + nherm(lab) + nherm(lcd);
 }
+// Which J-engine classes may run one ordered item per thread instead of one per
+// warp: up to kJThread values, most of them in lane-interleaved local memory
+// beyond the register file, which costs little beside the FP64 pipe.  Measured on
+// GB300, 520 functions, FP64: (ps|fd) 46.1 -> 6.5 ms, (dp|fp) 37.3 -> 12.5 ms, (fp|fp)
+// 28.2 -> 12.5 ms; its FP32 tier (fp|fp) 2.26 -> 0.32 ms.  Beyond 260 the long ones
+// are no faster ((fd|fp) 3.8 against 3.9 ms, (ff|ff) 0.12 against 1.04 ms) and take
+// minutes to compile.  Above kJAlways values only long lists do (more than kJLong
+// items per SM): few items leave the lanes idle ((dd|dd), 930 items: 0.025 ms per
+// warp, 0.090 ms per lane; (fp|dd), 2182 items: 0.105 against 0.092 ms).
+constexpr int kJAlways = 130, kJThread = 260, kJLong = 8;
+__host__ __device__ constexpr bool use_j_thread(int lab, int lcd) { return j_footprint(lab, lcd) <= kJThread; }
 
 // J-engine (Eq. j_formula), one ordered (bra, ket) shell-pair item per lane:
 // for each bra primitive pair, J_P += sum_{ket prims} sum_Q R_{P+Q} D_Q with

@@ -115,6 +115,20 @@ def test_primitive_screening(eri):
     assert fl[0] < fl[1]
 
 
+# Lists of 8 items per SM and shorter run a warp per item in the J-engine's large
+# classes, longer ones a lane; FP32 items are below the tier bound (1e-5 each, some
+# 1e2 per element, 1e-5 of it at most lost with Hermite cancellation): 1e-8.
+@pytest.mark.parametrize("mixed,tol", [(False, TOL), (True, 1e-8)])
+@pytest.mark.parametrize("copies", [1, 1300])
+def test_jengine_large_classes(eri, copies, mixed, tol):
+    b, D = W.small_system(["1s1p1d1f", "1f"], seed=31)
+    plan = eri.Plan([b] * copies, precision=eri.ERI_MIXED if mixed else eri.ERI_FP64, mixed_tau=1e-5)
+    J, _ = plan.build_jk(plan.pack([_t(D)] * copies), want_k=False)
+    Jo, _ = oracle.Oracle(b).jk(D)
+    for m in (0, copies - 1):
+        assert np.abs(plan.unpack(J)[m].cpu().numpy() - Jo).max() < tol
+
+
 @pytest.mark.parametrize("copies", [1, 120])
 def test_captured_before_the_first_build(eri, copies):
     import torch
