@@ -210,9 +210,11 @@ __device__ __forceinline__ int64_t item_tile(const WorkList& wl, int64_t items, 
   return t < 1 ? 1 : (t < wl.tile ? t : wl.tile);
 }
 
-// an item's primitive quartets in 16 steps of its class pair's largest
+// an item's primitive quartets in 16 steps of its class pair's largest (0 .. 15: it
+// indexes the counters of k_tier_split)
 __device__ __forceinline__ int work_bucket(const WorkList& wl, int npb, int npk) {
-  return (int)((int64_t)(npb * npk - 1) * 16 / ((int64_t)wl.mpb * wl.mpk));
+  const int64_t b = ((int64_t)npb * npk - 1) * 16 / ((int64_t)wl.mpb * wl.mpk);
+  return b < 0 ? 0 : (b > 15 ? 15 : (int)b);
 }
 
 // Ket position of list item ik of a bra pair with `count` kets.  Primitive

@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
       }
       int pb0, pb1, pk0, pk1;
       sp.range(part, npb, npk, pb0, pb1, pk0, pk1);
-      if (pb0 >= pb1) continue;  // uniform over the block
+      if (pb0 >= pb1 || npk == 0) continue;  // uniform over the block; W has no value without a ket primitive
       __syncthreads();  // the previous item's shared memory (first item: the tables) is done with
       const T* Dp = dens<T>(a) + mbase;
       for (int x = tid; x < S::NDB; x += NT) {

@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(GShape<LA, LB, LC, LD, T>::NT) grad_block_kern
       }
       int pb0, pb1, pk0, pk1;
       sp.range(part, npb, npk, pb0, pb1, pk0, pk1);
-      if (pb0 >= pb1) continue;  // uniform over the block
+      if (pb0 >= pb1 || npk == 0) continue;  // uniform over the block; W has no value without a ket primitive
       // items of a tile usually share the bra atoms: their sums go out together
       // (FP32 sums and deterministic builds: once per item)
       const int nA = __ldg(a.sh_atom + s1), nB = __ldg(a.sh_atom + s2);

@@ -407,8 +407,8 @@ __global__ void __launch_bounds__(32 * kSchwarzWarps)
 // units of pref), and |(ab|cd)| <= q_ab q_cd for every primitive quartet.
 // k_primpack moves the primitive pairs with q qmax >= kPrimEps thresh to the
 // front of their shell pair and counts them; the J/K, J-engine and gradient
-// kernels run over those.  Each dropped primitive quartet is below 1e-8 of the
-// quartet threshold (thresh = 0 drops none).
+// kernels run over those (a pair keeps at least one).  Each dropped primitive
+// quartet is below 1e-8 of the quartet threshold (thresh = 0 drops none).
 constexpr double kPrimEps = 1e-8;
 __global__ void __launch_bounds__(128)
     k_primq(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,
@@ -505,7 +505,10 @@ __global__ void k_primpack(int npair, const int* __restrict__ s1, const int* __r
     }
     ++m;
   }
-  if (lane == 0) nkeep[ip] = m;
+  // Never none: a pair of frozen lists that the atoms have pulled apart stays listed,
+  // and the kernels count on a first primitive pair (whose integrals are as small as
+  // its bound; it is in place already).
+  if (lane == 0) nkeep[ip] = max(m, 1);
 }
 
 // Per-molecule Schwarz maximum (pairs never cross molecules).  Q >= 0, so

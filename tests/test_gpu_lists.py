@@ -1,0 +1,83 @@
+"""GPU tests of the lists that the builds run over:
+
+- lists frozen at one geometry while the atoms move far apart: shell pairs that
+  stay listed although none of their primitive pairs is above the screening
+  bound any more, in every kernel (J+K, J-engine, gradient; FP64 and mixed
+  precision; short lists and lists ordered by work), against the oracle on the
+  same frozen lists.
+
+Tolerances: 1e-10 (J, K) and 1e-9 (gradients), the parity tolerances of the
+library.  Mixed precision with a tier bound of 1e-7: an FP32 quartet is at most
+1e-7 and off by at most 1e-5 of it (rounding 6e-8 times Hermite cancellation),
+some 1e3 of them per element: 1e-9, taken as 1e-8; a derivative brings a factor
+2 sqrt(p) of up to 10: 1e-7.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+THRESH = 1e-12
+
+
+@pytest.fixture(scope="module")
+def eri():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2406_14920_gb300.build import build
+    build()
+    import paper_2406_14920_gb300 as m
+    return m
+
+
+def _t(x):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(x, np.float64)).cuda()
+
+
+def _basis(shells, coords, seed=5):
+    """shells: (atom, l, exponents)"""
+    rng = np.random.default_rng(seed)
+    n = np.array([len(s[2]) for s in shells], np.int32)
+    off = np.concatenate([[0], np.cumsum(n)[:-1]]).astype(np.int32)
+    return W.Basis(np.array([s[0] for s in shells], np.int32), np.array([s[1] for s in shells], np.int32), n, off,
+                   np.concatenate([np.asarray(s[2], float) for s in shells]),
+                   rng.uniform(0.3, 1.0, int(n.sum())), np.asarray(coords, float))
+
+
+# single tight primitives of every angular momentum beside one diffuse s shell per
+# atom; contracted s and p shells (lists ordered by work in FP64 builds too)
+_SINGLE = [(a, l, [e + 0.5 * a]) for a in range(2) for l, e in ((0, 0.4), (0, 5.0), (1, 5.0), (2, 6.0), (3, 7.0))]
+_CONTRACTED = [(a, l, e) for a in range(2) for l, e in ((0, [0.4]), (0, [9.0, 4.0]), (1, [8.0, 4.5]))]
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("shells,copies", [(_SINGLE, 1), (_SINGLE, 3), (_CONTRACTED, 1), (_CONTRACTED, 4000)])
+def test_frozen_lists_with_atoms_pulled_apart(eri, shells, copies, mixed):
+    near = np.array([[0.0, 0.0, 0.0], [0.2, 0.3, 0.9]])
+    far = near + np.array([[0.0, 0.0, 0.0], [1.0, 2.0, 6.0]])
+    b = _basis(shells, near)
+    D = W.density_from_orbitals(np.random.default_rng(1), b.nbf, 4)
+    plan = eri.Plan([b] * copies, thresh=THRESH, precision=eri.ERI_MIXED if mixed else eri.ERI_FP64, mixed_tau=1e-7)
+    plan.set_coords(_t(np.concatenate([far] * copies)), freeze_lists=True)
+    # the case: every pair is listed, the tight ones on two centres (exponents 4 and more: exp(-2 R^2)) are nothing
+    lists = plan.lists()
+    assert lists["sig"].all() and np.exp(-2.0 * ((far[1] - far[0]) ** 2).sum()) < 1e-40
+    o = oracle.Oracle(b.with_coords(far))
+    Q = lists["Q"][:b.nshell * (b.nshell + 1) // 2]
+    Jo, Ko = o.jk(D, THRESH, Q)
+    go = o.grad(D, THRESH, Q)
+    Dp = plan.pack([_t(D)] * copies)
+    tol, gtol = (1e-8, 1e-7) if mixed else (1e-10, 1e-9)
+    for _ in range(2):
+        J, K = plan.build_jk(Dp)
+        Je, _ = plan.build_jk(Dp, want_k=False)
+        g = plan.grad(Dp, precision=eri.ERI_MIXED if mixed else eri.ERI_FP64).cpu().numpy().reshape(copies, -1, 3)
+        for m in {0, copies // 2, copies - 1}:
+            for x, ref in ((J, Jo), (K, Ko), (Je, Jo)):
+                assert np.abs(plan.unpack(x)[m].cpu().numpy() - ref).max() < tol
+            assert np.abs(g[m] - go).max() < gtol
