@@ -510,9 +510,11 @@ __global__ void __launch_bounds__(128) j_thread_kernel(JArgs a) {
           doneb += npb;
         }
       }
-      // lane 0's item is always valid here
+      // lane 0's item is always valid here.  Deterministic builds add every item by
+      // itself: a compacted list's order, and with it which items share a warp, may
+      // differ from call to call.
       const int pair0 = __shfl_sync(0xffffffffu, pb_id, 0);
-      const bool uni = __all_sync(0xffffffffu, !ok || pb_id == pair0);
+      const bool uni = __all_sync(0xffffffffu, !ok || pb_id == pair0) && !a.det;
       if (uni) npb = __shfl_sync(0xffffffffu, npb, 0);
       int pb0, pb1, pk0, pk1;
       sp.range(part, npb, npk, pb0, pb1, pk0, pk1);

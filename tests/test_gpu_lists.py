@@ -4,7 +4,10 @@
   stay listed although none of their primitive pairs is above the screening
   bound any more, in every kernel (J+K, J-engine, gradient; FP64 and mixed
   precision; short lists and lists ordered by work), against the oracle on the
-  same frozen lists.
+  same frozen lists;
+- deterministic mixed J-only builds: bit for bit the same from call to call and
+  in graph replays, over compacted lists of several runs (their order is not
+  fixed).
 
 Tolerances: 1e-10 (J, K) and 1e-9 (gradients), the parity tolerances of the
 library.  Mixed precision with a tier bound of 1e-7: an FP32 quartet is at most
@@ -81,3 +84,20 @@ def test_frozen_lists_with_atoms_pulled_apart(eri, shells, copies, mixed):
             for x, ref in ((J, Jo), (K, Ko), (Je, Jo)):
                 assert np.abs(plan.unpack(x)[m].cpu().numpy() - ref).max() < tol
             assert np.abs(g[m] - go).max() < gtol
+
+
+@pytest.mark.parametrize("copies", [3, 60])
+def test_deterministic_mixed_j_engine(eri, copies):
+    import torch
+    b, D = W.small_system(["2s2p1d1f", "1s1p1d"], seed=13)
+    plan = eri.Plan([b] * copies, precision=eri.ERI_MIXED, mixed_tau=1e-2, deterministic=True)
+    Dp = plan.pack([_t(D)] * copies)
+    J = plan.build_jk(Dp, want_k=False)[0].clone()
+    assert plan.stats()["quartets_j_fp32"] > 0
+    for _ in range(5):
+        assert torch.equal(plan.build_jk(Dp, want_k=False)[0], J)
+    Jg = torch.empty_like(J)
+    for _ in range(2):
+        plan.build_jk_graph(Dp, Jg, None)
+        assert torch.equal(Jg, J)
+    plan.check()
