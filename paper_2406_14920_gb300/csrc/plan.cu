@@ -1866,6 +1866,13 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
     if (!split && P->tier_nb >= std::max(1, std::min(nbranch, eri_plan_impl::kBranches)))
       for (const ClassLaunch& l : order) ordered = ordered || order_first(P, l.X, l.Y);
     if (ordered) nbranch = std::min(nbranch, P->tier_nb);
+    // (Deterministic builds order only lists that fit one window: the windows follow
+    // the size of the plan's lists, which may change between two calls, and a short
+    // last window takes other kernels and primitive splits than the list as a whole.)
+    auto by_work = [&](int X, int Y) {
+      return ordered && order_first(P, X, Y) &&
+             !(P->opts.deterministic && P->h_ktot[X * NPAIRCLASS + Y] > P->tier_cap);
+    };
     nbranch = assign_branches(order, nbranch);
     if (concurrent) {
       const int rc = P->fork(s, nbranch);
@@ -1892,7 +1899,7 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       const int b = l.branch;
       const cudaStream_t ls = concurrent ? P->branch[b] : s;
       ka.same_class = l.X == l.Y;
-      if (!split && !(ordered && order_first(P, l.X, l.Y))) {
+      if (!split && !by_work(l.X, l.Y)) {
         ka.wl = P->klist(l.X, l.Y);
         ka.items = nullptr;
         ka.nitems = nullptr;

@@ -7,7 +7,9 @@
   same frozen lists;
 - deterministic mixed J-only builds: bit for bit the same from call to call and
   in graph replays, over compacted lists of several runs (their order is not
-  fixed).
+  fixed);
+- deterministic FP64 builds over lists that have grown beyond the plan's order
+  lists: the same bits before and after those lists are made larger.
 
 Tolerances: 1e-10 (J, K) and 1e-9 (gradients), the parity tolerances of the
 library.  Mixed precision with a tier bound of 1e-7: an FP32 quartet is at most
@@ -101,3 +103,32 @@ def test_deterministic_mixed_j_engine(eri, copies):
         plan.build_jk_graph(Dp, Jg, None)
         assert torch.equal(Jg, J)
     plan.check()
+
+
+def _s_atoms(counts, nprim, seed=11):
+    """counts[a] s shells of nprim primitives on atom a, atoms 1.5 bohr apart in a row."""
+    rng = np.random.default_rng(seed)
+    atoms = np.repeat(np.arange(len(counts)), counts)
+    return _basis([(a, 0, np.exp(rng.uniform(np.log(0.2), np.log(3.0), nprim))) for a in atoms],
+                  [[0.0, 0.0, 1.5 * a] for a in range(len(counts))], seed)
+
+
+def test_deterministic_builds_do_not_depend_on_the_order_lists(eri):
+    import torch
+    b, copies = _s_atoms([15, 5], 2), 5
+    D = W.density_from_orbitals(np.random.default_rng(3), b.nbf, 4)
+    apart = b.coords + np.array([[0.0, 0.0, 0.0], [0.0, 0.0, 60.0]])
+    plan = eri.Plan([b.with_coords(apart)] * copies, deterministic=True)  # long enough to be ordered by work
+    n0 = plan.stats()["quartets_j"]
+    plan.set_coords(_t(np.concatenate([b.coords] * copies)))
+    assert 38912 < n0 < plan.stats()["quartets_k"] < 2 * n0  # (152 SMs: 256 quartets per SM) now one window and a bit
+    Dp = plan.pack([_t(D)] * copies)
+    J, K = (x.clone() for x in plan.build_jk(Dp))
+    Jg, Kg = torch.empty_like(J), torch.empty_like(K)
+    plan.build_jk_graph(Dp, Jg, Kg)  # makes the lists as long as the items
+    assert torch.equal(Jg, J) and torch.equal(Kg, K)
+    J2, K2 = plan.build_jk(Dp)
+    assert torch.equal(J2, J) and torch.equal(K2, K)
+    Jo, Ko = oracle.Oracle(b).jk(D)
+    assert np.abs(plan.unpack(J)[0].cpu().numpy() - Jo).max() < 1e-10
+    assert np.abs(plan.unpack(K)[0].cpu().numpy() - Ko).max() < 1e-10
