@@ -1054,6 +1054,10 @@ int eri_plan_impl::build_lists(double th, cudaStream_t s) {
   CK(cudaMemcpyAsync(h_jtot, d_jtot, sizeof(h_jtot), cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(h_kprim, d_kprim, sizeof(h_kprim), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  // Tier lists that have become too short are replaced here and by no later call: a
+  // build that the caller captures, in FP64 too, holds their addresses, and it is
+  // good until the next list rebuild.  (Without room for them the plan has none.)
+  if (tier_nb > 0 && tier_len() > tier_cap && ensure_tier_bufs(tier_nb) != ERI_OK) cudaGetLastError();
   return ERI_OK;
 }
 
@@ -1183,12 +1187,15 @@ int eri_plan_impl::eager_branches(bool lists) const {
 // Compacted tier lists of mixed-precision builds: per branch, two lists of
 // tier_cap items (int2 bra / ket positions) and two counters.  tier_cap is the
 // longest class-pair list, at most kTierCap; longer lists are split in windows.
-
-int eri_plan_impl::ensure_tier_bufs(int nb) {
+int64_t eri_plan_impl::tier_len() const {
   int64_t mx = 1;
   for (int X = 0; X < NPAIRCLASS; ++X)
     for (int Y = 0; Y <= X; ++Y) mx = std::max(mx, h_ktot[X * NPAIRCLASS + Y]);
-  const int64_t cap = std::min(mx, kTierCap);
+  return std::min(mx, kTierCap);
+}
+
+int eri_plan_impl::ensure_tier_bufs(int nb) {
+  const int64_t cap = tier_len();
   if (cap > tier_cap) {
     CK(cudaDeviceSynchronize());
     for (int b = 0; b < kStreams; ++b) {

@@ -102,6 +102,7 @@ struct eri_plan_impl {
   unsigned int* tcnt = nullptr;
   int64_t tier_cap = 0;
   int tier_nb = 0;
+  int64_t tier_len() const;  // items a tier list has to hold for the present lists
   int ensure_tier_bufs(int nb);
   // work-tile length (items per worker tile) per (bra class, ket class, tier),
   // set by eri_autotune or eri_set_tiles; 0 = the built-in default

@@ -9,7 +9,9 @@
   in graph replays, over compacted lists of several runs (their order is not
   fixed);
 - deterministic FP64 builds over lists that have grown beyond the plan's order
-  lists: the same bits before and after those lists are made larger.
+  lists: the same bits before and after those lists are made larger;
+- an FP64 build captured by the caller over grown lists, replayed after other
+  builds of the plan.
 
 Tolerances: 1e-10 (J, K) and 1e-9 (gradients), the parity tolerances of the
 library.  Mixed precision with a tier bound of 1e-7: an FP32 quartet is at most
@@ -119,9 +121,9 @@ def test_deterministic_builds_do_not_depend_on_the_order_lists(eri):
     D = W.density_from_orbitals(np.random.default_rng(3), b.nbf, 4)
     apart = b.coords + np.array([[0.0, 0.0, 0.0], [0.0, 0.0, 60.0]])
     plan = eri.Plan([b.with_coords(apart)] * copies, deterministic=True)  # long enough to be ordered by work
-    n0 = plan.stats()["quartets_j"]
+    n0 = plan.stats()["quartets_k"]
     plan.set_coords(_t(np.concatenate([b.coords] * copies)))
-    assert 38912 < n0 < plan.stats()["quartets_k"] < 2 * n0  # (152 SMs: 256 quartets per SM) now one window and a bit
+    assert n0 >= 256 * 152 and plan.stats()["quartets_k"] > 2 * n0  # (256 per SM are ordered)
     Dp = plan.pack([_t(D)] * copies)
     J, K = (x.clone() for x in plan.build_jk(Dp))
     Jg, Kg = torch.empty_like(J), torch.empty_like(K)
@@ -132,3 +134,41 @@ def test_deterministic_builds_do_not_depend_on_the_order_lists(eri):
     Jo, Ko = oracle.Oracle(b).jk(D)
     assert np.abs(plan.unpack(J)[0].cpu().numpy() - Jo).max() < 1e-10
     assert np.abs(plan.unpack(K)[0].cpu().numpy() - Ko).max() < 1e-10
+
+
+def _captured(build):
+    import torch
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s):
+        g.capture_begin()
+        try:
+            build()
+        finally:
+            g.capture_end()
+    torch.cuda.current_stream().wait_stream(s)
+    return g
+
+
+def test_captured_build_outlives_other_builds(eri):
+    import torch
+    b, copies = _s_atoms([15, 5], 2), 5
+    D = W.density_from_orbitals(np.random.default_rng(3), b.nbf, 4)
+    apart = b.coords + np.array([[0.0, 0.0, 0.0], [0.0, 0.0, 60.0]])
+    plan = eri.Plan([b.with_coords(apart)] * copies)  # holds order lists
+    plan.set_coords(_t(np.concatenate([b.coords] * copies)))  # longer lists
+    Dp = plan.pack([_t(D)] * copies)
+    J, K = torch.zeros_like(Dp), torch.zeros_like(Dp)
+    g = _captured(lambda: plan.build_jk(Dp, J, K))
+    Jg, Kg = torch.empty_like(J), torch.empty_like(K)
+    for precision in (eri.ERI_FP64, eri.ERI_MIXED):
+        plan.build_jk_graph(Dp, Jg, Kg, precision=precision)
+        plan.build_jk(Dp, Jg, Kg, precision=precision)
+    plan.grad(Dp, precision=eri.ERI_MIXED)
+    g.replay()
+    torch.cuda.synchronize()
+    Jo, Ko = oracle.Oracle(b).jk(D)
+    for m in (0, copies - 1):
+        assert np.abs(plan.unpack(J)[m].cpu().numpy() - Jo).max() < 1e-10
+        assert np.abs(plan.unpack(K)[m].cpu().numpy() - Ko).max() < 1e-10
