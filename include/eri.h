@@ -169,12 +169,14 @@ int eri_plan_set_coords(eri_plan_t* plan, const double* coords_dev, int32_t free
  * precision: ERI_FP64 or ERI_MIXED (tier split at the plan's mixed_tau: a device
  * pass writes each class pair's FP64-tier and FP32-tier quartets to two compacted
  * lists, then each tier runs over its own list; the plan holds these lists, up
- * to 2^23 quartets per tier and 512 MB in all, allocated by the first mixed build
- * or graph capture, or with the plan where its FP64 builds order long lists in them).
+ * to 2^23 quartets per tier and 512 MB in all, allocated by the first mixed build,
+ * mixed gradient or graph build, or with the plan where its FP64 builds order long
+ * lists in them; a list rebuild replaces them when they have become too short).
  * With thresh < 0 and opts.profile = 0 the call only enqueues work: class launches
  * fork from `stream` onto side streams of the plan and join it before the call
- * returns (no host wait, no allocation in FP64 and after the first mixed build), so
- * it may be captured into a CUDA graph.  Calls on one plan share its workspace and
+ * returns (no host wait; no allocation in FP64, nor in mixed precision once the plan
+ * has its tier lists), so it may be captured into a CUDA graph, which is good until
+ * the next list rebuild.  Calls on one plan share its workspace and
  * its side streams and must be ordered by the caller.
  */
 int eri_build_jk(eri_plan_t* plan, const double* D, double* J, double* K, double thresh, int32_t precision,

@@ -1057,7 +1057,7 @@ int eri_plan_impl::build_lists(double th, cudaStream_t s) {
   // Tier lists that have become too short are replaced here and by no later call: a
   // build that the caller captures, in FP64 too, holds their addresses, and it is
   // good until the next list rebuild.  (Without room for them the plan has none.)
-  if (tier_nb > 0 && tier_len() > tier_cap && ensure_tier_bufs(tier_nb) != ERI_OK) cudaGetLastError();
+  if (tier_nb > 0 && tier_len() > tier_cap && ensure_tier_bufs(1) != ERI_OK) cudaGetLastError();
   return ERI_OK;
 }
 
@@ -1172,14 +1172,15 @@ int eri_plan_impl::join(cudaStream_t s, int n) {
 // Profiled calls run in order on the caller's stream, so that an event pair
 // times one launch.
 // With tier lists the streams are as many (4 to kStreams) as keep the lists
-// within 512 MB.
+// within 512 MB, at the length they have or would get.
 int eri_plan_impl::eager_branches(bool lists) const {
   if (opts.profile) return 0;
   int n = kStreams;
   if (lists) {
     int64_t mx = 1;
     for (int64_t t : h_jtot) mx = std::max(mx, t);
-    while (n > kBranches && n * std::min(mx, kTierCap) > (int64_t)1 << 25) n /= 2;
+    mx = std::max(tier_cap, std::min(mx, kTierCap));
+    while (n > kBranches && n * mx > (int64_t)1 << 25) n /= 2;
   }
   return n;
 }
@@ -1187,6 +1188,9 @@ int eri_plan_impl::eager_branches(bool lists) const {
 // Compacted tier lists of mixed-precision builds: per branch, two lists of
 // tier_cap items (int2 bra / ket positions) and two counters.  tier_cap is the
 // longest class-pair list, at most kTierCap; longer lists are split in windows.
+// The first call that needs lists takes those of every stream of an eager build, so
+// that no later call allocates until the lists grow; builds run over no more
+// streams than there are lists.  An error only if fewer than `need` could be had.
 int64_t eri_plan_impl::tier_len() const {
   int64_t mx = 1;
   for (int X = 0; X < NPAIRCLASS; ++X)
@@ -1194,7 +1198,7 @@ int64_t eri_plan_impl::tier_len() const {
   return std::min(mx, kTierCap);
 }
 
-int eri_plan_impl::ensure_tier_bufs(int nb) {
+int eri_plan_impl::ensure_tier_bufs(int need) {
   const int64_t cap = tier_len();
   if (cap > tier_cap) {
     CK(cudaDeviceSynchronize());
@@ -1206,9 +1210,14 @@ int eri_plan_impl::ensure_tier_bufs(int nb) {
     tier_cap = cap;
   }
   if (!tcnt) CK(dalloc(&tcnt, 2 * kStreams));
-  for (int b = tier_nb; b < nb; ++b)
-    if (!tbuf[b]) CK(dalloc(&tbuf[b], 2 * (size_t)tier_cap));
-  tier_nb = std::max(tier_nb, nb);
+  const int want = tier_nb == 0 ? std::max(need, eager_branches(true)) : need;
+  for (; tier_nb < want; ++tier_nb)
+    if (const cudaError_t e = dalloc(&tbuf[tier_nb], 2 * (size_t)tier_cap)) {
+      tbuf[tier_nb] = nullptr;
+      if (tier_nb < need) return eri_fail(e);
+      cudaGetLastError();  // fewer streams
+      break;
+    }
   return ERI_OK;
 }
 
@@ -1695,7 +1704,7 @@ static void ensure_order_bufs(eri_plan_impl* P) {
   bool any = false;
   for (int X = 0; X < NPAIRCLASS; ++X)
     for (int Y = 0; Y <= X; ++Y) any = any || order_first(P, X, Y);
-  if (any && P->ensure_tier_bufs(std::max(1, P->eager_branches(true))) != ERI_OK) cudaGetLastError();
+  if (any && P->ensure_tier_bufs(1) != ERI_OK) cudaGetLastError();
 }
 
 // One J/K build on stream s, lists as they stand.  nbranch > 0: the class
@@ -1725,8 +1734,9 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       k_dmax<<<grid1(P->npair, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_sh_l, P->d_pao1, P->d_pao2,
                                                   P->d_pmol, P->d_mat_off, P->d_mat_n, P->d_Dp, P->d_dmax);
       CK(cudaGetLastError());
-      const int rc = P->ensure_tier_bufs(std::max(1, nbranch));  // (a graph capture has them already)
+      const int rc = P->ensure_tier_bufs(1);  // (a graph capture has them already)
       if (rc != ERI_OK) return rc;
+      nbranch = std::min(nbranch, P->tier_nb);
     }
     JArgs ja{};
     ja.pd = P->pairdata(); ja.sp = P->spinfo(); ja.bt = P->boystabs();
@@ -1863,8 +1873,9 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
                                            J != nullptr, K != nullptr), 0});
       }
     if (split) {
-      const int rc = P->ensure_tier_bufs(std::max(1, nbranch));  // (a graph capture has them already)
+      const int rc = P->ensure_tier_bufs(1);  // (a graph capture has them already)
       if (rc != ERI_OK) return rc;
+      nbranch = std::min(nbranch, P->tier_nb);
     }
     // Plain FP64 builds order the long lists of the thread kernels the same way
     // (every quartet in one list, see k_tier_split) where the plan holds the lists
@@ -2342,7 +2353,7 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
     k_dmax<<<grid1(P->npair, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_sh_l, P->d_pao1, P->d_pao2,
                                                 P->d_pmol, P->d_mat_off, P->d_mat_n, P->d_Dp, P->d_dmax);
     CK(cudaGetLastError());
-    const int rc = P->ensure_tier_bufs(std::max(1, P->eager_branches(true)));
+    const int rc = P->ensure_tier_bufs(1);
     if (rc != ERI_OK) return rc;
   }
   GradArgs ga{};
@@ -2377,6 +2388,7 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
     return ERI_OK;
   };
   int nbranch = P->eager_branches(mixed);
+  if (mixed) nbranch = std::min(nbranch, P->tier_nb);
   std::vector<ClassLaunch> order;
   for (int X = 0; X < NPAIRCLASS; ++X)
     for (int Y = 0; Y < NPAIRCLASS; ++Y) {

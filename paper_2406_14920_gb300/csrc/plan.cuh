@@ -103,7 +103,7 @@ struct eri_plan_impl {
   int64_t tier_cap = 0;
   int tier_nb = 0;
   int64_t tier_len() const;  // items a tier list has to hold for the present lists
-  int ensure_tier_bufs(int nb);
+  int ensure_tier_bufs(int need);
   // work-tile length (items per worker tile) per (bra class, ket class, tier),
   // set by eri_autotune or eri_set_tiles; 0 = the built-in default
   int tile_k[eri::NPAIRCLASS * eri::NPAIRCLASS * 2] = {};

@@ -11,7 +11,9 @@
 - deterministic FP64 builds over lists that have grown beyond the plan's order
   lists: the same bits before and after those lists are made larger;
 - an FP64 build captured by the caller over grown lists, replayed after other
-  builds of the plan.
+  builds of the plan;
+- tier lists taken once: mixed builds over shorter lists, or after a graph build,
+  allocate nothing more and can be captured.
 
 Tolerances: 1e-10 (J, K) and 1e-9 (gradients), the parity tolerances of the
 library.  Mixed precision with a tier bound of 1e-7: an FP32 quartet is at most
@@ -172,3 +174,46 @@ def test_captured_build_outlives_other_builds(eri):
     for m in (0, copies - 1):
         assert np.abs(plan.unpack(J)[m].cpu().numpy() - Jo).max() < 1e-10
         assert np.abs(plan.unpack(K)[m].cpu().numpy() - Ko).max() < 1e-10
+
+
+def test_tier_lists_are_taken_once(eri):
+    import torch
+    b, copies = _s_atoms([10, 10], 1), 64
+    D = W.density_from_orbitals(np.random.default_rng(3), b.nbf, 4)
+    plan = eri.Plan([b] * copies, precision=eri.ERI_MIXED)
+    Dp = plan.pack([_t(D)] * copies)
+    J, K = torch.empty_like(Dp), torch.empty_like(Dp)
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    f0 = free()
+    plan.build_jk(Dp, J, K)  # long lists: fewer than 16 streams
+    f1 = free()
+    assert 0 < f0 - f1 < 544 << 20
+    plan.build_jk(Dp, J, K, thresh=0.3)  # short lists
+    plan.grad(Dp, precision=eri.ERI_MIXED)
+    plan.build_jk(Dp, J, None)
+    assert abs(free() - f1) < 16 << 20
+    apart = np.concatenate([b.coords + np.array([[0.0, 0.0, 0.0], [0.0, 0.0, 60.0]])] * copies)
+    plan.set_coords(_t(apart))
+    J2, K2 = torch.zeros_like(J), torch.zeros_like(K)
+    g = _captured(lambda: plan.build_jk(Dp, J2, K2))
+    plan.build_jk(Dp, J, K)
+    g.replay()
+    torch.cuda.synchronize()
+    assert float((J - J2).abs().max()) < 1e-10 and float((K - K2).abs().max()) < 1e-10
+
+
+def test_mixed_build_captured_after_a_graph_build(eri):
+    import torch
+    b, D = W.small_system(["2s1p1d", "1s1p"], seed=8)
+    plan = eri.Plan(b, precision=eri.ERI_MIXED)
+    Dt = _t(D)
+    J, K = torch.empty_like(Dt), torch.empty_like(Dt)
+    plan.build_jk_graph(Dt, J, K)
+    J2, K2 = torch.zeros_like(J), torch.zeros_like(K)
+    _captured(lambda: plan.build_jk(Dt, J2, K2)).replay()
+    torch.cuda.synchronize()
+    assert float((J - J2).abs().max()) < 1e-10 and float((K - K2).abs().max()) < 1e-10
