@@ -350,7 +350,8 @@ extern "C" int eri_nuclear(eri_plan_t* plan, int32_t ncharge, const double* q, c
   if ((rc = ensure_nuc(P)) != ERI_OK) return rc;
   NCK(cudaMemsetAsync(P->d_Jherm, 0, sizeof(double) * (size_t)P->nherm_tot, s));
   // independent sums (atomics), one of the plan's streams each
-  if ((rc = P->fork(s, 2 * LMAX + 1)) != ERI_OK) return rc;
+  Fork side(s, P->branch, P->fork_ev, P->join_ev);
+  NCK(side.open(2 * LMAX + 1));
   NCK(launch_herm<6>(P, ncharge, q, xyz, P->branch[0]));
   NCK(launch_herm<5>(P, ncharge, q, xyz, P->branch[1]));
   NCK(launch_herm<4>(P, ncharge, q, xyz, P->branch[2]));
@@ -358,7 +359,7 @@ extern "C" int eri_nuclear(eri_plan_t* plan, int32_t ncharge, const double* q, c
   NCK(launch_herm<2>(P, ncharge, q, xyz, P->branch[4]));
   NCK(launch_herm<1>(P, ncharge, q, xyz, P->branch[5]));
   NCK(launch_herm<0>(P, ncharge, q, xyz, P->branch[6]));
-  if ((rc = P->join(s, 2 * LMAX + 1)) != ERI_OK) return rc;
+  NCK(side.join());
   const MolMats mm = molmats(P);
   k_post_j<<<(int)(((int64_t)P->npair * 100 + 127) / 128), 128, 0, s>>>(
       P->npair, P->d_ps1, P->d_ps2, P->d_pnp, P->d_phoff, P->d_peoff, P->d_sh_l, P->d_pao1, P->d_pao2, P->d_pmol, mm,
@@ -385,7 +386,8 @@ extern "C" int eri_nuclear_grad(eri_plan_t* plan, const double* D, int32_t nchar
   NCK(cudaMemsetAsync(dEdR, 0, sizeof(double) * 3 * (size_t)P->natom, s));
   if (dEdC && ncharge > 0) NCK(cudaMemsetAsync(dEdC, 0, sizeof(double) * 3 * (size_t)ncharge, s));
   // independent sums (atomics), one of the plan's streams each
-  if ((rc = P->fork(s, 2 * LMAX + 1)) != ERI_OK) return rc;
+  Fork side(s, P->branch, P->fork_ev, P->join_ev);
+  NCK(side.open(2 * LMAX + 1));
   NCK(launch_grad<6>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[0]));
   NCK(launch_grad<5>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[1]));
   NCK(launch_grad<4>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[2]));
@@ -393,6 +395,6 @@ extern "C" int eri_nuclear_grad(eri_plan_t* plan, const double* D, int32_t nchar
   NCK(launch_grad<2>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[4]));
   NCK(launch_grad<1>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[5]));
   NCK(launch_grad<0>(P, ncharge, q, xyz, dEdR, dEdC, P->branch[6]));
-  if ((rc = P->join(s, 2 * LMAX + 1)) != ERI_OK) return rc;
+  NCK(side.join());
   return ERI_OK;
 }

@@ -1152,20 +1152,6 @@ int eri_plan_impl::ensure_streams() {
 // longest compacted tier list (items); longer class-pair lists are split in windows
 static const int64_t kTierCap = 1 << 23;
 
-int eri_plan_impl::fork(cudaStream_t s, int n) {
-  CK(cudaEventRecord(fork_ev, s));
-  for (int b = 0; b < n; ++b) CK(cudaStreamWaitEvent(branch[b], fork_ev, 0));
-  return ERI_OK;
-}
-
-int eri_plan_impl::join(cudaStream_t s, int n) {
-  for (int b = 0; b < n; ++b) {
-    CK(cudaEventRecord(join_ev[b], branch[b]));
-    CK(cudaStreamWaitEvent(s, join_ev[b], 0));
-  }
-  return ERI_OK;
-}
-
 // Eager calls overlap their class launches (independent sums into the same
 // accumulators) on the plan's side streams: a small molecule's fifty launches
 // hold a few blocks each, and one after another they leave most SMs idle.
@@ -1788,10 +1774,8 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
         if (tot > 0) order.push_back({X, Y, jengine_flops(X, Y, (double)tot * P->h_maxnp[X] * P->h_maxnp[Y]), 0});
       }
     nbranch = assign_branches(order, nbranch);
-    if (concurrent) {
-      const int rc = P->fork(s, nbranch);
-      if (rc != ERI_OK) return rc;
-    }
+    Fork side(s, P->branch, P->fork_ev, P->join_ev);
+    if (concurrent) CK(side.open(nbranch));
     for (const ClassLaunch& l : order) {
         const int X = l.X, Y = l.Y, b = l.branch;
         const WorkList full = P->jlist(X, Y);
@@ -1824,10 +1808,7 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
         ja.items = nullptr;
         ja.nitems = nullptr;
     }
-    if (concurrent) {
-      const int rc = P->join(s, nbranch);
-      if (rc != ERI_OK) return rc;
-    }
+    CK(side.join());
     CK(cudaMemsetAsync(J, 0, sizeof(double) * nn, s));
     k_post_j<<<grid1((int64_t)P->npair * 100, 128), 128, 0, s>>>(P->npair, P->d_ps1, P->d_ps2, P->d_pnk, P->d_phoff,
                                                                  P->d_peoff, P->d_sh_l, P->d_pao1, P->d_pao2,
@@ -1892,10 +1873,8 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
              !(P->opts.deterministic && P->h_ktot[X * NPAIRCLASS + Y] > P->tier_cap);
     };
     nbranch = assign_branches(order, nbranch);
-    if (concurrent) {
-      const int rc = P->fork(s, nbranch);
-      if (rc != ERI_OK) return rc;
-    }
+    Fork side(s, P->branch, P->fork_ev, P->join_ev);
+    if (concurrent) CK(side.open(nbranch));
     const bool prof = P->opts.profile && !concurrent;
     auto launch = [&](int X, int Y, int tier, cudaStream_t ls) -> int {
       ka.tier_want = tier;
@@ -1951,10 +1930,7 @@ static int build_impl(eri_plan_impl* P, const double* D, double* J, double* K, i
       ka.items = nullptr;
       ka.nitems = nullptr;
     }
-    if (concurrent) {
-      const int rc = P->join(s, nbranch);
-      if (rc != ERI_OK) return rc;
-    }
+    CK(side.join());
     P->prof_builds += P->opts.profile ? 1 : 0;
     if (K) {
       k_post_k<<<P->mat_grid(256), 256, 0, s>>>(mm, P->d_Kh, P->d_f, K, ka.det, P->d_status);
@@ -2396,10 +2372,8 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
       if (tot > 0.0) order.push_back({X, Y, grad_flops(X, Y, tot, tot * mb * mk, tot * mb), 0});
     }
   nbranch = assign_branches(order, nbranch);
-  if (nbranch > 0) {
-    const int rc = P->fork(s, nbranch);
-    if (rc != ERI_OK) return rc;
-  }
+  Fork side(s, P->branch, P->fork_ev, P->join_ev);
+  CK(side.open(nbranch));
   for (const ClassLaunch& l : order) {
     const WorkList full = P->jlist(l.X, l.Y);
     const cudaStream_t ls = nbranch > 0 ? P->branch[l.branch] : s;
@@ -2430,10 +2404,7 @@ extern "C" int eri_jk_grad_prec(eri_plan_t* plan, const double* D, double* dEdR,
       }
     }
   }
-  if (nbranch > 0) {
-    const int rc = P->join(s, nbranch);
-    if (rc != ERI_OK) return rc;
-  }
+  CK(side.join());
   if (ga.det) {
     k_fix_to_double<<<grid1(3 * P->natom, 128), 128, 0, s>>>(3 * P->natom, dEdR, P->d_status);
     CK(cudaGetLastError());

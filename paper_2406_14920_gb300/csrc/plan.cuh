@@ -5,6 +5,7 @@
 #include <vector>
 #include <cuda_runtime.h>
 #include "common.cuh"
+#include "fork.cuh"
 #include "../../include/eri.h"
 #include "xc_state.cuh"
 
@@ -93,8 +94,6 @@ struct eri_plan_impl {
   int gprec = -1;
   int gbranches = 0;  // branches of the kept graph (1: serial chain, kBranches: forked)
   int ensure_streams();
-  int fork(cudaStream_t s, int n);  // branch[0 .. n) continue from s
-  int join(cudaStream_t s, int n);  // s continues after branch[0 .. n)
   int eager_branches(bool lists) const;  // streams an eager call forks over (0: none, one launch after another on s)
   // compacted tier lists of mixed builds (per branch), see ensure_tier_bufs; FP64
   // builds order their long lists in them
