@@ -422,7 +422,10 @@ int eri_nuclear_grad(eri_plan_t* plan, const double* D, int32_t ncharge, const d
  * shells that reach each block, and evaluates the basis functions and their
  * gradients there; when those values fit in cap_bytes (<= 0: 16 GiB) they stay
  * resident in device memory for every later call, otherwise each call
- * recomputes them in chunks of that size.  Waits for the device (a previous
+ * recomputes them in chunks of that size.  Beside them, and not under cap_bytes,
+ * the grid holds 16 nbf^2 bytes (the density as digits), at most 1 GiB of partial
+ * sums of V, and the points, potentials and function lists (4 nbf + 8 nshell
+ * bytes per block of points).  Waits for the device (a previous
  * grid's buffers are released; host bookkeeping of the block sizes).  The grid
  * follows eri_plan_set_coords: it is rebuilt, with the same parameters, at the
  * next XC call after a change (that call waits for the device too).
