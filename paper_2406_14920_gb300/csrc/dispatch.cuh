@@ -68,11 +68,36 @@ cudaError_t launch_over(const Args& a, int64_t workers, int per_block, int threa
   return r;
 }
 
-// work items of a thread kernel over a list of n items (with the parts of a
-// short list, see prim_split; longer lists fill the grid by themselves)
+// lanes that a list of n items can use: those of the largest split of a short list,
+// see prim_split; longer lists fill the grid by themselves
 template <typename T>
-inline int64_t split_items(const WorkList& wl, int64_t n, bool kets = true) {
-  return sizeof(T) == 4 || wl.nshard > 1 ? n : n * wl.mpb * (kets ? wl.mpk : 1);
+inline int64_t split_items(const WorkList& wl, int64_t n, SplitBy by) {
+  const PrimSplit s = prim_split<T>(wl, 1, INT32_MAX, by);
+  const int per = 32 / s.g;
+  return (n * s.n * 32 + per - 1) / per;
+}
+
+// Thread kernel of a class in its form for short lists (where it has one: while the
+// launch has two lanes and more for every item) or in the other one.
+template <auto Short, auto Long, typename T, bool HAS_SHORT, typename Args>
+cudaError_t launch_thread(const Args& a, const WorkList& wl, int64_t n, cudaStream_t s, int nsm) {
+  if constexpr (HAS_SHORT) {
+    int occ = 0;
+    const cudaError_t e = blocks_per_sm<Short>(128, 0, &occ);
+    if (e != cudaSuccess) return e;
+    if (wl.nshard == 1 && 2 * n <= (int64_t)nsm * occ * 128)
+      return launch_over<Short>(a, split_items<T>(wl, n, SplitBy::lanes), 128, 128, 0, s, nsm);
+  }
+  return launch_over<Long>(a, split_items<T>(wl, n, SplitBy::parts), 128, 128, 0, s, nsm);
+}
+
+// Blocks of a block kernel over a list of n items: short lists are split (by bra
+// primitives, see prim_split) while that leaves SMs without a block.  More parts would
+// be additions for nothing: other classes' launches run beside this one (split to
+// every resident block, 75 functions took 1.53 ms, now 1.46).
+template <typename T>
+inline int64_t split_blocks(const WorkList& wl, int64_t n, int nsm) {
+  return n * prim_split<T>(wl, n, nsm, SplitBy::blocks).n;
 }
 
 template <int LA, int LB, int LC, int LD, typename T>
@@ -80,16 +105,20 @@ cudaError_t launch_jk_t(const JKArgs& a, cudaStream_t s, int nsm) {
   const int64_t n = a.k.wl.total - a.k.wl.first;
   if (n <= 0) return cudaSuccess;
   if constexpr (use_thread_kernel(LA, LB, LC, LD, sizeof(T) == 4)) {
-    if constexpr (block_when_short<LA, LB, LC, LD, T>()) {
+    constexpr bool blocks = block_when_short<LA, LB, LC, LD, T>();
+    if constexpr (blocks) {
       using S = CShape<LA, LB, LC, LD, T>;
       if (n <= (int64_t)kShortList * nsm)
-        return launch_over<jk_block_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.k.wl, n, false), 1, S::NT, S::smem(), s, nsm);
+        return launch_over<jk_block_kernel<LA, LB, LC, LD, T>>(a, split_blocks<T>(a.k.wl, n, nsm), 1, S::NT, S::smem(), s, nsm);
     }
-    return launch_over<jk_thread_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.k.wl, n), 128, 128, 0, s, nsm);
+    // (the lane form of these larger classes would hold up to 108 sums through the
+    // shuffles: ptxas spills all of it)
+    return launch_thread<jk_thread_kernel<LA, LB, LC, LD, T, sizeof(T) == 8 && !blocks>,
+                         jk_thread_kernel<LA, LB, LC, LD, T, false>, T, sizeof(T) == 8 && !blocks>(a, a.k.wl, n, s, nsm);
   } else if constexpr (use_block_kernel<LA, LB, LC, LD, T>()) {
     using S = CShape<LA, LB, LC, LD, T>;
     static_assert(S::smem() <= 227 * 1024, "block kernel exceeds 227 KB");
-    return launch_over<jk_block_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.k.wl, n, false), 1, S::NT, S::smem(), s, nsm);
+    return launch_over<jk_block_kernel<LA, LB, LC, LD, T>>(a, split_blocks<T>(a.k.wl, n, nsm), 1, S::NT, S::smem(), s, nsm);
   } else {
     using S = BShape<LA, LB, LC, LD, T>;
     constexpr int WPB = 4;
@@ -131,14 +160,15 @@ cudaError_t launch_grad_unit(int y, const GradArgs& a, cudaStream_t s, int nsm) 
         if constexpr (grad_block_when_short<LA, LB, LC, LD, T>()) {
           using S = GShape<LA, LB, LC, LD, T>;
           if (n <= (int64_t)kShortList * nsm)
-            return launch_over<grad_block_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.wl, n, false), 1, S::NT,
+            return launch_over<grad_block_kernel<LA, LB, LC, LD, T>>(a, split_blocks<T>(a.wl, n, nsm), 1, S::NT,
                                                                      S::smem(), s, nsm);
         }
-        return launch_over<grad_thread_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.wl, n), 128, 128, 0, s, nsm);
+        return launch_thread<grad_thread_kernel<LA, LB, LC, LD, T, P == 0>, grad_thread_kernel<LA, LB, LC, LD, T, false>, T,
+                             P == 0>(a, a.wl, n, s, nsm);
       } else {
         using S = GShape<LA, LB, LC, LD, T>;
         static_assert(S::smem() <= 227 * 1024, "gradient block exceeds 227 KB");
-        return launch_over<grad_block_kernel<LA, LB, LC, LD, T>>(a, split_items<T>(a.wl, n, false), 1, S::NT, S::smem(), s, nsm);
+        return launch_over<grad_block_kernel<LA, LB, LC, LD, T>>(a, split_blocks<T>(a.wl, n, nsm), 1, S::NT, S::smem(), s, nsm);
       }
     }
     return launch_grad_unit<X, P, Y + 1>(y, a, s, nsm);
@@ -152,7 +182,7 @@ cudaError_t launch_j_t(const JArgs& a, cudaStream_t s, int nsm) {
   constexpr bool small = j_footprint(LAB, LCD) <= kJAlways;
   if constexpr (use_j_thread(LAB, LCD)) {
     if (small || n > (int64_t)kJLong * nsm)
-      return launch_over<j_thread_kernel<LAB, LCD, T>>(a, split_items<T>(a.wl, n), 128, 128, 0, s, nsm);
+      return launch_over<j_thread_kernel<LAB, LCD, T>>(a, split_items<T>(a.wl, n, SplitBy::parts), 128, 128, 0, s, nsm);
   }
   if constexpr (small) {
     return cudaErrorInvalidValue;  // (not reached)

@@ -154,36 +154,89 @@ struct BraCursor {
   }
 };
 
-// Thread kernels on short lists: an item's primitive quartets are split into n =
-// sb * sk parts (sb ranges of bra primitives times sk of ket primitives), each a
-// work item of its own whose sums are added like any other, so that a contracted
-// (81 primitive quartets) item of a small molecule is not one thread's serial
-// chain.  n is the largest split that still gives every lane of the launch at
-// most one part; lists longer than the launch's lanes are not split (a part
-// repeats the contraction with D).  FP64 only: an FP32 item's sum is taken whole,
-// so that its rounding does not depend on the list it is in.  A split over GPUs
-// keeps whole items.
+// Short lists: an item's primitive quartets are split, so that a contracted (81
+// primitive quartets) item of a small molecule is not one thread's serial chain.
+// The split is the largest that still gives every lane (block) of the launch at most
+// one part; lists longer than the launch's lanes are not split.
+//   lanes: g <= 32 neighbouring lanes take an item, gb ranges of bra primitives times
+//     gk of ket primitives, and sum their parts by shuffles, so that the item is added
+//     once (what they do not reach is further work items).
+//   parts: every part is a work item of its own and added by itself.
+//   blocks: the same over bra primitives.
+// J/K and gradients take lanes where the host knows that the list is short (plain
+// FP64): 81 parts added by themselves into a global sum left 1e-15 to 3e-15 of a
+// diatomic's J and K and 1e-14 of a gradient, whole items 4e-16 and 2e-15, lanes 4e-16
+// to 1e-15 and 3e-15 (the diatomic's build 93 us with parts, 62 with lanes).  Parts are
+// left for compacted lists that only the device knows to be short (FP64 tiers of
+// mixed builds: the lane form's code costs the long lists up to 10 %), for lists of
+// the larger J/K classes too long for a block per quartet, and for the J-engine,
+// whose sums are per bra primitive.  FP64 only: an FP32 item's sum
+// is taken whole, so that its rounding does not depend on the list it is in.  A
+// split over GPUs keeps whole items.
+enum class SplitBy { lanes, parts, blocks };
 struct PrimSplit {
-  int n, sb, sk;
-  __device__ __forceinline__ void range(int part, int npb, int npk, int& b0, int& b1, int& k0, int& k1) const {
-    const int pb = part / sk, pk = part - pb * sk;
-    b0 = npb * pb / sb;
-    b1 = npb * (pb + 1) / sb;
-    k0 = npk * pk / sk;
-    k1 = npk * (pk + 1) / sk;
+  int n, nk, gb, gk, g;
+  // of part `part`, lane `sub` < g: bra primitives [b0, b1), ket primitives [k0, k1)
+  __device__ __forceinline__ void range(int part, int sub, int npb, int npk, int& b0, int& b1, int& k0, int& k1) const {
+    const int pb = part / nk * gb + sub / gk, pk = part % nk * gk + sub % gk, nb = n / nk * gb, nkk = nk * gk;
+    b0 = npb * pb / nb;
+    b1 = npb * (pb + 1) / nb;
+    k0 = npk * pk / nkk;
+    k1 = npk * (pk + 1) / nkk;
   }
 };
-// (kets = false: bra primitives only, for the block kernels.)
 template <typename T>
-__device__ __forceinline__ PrimSplit prim_split(const WorkList& wl, int64_t items, int64_t lanes, bool kets = true) {
-  PrimSplit s{1, 1, 1};
+__host__ __device__ __forceinline__ PrimSplit prim_split(const WorkList& wl, int64_t items, int64_t lanes, SplitBy by) {
+  PrimSplit s{1, 1, 1, 1, 1};
   if (sizeof(T) == 4 || wl.nshard > 1 || items <= 0 || 2 * items > lanes) return s;
   const int64_t room = lanes / items;
-  s.sb = (int)(room < wl.mpb ? room : wl.mpb);
-  const int64_t rk = room / s.sb;
-  s.sk = kets ? (int)(rk < wl.mpk ? rk : wl.mpk) : 1;
-  s.n = s.sb * s.sk;
+  if (by != SplitBy::lanes) {
+    const int sb = (int)(room < wl.mpb ? room : wl.mpb);
+    const int64_t rk = room / sb;
+    s.nk = by == SplitBy::blocks ? 1 : (int)(rk < wl.mpk ? rk : wl.mpk);
+    s.n = sb * s.nk;
+    return s;
+  }
+  // A warp takes 32 / g items.  The group whose lanes have least to do, over chains of
+  // c bra primitives: per bra primitive a chain of ket primitives and the bra transform
+  // (two of them or more: lanes that share a bra primitive repeat it); of equals the
+  // smaller group.
+  const int width = room < 32 ? 32 / (int)((31 + room) / room) : 32;
+  int best = 1 << 30;
+  for (int c = (wl.mpb + width - 1) / width, i = 0; i < 3 && c <= wl.mpb; ++c, ++i) {
+    const int gb = (wl.mpb + c - 1) / c, gk = wl.mpk < width / gb ? wl.mpk : width / gb;
+    const int cost = 32 * c * ((wl.mpk + gk - 1) / gk + 2) + gb * gk;
+    if (cost < best) {
+      best = cost;
+      s.gb = gb;
+      s.gk = gk;
+      s.g = gb * gk;
+    }
+  }
+  const int64_t more = room * (32 / s.g) / 32;  // >= 1
+  const int lb = (wl.mpb + s.gb - 1) / s.gb, lk = (wl.mpk + s.gk - 1) / s.gk;
+  const int nb = (int)(more < lb ? more : lb);
+  s.nk = (int)(more / nb < lk ? more / nb : lk);
+  s.n = nb * s.nk;
   return s;
+}
+// Sums of x[0 .. N) over a group of g neighbouring lanes (`lanes`), in its first lane
+// (sub = 0): each step adds the lanes from o on to those below, where there are any
+template <int N, typename T>
+__device__ __forceinline__ void group_sum(T* x, int g, int sub, unsigned lanes) {
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+    if (o >= g) continue;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const T w = __shfl_down_sync(lanes, x[i], o);  // (of another group or none: not used)
+      if (sub + o < g) x[i] += w;
+    }
+  }
+}
+// lanes of the group of g that this lane belongs to (li: its number in the warp)
+__device__ __forceinline__ unsigned group_lanes(int g, int li) {
+  return li < 32 / g ? (0xffffffffu >> (32 - g)) << (li * g) : 0u;
 }
 
 // Tile of a warp's turn: turns of nwarps tiles, the warps shifted by three from
@@ -470,7 +523,7 @@ __global__ void __launch_bounds__(128) j_thread_kernel(JArgs a) {
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t span = 32 * thread_tile(a.wl, total - first, nwarps), ntiles = (total - first + span - 1) / span;
   unsigned long long done = 0, doneq = 0, doneb = 0;
-  const PrimSplit sp = prim_split<T>(a.wl, total - first, 32 * nwarps);
+  const PrimSplit sp = prim_split<T>(a.wl, total - first, 32 * nwarps, SplitBy::parts);
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   for (int64_t turn = 0; turn * nwarps * nshard < ntiles * sp.n; ++turn) {
     const int64_t tl = warp_tile(turn, warp, nwarps) * nshard + shard;
@@ -517,7 +570,7 @@ __global__ void __launch_bounds__(128) j_thread_kernel(JArgs a) {
       const bool uni = __all_sync(0xffffffffu, !ok || pb_id == pair0) && !a.det;
       if (uni) npb = __shfl_sync(0xffffffffu, npb, 0);
       int pb0, pb1, pk0, pk1;
-      sp.range(part, npb, npk, pb0, pb1, pk0, pk1);
+      sp.range(part, 0, npb, npk, pb0, pb1, pk0, pk1);
       for (int pb = pb0; pb < pb1; ++pb) {
         T acc[HAB];
 #pragma unroll
@@ -565,7 +618,7 @@ __global__ void __launch_bounds__(128) j_thread_kernel(JArgs a) {
             for (int x = 0; x < HAB; ++x) acc_add(a.Jherm + hb + (size_t)pb * HAB + x, (double)acc[x], a.det);
         } else if (ok) {
 #pragma unroll
-          for (int x = 0; x < HAB; ++x) acc_add(a.Jherm + hb + (size_t)pb * HAB + x, (double)acc[x], a.det);
+            for (int x = 0; x < HAB; ++x) acc_add(a.Jherm + hb + (size_t)pb * HAB + x, (double)acc[x], a.det);
         }
       }
     }

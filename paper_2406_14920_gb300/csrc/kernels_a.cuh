@@ -291,11 +291,12 @@ __device__ __forceinline__ void contract_block(const JKArgs& A, const T* X, T w,
   }
 }
 
-// One quartet (bra position ib, ket position ik of the work list) of a thread-kernel class.
-template <int LA, int LB, int LC, int LD, typename T>
+// One quartet (bra position ib, ket position ik of the work list) of a thread-kernel
+// class: part `part` of it, by this lane or (SHORT) by its group of lanes.
+template <int LA, int LB, int LC, int LD, typename T, bool SHORT>
 __device__ __forceinline__ void thread_item(const JKArgs& A, int ib, int ik, int64_t nket, const PrimSplit& sp, int part,
-                                            unsigned long long& done, unsigned long long& doneq,
-                                            unsigned long long& doneb) {
+                                            int sub, unsigned lanes, unsigned long long& done,
+                                            unsigned long long& doneq, unsigned long long& doneb) {
   using S = AShape<LA, LB, LC, LD>;
   const KArgs& a = A.k;
   const int pb_id = __ldg(a.wl.bra + ib);
@@ -305,14 +306,14 @@ __device__ __forceinline__ void thread_item(const JKArgs& A, int ib, int ik, int
   const int s1 = __ldg(a.sp.s1 + pb_id), s2 = __ldg(a.sp.s2 + pb_id);
   const int s3 = __ldg(a.sp.s1 + pk_id), s4 = __ldg(a.sp.s2 + pk_id);
   const int npb_ = __ldg(a.sp.np + pb_id), npk_ = __ldg(a.sp.np + pk_id);
-  if (part == 0) {
+  if (part == 0 && sub == 0) {
     ++done;
     doneq += (unsigned long long)npb_ * npk_;
     doneb += npb_;
   }
   int pb0, pb1, pk0, pk1;
-  sp.range(part, npb_, npk_, pb0, pb1, pk0, pk1);
-  if (pb0 >= pb1 || pk0 >= pk1) return;
+  sp.range(part, sub, npb_, npk_, pb0, pb1, pk0, pk1);
+  if (!SHORT && (pb0 >= pb1 || pk0 >= pk1)) return;
   T w = T(1);
   if (s1 == s2) w *= T(0.5);
   if (s3 == s4) w *= T(0.5);
@@ -324,13 +325,18 @@ __device__ __forceinline__ void thread_item(const JKArgs& A, int ib, int ik, int
   else
     eri_block_reg_pq<LA, LB, LC, LD, T>(a, __ldg(a.sp.poff + pb_id), pb0, pb1, __ldg(a.sp.eoff + pb_id),
                                         __ldg(a.sp.poff + pk_id), pk0, pk1, __ldg(a.sp.eoff + pk_id), X);
+  if constexpr (SHORT) {
+    group_sum<S::NAB * S::NCD>(X, sp.g, sub, lanes);
+    if (sub != 0) return;
+  }
   const int ao1 = __ldg(a.sp.ao1 + pb_id), ao2 = __ldg(a.sp.ao2 + pb_id);
   const int64_t base = __ldg(a.sp.mat_off + mol);
   const int n = __ldg(a.sp.mat_n + mol);
   contract_block<LA, LB, LC, LD, T>(A, X, w, ao1, ao2, __ldg(a.sp.ao1 + pk_id), __ldg(a.sp.ao2 + pk_id), base, n);
 }
 
-template <int LA, int LB, int LC, int LD, typename T>
+// SHORT: the form for short lists, a group of lanes per item (see prim_split)
+template <int LA, int LB, int LC, int LD, typename T, bool SHORT>
 __global__ void __launch_bounds__(128) jk_thread_kernel(JKArgs A) {
   const KArgs& a = A.k;
   // items: positions in the work list, or (mixed precision) this tier's compacted list
@@ -341,9 +347,12 @@ __global__ void __launch_bounds__(128) jk_thread_kernel(JKArgs A) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   unsigned long long done = 0, doneq = 0, doneb = 0;
   // a warp shares a tile of 32 * tile consecutive items, lane l takes items l, l + 32, ...
-  const int64_t span = 32 * (int64_t)a.wl.tile, ntiles = (total - first + span - 1) / span;
+  // (SHORT: of 32 / g items, each with g lanes)
   const int lane = threadIdx.x & 31;
-  const PrimSplit sp = prim_split<T>(a.wl, total - first, stride);
+  const PrimSplit sp = prim_split<T>(a.wl, total - first, stride, SHORT ? SplitBy::lanes : SplitBy::parts);
+  const int per = SHORT ? 32 / sp.g : 32, li = SHORT ? lane / sp.g : lane, sub = SHORT ? lane % sp.g : 0;
+  const unsigned lanes = SHORT ? group_lanes(sp.g, li) : 0u;
+  const int64_t span = SHORT ? per : 32 * (int64_t)a.wl.tile, ntiles = (total - first + span - 1) / span;
   const int64_t nwarps = stride >> 5, warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   for (int64_t turn = 0; turn * nwarps * nshard < ntiles * sp.n; ++turn) {
     const int64_t tl = warp_tile(turn, warp, nwarps) * nshard + shard;
@@ -351,18 +360,18 @@ __global__ void __launch_bounds__(128) jk_thread_kernel(JKArgs A) {
     const int part = (int)(tl / ntiles);
     const int64_t t0 = first + (tl - part * ntiles) * span;
     const int64_t i1 = t0 + span < total ? t0 + span : total;
-    const int64_t i0 = t0 + lane;
+    const int64_t i0 = t0 + li;
     if (i0 >= i1) continue;
     if (compact) {
-      for (int64_t item = i0; item < i1; item += 32) {
+      for (int64_t item = i0; item < i1; item += per) {
         const int2 v = __ldg(a.items + item);
-        thread_item<LA, LB, LC, LD, T>(A, v.x, v.y, 0, sp, part, done, doneq, doneb);
+        thread_item<LA, LB, LC, LD, T, SHORT>(A, v.x, v.y, 0, sp, part, sub, lanes, done, doneq, doneb);
       }
     } else {
       BraCursor cur(a.wl, i0);
-      for (int64_t item = i0; item < i1; item += 32) {
+      for (int64_t item = i0; item < i1; item += per) {
         const int ik = cur.at(a.wl, item);
-        thread_item<LA, LB, LC, LD, T>(A, cur.ib, ik, cur.be - cur.bs, sp, part, done, doneq, doneb);
+        thread_item<LA, LB, LC, LD, T, SHORT>(A, cur.ib, ik, cur.be - cur.bs, sp, part, sub, lanes, done, doneq, doneb);
       }
     }
   }

@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
   const int nshard = compact ? 1 : a.wl.nshard, shard = compact ? 0 : a.wl.shard;
   unsigned long long done = 0, doneq = 0, doneb = 0;
   const int64_t tile = item_tile(a.wl, total - first, gridDim.x), ntiles = (total - first + tile - 1) / tile;
-  const PrimSplit sp = prim_split<T>(a.wl, total - first, gridDim.x, false);
+  const PrimSplit sp = prim_split<T>(a.wl, total - first, gridDim.x, SplitBy::blocks);
   for (int64_t tl = (int64_t)blockIdx.x * nshard + shard; tl < ntiles * sp.n; tl += (int64_t)gridDim.x * nshard) {
     const int part = (int)(tl / ntiles);
     const int64_t t0 = first + (tl - part * ntiles) * tile, t1 = t0 + tile < total ? t0 + tile : total;
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(CShape<LA, LB, LC, LD, T>::NT) jk_block_kernel
         doneb += npb;
       }
       int pb0, pb1, pk0, pk1;
-      sp.range(part, npb, npk, pb0, pb1, pk0, pk1);
+      sp.range(part, 0, npb, npk, pb0, pb1, pk0, pk1);
       if (pb0 >= pb1 || npk == 0) continue;  // uniform over the block; W has no value without a ket primitive
       __syncthreads();  // the previous item's shared memory (first item: the tables) is done with
       const T* Dp = dens<T>(a) + mbase;

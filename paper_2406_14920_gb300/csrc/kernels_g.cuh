@@ -65,6 +65,13 @@ template <typename T> __device__ __forceinline__ const T* gdens(const GradArgs& 
 template <> __device__ __forceinline__ const double* gdens<double>(const GradArgs& a) { return a.Dp; }
 template <> __device__ __forceinline__ const float* gdens<float>(const GradArgs& a) { return a.Dpf; }
 
+// dE/dA and dE/dB of direction d.  Of two shells on one atom the sum: the parts that
+// move the shells against each other cancel in it and not in the gradient's rounding.
+__device__ __forceinline__ void add_pair(const GradArgs& a, int d, int atA, int atB, double x, double y) {
+  acc_add(a.grad + 3 * atA + d, atA == atB ? x + y : x, a.det);
+  if (atA != atB) acc_add(a.grad + 3 * atB + d, y, a.det);
+}
+
 // ---------------------------------------------------------------------------
 // one item per thread
 // ---------------------------------------------------------------------------
@@ -239,7 +246,8 @@ __device__ __forceinline__ void grad_item(const GradArgs& a, int pb_id, int pk_i
   }
 }
 
-template <int LA, int LB, int LC, int LD, typename T>
+// SHORT: the form for short lists, a group of lanes per item (see prim_split)
+template <int LA, int LB, int LC, int LD, typename T, bool SHORT>
 __global__ void __launch_bounds__(128) grad_thread_kernel(GradArgs a) {
   const bool compact = a.items != nullptr;
   const int64_t total = compact ? (int64_t)__ldg(a.nitems) : a.wl.total;
@@ -247,8 +255,12 @@ __global__ void __launch_bounds__(128) grad_thread_kernel(GradArgs a) {
   const int nshard = compact ? 1 : a.wl.nshard, shard = compact ? 0 : a.wl.shard;
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const PrimSplit sp = prim_split<T>(a.wl, total - first, 32 * nwarps);
-  const int64_t span = 32 * thread_tile(a.wl, total - first, nwarps), ntiles = (total - first + span - 1) / span;
+  const PrimSplit sp = prim_split<T>(a.wl, total - first, 32 * nwarps, SHORT ? SplitBy::lanes : SplitBy::parts);
+  // items a warp takes at a time; this lane's of them, and its place in the item's group
+  const int per = SHORT ? 32 / sp.g : 32, li = SHORT ? lane / sp.g : lane, sub = SHORT ? lane % sp.g : 0;
+  const unsigned lanes = SHORT ? group_lanes(sp.g, li) : 0u;
+  const int64_t span = SHORT ? per : 32 * thread_tile(a.wl, total - first, nwarps),
+                ntiles = (total - first + span - 1) / span;
   unsigned long long done = 0, doneq = 0, doneb = 0;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   for (int64_t turn = 0; turn * nwarps * nshard < ntiles * sp.n; ++turn) {
@@ -257,9 +269,9 @@ __global__ void __launch_bounds__(128) grad_thread_kernel(GradArgs a) {
     const int part = (int)(tl / ntiles);
     const int64_t t0 = first + (tl - part * ntiles) * span, i1 = t0 + span < total ? t0 + span : total;
     BraCursor cur;
-    if (!compact) cur.seek(a.wl, t0 + lane < i1 ? t0 + lane : t0);
-    for (int64_t base = t0; base < i1; base += 32) {  // uniform over the warp
-      const int64_t item = base + lane;
+    if (!compact) cur.seek(a.wl, t0 + li < i1 ? t0 + li : t0);
+    for (int64_t base = t0; base < i1; base += per) {  // uniform over the warp
+      const int64_t item = base + li;
       const bool ok = item < i1;
       T gA[3] = {T(0), T(0), T(0)}, gB[3] = {T(0), T(0), T(0)};
       int atA = -1, atB = -1;
@@ -278,7 +290,7 @@ __global__ void __launch_bounds__(128) grad_thread_kernel(GradArgs a) {
         if (!compact) ik = ket_pos(a.wl, seg, ik, cur.be - cur.bs);
         const int pk_id = __ldg(a.wl.ket + seg + ik);
         const int npb = __ldg(a.sp.np + pb_id), npk = __ldg(a.sp.np + pk_id);
-        if (part == 0) {
+        if (part == 0 && sub == 0) {
           ++done;
           doneq += (unsigned long long)npb * npk;
           doneb += npb;
@@ -286,9 +298,17 @@ __global__ void __launch_bounds__(128) grad_thread_kernel(GradArgs a) {
         atA = __ldg(a.sh_atom + __ldg(a.sp.s1 + pb_id));
         atB = __ldg(a.sh_atom + __ldg(a.sp.s2 + pb_id));
         int pb0, pb1, pk0, pk1;
-        sp.range(part, npb, npk, pb0, pb1, pk0, pk1);
+        sp.range(part, sub, npb, npk, pb0, pb1, pk0, pk1);
         if (pb0 < pb1 && pk0 < pk1) grad_item<LA, LB, LC, LD, T>(a, pb_id, pk_id, mol, pb0, pb1, pk0, pk1, gA, gB);
       }
+      if constexpr (SHORT)
+        if (ok) {  // the item's sums, in the first lane of its group
+          group_sum<3>(gA, sp.g, sub, lanes);
+          group_sum<3>(gB, sp.g, sub, lanes);
+          if (sub != 0)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) gA[d] = gB[d] = T(0);
+        }
       // the lists are bra-major: a warp's items usually share the two atoms, and
       // their sums go out as one atomic each (deterministic builds keep one
       // fixed-point add per item, whose sum does not depend on the grouping)
@@ -303,16 +323,13 @@ __global__ void __launch_bounds__(128) grad_thread_kernel(GradArgs a) {
             y += __shfl_xor_sync(0xffffffffu, y, o);
           }
           if (lane == 0) {
-            atomicAdd(a.grad + 3 * a0 + d, x);
-            atomicAdd(a.grad + 3 * b0 + d, y);
+            atomicAdd(a.grad + 3 * a0 + d, a0 == b0 ? x + y : x);  // (see add_pair)
+            if (a0 != b0) atomicAdd(a.grad + 3 * b0 + d, y);
           }
         }
-      } else if (ok) {
+      } else if (ok && sub == 0) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          acc_add(a.grad + 3 * atA + d, (double)gA[d], a.det);
-          acc_add(a.grad + 3 * atB + d, (double)gB[d], a.det);
-        }
+        for (int d = 0; d < 3; ++d) add_pair(a, d, atA, atB, (double)gA[d], (double)gB[d]);
       }
     }
   }
@@ -439,15 +456,18 @@ __global__ void __launch_bounds__(GShape<LA, LB, LC, LD, T>::NT) grad_block_kern
       if (lane == 0) red[d * 8 + wp] = v;
     }
     __syncthreads();
-    if (tid < 6) {
-      double v = 0.0;
-      for (int x = 0; x < NT / 32; ++x) v += (double)red[tid * 8 + x];
-      acc_add(a.grad + 3 * (tid < 3 ? atA : atB) + tid % 3, v, a.det);
+    if (tid < 3) {
+      double v = 0.0, u = 0.0;
+      for (int x = 0; x < NT / 32; ++x) {
+        v += (double)red[tid * 8 + x];
+        u += (double)red[(tid + 3) * 8 + x];
+      }
+      add_pair(a, tid, atA, atB, v, u);
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) gA[d] = gB[d] = T(0);
   };
-  const PrimSplit sp = prim_split<T>(a.wl, total - first, gridDim.x, false);
+  const PrimSplit sp = prim_split<T>(a.wl, total - first, gridDim.x, SplitBy::blocks);
   for (int64_t tl = (int64_t)blockIdx.x * nshard + shard; tl < ntiles * sp.n; tl += (int64_t)gridDim.x * nshard) {
     const int part = (int)(tl / ntiles);
     const int64_t t0 = first + (tl - part * ntiles) * tile, t1 = t0 + tile < total ? t0 + tile : total;
@@ -477,7 +497,7 @@ __global__ void __launch_bounds__(GShape<LA, LB, LC, LD, T>::NT) grad_block_kern
         doneb += npb;
       }
       int pb0, pb1, pk0, pk1;
-      sp.range(part, npb, npk, pb0, pb1, pk0, pk1);
+      sp.range(part, 0, npb, npk, pb0, pb1, pk0, pk1);
       if (pb0 >= pb1 || npk == 0) continue;  // uniform over the block; W has no value without a ket primitive
       // items of a tile usually share the bra atoms: their sums go out together
       // (FP32 sums and deterministic builds: once per item)

@@ -13,7 +13,9 @@
 - an FP64 build captured by the caller over grown lists, replayed after other
   builds of the plan;
 - tier lists taken once: mixed builds over shorter lists, or after a graph build,
-  allocate nothing more and can be captured.
+  allocate nothing more and can be captured;
+- short lists whose items are split over lanes: an item is added a few times at
+  most, as the rounding of fixed-point sums shows, and every primitive once.
 
 Tolerances: 1e-10 (J, K) and 1e-9 (gradients), the parity tolerances of the
 library.  Mixed precision with a tier bound of 1e-7: an FP32 quartet is at most
@@ -217,3 +219,24 @@ def test_mixed_build_captured_after_a_graph_build(eri):
     _captured(lambda: plan.build_jk(Dt, J2, K2)).replay()
     torch.cuda.synchronize()
     assert float((J - J2).abs().max()) < 1e-10 and float((K - K2).abs().max()) < 1e-10
+
+
+# A deterministic build rounds every addition to 2^-46, so its error shows how often
+# an item is added.  A plan that takes a share of the work keeps whole items: two
+# shares together are the reference.  A split item is added once per group of lanes
+# (three of them cover 81 primitive quartets) or per bra primitive in the block
+# kernels, nine times at most: at most three times the rms error, and four with the
+# scatter of small matrices (81 additions: nine times).
+@pytest.mark.parametrize("comp", [["2s1p", "2s1p"], ["2s1p", "1s"], ["1s1p", "1s1p"], ["1s1p1d", "1s1p"]])
+def test_split_items_are_added_a_few_times_at_most(eri, comp):
+    b, D = W.small_system(comp, seed=17)
+    plan = eri.Plan(b, thresh=0.0, deterministic=True)
+    split = [x.cpu().numpy() for x in plan.build_jk(_t(D))]
+    whole = 0.0
+    for shard in range(2):
+        plan.set_shard(shard, 2)
+        whole = whole + np.array([x.cpu().numpy() for x in plan.build_jk(_t(D))])
+    ref = np.array(oracle.Oracle(b).jk(D, 0.0))
+    assert np.abs(split - ref).max() < 1e-10
+    rms = [np.sqrt(((x - ref) ** 2).mean()) for x in (split, whole)]
+    assert rms[0] < 4.0 * rms[1]
