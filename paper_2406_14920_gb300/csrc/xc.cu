@@ -54,8 +54,9 @@ constexpr int kVC = 128;          // k_xc_vmat: functions of Phi_b staged at a t
 // V is summed in up to kParts half matrices, 2^kPartShift consecutive blocks to
 // one (two or three are in L2 at a time), and these are added at the end: one sum
 // over the thousands of blocks of an element loses sqrt(blocks) roundings (60
-// atoms: 5.7e-15 of V against 1.6e-15).  The first part is V itself; the others
-// take at most kPartBytes (from 11,585 functions on there are none).
+// atoms: 5.7e-15 of V against 1.6e-15).  They take at most kPartBytes: where that is
+// too little for all of them (from 2,900 functions on), V itself is the first and the
+// others are as many as fit (none from 11,586 functions on).
 constexpr int kParts = 16, kPartShift = 8;
 constexpr size_t kPartBytes = size_t(1) << 30;
 constexpr int kSlots = 5;         // workspace rows per function: phi, d/dx, d/dy, d/dz, Z
@@ -697,7 +698,7 @@ struct VmatSmem {
 __global__ void __launch_bounds__(32 * kVWarps, 2)
     k_xc_vmat(int b0, int nbf, const int* __restrict__ nbfb, const int* __restrict__ bfl,
               const int64_t* __restrict__ woff, const double* __restrict__ work, const int* __restrict__ bad, int parts,
-              double* __restrict__ V, double* __restrict__ Vparts) {
+              double* V, double* Vparts) {
   extern __shared__ __align__(16) unsigned char smraw[];
   VmatSmem& S = *reinterpret_cast<VmatSmem*>(smraw);
   const int b = b0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
@@ -706,7 +707,8 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
   const double* phi = work + woff[b];
   const double* Z = phi + (int64_t)4 * n * kBP;
   const int part = (b >> kPartShift) % parts;
-  double* Vh = part == 0 ? V : Vparts + (int64_t)(part - 1) * nbf * nbf;
+  double* Vh = Vparts + (int64_t)part * nbf * nbf;
+  if (V) Vh = part == 0 ? V : Vh - (int64_t)nbf * nbf;  // V is the first part
   if (bad[b]) {  // an infinity or NaN: plain sums
     for (int64_t o = tid; o < (int64_t)n * n; o += 32 * kVWarps) {
       const int i = (int)(o / n), j = (int)(o - (int64_t)i * n);
@@ -788,13 +790,14 @@ __global__ void __launch_bounds__(32 * kVWarps, 2)
   }
 }
 
-// V = Vh + Vh^T, Vh = sum of the parts (the first is V: its elements (i, j) and
-// (j, i) are read and written by one thread)
-__global__ void k_xc_symm(int nbf, int parts, const double* __restrict__ Vparts, double* __restrict__ V) {
+// V = Vh + Vh^T, Vh = sum of the parts: those of Vparts and (IN_V) V itself, whose
+// elements (i, j) and (j, i) are read and written by one thread
+template <bool IN_V>
+__global__ void k_xc_symm(int nbf, int parts, const double* __restrict__ Vparts, double* V) {
   const int i = blockIdx.x;
   for (int j = threadIdx.x; j <= i; j += blockDim.x) {
-    double v = V[(int64_t)i * nbf + j] + V[(int64_t)j * nbf + i];
-    for (int p = 0; p + 1 < parts; ++p) {
+    double v = IN_V ? V[(int64_t)i * nbf + j] + V[(int64_t)j * nbf + i] : 0.0;
+    for (int p = 0; p < parts - IN_V; ++p) {
       const double* Vh = Vparts + (int64_t)p * nbf * nbf;
       v += Vh[(int64_t)i * nbf + j] + Vh[(int64_t)j * nbf + i];
     }
@@ -870,8 +873,10 @@ static int xc_build(eri_plan_impl* P, cudaStream_t s) {
   XCK(xalloc(&X.d_dexp, (size_t)nbf));
   XCK(xalloc(&X.d_zbad, (size_t)nb));
   const size_t nn8 = sizeof(double) * (size_t)nbf * nbf;
-  X.parts = (int)std::min<size_t>({(size_t)kParts, 1 + kPartBytes / nn8, (size_t)(nb >> kPartShift) + 1});
-  XCK(xalloc(&X.d_vpart, (size_t)(X.parts - 1) * nbf * nbf));
+  X.parts = (int)std::min<size_t>(kParts, (size_t)(nb >> kPartShift) + 1);
+  X.in_v = (size_t)X.parts * nn8 > kPartBytes;
+  if (X.in_v) X.parts = (int)std::min<size_t>(X.parts, 1 + kPartBytes / nn8);
+  XCK(xalloc(&X.d_vpart, (size_t)(X.parts - X.in_v) * nbf * nbf));
   XCK(cudaMemcpyAsync(X.d_perm, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice, s));
   const int nt = std::max(nrad, nth);
   k_xc_nodes<<<(nt + 127) / 128, 128, 0, s>>>(nrad, nth, X.radius, X.d_rad, X.d_ang);
@@ -978,8 +983,10 @@ static int xc_density_impl(eri_plan_impl* P, const double* D, double* rho, doubl
 static int xc_matrix_impl(eri_plan_impl* P, const double* vrho, const double* vgrad, double* V, cudaStream_t s) {
   XcState& X = P->xc;
   const int nbf = P->nbf;
-  XCK(cudaMemsetAsync(V, 0, sizeof(double) * (size_t)nbf * nbf, s));
-  if (X.parts > 1) XCK(cudaMemsetAsync(X.d_vpart, 0, sizeof(double) * (size_t)(X.parts - 1) * nbf * nbf, s));
+  double* first = X.in_v ? V : nullptr;
+  if (first) XCK(cudaMemsetAsync(V, 0, sizeof(double) * (size_t)nbf * nbf, s));
+  if (X.parts > X.in_v)
+    XCK(cudaMemsetAsync(X.d_vpart, 0, sizeof(double) * (size_t)(X.parts - X.in_v) * nbf * nbf, s));
   XCK(cudaFuncSetAttribute(k_xc_vmat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(VmatSmem)));
   for (size_t c = 0; c + 1 < X.chunk.size(); ++c) {
     const int b0 = X.chunk[c], b1 = X.chunk[c + 1];
@@ -987,10 +994,11 @@ static int xc_matrix_impl(eri_plan_impl* P, const double* vrho, const double* vg
     if (!X.resident) xc_launch_ao(P, b0, b1, s);
     k_xc_z<<<b1 - b0, kBP, 0, s>>>(b0, X.d_perm, X.d_nbfb, X.d_woff, X.d_w, vrho, vgrad, X.d_work, X.d_zbad);
     k_xc_vmat<<<b1 - b0, 32 * kVWarps, sizeof(VmatSmem), s>>>(b0, nbf, X.d_nbfb, X.d_bfl, X.d_woff, X.d_work, X.d_zbad,
-                                                             X.parts, V, X.d_vpart);
+                                                             X.parts, first, X.d_vpart);
     XCK(cudaGetLastError());
   }
-  k_xc_symm<<<nbf, 128, 0, s>>>(nbf, X.parts, X.d_vpart, V);
+  if (first) k_xc_symm<true><<<nbf, 128, 0, s>>>(nbf, X.parts, X.d_vpart, V);
+  else k_xc_symm<false><<<nbf, 128, 0, s>>>(nbf, X.parts, X.d_vpart, V);
   XCK(cudaGetLastError());
   return ERI_OK;
 }

@@ -29,7 +29,8 @@ struct XcState {
   int* d_pexp = nullptr;      // largest exponent of phi per block slot (xc_mma.cuh)
   uint4* d_ddig = nullptr;    // digits of D and its row exponents (written by each call)
   int *d_dexp = nullptr, *d_zbad = nullptr;  // d_zbad: blocks with an infinity or NaN in Z
-  int parts = 1;              // half matrices V is summed in: V itself and parts - 1 more
+  int parts = 1;              // half matrices V is summed in
+  int in_v = 0;               // 1: V itself is the first of them, d_vpart holds the others
   double* d_vpart = nullptr;
   double *d_rho = nullptr, *d_grad = nullptr, *d_vrho = nullptr, *d_vgrad = nullptr;
   double sum_nb = 0.0, sum_nb2 = 0.0;  // sum over blocks of n_b and n_b^2 (significant functions)
