@@ -175,8 +175,8 @@ def oracle_rate(basis, quartets, target_s):
 
 # sources of the J/K class kernels and their launches: the DRAM traffic figures
 # of profiles/ hold only while these are unchanged
-JK_SOURCES = ["common.cuh", "kernels.cuh", "kernels_a.cuh", "kernels_b.cuh", "dispatch.cuh", "units.h",
-              "k_unit.cu", "plan.cu", "plan.cuh"]
+JK_SOURCES = ["common.cuh", "kernels.cuh", "kernels_a.cuh", "kernels_b.cuh", "kernels_c.cuh", "dispatch.cuh",
+              "fork.cuh", "units.h", "k_unit.cu", "plan.cu", "plan.cuh"]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "jk_dram_traffic_w1.md")
 
 

@@ -9,7 +9,13 @@
  *   point charges        Sec. 2.4, Eq. v1e_definition, Eq. v1e_formula; SI Sec. 1.3
  *   J and K              Eq. j_definition (J_mn = sum_ls (mn|ls) D_ls),
  *                        Eq. k_definition (K_ml = sum_ns (mn|ls) D_ns)
- *   screening            Eq. cauchy_schwarz_bound, Eq. kernel_upperbound
+ *   screening            Eq. cauchy_schwarz_bound, Eq. kernel_upperbound; inside a listed
+ *                        pair, primitive pairs whose every quartet is bounded below 1e-8
+ *                        of the quartet threshold are not run (builds and gradients; a
+ *                        threshold of 0 runs all).  The bound is on the integral: a
+ *                        derivative may be larger by about sqrt((2 l + 1) p) + 2 (ab/p) |AB|
+ *                        (l: angular momentum of the pair, p = a + b its exponents), some
+ *                        1e2 to 1e3 for the tightest pairs
  *   energies, gradient   SI Eq. si_E_J_K, SI Eq. si_dE_J, SI Eq. si_dE_K
  *
  * Conventions (all calls):
@@ -152,7 +158,8 @@ int eri_plan_layout(eri_plan_t* plan, int32_t* nmol, int64_t* mat_off, int32_t* 
  * data, Schwarz bounds and lists are rebuilt on `stream`, then the call waits
  * for the new list sizes (a device->host copy).  Use for finite differences
  * and for autograd.  If freeze_lists != 0 the lists and Q of the previous
- * geometry are kept (so energies are smooth functions of the coordinates).
+ * geometry are kept (so energies are smooth functions of the coordinates; which
+ * primitive pairs of a listed pair are run is decided anew, at least one is).
  */
 int eri_plan_set_coords(eri_plan_t* plan, const double* coords_dev, int32_t freeze_lists, void* stream);
 
@@ -407,7 +414,14 @@ int eri_nuclear_grad(eri_plan_t* plan, const double* D, int32_t ncharge, const d
 /*
  * Exchange-correlation quadrature on a molecular grid (Sec. 2.6; the paper's
  * four steps: grid, density, functional, matrix).  Plans of one molecule only
- * (a batched plan gets ERI_EUNSUPPORTED).  All arithmetic is FP64.
+ * (a batched plan gets ERI_EUNSUPPORTED).  All arithmetic is FP64, but for the two
+ * products with the basis values (D phi in the density, Z phi^T in the matrix, Z = the
+ * weighted potentials times phi and its gradient): these are exact sums of operands
+ * rounded to 2^-56 of the largest value of their row of D, of their point's phi, or of
+ * their function's 32 values in a block.  Their error is bounded as that of an FP64
+ * sum in the norm (absolutely, by the largest products of a block), not for each
+ * element by itself: elements of V many orders of magnitude below the others keep
+ * fewer correct digits, and operands below 2^-1022 count as zero.
  *
  * eri_xc_grid builds the plan's grid on the device (step 1): for every atom,
  * nrad radial nodes (Gauss-Chebyshev of the second kind, x_i = cos(i pi /

@@ -408,7 +408,10 @@ __global__ void __launch_bounds__(32 * kSchwarzWarps)
 // k_primpack moves the primitive pairs with q qmax >= kPrimEps thresh to the
 // front of their shell pair and counts them; the J/K, J-engine and gradient
 // kernels run over those (a pair keeps at least one).  Each dropped primitive
-// quartet is below 1e-8 of the quartet threshold (thresh = 0 drops none).
+// quartet is below 1e-8 of the quartet threshold (thresh = 0 drops none).  That
+// bounds the integral; the gradient's derivatives raise a Hermite index or bring
+// down an exponent, up to about sqrt((2l + 1) p) + 2 (ab/p) |AB| times it, 1e2 to 1e3
+// for the tightest pairs, which leaves 1e-5 of the threshold and less.
 constexpr double kPrimEps = 1e-8;
 __global__ void __launch_bounds__(128)
     k_primq(int npair, const int* __restrict__ s1, const int* __restrict__ s2, const int* __restrict__ np,

@@ -1,17 +1,27 @@
 // FP64 products on the tensor cores for the exchange-correlation contractions.
 //
-// What bounds them otherwise: GB300's FP64 pipe, 1.06 TFLOP/s, against 0.6
-// PFLOP/s of mma.sync f16 (both measured).  A row of operands is written as
-// integers q = rint(v 2^(55 - e)) under the row's common power of two 2^e >
-// max |v|, and q as 8 signed digits of 7 bits, |digit| <= 64, which f16 holds
+// What bounds them otherwise: GB300's FP64 pipe, 1.06 TFLOP/s (eri_peak_probe), against
+// 0.6 PFLOP/s of mma.sync f16 (independent m16n8k16 products on every SM, timed
+// apart from the library).  The products are taken by slices, as in Ozaki's scheme
+// (Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012): a row of operands is
+// written as integers q = rint(v 2^(55 - e)) under the row's common power of two
+// 2^e > max |v|, and q as 8 signed digits of 7 bits, |digit| <= 64, which f16 holds
 // exactly.  A product of two digits is at most 2^12, so the FP32 accumulator of
 // the tensor core holds the sum of the up to 8 digit products of one weight
 // (i + j = k) over 512 terms exactly (8 x 512 x 2^12 = 2^24): no rounding
 // happens before the nine sums of weights k = 0..8 are put together, in
-// integers and rounded once.  43 f16 products replace one FP64 product; the
-// pairs left out (k > 8) are below 2^-63 of 2^(e_a + e_b) per term, and the
-// digits represent an operand to 2^-56 of its row's maximum, where a plain FP64
-// sum rounds every step to 2^-53 of its partial sum.
+// integers and rounded once.  43 f16 products replace one FP64 product.
+// Accuracy: the digits represent an operand to 2^-56 of its row's maximum, and the
+// pairs left out (k > 8, six of weight 9) are together below 2^-60 of 2^(e_a + e_b)
+// per term.  That is an absolute bound, about 2^-54 max|a| max|b| per term over the
+// rows (of D, of one point's phi, of one function's 32 values of Z or phi): in the
+// norm no more than the roundings of a plain FP64 sum (measured rms error of V 9e-16
+// to 1.4e-15 with either), but not element by element.  An operand 2^-k of its row's
+// maximum keeps 55 - k bits, so a sum that is small because each operand is small
+// where the other is large has fewer correct digits than a plain sum would give it:
+// of two Gaussians that both peak inside the block, 4 bohr apart (3.8e-6 beside
+// products of 1) it is right to 5e-12 of itself, 6 bohr apart (1e-14) to 1e-3; over
+// points near one of them only, to 1e-17 at any distance.
 // mma.sync rather than tcgen05: nine accumulators of 128 x N FP32 fill the 512
 // columns of TMEM at N = 56, and at such N a tcgen05.mma is bound by reading A
 // from shared memory; the register form also takes its A operand as it is
@@ -71,8 +81,8 @@ __device__ __forceinline__ void mma_f16(float* c, const uint32_t* a, const uint2
 }
 
 // Accumulators of products with at most kShortTerms terms may start at kMagic =
-// 1.5 2^23: a sum below 2^22 is then the low bits of the FP32 word, which saves
-// the conversions.
+// 1.5 2^23: a sum of at most 2^22 is then the difference of the FP32 words, which
+// saves the conversions.
 constexpr int kShortTerms = 128;
 constexpr float kMagic = 12582912.0f;
 constexpr int kMagicBits = 0x4b400000;
@@ -109,7 +119,7 @@ __device__ __forceinline__ double combine(const float (&acc)[kWeights][4], int c
   return __longlong_as_double((long long)r);
 }
 
-// The same value (accumulators started at kMagic, sums below 2^20) with three FP64
+// The same value (accumulators started at kMagic, sums of at most 2^20) with three FP64
 // operations: hi and lo become doubles as the low bits of 1.5 2^52, the sum is
 // rounded once, and the exponents are added to the word.
 __device__ __forceinline__ double combine_fp64(const float (&acc)[kWeights][4], int c, int Ea, int Eb) {
