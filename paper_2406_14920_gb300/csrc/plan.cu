@@ -1189,14 +1189,17 @@ int64_t eri_plan_impl::tier_len() const {
 
 int eri_plan_impl::ensure_tier_bufs(int need) {
   const int64_t cap = tier_len();
-  if (cap > tier_cap) {
+  if (tier_nb == 0) {
+    tier_cap = cap;
+  } else if (cap > tier_cap) {
     CK(cudaDeviceSynchronize());
     for (int b = 0; b < kStreams; ++b) {
       if (tbuf[b]) cudaFree(tbuf[b]);
       tbuf[b] = nullptr;
     }
     tier_nb = 0;
-    tier_cap = cap;
+    // (lists that grow once, atoms moving closer, grow again: an eighth to spare)
+    tier_cap = std::min(kTierCap, cap + cap / 8);
   }
   if (!tcnt) CK(dalloc(&tcnt, 2 * kStreams));
   const int want = tier_nb == 0 ? std::max(need, eager_branches(true)) : need;
